@@ -1,0 +1,13 @@
+// FP64 forward on the tensor cores (lr_fx64.cu): eligibility, tables and launch.
+#pragma once
+#include "lr_internal.h"
+
+namespace lr {
+// largest tile (outputs per block) that the tensor-core kernels take for this plan's halos, bounds and
+// order; 0 when they do not apply
+int fx_max_tile(const FwdParams &P, int order);
+// expansion nodes and transforms of the launch parameters
+void fx_tables(FwdParams &P);
+// returns a cudaError_t value; P.tile + P.HL + P.HR (P.tile for KIND_PROJECT) is at most FX_ROWS
+int launch_fx64(int kind, int order, const FwdParams &P, int sms, void *stream);
+}  // namespace lr

@@ -11,6 +11,7 @@
 
 #include "lr_internal.h"
 #include "lr_bwd.h"
+#include "lr_fx64.h"
 #include "lr_launch.h"
 #include "lr_pipeline.h"
 #include "lr_planview.h"
@@ -40,6 +41,7 @@ struct lr_plan {
     lr_plan_desc desc;
     lr::FwdParams base;
     int T, h;
+    int tile;  // outputs per tile as the caller sees it (a multiple of base.tile)
     int threads;
     int *d_err;
     int64_t *d_tile_off;
@@ -307,6 +309,23 @@ int constant_delay_table(lr_plan *p, const lr_orbit *o)
     }
     P.cd_w = p->d_cdw;
     return LR_OK;
+}
+
+// FP64 plans whose stencils fit run on the tensor-core kernels (lr_fx64.cu).  Their blocks hold at most
+// fx_max_tile outputs; a larger tile is worked in equal parts, so that a time split in units of the tile
+// keeps every block whole.  Nested delays that vary keep the sample-by-sample kernels.
+void fx_setup(lr_plan *p)
+{
+    lr::FwdParams &P = p->base;
+    P.fx.tile = 0;
+    if (p->desc.precision != LR_FP64 || (P.delay_nested && !P.cd_w)) return;
+    const int most = lr::fx_max_tile(P, p->desc.order);
+    int block = p->tile < most ? p->tile : most;
+    while (block >= 128 && p->tile % block) --block;
+    if (block < 128 && p->tile >= 128) return;  // no part of at least 128 outputs
+    P.fx.tile = block;
+    P.tile = block;
+    lr::fx_tables(P);
 }
 
 bool all_finite(const double *p, size_t n)
@@ -612,7 +631,15 @@ LR_API int lr_plan_create(lr_ctx *ctx, const lr_plan_desc *d, lr_plan **out)
             delete p;
             return st;
         }
+        if (d->tile == 0 && (!P.delay_nested || P.cd_w)) {
+            const int most = lr::fx_max_tile(P, d->order);
+            if (most >= 128) P.tile = most;
+        }
     }
+    P.ymax = P.tile + P.HL + P.HR;
+    P.wmax = P.ymax + 2 * P.sig_b + P.lproj_b + p->T + 4;
+    p->tile = P.tile;
+    fx_setup(p);
     *out = p;
     return LR_OK;
 }
@@ -645,7 +672,7 @@ LR_API int lr_required_margin(const lr_plan *plan, int64_t *left, int64_t *right
 LR_API int lr_plan_tile(const lr_plan *plan, int *tile)
 {
     if (!plan || !tile) return LR_ERR_INVALID_ARG;
-    *tile = plan->base.tile;
+    *tile = plan->tile;
     return LR_OK;
 }
 
@@ -1169,6 +1196,8 @@ int plan_set_tile(lr_plan *plan, int tile)
     P.tile = tile;
     P.ymax = ymax;
     P.wmax = P.ymax + 2 * P.sig_b + P.lproj_b + plan->T + 4;
+    plan->tile = tile;
+    fx_setup(plan);
     return LR_OK;
 }
 

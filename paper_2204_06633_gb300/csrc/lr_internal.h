@@ -95,6 +95,18 @@ struct LikeArgs {
     int64_t n_total;     // samples the data array holds per channel block (sum of N_s)
 };
 
+// Tensor-core FP64 kernels (lr_fx64.cu): rows of a block, expansion nodes, byte counts of the staged
+// digit planes and stencils
+constexpr int FX_ROWS = 512, FX_NODES = 8, FX_TDI_NODES = 4;
+constexpr int FX_PROJ_PLANES = 14 * (FX_ROWS + 64) * 2, FX_PROJ_W = 12 * 38 * 72;
+constexpr int FX_TDI_PLANES = 42 * (FX_ROWS + 64) * 2, FX_TDI_W = 12 * 19 * 72;
+struct FxTab {
+    int tile;                                     // outputs per block (0: the plan does not use these kernels)
+    double icdt;                                  // 1 / (c dt)
+    double node_j[FX_NODES], cheb[FX_NODES][FX_NODES / 2];           // node rows, transform (half by symmetry)
+    double tnode_j[FX_TDI_NODES], tcheb[FX_TDI_NODES][FX_TDI_NODES / 2];
+};
+
 struct FwdParams {
     double dt, inv_dt, t0;
     OrbitDev po, to;      // projection orbit, TDI orbit
@@ -130,6 +142,7 @@ struct FwdParams {
     // null when the delays vary (FP64 kernels only)
     const double *cd_w;
     int cd_off[3][2][CHAIN_TERMS];
+    FxTab fx;
 };
 
 // generated strain: the source's waveform sampled on the output grid at every index (the

@@ -20,6 +20,7 @@
 #include <string>
 #include <vector>
 
+#include "lr_fx64.h"
 #include "lr_launch.h"
 #include "lr_planview.h"
 
@@ -52,7 +53,8 @@ std::string tune_key(const lr::PlanView &v, int generation, int64_t n)
         if (c == ' ') c = '_';
     int bucket = n > 0 ? (int)std::floor(std::log2((double)n)) : 0;
     char buf[256];
-    std::snprintf(buf, sizeof(buf), "%s|p%d|o%d|g%d|b%d", name.c_str(), v.precision, v.order, generation, bucket);
+    std::snprintf(buf, sizeof(buf), "%s|p%d%s|o%d|g%d|b%d", name.c_str(), v.precision, v.base.fx.tile ? "x" : "", v.order,
+                  generation, bucket);
     return buf;
 }
 
@@ -89,6 +91,8 @@ std::vector<int> tile_candidates(const lr::PlanView &v)
         cand.push_back(tmax);
         for (int t : {256, 192, 128})
             if (t < tmax) cand.push_back(t);
+    } else if (v.base.fx.tile) {
+        cand.push_back(lr::fx_max_tile(v.base, v.order));  // the largest block: the work per block hardly depends on it
     } else {
         for (int t : {256, 384, 512, 768, 1024}) cand.push_back(t);
     }

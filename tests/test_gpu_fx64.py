@@ -1,0 +1,102 @@
+"""The tensor-core FP64 kernels at the places where their blocks can go wrong, against the oracle and
+against the sample-by-sample kernels (reached with a tile that has no part of 128 to 478 outputs)."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+import oracle  # noqa: E402
+import paper_2204_06633_gb300 as lr  # noqa: E402
+import synth  # noqa: E402
+from _gpu import DT, T0, Pair, assert_close, dev, host, run_case, sky  # noqa: E402
+
+BY_SAMPLE = 509   # a prime tile above the largest block
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    return lr.Context(0)
+
+
+@pytest.fixture(scope="module")
+def flex(ctx):
+    return Pair(ctx, synth.orbit_flexing(-2e6, 2e6))
+
+
+@pytest.mark.parametrize("kind", ["response", "project", "tdi"])
+@pytest.mark.parametrize("N", [1, 31, 477, 478, 479, 957, 20000])
+def test_block_edges_and_steps(ctx, flex, kind, N):
+    """Partial and whole blocks; 20 000 outputs hold knots and stencil steps of every read.  A source
+    near the ecliptic drifts fastest."""
+    src = dataclasses.replace(synth.draw_sources(1, seed=N)[0], f=2e-3, beta=0.02)
+    run_case(ctx, src, N, 25, flex, kind=kind)
+
+
+@pytest.mark.parametrize("p", [1, 3, 9, 17, 31, 41])
+@pytest.mark.parametrize("gen", [1, 2])
+def test_orders(ctx, flex, p, gen):
+    run_case(ctx, synth.draw_sources(1, seed=p)[0], 3000, p, flex, gen=gen)
+
+
+@pytest.mark.parametrize("dt", [2.5, 5.0, 15.0, 100.0])
+def test_sampling_steps(ctx, dt):
+    """Chained delays from under one to 24 samples: one merged stencil per link in each case."""
+    N, p = 3000, 25
+    orb = synth.orbit_flexing(T0 - 3e5, T0 + N * dt + 3e5)
+    pair = Pair(ctx, orb)
+    src = dataclasses.replace(synth.draw_sources(1, seed=9)[0], f=0.01 / dt)
+    t0h, hp, hc = synth.gb_input(src, T0, dt, N, p)
+    plan = lr.Plan(ctx, p, N, dt, pair.gpu, t0=T0)
+    got = host(plan.response(dev(hp), dev(hc), t0h, sky(src)))
+    plan.check()
+    args = (p, 2, dt, T0, N, pair.orc, pair.orc, hp, hc, t0h, src.lam, src.beta, src.psi)
+    assert_close(got, oracle.response(*args), oracle.response(*args, absval=True), p + 1, 1e-12)
+
+
+def test_source_along_an_arm(ctx, flex):
+    """Near an arm direction the patterns turn within a block: the block's expansion does not apply."""
+    t = 10000.0
+    pos = synth.keplerian_flexing(np.array([t]))[:, :, 0]
+    d = (pos[0] - pos[1]) / np.linalg.norm(pos[0] - pos[1])
+    for off in (1e-3, 5e-3, 2e-2):
+        src = dataclasses.replace(synth.draw_sources(1, seed=4)[0], lam=float(np.arctan2(-d[1], -d[0]) + off),
+                                  beta=float(np.arcsin(-d[2])))
+        run_case(ctx, src, 2500, 25, flex)
+
+
+@pytest.mark.parametrize("p", [11, 41])
+def test_wide_range_and_nonfinite_blocks_match_the_sample_kernels(ctx, flex, p):
+    """A loud sample, a NaN and an infinity: the blocks that read them are evaluated sample by sample (same
+    arithmetic as the sample kernels), with the same outputs undefined; the others agree to rounding."""
+    N = 6000
+    src = dataclasses.replace(synth.draw_sources(1, seed=7)[0], f=3e-3)
+    t0h, hp, hc = synth.gb_input(src, T0, DT, N, p)
+    hp[2000] *= 1e9
+    hp[3500] = np.nan
+    hc[5000] = np.inf
+    out = []
+    for tile in (0, BY_SAMPLE):
+        plan = lr.Plan(ctx, p, N, DT, flex.gpu, t0=T0, tile=tile)
+        out.append(host(plan.response(dev(hp), dev(hc), t0h, sky(src))))
+        with pytest.raises(lr.LRError):
+            plan.check()
+    a, b = out
+    assert np.array_equal(np.isfinite(a), np.isfinite(b)) and not np.isfinite(b).all()
+    ok = np.isfinite(b)
+    quiet = ok.copy()
+    quiet[:, 1700:2300] = False   # outputs that read the loud sample
+    assert np.linalg.norm((a - b)[ok]) <= 1e-12 * np.linalg.norm(b[ok])
+    assert np.linalg.norm((a - b)[quiet]) <= 1e-12 * np.linalg.norm(b[quiet])
+
+
+def test_zero_strain_gives_zero(ctx, flex):
+    plan = lr.Plan(ctx, 25, 2000, DT, flex.gpu, t0=T0)
+    z = torch.zeros(2200, dtype=torch.float64, device="cuda:0")
+    assert not plan.response(z, z, -100 * DT, (0.3, 0.2, 0.1)).any()
+    plan.check()
