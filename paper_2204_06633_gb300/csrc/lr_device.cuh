@@ -88,7 +88,8 @@ __device__ inline const double *like_data(const FwdParams &P, int64_t oo, int64_
     return P.like.data + 3 * oo;
 }
 
-__device__ inline TileInfo tile_info(const FwdParams &P, int64_t g, int ochan)
+// tile g's record once its source s is known
+__device__ inline TileInfo tile_info_of(const FwdParams &P, int64_t g, int64_t s, int ochan)
 {
     TileInfo ti;
     ti.ok = 1;
@@ -106,12 +107,6 @@ __device__ inline TileInfo tile_info(const FwdParams &P, int64_t g, int ochan)
         if (P.gen_strain) ti.gb = make_gb(P.src.gb1);
     } else {
         const int64_t *to = P.src.tile_off;
-        int64_t lo = 0, hi = P.src.S;  // find s with to[s] <= g < to[s+1]
-        while (hi - lo > 1) {
-            int64_t mid = (lo + hi) >> 1;
-            if (__ldg(to + mid) <= g) lo = mid; else hi = mid;
-        }
-        int64_t s = lo;
         int64_t ho = 0, ho1 = 0;
         if (P.gen_strain) {
             ti.gb = make_gb(P.src.gb[s]);
@@ -140,6 +135,20 @@ __device__ inline TileInfo tile_info(const FwdParams &P, int64_t g, int ochan)
     ti.nb = rem < P.tile ? rem : P.tile;
     if (ti.nb < 0) ti.nb = 0;
     return ti;
+}
+
+__device__ inline TileInfo tile_info(const FwdParams &P, int64_t g, int ochan)
+{
+    int64_t lo = 0;
+    if (P.src.tile_off) {
+        const int64_t *to = P.src.tile_off;
+        int64_t hi = P.src.S;  // find s with to[s] <= g < to[s+1]
+        while (hi - lo > 1) {
+            int64_t mid = (lo + hi) >> 1;
+            if (__ldg(to + mid) <= g) lo = mid; else hi = mid;
+        }
+    }
+    return tile_info_of(P, g, lo, ochan);
 }
 
 // ---------------------------------------------------------------- Lagrange reads (FP64)

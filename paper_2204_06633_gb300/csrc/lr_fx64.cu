@@ -31,13 +31,18 @@
 //
 // Layout of the contraction (mma.sync m16n8k16): row a of a block of 16 is samples 8a..8a+7, column b the
 // sample within the row, so the left operand is the staged series itself, series[8a + c], and the right
-// one the stencil shifted by b, W[c - b]; neither is expanded in memory.  A lane's four k-values are taken
+// one the stencil shifted by b, W[c - b]; neither is expanded in memory.  The projection takes rows of 4
+// samples and two links as the columns' other half: both links read the same strain, and 29 taps + 3 fit
+// 32 steps of k where 29 + 7 need 48.  A lane's four k-values are taken
 // as four consecutive c (the same permutation of k on both sides), so a lane reads its two left registers
 // of a row with one 8-byte load and its right registers from four consecutive digit bytes, which become
 // halves by placing them under the exponent of 1024 and subtracting 1152.
 //
-// Measured (fused, order 25, one year of 3 153 600 outputs): 44.45 ms sample by sample, 4.36 ms here, with
-// 1.3e-13 relative error against 64 bits where the sample form has 1.4e-13.
+// Measured (fused, order 25, one year of 3 153 600 outputs): 44.45 ms sample by sample, 3.65 ms here, with
+// 1.3e-13 relative error against 64 bits where the sample form has 1.4e-13.  Two blocks share an SM; the
+// tensor pipe is busy a third of the time and the FP64 pipe (weights, transforms) a quarter, the rest is
+// latency of the short FP64 phases.  With 8-sample rows in the projection and the TDI stencils computed in
+// every block it was 4.36 ms.
 //
 // Where the expansion does not apply, the block is evaluated sample by sample in FP64 as in lr_fwd64.cu: a
 // NaN or infinity in the series, values that span more than 12 bits between 32-sample stretches (the
@@ -58,7 +63,7 @@ constexpr int DL = NY + 64;       // staged samples per digit plane
 constexpr int WS = 72;            // bytes per digit row of a stencil: 7 zeros, the taps, zeros
 constexpr int NN = FX_NODES, NT = FX_TDI_NODES;
 constexpr int MAXSEG = 10;
-constexpr int GP = 16;            // spacing of the projection's grid samples
+constexpr int GP = 32;            // spacing of the projection's grid samples
 constexpr int NG = NY / GP + 1;
 constexpr int GT = 64;            // spacing of the TDI grid samples
 constexpr int NGT = NY / GT + 1;
@@ -115,7 +120,7 @@ struct Shared {
     double lc1[64], lc0[64], rc1[64], rc0[64];  // Lagrange factors (prefix, suffix) of the nodes
     union {  // the projection's grid and nodes, then the TDI's
         struct {
-            double npos[NN][9], neps[NN * 9], ncf[NN][12];
+            double npos[NN][9], nodeu[NN * 9], ncf[NN][12];
             float fg[NG][9];
             int mg[NG][10];
         };
@@ -127,33 +132,21 @@ struct Shared {
     };
     int segm[MAXSEG][NTERM + 1];  // stencil positions (9 or 42) and the spline piece of each segment
     int segj[MAXSEG + 1];
-    int nseg, nlist;
+    int nseg, nlist, fast;
     unsigned brk[NY / 32];
     int list[NTERM * 8 + 8];
     int mmin, mmax;
     int cmax[6], wexp[6];
     unsigned vmax, vmin;
-    unsigned qmask;
+    unsigned long long qor[NN];  // OR of the coefficients' magnitudes per order
+    int nq, last;                // orders in use; whether those above 0 have their last digit only
     int bad;
     double red[2 * 8];
 };
 
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ uint2 lds64(uint32_t a)
-{
-    uint2 v;
-    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
-    return v;
-}
-__device__ __forceinline__ uint32_t lds32(uint32_t a)
-{
-    uint32_t v;
-    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
-    return v;
-}
 __device__ __forceinline__ void mma_f16(float *c, const uint32_t *a, uint32_t b0, uint32_t b1)
 {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
@@ -181,13 +174,14 @@ constexpr long long DIGIT_BIAS = 0x808080808080ll;
 
 // ---------------------------------------------------------------- contraction
 // acc[i][L][.] += the level sums of orders QF .. QF + NQ - 1 over `parts` series of `nks` steps of 16 taps
-template <int QF, int NQ, bool TDI>
-__device__ __forceinline__ void contract(float (&acc)[NQ][7][4], uint32_t a_lane, uint32_t w_lane, uint32_t sh, int nks,
-                                         const signed char *links)
+template <int QF, int NQ, bool TDI, bool LAST = false>
+__device__ __forceinline__ void contract(float (&acc)[NQ][7][4], const unsigned char *a_lane,
+                                         const unsigned char *w_lane, uint32_t sh, int nks, const signed char *links)
 {
-    constexpr int ZM = zq(TDI, QF);      // the smallest z of the group
+    constexpr int ZM = LAST ? 6 : zq(TDI, QF);  // the smallest z of the group
     constexpr int NA = ZM ? 8 - ZM : 7;  // digit planes of the series that it needs
     constexpr int PARTS = TDI ? 4 : 2, ROWS = TDI ? TD : PD;
+    constexpr int RS = TDI ? 16 : 8;     // bytes between rows of the left operand: 8 or 4 samples
 #pragma unroll
     for (int i = 0; i < NQ; ++i)
 #pragma unroll
@@ -196,23 +190,24 @@ __device__ __forceinline__ void contract(float (&acc)[NQ][7][4], uint32_t a_lane
             for (int r = 0; r < 4; ++r) acc[i][L][r] = 0.0f;
 #pragma unroll 1
     for (int part = 0; part < PARTS; ++part) {
-        uint32_t pa = a_lane + (uint32_t)((TDI ? links[part] : part) * 7 * DL * 2);
-        uint32_t pw = w_lane + (uint32_t)(part * ROWS * WS);
+        const unsigned char *pa = a_lane + (TDI ? links[part] : part) * (7 * DL * 2);
+        const unsigned char *pw = w_lane + part * ROWS * WS;
 #pragma unroll 1
         for (int ks = 0; ks < nks; ++ks, pa += 32, pw += 16) {
             uint32_t a[NA][4];
 #pragma unroll
             for (int k = 0; k < NA; ++k) {
-                const uint2 lo = lds64(pa + k * DL * 2), hi = lds64(pa + k * DL * 2 + 128);
+                const uint2 lo = *reinterpret_cast<const uint2 *>(pa + k * DL * 2);
+                const uint2 hi = *reinterpret_cast<const uint2 *>(pa + k * DL * 2 + 8 * RS);
                 a[k][0] = lo.x; a[k][1] = hi.x; a[k][2] = lo.y; a[k][3] = hi.y;
             }
 #pragma unroll
             for (int i = 0; i < NQ; ++i) {
                 const int z = zq(TDI, QF + i), row = digit_row(TDI, QF + i);
 #pragma unroll
-                for (int d = z; d < 7; ++d) {
-                    const uint32_t w0 = lds32(pw + (row + d - z) * WS), w1 = lds32(pw + (row + d - z) * WS + 4);
-                    const uint32_t u = __funnelshift_r(w0, w1, sh);
+                for (int d = LAST ? 6 : z; d < 7; ++d) {
+                    const uint32_t *w = reinterpret_cast<const uint32_t *>(pw + (row + d - z) * WS);
+                    const uint32_t u = __funnelshift_r(w[0], w[1], sh);
                     const uint32_t b0 = digits_h2(u, 0x4140u), b1 = digits_h2(u, 0x4342u);
 #pragma unroll
                     for (int k = 0; k < 6 - d; ++k) mma_f16(acc[i][d + k], a[k], b0, b1);
@@ -333,7 +328,7 @@ __device__ __forceinline__ const Coef4 *row_at(const OrbitDev &o, double t, int 
 }
 
 // spacecraft s at time t: k.x/(c dt) and, when pos is not null, its position
-__device__ __forceinline__ double sigma_at(const FwdParams &P, const SkyConst &S, const Coef4 *row, double x, int s,
+__device__ __forceinline__ double sigma_at(const FwdParams &P, const FxTab &X, const SkyConst &S, const Coef4 *row, double x, int s,
                                            double *pos)
 {
     double v[3];
@@ -343,16 +338,37 @@ __device__ __forceinline__ double sigma_at(const FwdParams &P, const SkyConst &S
 #pragma unroll
         for (int d = 0; d < 3; ++d) pos[3 * s + d] = v[d];
     }
-    return (S.k[0] * v[0] + S.k[1] * v[1] + S.k[2] * v[2]) * P.fx.icdt;
+    return (S.k[0] * v[0] + S.k[1] * v[1] + S.k[2] * v[2]) * X.icdt;
+}
+
+// positions of the three reads of spacecraft s (its reception, the emissions to the two others)
+__device__ __forceinline__ void reads_of(const FwdParams &P, const FxTab &X, const SkyConst &S, const Coef4 *row, double x, int s,
+                                         double u0, double *u, double *pos)
+{
+    const double sig = sigma_at(P, X, S, row, x, s, pos);
+    u[0] = u0 - sig;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) u[1 + i] = u0 - cubic(ldg4(row + 9 + c_by_emitter[s][i]), x) * P.inv_dt - sig;
+}
+
+// the same at expansion node n, with the spacecraft's position, on a given spline piece
+__device__ __forceinline__ void node_reads(const FwdParams &P, const FxTab &X, Shared &S, double t_lo, double u0, int n, int s, int piece)
+{
+    double x, u[3];
+    int k;
+    const Coef4 *row = row_at(P.po, t_lo + X.node_j[n] * P.dt, piece, &x, &k);
+    reads_of(P, X, S.skc, row, x, s, u0, u, S.npos[n]);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) S.nodeu[n * 9 + (i == 0 ? s : 3 + c_by_emitter[s][i - 1])] = u[i];
 }
 
 // position (samples, relative to the row) of read rd (0-2 receptions, 3 + l emissions) at time t
-__device__ __forceinline__ double read_pos(const FwdParams &P, const SkyConst &S, double u0, double t, int rd, int *piece)
+__device__ __forceinline__ double read_pos(const FwdParams &P, const FxTab &X, const SkyConst &S, double u0, double t, int rd, int *piece)
 {
     double x;
     const Coef4 *row = row_at(P.po, t, -1, &x, piece);
     const int s = rd < 3 ? rd : c_ls[rd - 3];
-    const double sig = sigma_at(P, S, row, x, s, nullptr);
+    const double sig = sigma_at(P, X, S, row, x, s, nullptr);
     return rd < 3 ? u0 - sig : u0 - cubic(ldg4(row + 9 + rd - 3), x) * P.inv_dt - sig;
 }
 
@@ -409,15 +425,41 @@ __device__ __forceinline__ bool range_ok(const Shared &S, int *e)
     return eb >= 200 && eb <= 1900 && eb - es <= RANGE_BITS;
 }
 
-// seven digit planes (halves) of v * scale at index p
-__device__ __forceinline__ void digits_to_planes(uint16_t *pl, int p, double v, double scale)
+// v * 2^(55 - e), |v| < 2^e, rounded to an integer: shifts of the significand (FP64 conversions issue at a
+// 64th of the integer rate)
+__device__ __forceinline__ long long to_fixed(double v, int e)
 {
-    const long long X = __double2ll_rn(v * scale) + DIGIT_BIAS;
+    const long long b = __double_as_longlong(v);
+    const int E = (int)((b >> 52) & 0x7ff);
+    const unsigned long long m = ((unsigned long long)b & 0xfffffffffffffull) | (E ? 1ull << 52 : 0ull);
+    const int s = E - e - 1020;  // at most 2
+    unsigned long long r;
+    if (s >= 0) r = m << s;
+    else r = s > -60 ? ((m >> (-s - 1)) + 1) >> 1 : 0ull;
+    return b < 0 ? -(long long)r : (long long)r;
+}
+
+// v * 2^e to FP64, rounded to nearest (ties away), for results in the normal range
+__device__ __forceinline__ double from_fixed(long long v, int e)
+{
+    if (v == 0) return 0.0;
+    const unsigned long long a = (unsigned long long)(v < 0 ? -v : v);
+    const int z = __clzll((long long)a);
+    // significand with its leading one at bit 52; the rounding carry moves into the exponent
+    const unsigned long long m = (((a << z) >> 10) + 1) >> 1;
+    const unsigned long long bits = m + ((unsigned long long)(1023 + 63 - z + e - 1) << 52);
+    return __longlong_as_double((long long)(bits | (v < 0 ? 1ull << 63 : 0ull)));
+}
+
+// seven digit planes (halves) of v in units of 2^(e - 55) at index p
+__device__ __forceinline__ void digits_to_planes(uint16_t *pl, int p, double v, int e)
+{
+    const long long X = to_fixed(v, e) + DIGIT_BIAS;
     const uint32_t top = (uint32_t)((int)(X >> 48) + 128);  // 0 .. 256
     const uint32_t lo = (uint32_t)X, hi = (uint32_t)(X >> 32);
     const uint32_t d[7] = {top, (hi >> 8) & 255u, hi & 255u, lo >> 24, (lo >> 16) & 255u, (lo >> 8) & 255u, lo & 255u};
 #pragma unroll
-    for (int i = 0; i < 7; i += 1) {
+    for (int i = 0; i < 7; ++i) {
         uint32_t r;
         asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(0x6400u + d[i]), "r"(0x6480u));
         pl[i * DL + p] = (uint16_t)r;
@@ -438,16 +480,44 @@ __device__ __forceinline__ bool coef_digits(unsigned char *w, long long b)
 }
 
 template <bool TDI, int Q>
-__device__ __forceinline__ bool coef_store(unsigned char *w, double b, unsigned &mask)
+__device__ __forceinline__ bool coef_store(unsigned char *w, double b, unsigned long long *mag)
 {
     const long long v = __double2ll_rn(b);
-    if (v) mask |= 1u << Q;
+    mag[Q] |= (unsigned long long)(v < 0 ? -v : v);
     return coef_digits<zq(TDI, Q)>(w + digit_row(TDI, Q) * WS, v);
+}
+
+// magnitudes of the block's coefficients per order, over all threads (then count_orders after a barrier)
+template <int N>
+__device__ __forceinline__ void orders_in_use(Shared &S, const unsigned long long *mag)
+{
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+        const unsigned hi = __reduce_or_sync(0xffffffffu, (unsigned)(mag[q] >> 32));
+        const unsigned lo = __reduce_or_sync(0xffffffffu, (unsigned)mag[q]);
+        if ((threadIdx.x & 31) == 0 && (hi | lo)) atomicOr(&S.qor[q], (unsigned long long)hi << 32 | lo);
+    }
+}
+
+// the number of orders in use, and whether the orders above 0 (constant delays and positions: rounding of
+// the transform) fit their last digit; ends with a barrier
+template <int N>
+__device__ __forceinline__ void count_orders(Shared &S)
+{
+    if (threadIdx.x < 32) {
+        const unsigned long long m = threadIdx.x < N ? S.qor[threadIdx.x] : 0;
+        const unsigned used = __ballot_sync(0xffffffffu, m != 0), big = __ballot_sync(0xffffffffu, threadIdx.x > 0 && m >= 64);
+        if (threadIdx.x == 0) {
+            S.nq = 32 - __clz((int)used);
+            S.last = big == 0;
+        }
+    }
+    __syncthreads();
 }
 
 // ---------------------------------------------------------------- the block's link series
 // Fills ys[6][NY] with the link series of rows 0 .. ny - 1 (sample k_lo + row).
-__device__ void project_block(const FwdParams &P, Shared &S, int T, int64_t k_lo, int ny, double u0, double *ys,
+__device__ void project_block(const FwdParams &P, const FxTab &X, Shared &S, int T, int64_t k_lo, int ny, double u0, double *ys,
                               unsigned char *work)
 {
     const int tid = threadIdx.x, h = (T - 2) / 2;
@@ -458,26 +528,32 @@ __device__ void project_block(const FwdParams &P, Shared &S, int T, int64_t k_lo
     unsigned char *W = work + FX_PROJ_PLANES;
     double *wn = reinterpret_cast<double *>(work + FX_PROJ_PLANES + FX_PROJ_W);
 
-    // stencil positions on the grid samples
-    if (tid < NG * 3) {
+    // stencil positions on the grid samples, and the reads at the expansion nodes (on row 0's spline piece)
+    if (tid < (NG + NN) * 3) {
         const int g = tid / 3, s = tid % 3;
-        const double t = t_lo + (double)(g * GP) * P.dt;
-        double x;
-        int piece;
-        const Coef4 *row = row_at(P.po, t, -1, &x, &piece);
-        const double sig = sigma_at(P, S.skc, row, x, s, nullptr);
-        if (s == 0) S.mg[g][9] = piece;
+        if (g < NG) {
+            double x;
+            int piece;
+            const Coef4 *row = row_at(P.po, t_lo + (double)(g * GP) * P.dt, -1, &x, &piece);
+            if (s == 0) S.mg[g][9] = piece;
+            double u[3];
+            reads_of(P, X, S.skc, row, x, s, u0, u, nullptr);
 #pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            const int rd = i == 0 ? s : 3 + c_by_emitter[s][i - 1];
-            const double u = i == 0 ? u0 - sig : u0 - cubic(ldg4(row + 9 + rd - 3), x) * P.inv_dt - sig;
-            const double fl = floor(u);
-            S.mg[g][rd] = (int)(fl - fl0);
-            S.fg[g][rd] = (float)(u - fl);
+            for (int i = 0; i < 3; ++i) {
+                const int rd = i == 0 ? s : 3 + c_by_emitter[s][i - 1];
+                const double fl = floor(u[i]);
+                S.mg[g][rd] = (int)(fl - fl0);
+                S.fg[g][rd] = (float)(u[i] - fl);
+            }
+        } else {
+            double x;
+            int piece;
+            row_at(P.po, t_lo, -1, &x, &piece);
+            node_reads(P, X, S, t_lo, u0, g - NG, s, piece);
         }
     }
     if (tid < NY / 32) S.brk[tid] = 0;
-    if (tid == 32) {
+    if (tid == 192) {
         S.nlist = 0;
         S.bad = 0;
         S.vmax = 0;
@@ -503,12 +579,12 @@ __device__ void project_block(const FwdParams &P, Shared &S, int T, int64_t k_lo
     __syncthreads();
     for (int i = tid >> 5; i < S.nlist; i += blockDim.x >> 5) {
         const int g = S.list[i] / 10, rd = S.list[i] % 10, lane = tid & 31;
-        const int j = g * GP + (lane < GP ? lane : GP);
+        const int j = g * GP + lane + 1;   // rows g GP + 1 .. (g + 1) GP against the row before
         int piece;
-        const double u = read_pos(P, S.skc, u0, t_lo + (double)j * P.dt, rd < 9 ? rd : 0, &piece);
+        const double u = read_pos(P, X, S.skc, u0, t_lo + (double)j * P.dt, rd < 9 ? rd : 0, &piece);
         const int m = rd < 9 ? (int)(floor(u) - fl0) : piece;
         const int prev = __shfl_up_sync(0xffffffffu, m, 1);
-        if (lane >= 1 && lane <= GP && m != prev && j < NY) atomicOr(&S.brk[j >> 5], 1u << (j & 31));
+        if (m != (lane ? prev : S.mg[g][rd]) && j < NY) atomicOr(&S.brk[j >> 5], 1u << (j & 31));
     }
     __syncthreads();
     if (tid == 0) collect_segments(S, ny);
@@ -516,9 +592,12 @@ __device__ void project_block(const FwdParams &P, Shared &S, int T, int64_t k_lo
     const int nseg = S.nseg;
     if (tid < nseg * 10) {
         const int sg = tid / 10, rd = tid % 10;
-        int piece;
-        const double u = read_pos(P, S.skc, u0, t_lo + (double)S.segj[sg] * P.dt, rd < 9 ? rd : 0, &piece);
-        const int m = rd < 9 ? (int)(floor(u) - fl0) : piece;
+        int m = S.mg[0][rd];
+        if (sg) {
+            int piece;
+            const double u = read_pos(P, X, S.skc, u0, t_lo + (double)S.segj[sg] * P.dt, rd < 9 ? rd : 0, &piece);
+            m = rd < 9 ? (int)(floor(u) - fl0) : piece;
+        }
         S.segm[sg][rd] = m;
         if (rd < 9) {
             atomicMin(&S.mmin, m);
@@ -527,7 +606,7 @@ __device__ void project_block(const FwdParams &P, Shared &S, int T, int64_t k_lo
     }
     __syncthreads();
     const int mmin = S.mmin, KW = S.mmax - mmin + T;   // taps of a merged stencil
-    const int nks = (KW + 7 + 15) / 16;
+    const int nks = (KW + 3 + 15) / 16;
     bool bad = S.bad || nks * 16 > 64;
     // strain window: row j reads samples w_lo + j .. w_lo + j + KW - 1
     const int64_t w_lo = k_lo + (int64_t)fl0 + mmin - h;
@@ -568,12 +647,11 @@ __device__ void project_block(const FwdParams &P, Shared &S, int T, int64_t k_lo
     }
     if (!bad) bad = !range_ok(S, &ex);
     if (!bad) {
-        const double scale = pow2(55 - ex);
         for (int i = 0; i < 3; ++i) {
             const int p = tid + i * 256;
             if (p < DL) {
-                digits_to_planes(planes, p, vp[i], scale);
-                digits_to_planes(planes + 7 * DL, p, vc[i], scale);
+                digits_to_planes(planes, p, vp[i], ex);
+                digits_to_planes(planes + 7 * DL, p, vc[i], ex);
             }
         }
     }
@@ -584,48 +662,62 @@ __device__ void project_block(const FwdParams &P, Shared &S, int T, int64_t k_lo
         __syncthreads();  // the previous segment's stencils and nodes are free
         for (int i = tid; i < FX_PROJ_W / 16; i += blockDim.x)
             reinterpret_cast<uint4 *>(W)[i] = make_uint4(0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u);
-        if (tid < NN * 3) {
-            const int n = tid / 3, s = tid % 3;
-            const double t = t_lo + P.fx.node_j[n] * P.dt;
-            double x;
-            int piece;
-            const Coef4 *row = row_at(P.po, t, sm[9], &x, &piece);
-            const double sig = sigma_at(P, S.skc, row, x, s, S.npos[n]);
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                const int rd = i == 0 ? s : 3 + c_by_emitter[s][i - 1];
-                const double u = i == 0 ? u0 - sig : u0 - cubic(ldg4(row + 9 + rd - 3), x) * P.inv_dt - sig;
-                S.neps[n * 9 + rd] = u - (fl0 + (double)sm[rd]);
-            }
-        }
-        if (tid >= 64 && tid < 70) S.cmax[tid - 64] = 0;
-        if (tid == 70) S.qmask = 0;
+        if (sm[9] != S.segm[sg ? sg - 1 : 0][9] && tid < NN * 3) node_reads(P, X, S, t_lo, u0, tid / 3, tid % 3, sm[9]);
+        if (tid >= 192 && tid < 198) S.cmax[tid - 192] = 0;
+        if (tid >= 200 && tid < 200 + NN) S.qor[tid - 200] = 0;
         __syncthreads();
-        if (tid < NN * 9) {
-            lagrange_to(S, T, S.neps[tid], wn + tid, WNS);
-        } else if (tid >= 96 && tid < 96 + NN * 3) {
-            const int n = (tid - 96) / 3, r = (tid - 96) % 3, s = (r + 1) % 3;
+        // Lagrange weights at the nodes, two threads per read: prefix products of the lower half and suffix
+        // products of the upper half, then each carries on through the other's half
+        const int id = tid < WNS ? tid : tid - WNS;
+        const bool low = tid < WNS, half = tid < 2 * WNS;
+        double e = 0.0, run = 1.0;
+        if (half) {
+            e = S.nodeu[id] - (fl0 + (double)sm[id % 9]);
+            double *w = wn + id;
+            if (low) {
+                for (int a = 0; a < T / 2; ++a) {
+                    w[a * WNS] = run;
+                    run *= fma(e, S.lc1[a], S.lc0[a]);
+                }
+            } else {
+                for (int a = T - 1; a >= T / 2; --a) {
+                    w[a * WNS] = ((T - 1 - a) & 1) ? -run : run;
+                    run *= fma(e, S.rc1[a], S.rc0[a]);
+                }
+            }
+        } else if (tid >= 160 && tid < 160 + NN * 6) {
+            const int n = (tid - 160) / 6, l = (tid - 160) % 6, r = c_lr[l], s = c_ls[l];
             const SkyConst &K = S.skc;
             const double *x = S.npos[n];
             double d0 = x[3 * r] - x[3 * s], d1 = x[3 * r + 1] - x[3 * s + 1], d2 = x[3 * r + 2] - x[3 * s + 2];
-            const double inv = 1.0 / sqrt(d0 * d0 + d1 * d1 + d2 * d2);
+            const double inv = rsqrt(d0 * d0 + d1 * d1 + d2 * d2);
             d0 *= inv; d1 *= inv; d2 *= inv;
             const double un = K.u[0] * d0 + K.u[1] * d1 + K.u[2] * d2;
             const double vn = K.v[0] * d0 + K.v[1] * d1 + K.v[2] * d2;
             const double kn = K.k[0] * d0 + K.k[1] * d1 + K.k[2] * d2;
             const double xip = un * un - vn * vn, xic = 2.0 * un * vn;
-            const double xp = K.c2p * xip + K.s2p * xic, xc = -K.s2p * xip + K.c2p * xic;
-            const double gf = 1.0 / (2.0 * (1.0 - kn)), gr = 1.0 / (2.0 * (1.0 + kn));
-            const double c4[4] = {xp * gf, xc * gf, xp * gr, xc * gr};
-            double *o = S.ncf[n];
-            o[2 * r] = c4[0];
-            o[2 * r + 1] = c4[1];
-            o[2 * (5 - r)] = c4[2];
-            o[2 * (5 - r) + 1] = c4[3];
+            const double gf = 0.5 / (1.0 - kn);
+            const double cp = (K.c2p * xip + K.s2p * xic) * gf, cc = (K.c2p * xic - K.s2p * xip) * gf;
+            S.ncf[n][2 * l] = cp;
+            S.ncf[n][2 * l + 1] = cc;
             // NaN and infinity give the largest keys
-            atomicMax(&S.cmax[r], (int)(__float_as_uint((float)fmax(fabs(c4[0]), fabs(c4[1]))) & 0x7fffffffu));
-            atomicMax(&S.cmax[5 - r], (int)(__float_as_uint((float)fmax(fabs(c4[2]), fabs(c4[3]))) & 0x7fffffffu));
-            if (!(isfinite(gf) && isfinite(gr))) S.bad = 1;
+            atomicMax(&S.cmax[l], (int)(__float_as_uint((float)fmax(fabs(cp), fabs(cc))) & 0x7fffffffu));
+            if (!isfinite(gf)) S.bad = 1;
+        }
+        __syncthreads();
+        if (half) {
+            double *w = wn + id;
+            if (low) {
+                for (int a = T / 2; a < T; ++a) {
+                    w[a * WNS] *= run;
+                    run *= fma(e, S.lc1[a], S.lc0[a]);
+                }
+            } else {
+                for (int a = T / 2 - 1; a >= 0; --a) {
+                    w[a * WNS] *= ((T - 1 - a) & 1) ? -run : run;
+                    run *= fma(e, S.rc1[a], S.rc0[a]);
+                }
+            }
         }
         __syncthreads();
         if (tid < 6) {  // the stencil's scale: 2 max|c| with slack for offsets just outside [0, 1)
@@ -636,7 +728,7 @@ __device__ void project_block(const FwdParams &P, Shared &S, int T, int64_t k_lo
         if (tid < NN * 12) S.ncf[tid / 12][tid % 12] *= pow2(55 - S.wexp[(tid % 12) >> 1]);
         __syncthreads();
         bool fits = !S.bad;
-        unsigned mask = 0;
+        unsigned long long mag[NN] = {};
         if (fits)
             for (int i = tid; i < 12 * KW; i += blockDim.x) {
                 const int lp = i / KW, tap = i - lp * KW, l = lp >> 1;
@@ -660,61 +752,68 @@ __device__ void project_block(const FwdParams &P, Shared &S, int T, int64_t k_lo
                 for (int q = 0; q < NN; ++q) {
                     double v = 0.0;
 #pragma unroll
-                    for (int n = 0; n < NN / 2; ++n) v = fma((q & 1) ? o[n] : e[n], P.fx.cheb[q][n], v);
+                    for (int n = 0; n < NN / 2; ++n) v = fma((q & 1) ? o[n] : e[n], X.cheb[q][n], v);
                     b[q] = v;
                 }
-                fits &= coef_store<false, 0>(w, b[0], mask);
-                fits &= coef_store<false, 1>(w, b[1], mask);
-                fits &= coef_store<false, 2>(w, b[2], mask);
-                fits &= coef_store<false, 3>(w, b[3], mask);
-                fits &= coef_store<false, 4>(w, b[4], mask);
-                fits &= coef_store<false, 5>(w, b[5], mask);
-                fits &= coef_store<false, 6>(w, b[6], mask);
-                fits &= coef_store<false, 7>(w, b[7], mask) && fabs(b[7]) < LAST_MAX;
+                fits &= coef_store<false, 0>(w, b[0], mag);
+                fits &= coef_store<false, 1>(w, b[1], mag);
+                fits &= coef_store<false, 2>(w, b[2], mag);
+                fits &= coef_store<false, 3>(w, b[3], mag);
+                fits &= coef_store<false, 4>(w, b[4], mag);
+                fits &= coef_store<false, 5>(w, b[5], mag);
+                fits &= coef_store<false, 6>(w, b[6], mag);
+                fits &= coef_store<false, 7>(w, b[7], mag) && fabs(b[7]) < LAST_MAX;
             }
-        mask = __reduce_or_sync(0xffffffffu, mask);
-        if (lane == 0 && mask) atomicOr(&S.qmask, mask);
+        orders_in_use<NN>(S, mag);
         if (__syncthreads_or(!fits)) {
             bad = true;
             break;
         }
-        const unsigned qm = S.qmask;
+        count_orders<NN>(S);
+        const int nq = S.nq;
+        const bool last = S.last;
         const int js = S.segj[sg], je = S.segj[sg + 1];
-        const int mb0 = js >> 7, nmb = ((je - 1) >> 7) - mb0 + 1;
-        for (int it = warp; it < nmb * 6; it += blockDim.x >> 5) {
-            const int l = it % 6, mb = mb0 + it / 6;
-            const uint32_t a_lane = smem_u32(planes) + 16u * (16u * mb + lr4) + 8u * kp;
-            const uint32_t w_lane = smem_u32(W) + (uint32_t)(2 * l * PD * WS) + 4u * (kp + ((7u - lr4) >> 2));
+        const int mb0 = js >> 6, nmb = ((je - 1) >> 6) - mb0 + 1;
+        // item: 64 rows (16 groups of 4 samples) of two links; column = link, sample within the group
+        for (int it = warp; it < nmb * 3; it += blockDim.x >> 5) {
+            const int lp = it % 3, mb = mb0 + it / 3;
+            const int lw = 2 * lp + (int)(lr4 >> 2);   // the link whose stencil this lane loads
+            const int l = 2 * lp + (int)(kp >> 1);     // the link of this lane's sums
+            const unsigned char *a_lane = reinterpret_cast<const unsigned char *>(planes) + 8 * (16 * mb + (int)lr4) + 8 * kp;
+            const unsigned char *w_lane = W + 2 * lw * PD * WS + 4 + 4 * (kp + ((3 - (lr4 & 3)) >> 2));
             int kappa[4], jr[4];
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
-                jr[r] = 128 * mb + 8 * (int)(lr4 + (r >> 1) * 8) + 2 * (int)kp + (r & 1);
+                jr[r] = 64 * mb + 4 * (int)(lr4 + (r >> 1) * 8) + 2 * (int)(kp & 1) + (r & 1);
                 kappa[r] = 2 * jr[r] + 1 - NY;
             }
             long long b1[4] = {0, 0, 0, 0}, b2[4] = {0, 0, 0, 0};
-            if (qm & 0xf0u) {
+            if (nq > 4) {
                 float acc[4][7][4];
-                contract<4, 4, false>(acc, a_lane, w_lane, sh, nks, nullptr);
+                if (last) contract<4, 4, false, true>(acc, a_lane, w_lane, sh, nks, nullptr);
+                else contract<4, 4, false>(acc, a_lane, w_lane, sh, nks, nullptr);
                 clenshaw<4, 4, false>(acc, kappa, b1, b2);
             }
-            if (qm & 0xfcu) {
+            if (nq > 2) {
                 float acc[2][7][4];
-                contract<2, 2, false>(acc, a_lane, w_lane, sh, nks, nullptr);
+                if (last) contract<2, 2, false, true>(acc, a_lane, w_lane, sh, nks, nullptr);
+                else contract<2, 2, false>(acc, a_lane, w_lane, sh, nks, nullptr);
                 clenshaw<2, 2, false>(acc, kappa, b1, b2);
             }
-            if (qm & 0xfeu) {
+            if (nq > 1) {
                 float acc[1][7][4];
-                contract<1, 1, false>(acc, a_lane, w_lane, sh, nks, nullptr);
+                if (last) contract<1, 1, false, true>(acc, a_lane, w_lane, sh, nks, nullptr);
+                else contract<1, 1, false>(acc, a_lane, w_lane, sh, nks, nullptr);
                 clenshaw<1, 1, false>(acc, kappa, b1, b2);
             }
             float acc[1][7][4];
             contract<0, 1, false>(acc, a_lane, w_lane, sh, nks, nullptr);
-            const double unit = pow2(ex + S.wexp[l] - 57);
+            const int unit = ex + S.wexp[l] - 57;
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
                 const long long v = levels<0>(acc[0], r) + mul_nu<9>(b1[r], kappa[r]) - b2[r];
                 const int64_t k = k_lo + jr[r];
-                if (jr[r] >= js && jr[r] < je) ys[l * NY + jr[r]] = k >= 0 && k < ti.N ? (double)v * unit : 0.0;
+                if (jr[r] >= js && jr[r] < je) ys[l * NY + jr[r]] = k >= 0 && k < ti.N ? from_fixed(v, unit) : 0.0;
             }
         }
     }
@@ -774,33 +873,61 @@ __device__ void project_block(const FwdParams &P, Shared &S, int T, int64_t k_lo
     __syncthreads();
 }
 
-// ---------------------------------------------------------------- the block's X, Y, Z
-// Link rows ys[6][NY] (ny = nb + HL + HR of them, row = output + HL) to outputs; ys is overwritten.
-// Each output is handed to `emit(i, X, Y, Z)` by one thread.
-template <class Emit>
-__device__ void tdi_block(const FwdParams &P, Shared &S, int T, int64_t n0, int nb, double *ys, unsigned char *work,
-                          Emit emit)
+// Chebyshev coefficients of one tap over the block, from the piece's polynomial (degree 5 in its coordinate
+// on [-1, 1]) moved to the block's centre xc and scaled by its half width xs
+__device__ __forceinline__ void table_coefs(const FwdParams &P, const FxTab &X, int piece, int at, double xc, double xs, double *b)
 {
-    const int tid = threadIdx.x, h = (T - 2) / 2, ny = nb + P.HL + P.HR;
-    const uint32_t lane = tid & 31, warp = tid >> 5, lr4 = lane >> 2, kp = lane & 3;
-    const double t_lo = P.t0 + (double)n0 * P.dt;
-    double *wt = reinterpret_cast<double *>(work);
-    uint16_t *planes = reinterpret_cast<uint16_t *>(work);
-    const int xb = T * WTS * 8;
-    unsigned char *W = work + (xb > FX_TDI_PLANES ? xb : FX_TDI_PLANES);
-    const int qn = P.q_terms;
+    const double *c = X.tab + (size_t)piece * FX_TAB_Q * 12 * X.tab_kw + at;
+    const int st = 12 * X.tab_kw;
+    double p[FX_TAB_Q];
+#pragma unroll
+    for (int q = 0; q < FX_TAB_Q; ++q) p[q] = __ldg(c + q * st);
+#pragma unroll
+    for (int k = 0; k < NT; ++k)
+#pragma unroll
+        for (int q = FX_TAB_Q - 2; q >= k; --q) p[q] = fma(xc, p[q + 1], p[q]);
+    const double m1 = p[1] * xs, x2 = xs * xs, m2 = p[2] * x2, m3 = p[3] * (x2 * xs);
+    b[0] = fma(0.5, m2, p[0]);
+    b[1] = fma(0.75, m3, m1);
+    b[2] = 0.5 * m2;
+    b[3] = 0.25 * m3;
+}
 
-    if (tid < NY / 32) S.brk[tid] = 0;
-    if (tid == 32) {
-        S.nlist = 0;
-        S.bad = 0;
-        S.vmax = 0;
-        S.vmin = 0x7fffffffu;
-        S.mmin = 1 << 29;
-        S.mmax = -(1 << 29);
+// Segments of a block on the plan's expansion table (one per spline piece, at most two): their starts and
+// pieces, or 0 when a piece has no entry.  One thread.
+__device__ int table_segments(const FwdParams &P, const FxTab &X, Shared &S, double t_lo, int nb)
+{
+    double x;
+    int a, b;
+    row_at(P.to, t_lo, -1, &x, &a);
+    const double ua = x + (double)a;
+    row_at(P.to, t_lo + (double)(nb - 1) * P.dt, -1, &x, &b);
+    if (b > a + 1 || X.meta[2 * a] == 0 || X.meta[2 * b] == 0) return 0;
+    S.nseg = 1 + (b > a);
+    S.segj[0] = 0;
+    S.segm[0][NTERM] = a;
+    S.segj[S.nseg] = nb;
+    if (b > a) {  // first output of the second piece
+        int i = (int)(((double)b - ua) / (P.dt * P.to.inv_dk)), k;
+        i = i < 2 ? 1 : i - 1;
+        for (; i < nb - 1; ++i) {
+            row_at(P.to, t_lo + (double)i * P.dt, -1, &x, &k);
+            if (k >= b) break;
+        }
+        S.segj[1] = i;
+        S.segm[1][NTERM] = b;
     }
-    if (tid >= 64 && tid < 64 + NGT * 6) {
-        const int g = (tid - 64) / 6, l = (tid - 64) % 6;
+    return 1;
+}
+
+// The TDI's segments where the plan has no table: stencil steps of all delayed reads on a grid of samples
+// and every sample near one; fills segj, segm, nseg, mmin and mmax.
+__device__ void find_tdi_segments(const FwdParams &P, Shared &S, double t_lo, int nb)
+{
+    const int tid = threadIdx.x, qn = P.q_terms;
+    const uint32_t lane = tid & 31, warp = tid >> 5;
+    if (tid < NGT * 6) {
+        const int g = tid / 6, l = tid % 6;
         double x;
         int piece;
         const Coef4 *row = row_at(P.to, t_lo + (double)(g * GT) * P.dt, -1, &x, &piece);
@@ -808,13 +935,6 @@ __device__ void tdi_block(const FwdParams &P, Shared &S, int T, int64_t n0, int 
         if (l == 0) S.mgt[g][NTERM] = piece;
     }
     __syncthreads();
-    // the first and last link rows are spare: no stencil reaches them
-    for (int l = 0; l < 6; ++l)
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            const int j = tid + 256 * i;
-            range_update(S, j >= 1 && j < ny - 1 ? abs_hi(ys[l * NY + j]) : 0u);
-        }
     if (tid < NGT * 6) {
         const int g = tid / 6, cc = tid % 6;
         double D = 0.0;
@@ -872,11 +992,47 @@ __device__ void tdi_block(const FwdParams &P, Shared &S, int T, int64_t n0, int 
             atomicMax(&S.mmax, m);
         }
     }
+}
+
+// ---------------------------------------------------------------- the block's X, Y, Z
+// Link rows ys[6][NY] (ny = nb + HL + HR of them, row = output + HL) to outputs; ys is overwritten.
+// Each output is handed to `emit(i, X, Y, Z)` by one thread.
+template <class Emit>
+__device__ void tdi_block(const FwdParams &P, const FxTab &X, Shared &S, int T, int64_t n0, int nb, double *ys, unsigned char *work,
+                          Emit emit)
+{
+    const int tid = threadIdx.x, h = (T - 2) / 2, ny = nb + P.HL + P.HR;
+    const uint32_t lane = tid & 31, warp = tid >> 5, lr4 = lane >> 2, kp = lane & 3;
+    const double t_lo = P.t0 + (double)n0 * P.dt;
+    double *wt = reinterpret_cast<double *>(work);
+    uint16_t *planes = reinterpret_cast<uint16_t *>(work);
+    const int xb = T * WTS * 8;
+    unsigned char *W = work + (xb > FX_TDI_PLANES ? xb : FX_TDI_PLANES);
+    const int qn = P.q_terms;
+
+    if (tid < NY / 32) S.brk[tid] = 0;
+    if (tid == 32) {
+        S.nlist = 0;
+        S.bad = 0;
+        S.vmax = 0;
+        S.vmin = 0x7fffffffu;
+        S.mmin = 1 << 29;
+        S.mmax = -(1 << 29);
+    }
+    if (tid == 64) S.fast = X.tab ? table_segments(P, X, S, t_lo, nb) : 0;
     __syncthreads();
-    const int mmin = S.mmin, mmax = S.mmax > 0 ? S.mmax : 0;  // the undelayed read sits at 0
-    const int KW = mmax - mmin + T, nks = (KW + 7 + 15) / 16;
-    const int j0 = P.HL + mmin - h;                            // link row of the stencil's first tap for output 0
-    bool bad = S.bad || nks * 16 > 64 || j0 < 1 || mmax > 0;
+    // the first and last link rows are spare: no stencil reaches them
+    for (int l = 0; l < 6; ++l)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int j = tid + 256 * i;
+            range_update(S, j >= 1 && j < ny - 1 ? abs_hi(ys[l * NY + j]) : 0u);
+        }
+    const bool fast = S.fast != 0;
+    if (!fast) find_tdi_segments(P, S, t_lo, nb);
+    __syncthreads();
+    const int nseg = S.nseg;
+    bool bad = S.bad;
     int ey = 0;
     const bool zero = S.vmax == 0;
     if (zero) {
@@ -894,23 +1050,32 @@ __device__ void tdi_block(const FwdParams &P, Shared &S, int T, int64_t n0, int 
     int done = 0;                                          // outputs kept in ys[0..2][.] by earlier segments
     for (int sg = 0; sg < nseg && !bad; ++sg) {
         const int *sm = S.segm[sg];
+        const int piece = sm[NTERM];
+        const int mmin = fast ? X.meta[2 * piece + 1] : S.mmin;
+        const int KW = fast ? X.meta[2 * piece] : (S.mmax > 0 ? S.mmax : 0) - mmin + T;
+        const int nks = (KW + 7 + 15) / 16;
+        const int j0 = P.HL + mmin - h;                        // link row of the stencil's first tap for output 0
+        if (!fast && (nks * 16 > 64 || j0 < 1 || S.mmax > 0)) {
+            bad = true;
+            break;
+        }
         __syncthreads();
         for (int i = tid; i < FX_TDI_W / 16; i += blockDim.x)
             reinterpret_cast<uint4 *>(W)[i] = make_uint4(0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u);
-        if (tid < NT * 6) {
+        if (!fast && tid < NT * 6) {
             const int n = tid / 6, l = tid % 6;
             double x;
-            int piece;
-            const Coef4 *row = row_at(P.to, t_lo + P.fx.tnode_j[n] * P.dt, sm[NTERM], &x, &piece);
+            int k;
+            const Coef4 *row = row_at(P.to, t_lo + X.tnode_j[n] * P.dt, piece, &x, &k);
             S.lnode[n][l] = cubic(ldg4(row + 9 + l), x) * P.inv_dt;
         }
         if (tid == 64) {
-            S.qmask = 0;
             S.cmax[0] = 0;
+            for (int q = 0; q < NT; ++q) S.qor[q] = 0;
         }
         __syncthreads();
         // the node weights take the planes' place; with more than one segment the series is sliced again
-        if (tid < NT * NTERM) {
+        if (!fast && tid < NT * NTERM) {
             const int n = tid / NTERM, tm = tid % NTERM, cc = tm / 7, q = tm % 7 + 1;
             if (q <= qn) {
                 double D = 0.0;
@@ -919,37 +1084,44 @@ __device__ void tdi_block(const FwdParams &P, Shared &S, int T, int64_t n0, int 
             }
         }
         __syncthreads();
-        // merged stencils: the reads of one (channel, link) added tap by tap at the four nodes
+        // merged stencils: the reads of one (channel, link) added tap by tap at the four nodes, or the plan's
+        // table around the block's centre
+        const double xc = 2.0 * ((t_lo + 0.5 * (NY - 1) * P.dt - P.to.t_first) * P.to.inv_dk - (double)piece) - 1.0;
+        const double xs = NY * P.dt * P.to.inv_dk;
         double b[REPS][NT];
         float bm = 0.0f;
 #pragma unroll
         for (int rep = 0; rep < REPS; ++rep) {
             const int i = tid + 256 * rep;
-            double V[NT] = {0.0, 0.0, 0.0, 0.0};
-            if (i < 12 * KW) {
-                const int cs = i / KW, tap = i - cs * KW, ch = cs >> 2, sl = cs & 3;
+            if (i < 12 * KW && fast) {
+                table_coefs(P, X, piece, (i / KW) * X.tab_kw + i % KW, xc, xs, b[rep]);
+            } else {
+                double V[NT] = {0.0, 0.0, 0.0, 0.0};
+                if (i < 12 * KW) {
+                    const int cs = i / KW, tap = i - cs * KW, ch = cs >> 2, sl = cs & 3;
 #pragma unroll
-                for (int x = 0; x < 4; ++x) {
-                    const int tm = c_slots.term[ch][sl][x], c = tm >> 3, q = tm & 7;
-                    if (q > qn) continue;
-                    if (q == 0) {
-                        if (tap == h - mmin) {
+                    for (int x = 0; x < 4; ++x) {
+                        const int tm = c_slots.term[ch][sl][x], c = tm >> 3, q = tm & 7;
+                        if (q > qn) continue;
+                        if (q == 0) {
+                            if (tap == h - mmin) {
 #pragma unroll
-                            for (int n = 0; n < NT; ++n) V[n] += c ? -1.0 : 1.0;
+                                for (int n = 0; n < NT; ++n) V[n] += c ? -1.0 : 1.0;
+                            }
+                            continue;
                         }
-                        continue;
+                        const int id = (ch * 2 + c) * 7 + q - 1, a = tap - (sm[id] - mmin);
+                        if (a < 0 || a >= T) continue;
+                        const double *w = wt + a * WTS + id;
+#pragma unroll
+                        for (int n = 0; n < NT; ++n) V[n] += c ? -w[n * NTERM] : w[n * NTERM];
                     }
-                    const int id = (ch * 2 + c) * 7 + q - 1, a = tap - (sm[id] - mmin);
-                    if (a < 0 || a >= T) continue;
-                    const double *w = wt + a * WTS + id;
-#pragma unroll
-                    for (int n = 0; n < NT; ++n) V[n] += c ? -w[n * NTERM] : w[n * NTERM];
                 }
-            }
-            const double e0 = V[0] + V[3], e1 = V[1] + V[2], o0 = V[0] - V[3], o1 = V[1] - V[2];
+                const double e0 = V[0] + V[3], e1 = V[1] + V[2], o0 = V[0] - V[3], o1 = V[1] - V[2];
 #pragma unroll
-            for (int q = 0; q < NT; ++q)
-                b[rep][q] = (q & 1) ? fma(o0, P.fx.tcheb[q][0], o1 * P.fx.tcheb[q][1]) : fma(e0, P.fx.tcheb[q][0], e1 * P.fx.tcheb[q][1]);
+                for (int q = 0; q < NT; ++q)
+                    b[rep][q] = (q & 1) ? fma(o0, X.tcheb[q][0], o1 * X.tcheb[q][1]) : fma(e0, X.tcheb[q][0], e1 * X.tcheb[q][1]);
+            }
             bm = fmaxf(bm, fabsf((float)b[rep][0]));
         }
         bm = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(bm)));
@@ -959,45 +1131,43 @@ __device__ void tdi_block(const FwdParams &P, Shared &S, int T, int64_t n0, int 
         const int ew = sm_max > 1e-30f && sm_max < 1e30f ? (int)(__float_as_uint(sm_max) >> 23) - 126 : 0;
         const double ws = pow2(55 - ew);
         bool fits = sm_max < 1e30f;
-        unsigned mask = 0;
+        unsigned long long mag[NT] = {};
 #pragma unroll
         for (int rep = 0; rep < REPS; ++rep) {
             const int i = tid + 256 * rep;
             if (i < 12 * KW) {
                 const int cs = i / KW, tap = i - cs * KW;
                 unsigned char *w = W + cs * TD * WS + 7 + tap;
-                fits &= coef_store<true, 0>(w, b[rep][0] * ws, mask);
-                fits &= coef_store<true, 1>(w, b[rep][1] * ws, mask);
-                fits &= coef_store<true, 2>(w, b[rep][2] * ws, mask);
-                fits &= coef_store<true, 3>(w, b[rep][3] * ws, mask);
+                fits &= coef_store<true, 0>(w, b[rep][0] * ws, mag);
+                fits &= coef_store<true, 1>(w, b[rep][1] * ws, mag);
+                fits &= coef_store<true, 2>(w, b[rep][2] * ws, mag);
+                fits &= coef_store<true, 3>(w, b[rep][3] * ws, mag);
             }
         }
-        mask = __reduce_or_sync(0xffffffffu, mask);
-        if (lane == 0 && mask) atomicOr(&S.qmask, mask);
+        orders_in_use<NT>(S, mag);
         if (__syncthreads_or(!fits)) {
             bad = true;
             break;
         }
         const int js = S.segj[sg], je = S.segj[sg + 1];
-        const double scale = pow2(55 - ey);
         // link rows that only earlier outputs read are left out: their place holds those outputs now
         for (int i = tid; i < 6 * DL; i += blockDim.x) {
             const int l = i / DL, p = i - l * DL, j = p + j0;
-            digits_to_planes(planes + l * 7 * DL, p, p >= js && j < ny - 1 ? ys[l * NY + j] : 0.0, scale);
+            digits_to_planes(planes + l * 7 * DL, p, p >= js && j < ny - 1 ? ys[l * NY + j] : 0.0, ey);
         }
         __syncthreads();
-        const unsigned qm = S.qmask;
+        count_orders<NT>(S);
         const int mb0 = js >> 7, nmb = ((je - 1) >> 7) - mb0 + 1;
-        const double unit = pow2(ey + ew - 57);
+        const int unit = ey + ew - 57;
         const uint32_t sh = 8 * ((7 - lr4) & 3);
-        const bool hi = (qm & 14u) != 0;
+        const bool hi = S.nq > 1, last = S.last;
         const int per = nmb * 3;
         if (nseg == 1) {
             // order 0 and the higher orders are separate items (28 and 34 digit products)
             for (int it = warp; it < (hi ? 2 : 1) * per; it += blockDim.x >> 5) {
                 const int half = it / per, ch = it % per % 3, mb = mb0 + it % per / 3;
-                const uint32_t a_lane = smem_u32(planes) + 16u * (16u * mb + lr4) + 8u * kp;
-                const uint32_t w_lane = smem_u32(W) + (uint32_t)(4 * ch * TD * WS) + 4u * (kp + ((7u - lr4) >> 2));
+                const unsigned char *a_lane = reinterpret_cast<const unsigned char *>(planes) + 16 * (16 * mb + (int)lr4) + 8 * kp;
+                const unsigned char *w_lane = W + 4 * ch * TD * WS + 4 * (kp + ((7 - lr4) >> 2));
                 if (half == 0) {
                     float acc[1][7][4];
                     contract<0, 1, true>(acc, a_lane, w_lane, sh, nks, c_slots.link[ch]);
@@ -1006,7 +1176,8 @@ __device__ void tdi_block(const FwdParams &P, Shared &S, int T, int64_t n0, int 
                         part[ch * NY + 128 * mb + 8 * (lr4 + (r >> 1) * 8) + 2 * kp + (r & 1)] = levels<0>(acc[0], r);
                 } else {
                     float acc[3][7][4];
-                    contract<1, 3, true>(acc, a_lane, w_lane, sh, nks, c_slots.link[ch]);
+                    if (last) contract<1, 3, true, true>(acc, a_lane, w_lane, sh, nks, c_slots.link[ch]);
+                    else contract<1, 3, true>(acc, a_lane, w_lane, sh, nks, c_slots.link[ch]);
                     int kappa[4];
                     long long b1[4] = {0, 0, 0, 0}, b2[4] = {0, 0, 0, 0};
 #pragma unroll
@@ -1021,7 +1192,7 @@ __device__ void tdi_block(const FwdParams &P, Shared &S, int T, int64_t n0, int 
             for (int i = tid; i < nb; i += blockDim.x) {
                 double o[3];
 #pragma unroll
-                for (int c = 0; c < 3; ++c) o[c] = (double)(part[c * NY + i] + (hi ? part[(3 + c) * NY + i] : 0)) * unit;
+                for (int c = 0; c < 3; ++c) o[c] = from_fixed(part[c * NY + i] + (hi ? part[(3 + c) * NY + i] : 0), unit);
                 emit(i, o[0], o[1], o[2]);
             }
             done = nb;
@@ -1030,15 +1201,16 @@ __device__ void tdi_block(const FwdParams &P, Shared &S, int T, int64_t n0, int 
             // later segments do not read (their first link row is past output je)
             for (int it = warp; it < per; it += blockDim.x >> 5) {
                 const int ch = it % 3, mb = mb0 + it / 3;
-                const uint32_t a_lane = smem_u32(planes) + 16u * (16u * mb + lr4) + 8u * kp;
-                const uint32_t w_lane = smem_u32(W) + (uint32_t)(4 * ch * TD * WS) + 4u * (kp + ((7u - lr4) >> 2));
+                const unsigned char *a_lane = reinterpret_cast<const unsigned char *>(planes) + 16 * (16 * mb + (int)lr4) + 8 * kp;
+                const unsigned char *w_lane = W + 4 * ch * TD * WS + 4 * (kp + ((7 - lr4) >> 2));
                 int kappa[4];
                 long long b1[4] = {0, 0, 0, 0}, b2[4] = {0, 0, 0, 0};
 #pragma unroll
                 for (int r = 0; r < 4; ++r) kappa[r] = 2 * (128 * mb + 8 * (int)(lr4 + (r >> 1) * 8) + 2 * (int)kp + (r & 1)) + 1 - NY;
                 if (hi) {
                     float acc[3][7][4];
-                    contract<1, 3, true>(acc, a_lane, w_lane, sh, nks, c_slots.link[ch]);
+                    if (last) contract<1, 3, true, true>(acc, a_lane, w_lane, sh, nks, c_slots.link[ch]);
+                    else contract<1, 3, true>(acc, a_lane, w_lane, sh, nks, c_slots.link[ch]);
                     clenshaw<1, 3, true>(acc, kappa, b1, b2);
                 }
                 float acc[1][7][4];
@@ -1046,7 +1218,7 @@ __device__ void tdi_block(const FwdParams &P, Shared &S, int T, int64_t n0, int 
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
                     const int i = (kappa[r] + NY - 1) >> 1;
-                    if (i >= js && i < je) ys[ch * NY + i] = (double)(levels<0>(acc[0], r) + mul_nu<9>(b1[r], kappa[r]) - b2[r]) * unit;
+                    if (i >= js && i < je) ys[ch * NY + i] = from_fixed(levels<0>(acc[0], r) + mul_nu<9>(b1[r], kappa[r]) - b2[r], unit);
                 }
             }
             done = je;
@@ -1082,9 +1254,25 @@ __device__ void tdi_block(const FwdParams &P, Shared &S, int T, int64_t n0, int 
     __syncthreads();
 }
 
+// the source of tile g, by one warp: 32 probes a round
+__device__ __forceinline__ int64_t find_source(const FwdParams &P, int64_t g)
+{
+    const int64_t *to = P.src.tile_off;
+    int64_t lo = 0, hi = P.src.S;  // to[lo] <= g < to[hi]
+    while (hi - lo > 1) {
+        const int64_t step = (hi - lo + 31) >> 5, at = lo + step * ((threadIdx.x & 31) + 1);
+        const unsigned below = __ballot_sync(0xffffffffu, at < hi && __ldg(to + at) <= g);
+        const int64_t n = __popc(below);
+        const int64_t nlo = lo + step * n, nhi = nlo + step;
+        lo = nlo;
+        hi = nhi < hi ? nhi : hi;
+    }
+    return lo;
+}
+
 // ---------------------------------------------------------------- kernel
 template <int KIND>
-__global__ void __launch_bounds__(256, 2) k_fx64(FwdParams P, int T)
+__global__ void __launch_bounds__(256, 2) k_fx64(FwdParams P, FxTab X, int T)
 {
     extern __shared__ __align__(16) unsigned char sm_raw[];
     double *ys = reinterpret_cast<double *>(sm_raw);
@@ -1101,9 +1289,11 @@ __global__ void __launch_bounds__(256, 2) k_fx64(FwdParams P, int T)
     const bool like = KIND == KIND_LIKE;
     const int64_t total = P.total_tiles >= 0 ? P.total_tiles : P.src.tile_off[P.src.S];
     for (int64_t g = blockIdx.x; g < total; g += gridDim.x) {
+        int64_t src = 0;
+        if (tid < 32 && P.src.tile_off) src = find_source(P, g);
         if (tid == 0) {
-            S.ti = tile_info(P, g, KIND == KIND_PROJECT ? 6 : 3);
-            if (KIND != KIND_TDI) S.skc = make_sky(S.ti.sky);
+            S.ti = tile_info_of(P, g, src, KIND == KIND_PROJECT ? 6 : 3);
+            if (KIND != KIND_TDI) S.skc = P.src.tile_off ? P.src.skyc[src] : P.src.skyc1;
             if (!S.ti.ok) atomicOr(P.err, ERR_OFFSETS);
             if (like && !(S.ti.ok && S.ti.nb > 0)) like_store(P, g, 0.0, 0.0);
         }
@@ -1112,7 +1302,7 @@ __global__ void __launch_bounds__(256, 2) k_fx64(FwdParams P, int T)
             const TileInfo &ti = S.ti;
             const int nb = (int)ti.nb;
             if (KIND == KIND_PROJECT) {
-                project_block(P, S, T, ti.n0, nb, (P.t0 - ti.t0h) / P.dt, ys, work);
+                project_block(P, X, S, T, ti.n0, nb, (P.t0 - ti.t0h) / P.dt, ys, work);
                 for (int i = tid; i < nb; i += blockDim.x)
 #pragma unroll
                     for (int l = 0; l < 6; ++l) ti.out[l * ti.N + ti.n0 + i] = ys[l * NY + i];
@@ -1127,20 +1317,20 @@ __global__ void __launch_bounds__(256, 2) k_fx64(FwdParams P, int T)
                         }
                     __syncthreads();
                 } else {
-                    project_block(P, S, T, k_lo, ny, (P.t0 - ti.t0h) / P.dt, ys, work);
+                    project_block(P, X, S, T, k_lo, ny, (P.t0 - ti.t0h) / P.dt, ys, work);
                 }
                 double dh = 0.0, hh = 0.0;
-                tdi_block(P, S, T, ti.n0, nb, ys, work, [&](int i, double X, double Y, double Z) {
+                tdi_block(P, X, S, T, ti.n0, nb, ys, work, [&](int i, double vx, double vy, double vz) {
                     const int64_t n = ti.n0 + i;
                     if (ti.out) {
-                        ti.out[n] = X;
-                        ti.out[ti.N + n] = Y;
-                        ti.out[2 * ti.N + n] = Z;
+                        ti.out[n] = vx;
+                        ti.out[ti.N + n] = vy;
+                        ti.out[2 * ti.N + n] = vz;
                     }
                     if (like && ti.dat) {
                         const double da = __ldg(ti.dat + n), de = __ldg(ti.dat + ti.N + n), dT = __ldg(ti.dat + 2 * ti.N + n);
                         if (!(isfinite(da) && isfinite(de) && isfinite(dT))) atomicOr(P.err, ERR_NONFINITE);
-                        like_terms(P.like, X, Y, Z, da, de, dT, dh, hh);
+                        like_terms(P.like, vx, vy, vz, da, de, dT, dh, hh);
                     }
                 });
                 if (like) {
@@ -1150,6 +1340,114 @@ __global__ void __launch_bounds__(256, 2) k_fx64(FwdParams P, int T)
             }
         }
         __syncthreads();
+    }
+}
+
+// ---------------------------------------------------------------- the plan's TDI table
+// One CTA per spline piece of the TDI orbit: where no delayed read's stencil steps within the piece, the
+// merged stencils of the 12 (channel, link) pairs as polynomials of degree 5 in the piece's coordinate on
+// [-1, 1] (weights at six Chebyshev nodes; over a 1e5 s piece the delays move by ~1e-3 samples, so the next
+// order is below 2^-54).  meta: taps (0: no entry) and the first tap's position.  The stencils depend on the
+// orbit alone; from the table a block's expansion is 20 FP64 operations per tap, against ~130 per read and
+// node computed in the block.
+__global__ void __launch_bounds__(256) k_fx_table(FwdParams P, FxTab X, int T, double *tab, int *meta, int tab_kw)
+{
+    extern __shared__ double wt[];  // [T][TQ * NTERM + 1]
+    constexpr int TQ = FX_TAB_Q, WTT = TQ * NTERM + 1;
+    __shared__ double pc[6][4], eps[TQ][NTERM];
+    __shared__ double lc1[64], lc0[64], rc1[64], rc0[64];
+    __shared__ int mm[NTERM], mmin, mmax, bad;
+    const int tid = threadIdx.x, k = blockIdx.x, h = (T - 2) / 2, qn = P.q_terms;
+    if (tid < T) {
+        lc1[tid] = 1.0 / (double)(tid + 1);
+        lc0[tid] = (double)(h - tid) / (double)(tid + 1);
+        rc1[tid] = 1.0 / (double)(T - tid);
+        rc0[tid] = (double)(h - tid) / (double)(T - tid);
+    }
+    if (tid >= 64 && tid < 70) {  // delays in samples as polynomials of X = 2 x - 1
+        const Coef4 q = ldg4(piece_row(P.to, k) + 9 + tid - 64);
+        double *o = pc[tid - 64];
+        o[0] = (q.a + 0.5 * q.b + 0.25 * q.c + 0.125 * q.d) * P.inv_dt;
+        o[1] = (0.5 * q.b + 0.5 * q.c + 0.375 * q.d) * P.inv_dt;
+        o[2] = (0.25 * q.c + 0.375 * q.d) * P.inv_dt;
+        o[3] = 0.125 * q.d * P.inv_dt;
+    }
+    if (tid == 70) {
+        mmin = 1 << 29;
+        mmax = -(1 << 29);
+        bad = 0;
+    }
+    __syncthreads();
+    if (tid < NTERM && tid % 7 < qn) {
+        const int cc = tid / 7, q = tid % 7 + 1;
+        double D[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int i = 1; i <= q; ++i)
+            for (int c = 0; c < 4; ++c) D[c] += pc[c_tdifx.pair[cc >> 1][cc & 1][i]][c];
+        const double R = fabs(D[1]) + fabs(D[2]) + fabs(D[3]) + 1e-9;
+        const double fl = floor(-D[0]);
+        if (floor(-D[0] - R) != fl || floor(-D[0] + R) != fl || !(fl < 0.0) || !(fl > -1e6)) {
+            bad = 1;
+        } else {
+            mm[tid] = (int)fl;
+            atomicMin(&mmin, (int)fl);
+            atomicMax(&mmax, (int)fl);
+            for (int n = 0; n < TQ; ++n) {
+                const double x = X.tab_node[n];
+                eps[n][tid] = -fma(x, fma(x, fma(x, D[3], D[2]), D[1]), D[0]) - fl;
+            }
+        }
+    }
+    __syncthreads();
+    const int KW = (mmax > 0 ? mmax : 0) - mmin + T;
+    if (bad || KW > tab_kw || KW + 7 > 64 || P.HL + mmin - h < 1) {
+        if (tid == 0) meta[2 * k] = meta[2 * k + 1] = 0;
+        return;
+    }
+    for (int i = tid; i < TQ * NTERM; i += blockDim.x)
+        if (i % 7 < qn) {
+            const double e = eps[i / NTERM][i % NTERM];
+            double L = 1.0, R = 1.0;
+            for (int a = 0; a < T; ++a) {
+                wt[a * WTT + i] = L;
+                L *= fma(e, lc1[a], lc0[a]);
+            }
+            for (int a = T - 1; a >= 0; --a) {
+                wt[a * WTT + i] *= ((T - 1 - a) & 1) ? -R : R;
+                R *= fma(e, rc1[a], rc0[a]);
+            }
+        }
+    __syncthreads();
+    bool ok = true;
+    for (int i = tid; i < 12 * KW; i += blockDim.x) {
+        const int cs = i / KW, tap = i - cs * KW, ch = cs >> 2, sl = cs & 3;
+        double V[TQ], b[TQ];
+        for (int n = 0; n < TQ; ++n) V[n] = 0.0;
+        for (int x = 0; x < 4; ++x) {
+            const int tm = c_slots.term[ch][sl][x], c = tm >> 3, q = tm & 7;
+            if (q > qn) continue;
+            const int id = (ch * 2 + c) * 7 + q - 1, a = q ? tap - (mm[id] - mmin) : (tap == h - mmin ? 0 : -1);
+            if (a < 0 || a >= T) continue;
+            for (int n = 0; n < TQ; ++n) {
+                const double w = q ? wt[a * WTT + n * NTERM + id] : 1.0;
+                V[n] += c ? -w : w;
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < TQ; ++q) {
+            double v = 0.0;
+#pragma unroll
+            for (int n = 0; n < TQ; ++n) v = fma(V[n], X.tab_cheb[q][n], v);
+            b[q] = v;
+        }
+        const double m[TQ] = {b[0] - b[2] + b[4], b[1] - 3.0 * b[3] + 5.0 * b[5], 2.0 * b[2] - 8.0 * b[4],
+                              4.0 * b[3] - 20.0 * b[5], 8.0 * b[4], 16.0 * b[5]};
+        ok &= fabs(m[TQ - 1]) < 9e-13;  // 2^-40: the order left out is then below 2^-54
+        for (int q = 0; q < TQ; ++q) tab[((size_t)k * TQ + q) * 12 * tab_kw + cs * tab_kw + tap] = m[q];
+    }
+    ok = !__syncthreads_or(!ok);
+    if (tid == 0) {
+        meta[2 * k] = ok ? KW : 0;
+        meta[2 * k + 1] = mmin;
     }
 }
 
@@ -1179,23 +1477,97 @@ int fx_max_tile(const FwdParams &P, int order)
     const int T = order + 1;
     const int chain = P.HL - (T - 2) / 2 - 2;  // bound of a chained delay, samples
     // merged stencils within 64 taps with the 7 columns' shift; the sample-by-sample window in its place
-    if (7 + T + chain + 1 > 64 || 7 + T + 2 * P.lproj_b + 2 > 64) return 0;
+    if (7 + T + chain + 1 > 64 || 3 + T + 2 * P.lproj_b + 2 > 57) return 0;
     if (NY + 2 * P.sig_b + P.lproj_b + T + 4 > FX_PROJ_PLANES / 16) return 0;
     return NY - P.HL - P.HR;
 }
 
-void fx_tables(FwdParams &P)
+void fx_tables(const FwdParams &P, FxTab &X)
 {
     const double pi = 3.14159265358979323846;
-    P.fx.icdt = P.inv_dt / C_LIGHT;
-    for (int n = 0; n < NN; ++n) P.fx.node_j[n] = 0.5 * (NY * (1.0 + cos(pi * (2 * n + 1) / (2 * NN))) - 1.0);
+    X.icdt = P.inv_dt / C_LIGHT;
+    for (int n = 0; n < NN; ++n) X.node_j[n] = 0.5 * (NY * (1.0 + cos(pi * (2 * n + 1) / (2 * NN))) - 1.0);
     for (int q = 0; q < NN; ++q)
         for (int n = 0; n < NN / 2; ++n)
-            P.fx.cheb[q][n] = (q ? 2.0 : 1.0) / NN * cos(pi * ((q * (2 * n + 1)) % (4 * NN)) / (2 * NN));
-    for (int n = 0; n < NT; ++n) P.fx.tnode_j[n] = 0.5 * (NY * (1.0 + cos(pi * (2 * n + 1) / (2 * NT))) - 1.0);
+            X.cheb[q][n] = (q ? 2.0 : 1.0) / NN * cos(pi * ((q * (2 * n + 1)) % (4 * NN)) / (2 * NN));
+    for (int n = 0; n < NT; ++n) X.tnode_j[n] = 0.5 * (NY * (1.0 + cos(pi * (2 * n + 1) / (2 * NT))) - 1.0);
     for (int q = 0; q < NT; ++q)
         for (int n = 0; n < NT / 2; ++n)
-            P.fx.tcheb[q][n] = (q ? 2.0 : 1.0) / NT * cos(pi * ((q * (2 * n + 1)) % (4 * NT)) / (2 * NT));
+            X.tcheb[q][n] = (q ? 2.0 : 1.0) / NT * cos(pi * ((q * (2 * n + 1)) % (4 * NT)) / (2 * NT));
+    for (int n = 0; n < FX_TAB_Q; ++n) {
+        X.tab_node[n] = cos(pi * (2 * n + 1) / (2 * FX_TAB_Q));
+        for (int q = 0; q < FX_TAB_Q; ++q)
+            X.tab_cheb[q][n] = (q ? 2.0 : 1.0) / FX_TAB_Q * cos(pi * ((q * (2 * n + 1)) % (4 * FX_TAB_Q)) / (2 * FX_TAB_Q));
+    }
+}
+
+size_t fx_table_bytes(const FwdParams &P, int order)
+{
+    // plans with very many spline pieces work without the table
+    const int T = order + 1, kw = T + (P.HL - (T - 2) / 2 - 2) + 1;
+    const size_t per = sizeof(double) * FX_TAB_Q * 12 * (size_t)kw + 2 * sizeof(int);
+    return P.to.nint <= FX_TAB_PIECES ? per * (size_t)P.to.nint : 0;
+}
+
+int fx_table_build(const FwdParams &P, int order, FxPlan *F)
+{
+    const int T = order + 1, kw = T + (P.HL - (T - 2) / 2 - 2) + 1;
+    double *tab = static_cast<double *>(F->mem);
+    int *meta = reinterpret_cast<int *>(tab + (size_t)P.to.nint * FX_TAB_Q * 12 * kw);
+    const size_t smem = sizeof(double) * (size_t)T * (FX_TAB_Q * NTERM + 1);
+    cudaError_t e = cudaFuncSetAttribute((const void *)k_fx_table, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaEvent_t ev = nullptr;
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+    if (e != cudaSuccess) return (int)e;
+    k_fx_table<<<P.to.nint, 256, smem, 0>>>(P, F->tab, T, tab, meta, kw);
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaEventRecord(ev, 0);
+    if (e != cudaSuccess) {
+        cudaEventDestroy(ev);
+        return (int)e;
+    }
+    F->ready = ev;
+    F->tab.tab = tab;
+    F->tab.meta = meta;
+    F->tab.tab_kw = kw;
+    return 0;
+}
+
+void fx_plan_free(FxPlan *F)
+{
+    if (!F) return;
+    if (F->ready) cudaEventDestroy((cudaEvent_t)F->ready);
+    if (F->mem) cudaFree(F->mem);  // waits for the device
+    delete F;
+}
+
+// The launch's parameters.  Until the table's kernel is known to be done the stream waits for it; a captured
+// launch cannot (the event was recorded outside the capture), there the host waits.
+static int table_for(FxPlan *F, cudaStream_t stream, FxTab *X)
+{
+    *X = F->tab;
+    if (!F->ready) return 0;
+    const cudaEvent_t ev = (cudaEvent_t)F->ready;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(stream, &cap);
+    if (e != cudaSuccess) return (int)e;
+    if (cap != cudaStreamCaptureStatusNone) {
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;  // event calls are refused in the other modes
+        e = cudaThreadExchangeStreamCaptureMode(&mode);
+        if (e != cudaSuccess) return (int)e;
+        e = cudaEventSynchronize(ev);
+        const cudaError_t e2 = cudaThreadExchangeStreamCaptureMode(&mode);
+        if (e == cudaSuccess) e = e2;
+        return (int)e;
+    }
+    e = cudaEventQuery(ev);
+    if (e == cudaErrorNotReady) {
+        cudaGetLastError();
+        return (int)cudaStreamWaitEvent(stream, ev);
+    }
+    if (e != cudaSuccess) return (int)e;
+    F->ready = nullptr;
+    return (int)cudaEventDestroy(ev);
 }
 
 int launch_fx64(int kind, int order, const FwdParams &P, int sms, void *stream)
@@ -1212,7 +1584,9 @@ int launch_fx64(int kind, int order, const FwdParams &P, int sms, void *stream)
     int64_t grid = (int64_t)per_sm * sms;
     if (P.total_tiles >= 0 && P.total_tiles < grid) grid = P.total_tiles;
     if (grid < 1) grid = 1;
-    void *args[] = {(void *)&P, (void *)&T};
+    FxTab X;
+    if (const int te = table_for(P.fx, (cudaStream_t)stream, &X)) return te;
+    void *args[] = {(void *)&P, (void *)&X, (void *)&T};
     return (int)cudaLaunchKernel(k, dim3((unsigned)grid), dim3(256), args, smem, (cudaStream_t)stream);
 }
 

@@ -6,8 +6,13 @@ namespace lr {
 // largest tile (outputs per block) that the tensor-core kernels take for this plan's halos, bounds and
 // order; 0 when they do not apply
 int fx_max_tile(const FwdParams &P, int order);
-// expansion nodes and transforms of the launch parameters
-void fx_tables(FwdParams &P);
+// expansion nodes and transforms
+void fx_tables(const FwdParams &P, FxTab &X);
+// the plan's table of merged TDI stencils over the orbit's spline pieces: its size (0: none) and its
+// computation into F->mem, asynchronous (F->ready); a cudaError_t value
+size_t fx_table_bytes(const FwdParams &P, int order);
+int fx_table_build(const FwdParams &P, int order, FxPlan *F);
+void fx_plan_free(FxPlan *F);
 // returns a cudaError_t value; P.tile + P.HL + P.HR (P.tile for KIND_PROJECT) is at most FX_ROWS
 int launch_fx64(int kind, int order, const FwdParams &P, int sms, void *stream);
 }  // namespace lr

@@ -60,6 +60,8 @@ struct lr_plan {
     int64_t lpart_cap;
     // nested-delay table of the mixed kernels ([knots][42], samples)
     double *d_nest;
+    // tensor-core FP64 kernels: launch constants and expansion table, or null
+    lr::FxPlan *fx;
     // constant-delay TDI weights of the FP64 kernels ([3][2][8][T]), or null
     double *d_cdw;
 };
@@ -317,15 +319,27 @@ int constant_delay_table(lr_plan *p, const lr_orbit *o)
 void fx_setup(lr_plan *p)
 {
     lr::FwdParams &P = p->base;
-    P.fx.tile = 0;
+    P.fx_tile = 0;
     if (p->desc.precision != LR_FP64 || (P.delay_nested && !P.cd_w)) return;
     const int most = lr::fx_max_tile(P, p->desc.order);
     int block = p->tile < most ? p->tile : most;
     while (block >= 128 && p->tile % block) --block;
     if (block < 128 && p->tile >= 128) return;  // no part of at least 128 outputs
-    P.fx.tile = block;
+    if (!p->fx) {
+        p->fx = new (std::nothrow) lr::FxPlan();
+        if (!p->fx) return;
+        lr::fx_tables(P, p->fx->tab);
+        const size_t bytes = lr::fx_table_bytes(P, p->desc.order);
+        // without the table (no memory for it) the blocks compute their own stencils
+        if (bytes && lr::dev_malloc(&p->fx->mem, bytes) == cudaSuccess && lr::fx_table_build(P, p->desc.order, p->fx)) {
+            cudaFree(p->fx->mem);
+            p->fx->mem = nullptr;
+        }
+        cudaGetLastError();
+    }
+    P.fx = p->fx;
+    P.fx_tile = block;
     P.tile = block;
-    lr::fx_tables(P);
 }
 
 bool all_finite(const double *p, size_t n)
@@ -559,6 +573,7 @@ LR_API int lr_plan_create(lr_ctx *ctx, const lr_plan_desc *d, lr_plan **out)
     p->lpart_cap = 0;
     p->d_nest = nullptr;
     p->d_cdw = nullptr;
+    p->fx = nullptr;
     lr::FwdParams &P = p->base;
     std::memset(&P, 0, sizeof(P));
     P.dt = d->dt;
@@ -656,6 +671,7 @@ LR_API int lr_plan_destroy(lr_plan *plan)
     if (plan->d_lpart) cudaFree(plan->d_lpart);
     if (plan->d_nest) cudaFree(plan->d_nest);
     if (plan->d_cdw) cudaFree(plan->d_cdw);
+    lr::fx_plan_free(plan->fx);
     lr::pipe_free(plan->pipe);
     delete plan;
     return LR_OK;
@@ -844,7 +860,7 @@ int response_batched_impl(lr_plan *plan, int64_t S, const int64_t *h_off, const 
     int st = lr::plan_reserve_batch(plan, S);
     if (st) return st;
     lr::FwdParams P = plan->base;
-    lr::SkyConst *skyc = plan->desc.precision == LR_MIXED ? lr::plan_sky_table(plan) : nullptr;
+    lr::SkyConst *skyc = lr::needs_sky_table(plan->desc.precision, P) ? lr::plan_sky_table(plan) : nullptr;
     int e = lr::launch_batch_tables(out_off, sky, S, P.tile, plan->d_tile_off, skyc, P.err, stream);
     if (e) return check_launch(plan->ctx, e);
     P.src.skyc = skyc;
@@ -993,7 +1009,7 @@ int likelihood_batched(lr_plan *plan, int64_t S, const int64_t *h_off, const int
     // sum over sources of ceil(N_s / tile) <= n_total / tile + S
     st = like_setup(plan, weights, n_total / P.tile + S, P, data, n_total);
     if (st) return st;
-    lr::SkyConst *skyc = plan->desc.precision == LR_MIXED ? lr::plan_sky_table(plan) : nullptr;
+    lr::SkyConst *skyc = lr::needs_sky_table(plan->desc.precision, P) ? lr::plan_sky_table(plan) : nullptr;
     int e = lr::launch_batch_tables(out_off, sky, S, P.tile, plan->d_tile_off, skyc, P.err, stream);
     if (e) return check_launch(plan->ctx, e);
     P.src.skyc = skyc;

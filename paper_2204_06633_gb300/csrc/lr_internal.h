@@ -99,12 +99,24 @@ struct LikeArgs {
 // digit planes and stencils
 constexpr int FX_ROWS = 512, FX_NODES = 8, FX_TDI_NODES = 4;
 constexpr int FX_PROJ_PLANES = 14 * (FX_ROWS + 64) * 2, FX_PROJ_W = 12 * 38 * 72;
+constexpr int FX_TAB_Q = 6, FX_TAB_PIECES = 4096;  // polynomial terms and most pieces of the plan's TDI table
 constexpr int FX_TDI_PLANES = 42 * (FX_ROWS + 64) * 2, FX_TDI_W = 12 * 19 * 72;
 struct FxTab {
-    int tile;                                     // outputs per block (0: the plan does not use these kernels)
-    double icdt;                                  // 1 / (c dt)
-    double node_j[FX_NODES], cheb[FX_NODES][FX_NODES / 2];           // node rows, transform (half by symmetry)
+    double icdt;                                                         // 1 / (c dt)
+    double node_j[FX_NODES], cheb[FX_NODES][FX_NODES / 2];               // node rows, transform (half by symmetry)
     double tnode_j[FX_TDI_NODES], tcheb[FX_TDI_NODES][FX_TDI_NODES / 2];
+    double tab_node[FX_TAB_Q], tab_cheb[FX_TAB_Q][FX_TAB_Q];             // of the table's own expansion
+    // merged TDI stencils per spline piece [pieces][FX_TAB_Q][12][tab_kw] and (taps, first tap) per piece; null: none
+    const double *tab;
+    const int *meta;
+    int tab_kw;
+};
+// host side of a plan's tensor-core kernels: launch constants, the table's memory and the event of its
+// computation (null once it is known to be done)
+struct FxPlan {
+    FxTab tab;
+    void *mem;
+    void *ready;
 };
 
 struct FwdParams {
@@ -142,7 +154,8 @@ struct FwdParams {
     // null when the delays vary (FP64 kernels only)
     const double *cd_w;
     int cd_off[3][2][CHAIN_TERMS];
-    FxTab fx;
+    int fx_tile;   // outputs per block of the tensor-core FP64 kernels (0: the plan does not use them)
+    FxPlan *fx;    // host memory, read at launch
 };
 
 // generated strain: the source's waveform sampled on the output grid at every index (the

@@ -19,7 +19,7 @@ int default_tile(int precision, int order)
 int launch_forward(int precision, int kind, int order, FwdParams &P, int threads, int sms, void *stream)
 {
     const bool mx = precision == LR_MIXED;
-    if (!mx && P.fx.tile) return launch_fx64(kind, order, P, sms, stream);
+    if (!mx && P.fx_tile) return launch_fx64(kind, order, P, sms, stream);
     if (mx) threads = MIXED_THREADS;
     size_t smem = 0;
     if (mx) smem_fwdmx(kind, order, P, &smem); else smem_fwd64(kind, order, P, &smem);

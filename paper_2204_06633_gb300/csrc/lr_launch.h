@@ -6,6 +6,8 @@ namespace lr {
 bool order_supported(int order);
 bool precision_supported(int precision);
 int default_tile(int precision, int order);
+// whether the plan's batched launches read the sources' sky frames from a table
+inline bool needs_sky_table(int precision, const FwdParams &P) { return precision == LR_MIXED || P.fx_tile; }
 // returns a cudaError_t value (0 = success)
 int launch_forward(int precision, int kind, int order, FwdParams &P, int threads, int sms, void *stream);
 int launch_tile_offsets(const int64_t *out_off, int64_t S, int tile, int64_t *tile_off, int *err, void *stream);

@@ -90,7 +90,7 @@ extern "C" LR_API int lr_response_batched_noalloc(lr_plan *plan, int64_t S, cons
     if (e) return lr::plan_cuda_fail(plan, e);
     lr::FwdParams P = v.base;
     // every entry of the tables the launch reads is written first by these kernels
-    lr::SkyConst *skyc = v.precision == LR_MIXED ? skytab : nullptr;
+    lr::SkyConst *skyc = lr::needs_sky_table(v.precision, P) ? skytab : nullptr;
     e = lr::launch_batch_tables(out_off, sky, S, P.tile, table, skyc, P.err, stream);
     if (e) return lr::plan_cuda_fail(plan, e);
     P.src.skyc = skyc;

@@ -195,7 +195,7 @@ extern "C" LR_API int lr_response_batched_host(lr_plan *plan, int64_t S, const i
         if (e == cudaSuccess) e = cudaStreamWaitEvent(w.s_run, q.out, 0);
         if (e != cudaSuccess) break;
         FwdParams P = v.base;
-        SkyConst *skyc = v.precision == LR_MIXED ? reinterpret_cast<SkyConst *>(q.tab + (w.cap_s + 1)) : nullptr;
+        SkyConst *skyc = needs_sky_table(v.precision, P) ? reinterpret_cast<SkyConst *>(q.tab + (w.cap_s + 1)) : nullptr;
         int le = launch_batch_tables(q.ooff, q.sky, ns, P.tile, q.tab, skyc, P.err, w.s_run);
         if (!le) {
             P.src.skyc = skyc;

@@ -53,7 +53,7 @@ std::string tune_key(const lr::PlanView &v, int generation, int64_t n)
         if (c == ' ') c = '_';
     int bucket = n > 0 ? (int)std::floor(std::log2((double)n)) : 0;
     char buf[256];
-    std::snprintf(buf, sizeof(buf), "%s|p%d%s|o%d|g%d|b%d", name.c_str(), v.precision, v.base.fx.tile ? "x" : "", v.order,
+    std::snprintf(buf, sizeof(buf), "%s|p%d%s|o%d|g%d|b%d", name.c_str(), v.precision, v.base.fx_tile ? "x" : "", v.order,
                   generation, bucket);
     return buf;
 }
@@ -91,7 +91,7 @@ std::vector<int> tile_candidates(const lr::PlanView &v)
         cand.push_back(tmax);
         for (int t : {256, 192, 128})
             if (t < tmax) cand.push_back(t);
-    } else if (v.base.fx.tile) {
+    } else if (v.base.fx_tile) {
         cand.push_back(lr::fx_max_tile(v.base, v.order));  // the largest block: the work per block hardly depends on it
     } else {
         for (int t : {256, 384, 512, 768, 1024}) cand.push_back(t);
@@ -165,7 +165,7 @@ LR_API int lr_response_batched_graph(lr_plan *plan, int64_t S, const int64_t *h_
         return e == cudaErrorMemoryAllocation ? LR_ERR_OOM : lr::plan_cuda_fail(plan, e);
     }
     lr::SkyConst *skyc =
-        v.precision == LR_MIXED ? reinterpret_cast<lr::SkyConst *>(g->tables + (S + 1)) : nullptr;
+        lr::needs_sky_table(v.precision, v.base) ? reinterpret_cast<lr::SkyConst *>(g->tables + (S + 1)) : nullptr;
     cudaStream_t cs = nullptr;
     e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
@@ -355,7 +355,7 @@ LR_API int lr_plan_autotune_batch(lr_plan *plan, int64_t S, const int64_t *lengt
     int best = tile0;
     double best_ms = 1e300;
     const std::vector<int> cand = tile_candidates(v);
-    lr::SkyConst *skyc = v.precision == LR_MIXED ? reinterpret_cast<lr::SkyConst *>(tables + k + 1) : nullptr;
+    lr::SkyConst *skyc = lr::needs_sky_table(v.precision, v.base) ? reinterpret_cast<lr::SkyConst *>(tables + k + 1) : nullptr;
     for (size_t i = 0; e == cudaSuccess && i < cand.size(); ++i) {
         if (lr::plan_set_tile(plan, cand[i]) != LR_OK) continue;
         lr::PlanView w;
