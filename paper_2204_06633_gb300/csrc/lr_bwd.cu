@@ -486,17 +486,30 @@ __global__ void __launch_bounds__(256) k_sky_adj64(FwdParams P, BwdParams B)
     }
 }
 
-// K4: per source, the tile partials in tile order
-__global__ void k_sky_reduce(const double *partial, const int64_t *tile_off, int64_t S, int64_t ntiles1,
-                             double *g_sky)
+// K4: per source the sum of its tiles' partials, one block per source in a fixed order (thread t takes tiles
+// t, t + 256, ..., then a tree), whatever the launch.  One thread per source walked the tiles one load at a
+// time: 1.89 ms for a year (12 319 tiles), now 31 us.
+__global__ void __launch_bounds__(256) k_sky_reduce(const double *__restrict__ partial, const int64_t *__restrict__ tile_off,
+                                                    int64_t S, int64_t ntiles1, double *__restrict__ g_sky)
 {
-    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= S) return;
-    const int64_t a = tile_off ? tile_off[s] : 0, b = tile_off ? tile_off[s + 1] : ntiles1;
-    double v[3] = {0.0, 0.0, 0.0};
-    for (int64_t t = a; t < b; ++t)
-        for (int c = 0; c < 3; ++c) v[c] += partial[3 * t + c];
-    for (int c = 0; c < 3; ++c) g_sky[3 * s + c] = v[c];
+    __shared__ double red[3][8];
+    for (int64_t s = blockIdx.x; s < S; s += gridDim.x) {
+        const int64_t a = tile_off ? tile_off[s] : 0, b = tile_off ? tile_off[s + 1] : ntiles1;
+        double v[3] = {0.0, 0.0, 0.0};
+        for (int64_t t = a + threadIdx.x; t < b; t += blockDim.x)
+            for (int c = 0; c < 3; ++c) v[c] += partial[3 * t + c];
+        for (int c = 0; c < 3; ++c) {
+            for (int o = 16; o > 0; o >>= 1) v[c] += __shfl_down_sync(0xffffffffu, v[c], o);
+            if ((threadIdx.x & 31) == 0) red[c][threadIdx.x >> 5] = v[c];
+        }
+        __syncthreads();
+        if (threadIdx.x < 3) {
+            double x = 0.0;
+            for (int w = 0; w < 8; ++w) x += red[threadIdx.x][w];
+            g_sky[3 * s + threadIdx.x] = x;
+        }
+        __syncthreads();
+    }
 }
 
 // ---------------------------------------------------------------- dispatch
@@ -547,9 +560,8 @@ int launch_bwd(int kind, int order, const FwdParams &P, const BwdParams &B, int 
 int launch_sky_reduce(const double *partial, const int64_t *tile_off, int64_t S, int64_t ntiles1, double *g_sky,
                       void *stream)
 {
-    const int threads = 128;
-    const int64_t blocks = (S + threads - 1) / threads;
-    k_sky_reduce<<<(unsigned)blocks, threads, 0, (cudaStream_t)stream>>>(partial, tile_off, S, ntiles1, g_sky);
+    const int64_t blocks = S < 4096 ? S : 4096;
+    k_sky_reduce<<<(unsigned)blocks, 256, 0, (cudaStream_t)stream>>>(partial, tile_off, S, ntiles1, g_sky);
     return (int)cudaGetLastError();
 }
 

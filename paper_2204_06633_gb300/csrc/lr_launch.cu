@@ -139,23 +139,24 @@ __global__ void __launch_bounds__(256) k_like_reduce(const double *__restrict__ 
 // respect to the template's X, Y, Z: g = scale * M^T W (d - M x), M the A, E, T map (rows
 // (-1, 0, 1)/sqrt 2, (1, -2, 1)/sqrt 6, (1, 1, 1)/sqrt 3).  Source s (of S) holds [3][N_s] at
 // 3 out_off[s] in x, d and g, which hold n1 samples per channel block (sources past them are
-// skipped and recorded); out_off == nullptr: one source of n1 samples.  Blocks walk sources,
-// threads walk samples.
+// skipped and recorded); out_off == nullptr: one source of n1 samples.  HBM bound (48 B read, 24 B written
+// per sample): grid rows walk sources, the blocks of a row share a source's samples (one block per source
+// left the chip idle for few sources: 400 us for 65536 samples, now 6).
 __global__ void __launch_bounds__(256) k_like_grad(const int64_t *__restrict__ out_off, int64_t S, int64_t n1,
                                                    const double *__restrict__ x, const double *__restrict__ d,
                                                    double w0, double w1, double w2, double scale,
                                                    double *__restrict__ g, int *err)
 {
     const double R2 = 0.70710678118654752440, R6 = 0.40824829046386301637, R3 = 0.57735026918962576451;
-    for (int64_t s = blockIdx.x; s < S; s += gridDim.x) {
+    for (int64_t s = blockIdx.y; s < S; s += gridDim.y) {
         const int64_t o = out_off ? out_off[s] : 0, N = out_off ? out_off[s + 1] - o : n1;
         if (N < 0 || o < 0 || o + N > n1) {
-            if (threadIdx.x == 0) atomicOr(err, ERR_OFFSETS);
+            if (threadIdx.x == 0 && blockIdx.x == 0) atomicOr(err, ERR_OFFSETS);
             continue;
         }
         const double *xs = x + 3 * o, *ds = d + 3 * o;
         double *gs = g + 3 * o;
-        for (int64_t i = threadIdx.x; i < N; i += blockDim.x) {
+        for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
             const double X = xs[i], Y = xs[N + i], Z = xs[2 * N + i];
             const double s2 = X + Z;
             const double ra = w0 * (ds[i] - (Z - X) * R2), re = w1 * (ds[N + i] - fma(-2.0, Y, s2) * R6),
@@ -171,8 +172,11 @@ __global__ void __launch_bounds__(256) k_like_grad(const int64_t *__restrict__ o
 int launch_like_grad(const int64_t *out_off, int64_t S, int64_t n1, const double *x, const double *d,
                      const double *w, double scale, double *g, int *err, void *stream)
 {
-    const int64_t blocks = S < 4096 ? S : 4096;
-    k_like_grad<<<(unsigned)blocks, 256, 0, (cudaStream_t)stream>>>(out_off, S, n1, x, d, w[0], w[1], w[2], scale, g,
+    const int64_t rows = S < 4096 ? S : 4096;
+    // about one pass of the threads over a source of mean length, at most ~16 blocks per SM in all
+    int64_t cols = (n1 / S + 255) / 256, most = (152 * 16 + rows - 1) / rows;
+    cols = cols < 1 ? 1 : (cols > most ? most : cols);
+    k_like_grad<<<dim3((unsigned)cols, (unsigned)rows), 256, 0, (cudaStream_t)stream>>>(out_off, S, n1, x, d, w[0], w[1], w[2], scale, g,
                                                                    err);
     return (int)cudaGetLastError();
 }
