@@ -1,0 +1,1016 @@
+// Adjoint kernels on the tensor cores: the transposes of the TDI and projection operators and the sky-angle
+// gradient, for FP64 and mixed plans alike (FP64 accuracy).
+//
+// The gathers of lr_bwd.cu (FP64) and lr_bwdmx.cu (float-float) spend ~50 FP64 or ~1000 FP32 operations per
+// tap on weights and sums.  Here the merged, expanded stencils of lr_fx64.cu are transposed: with
+// W(t) = sum_q b_q T_q(nu(t)) the transpose of  y[j] = sum_c W(t_j)[c] x[j + c]  is
+//      gx[i] = sum_q sum_c b_q[c] (T_q gy)[i - c],
+// a contraction with constant stencils (taps in reverse) of the series T_q(nu_j) gy_j, formed in fixed point by
+// Chebyshev's recurrence.  All orders, links and channels of one output meet in the same level sums.
+//   K1  g_y = T^T g_xyz    blocks of link samples; three channels, four orders, stencils of the plan's table.
+//   K2  g_h = P^T g_y      blocks of strain samples; six links, eight orders; h+ and hx are the columns' halves.
+//   K3  dLoss/d(lambda, beta, psi)   blocks of link samples: with y[k] = sum_n V_n(k) h[k + c] over the
+//       expansion nodes, the gradient is the inner product of dV_n/dtheta with the correlations
+//       C_q[c] = sum_k T_q(nu_k) gy[k] h[k + c], which are contractions over the block's samples; the node
+//       values (weights, their derivatives, geometry) are then needed 8 times per block, not per sample.
+// Segments (stencil steps, spline knots), ranges and the blocks evaluated sample by sample are as in lr_fx64.cu.
+//
+// Measured (one year at order 41, mixed plan): K1 5.97 -> 1.65, K2 12.16 -> 4.45, K3 12.2 -> 6.34 ms;
+// 65536 samples at order 25 (FP64 plan): K1 1.26 -> 0.063, K2 0.42 -> 0.116, K3 0.64 -> 0.175 ms.
+#include "lr_fx64.cuh"
+
+#include "lr_bwd.h"
+
+namespace lr {
+namespace {
+
+// digit planes of T_q g: digits that order q's products need (one more than its levels, up to seven)
+__host__ __device__ constexpr int gdigits(bool tdi, int q) { return zq(tdi, q) ? 8 - zq(tdi, q) : 7; }
+__host__ __device__ constexpr int gplane(bool tdi, int q)  // planes before order q
+{
+    return tdi ? (q == 0 ? 0 : q == 1 ? 7 : q == 2 ? 14 : q == 3 ? 19 : 22)
+               : (q <= 3 ? 7 * q : q == 4 ? 27 : q == 5 ? 32 : q == 6 ? 37 : q == 7 ? 41 : 44);
+}
+constexpr int TQP = gplane(true, NT);                         // 22 planes of a channel
+constexpr int QA = 3, PQA = gplane(false, QA), PQB = gplane(false, NN) - PQA;  // a link in two rounds: 21 and 23 planes
+constexpr int GB = 516;                                       // bytes of a digit row of T_q g (K3): distinct banks per link
+constexpr int GROWS = gplane(false, NN);                      // 44 rows per link
+
+constexpr int K1_PART = 3 * NY * 8, K1_PLANES = K1_PART + 6 * NY * 8;
+// the node weights of blocks off the table share the sums' and planes' place
+__host__ __device__ constexpr int k1_w(int T) { return K1_PART + (T * WTS * 8 > 6 * NY * 8 + TQP * DL * 2 ? T * WTS * 8 : 6 * NY * 8 + TQP * DL * 2); }
+constexpr int K2_PLANES = 6 * NY * 8, K2_W = K2_PLANES + PQB * DL * 2, K2_END = K2_W + FX_PROJ_W;
+constexpr int K3_G = FX_PROJ_PLANES, K3_GEND = K3_G + 2 * GROWS * GB;
+
+// acc[L] += the level sums of order Q, its digit planes at `a_lane`, its digit rows at `w_lane`
+template <int Q, bool TDI, bool LAST>
+__device__ __forceinline__ void contract_order(float (&acc)[7][4], const unsigned char *a_lane, const unsigned char *w_lane,
+                                               uint32_t sh, int nks)
+{
+    constexpr int Z = LAST ? 6 : zq(TDI, Q), Z0 = zq(TDI, Q), NA = Z ? 8 - Z : 7, RS = TDI ? 16 : 8;
+#pragma unroll 1
+    for (int ks = 0; ks < nks; ++ks, a_lane += 32, w_lane += 16) {
+        uint32_t a[NA][4];
+#pragma unroll
+        for (int k = 0; k < NA; ++k) {
+            const uint2 lo = *reinterpret_cast<const uint2 *>(a_lane + k * DL * 2);
+            const uint2 hi = *reinterpret_cast<const uint2 *>(a_lane + k * DL * 2 + 8 * RS);
+            a[k][0] = lo.x; a[k][1] = hi.x; a[k][2] = lo.y; a[k][3] = hi.y;
+        }
+#pragma unroll
+        for (int d = Z; d < 7; ++d) {
+            const uint32_t *w = reinterpret_cast<const uint32_t *>(w_lane + (d - Z0) * WS);
+            const uint32_t u = __funnelshift_r(w[0], w[1], sh);
+            const uint32_t b0 = digits_h2(u, 0x4140u), b1 = digits_h2(u, 0x4342u);
+#pragma unroll
+            for (int k = 0; k < 6 - d; ++k) mma_f16(acc[d + k], a[k], b0, b1);
+            if (d == 0) {
+                mma_f16(acc[6], a[6], b0, b1);
+            } else {
+                uint32_t x[4];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) x[r] = extend_h2(a[6 - d][r], a[7 - d][r]);
+                mma_f16(acc[6], x, b0, b1);
+            }
+        }
+    }
+}
+
+// digits 0 .. N - 1 of X (units of 2^-55) into planes
+template <int N>
+__device__ __forceinline__ void put_digits(uint16_t *pl, int p, long long X)
+{
+    X += DIGIT_BIAS;
+    const uint32_t lo = (uint32_t)X, hi = (uint32_t)(X >> 32);
+    const uint32_t d[7] = {(uint32_t)((int)(X >> 48) + 128), (hi >> 8) & 255u, hi & 255u, lo >> 24, (lo >> 16) & 255u, (lo >> 8) & 255u, lo & 255u};
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        uint32_t r;
+        asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(0x6400u + d[i]), "r"(0x6480u));
+        pl[i * DL + p] = (uint16_t)r;
+    }
+}
+
+__device__ __forceinline__ void reset_range(Shared &S)
+{
+    S.bad = 0;
+    S.vmax = 0;
+    S.vmin = 0x7fffffffu;
+}
+
+__device__ __forceinline__ void lagrange_tables(Shared &S, int T)
+{
+    const int tid = threadIdx.x, h = (T - 2) / 2;
+    if (tid < T) {
+        S.lc1[tid] = 1.0 / (double)(tid + 1);
+        S.lc0[tid] = (double)(h - tid) / (double)(tid + 1);
+        S.rc1[tid] = 1.0 / (double)(T - tid);
+        S.rc0[tid] = (double)(h - tid) / (double)(T - tid);
+    }
+}
+
+// the sky frame of a single-source launch, by the first warp (the three angles' sines on three lanes); the same
+// arithmetic as the batched launches' table
+__device__ __forceinline__ void sky_by_warp(const lr_sky &sky, SkyConst *out)
+{
+    const int lane = threadIdx.x & 31;
+    double s, c;
+    sincos(lane == 0 ? sky.lam : lane == 1 ? sky.beta : 2.0 * sky.psi, &s, &c);
+    const double sl = __shfl_sync(0xffffffffu, s, 0), cl = __shfl_sync(0xffffffffu, c, 0);
+    const double sb = __shfl_sync(0xffffffffu, s, 1), cb = __shfl_sync(0xffffffffu, c, 1);
+    const double s2 = __shfl_sync(0xffffffffu, s, 2), c2 = __shfl_sync(0xffffffffu, c, 2);
+    if (lane == 0) {
+        SkyConst k;
+        k.k[0] = -cb * cl; k.k[1] = -cb * sl; k.k[2] = -sb;
+        k.u[0] = sl;       k.u[1] = -cl;      k.u[2] = 0.0;
+        k.v[0] = -sb * cl; k.v[1] = -sb * sl; k.v[2] = cb;
+        k.c2p = c2; k.s2p = s2;
+        *out = k;
+    }
+}
+
+// ---------------------------------------------------------------- K1: TDI transpose
+// Chunks of 16 outputs: the weights of a chain's seven reads at each, then every link sample gathers the taps
+// that land on it (blocks that the table or the fixed point does not cover).
+__device__ void tdi_adj_scalar(const FwdParams &P, Shared &S, int T, int64_t k0, int nb, const double *gs, double *gy,
+                               int64_t N, double *w)
+{
+    const int tid = threadIdx.x, h = (T - 2) / 2, qn = P.q_terms;
+    const int64_t n_lo = k0 - h - 1;
+    int *mo = reinterpret_cast<int *>(w + 112 * T);
+    double acc[2][6];
+    for (int r = 0; r < 2; ++r)
+        for (int l = 0; l < 6; ++l) acc[r][l] = 0.0;
+    for (int p0 = 0; p0 < NY; p0 += 16)
+        for (int cc = 0; cc < 6; ++cc) {
+            const int ch = cc >> 1, c = cc & 1;
+            __syncthreads();
+            if (tid < 112) {
+                const int j = tid & 15, q = (tid >> 4) + 1;
+                if (q <= qn) {
+                    int piece;
+                    const double u = -chain_delay(P, P.t0 + (double)(n_lo + p0 + j) * P.dt, cc * 7 + q - 1, &piece), fl = floor(u);
+                    mo[tid] = (int)fl;
+                    lagrange_to(S, T, u - fl, w + tid, 112);
+                }
+            }
+            __syncthreads();
+            for (int r = 0; r < 2; ++r) {
+                const int i = tid + 256 * r;
+                if (i >= nb) continue;
+                for (int j = 0; j < 16; ++j) {
+                    const double g = gs[ch * NY + p0 + j];
+                    if (g == 0.0) continue;
+                    for (int q = 0; q <= qn; ++q) {
+                        const int64_t n = n_lo + p0 + j;
+                        double t;
+                        if (q == 0) {
+                            if (n != k0 + i) continue;
+                            t = g;
+                        } else {
+                            const int id = (q - 1) * 16 + j;
+                            const int a = (int)(k0 + i - (n + mo[id])) + h;
+                            if (a < 0 || a >= T) continue;
+                            t = w[a * 112 + id] * g;
+                        }
+                        const int l = c_tdifx.link[ch][c][q];
+#pragma unroll
+                        for (int m = 0; m < 6; ++m)
+                            if (m == l) acc[r][m] += c ? -t : t;
+                    }
+                }
+            }
+        }
+    for (int r = 0; r < 2; ++r)
+        if (tid + 256 * r < nb)
+            for (int l = 0; l < 6; ++l) gy[l * N + k0 + tid + 256 * r] = acc[r][l];
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(256, 2) k_fx_tdi_adj(FwdParams P, FxTab X, BwdParams B, int T)
+{
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    double *gs = reinterpret_cast<double *>(sm_raw);
+    long long *part = reinterpret_cast<long long *>(sm_raw + K1_PART);
+    uint16_t *planes = reinterpret_cast<uint16_t *>(sm_raw + K1_PLANES);
+    double *wt = reinterpret_cast<double *>(sm_raw + K1_PART);  // node weights, before the sums and planes
+    unsigned char *W = sm_raw + k1_w(T);
+    __shared__ Shared S;
+    const int tid = threadIdx.x, h = (T - 2) / 2;
+    const int lane = tid & 31, warp = tid >> 5, lr4 = lane >> 2, kp = lane & 3;
+    const uint32_t sh = 8 * ((7 - lr4) & 3);
+    lagrange_tables(S, T);
+    const int64_t total = P.total_tiles >= 0 ? P.total_tiles : P.src.tile_off[P.src.S];
+    for (int64_t g = blockIdx.x; g < total; g += gridDim.x) {
+        int64_t src = 0;
+        if (tid < 32 && P.src.tile_off) src = find_source(P, g);
+        if (tid == 0) {
+            S.ti = tile_info_of(P, g, src, 3);
+            if (!S.ti.ok) atomicOr(P.err, ERR_OFFSETS);
+            reset_range(S);
+        }
+        __syncthreads();
+        if (!S.ti.ok || S.ti.nb <= 0) {
+            __syncthreads();
+            continue;
+        }
+        const int64_t N = S.ti.N, k0 = S.ti.n0, n_lo = k0 - h - 1;
+        const int nb = (int)S.ti.nb;
+        const int rows = nb + X.tab_kw - 1 < NY ? nb + X.tab_kw - 1 : NY;
+        const double t_lo = P.t0 + (double)n_lo * P.dt;
+        const double *gx = B.g_xyz + (S.ti.out - P.out);
+        double *gy = B.g_y + 2 * (S.ti.out - P.out);
+        bool any = false;
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const int p = tid + 256 * r;
+                const int64_t n = n_lo + p;
+                const double v = p < rows && n >= 0 && n < N ? __ldg(gx + c * N + n) : 0.0;
+                gs[c * NY + p] = v;
+                any |= v != 0.0;
+                range_update(S, abs_hi(v));
+            }
+        if (tid < NY / 32) S.brk[tid] = 0;
+        if (tid == 0) {
+            S.fast = table_segments(P, X, S, t_lo, rows);
+            S.nlist = 0;
+            S.mmin = 1 << 29;
+            S.mmax = -(1 << 29);
+        }
+        if (!__syncthreads_or(any)) {
+            for (int i = tid; i < nb; i += blockDim.x)
+                for (int l = 0; l < 6; ++l) gy[l * N + k0 + i] = 0.0;
+            __syncthreads();
+            continue;
+        }
+        int eg = 0;
+        const bool fast = S.fast != 0;
+        if (!fast) find_tdi_segments(P, S, t_lo, rows);
+        __syncthreads();
+        bool bad = S.bad || !range_ok(S, &eg);
+        const int nseg = S.nseg;
+        for (int sg = 0; sg < nseg && !bad; ++sg) {
+            const int piece = S.segm[sg][NTERM], mmin = fast ? X.meta[2 * piece + 1] : S.mmin, KW = T - mmin, nks = (KW + 7 + 15) / 16;
+            const int js = S.segj[sg], je = S.segj[sg + 1];
+            int ew;
+            if (nks * 16 > 64 || nb + KW - 1 > rows || (!fast && S.mmax >= 0) ||
+                !tdi_stencils<true>(P, X, S, T, t_lo, sg, fast, KW, mmin, W, wt, &ew)) {
+                bad = true;
+                break;
+            }
+            count_orders<NT>(S);
+            const int nq = S.nq;
+            const bool last = S.last;
+            for (int ch = 0; ch < 3; ++ch) {
+                // the channel's series times T_q in digits, zero outside the segment
+                for (int p = tid; p < DL; p += blockDim.x) {
+                    const bool in = p >= js && p < je;
+                    const long long x0 = in ? to_fixed(gs[ch * NY + p], eg) : 0;
+                    const int kappa = 2 * p + 1 - NY;
+                    const long long x1 = in ? mul_nu<9>(x0, kappa) : 0;
+                    const long long x2 = in ? mul_nu<8>(x1, kappa) - x0 : 0;
+                    const long long x3 = in ? mul_nu<8>(x2, kappa) - x1 : 0;
+                    put_digits<gdigits(true, 0)>(planes + gplane(true, 0) * DL, p, x0);
+                    put_digits<gdigits(true, 1)>(planes + gplane(true, 1) * DL, p, x1);
+                    put_digits<gdigits(true, 2)>(planes + gplane(true, 2) * DL, p, x2);
+                    put_digits<gdigits(true, 3)>(planes + gplane(true, 3) * DL, p, x3);
+                }
+                __syncthreads();
+                for (int it = warp; it < 16; it += blockDim.x >> 5) {
+                    const int sl = it & 3, mb = it >> 2;
+                    if (128 * mb >= nb) continue;
+                    const int l = c_slots.link[ch][sl];
+                    const unsigned char *a_lane = reinterpret_cast<const unsigned char *>(planes) + 16 * (16 * mb + lr4) + 8 * kp;
+                    const unsigned char *w_lane = W + (ch * 4 + sl) * TD * WS + 4 * (kp + ((7 - lr4) >> 2));
+                    float acc[7][4] = {};
+                    contract_order<0, true, false>(acc, a_lane, w_lane, sh, nks);
+                    if (last) {
+                        if (nq > 1) contract_order<1, true, true>(acc, a_lane + gplane(true, 1) * DL * 2, w_lane + digit_row(true, 1) * WS, sh, nks);
+                        if (nq > 2) contract_order<2, true, true>(acc, a_lane + gplane(true, 2) * DL * 2, w_lane + digit_row(true, 2) * WS, sh, nks);
+                        if (nq > 3) contract_order<3, true, true>(acc, a_lane + gplane(true, 3) * DL * 2, w_lane + digit_row(true, 3) * WS, sh, nks);
+                    } else {
+                        if (nq > 1) contract_order<1, true, false>(acc, a_lane + gplane(true, 1) * DL * 2, w_lane + digit_row(true, 1) * WS, sh, nks);
+                        if (nq > 2) contract_order<2, true, false>(acc, a_lane + gplane(true, 2) * DL * 2, w_lane + digit_row(true, 2) * WS, sh, nks);
+                        if (nq > 3) contract_order<3, true, false>(acc, a_lane + gplane(true, 3) * DL * 2, w_lane + digit_row(true, 3) * WS, sh, nks);
+                    }
+                    bool first = true;   // each link is in two channels
+                    for (int c2 = 0; c2 < ch; ++c2)
+                        for (int s2 = 0; s2 < 4; ++s2) first &= c_slots.link[c2][s2] != l;
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        long long *o = part + l * NY + 128 * mb + 8 * (lr4 + (r >> 1) * 8) + 2 * kp + (r & 1);
+                        const long long v = levels<0>(acc, r);
+                        *o = first ? v : *o + v;
+                    }
+                }
+                __syncthreads();
+            }
+            const int unit = eg + ew - 57;
+            for (int i = tid; i < nb; i += blockDim.x)
+#pragma unroll
+                for (int l = 0; l < 6; ++l) {
+                    const double v = from_fixed(part[l * NY + i], unit);
+                    double *o = gy + l * N + k0 + i;
+                    *o = sg ? *o + v : v;
+                }
+        }
+        __syncthreads();
+        if (bad) tdi_adj_scalar(P, S, T, k0, nb, gs, gy, N, reinterpret_cast<double *>(sm_raw + K1_PART));
+        __syncthreads();
+    }
+}
+
+// ---------------------------------------------------------------- K2: projection transpose
+// the nine reads' coefficients of one link sample: U positions, CF[18] (read, polarisation)
+__device__ void proj_adj_sample(const FwdParams &P, const SkyConst &K, double u0, int64_t k, int64_t N, const double *gyk,
+                                double *U, double *CF, int st)
+{
+    for (int rd = 0; rd < 9; ++rd) {
+        U[rd * st] = u0;
+        CF[2 * rd * st] = CF[(2 * rd + 1) * st] = 0.0;
+    }
+    if (k < 0 || k >= N) return;
+    double x[9], L[6], sig[3];
+    orbit_all(P.po, P.t0 + (double)k * P.dt, x, L);
+    for (int i = 0; i < 3; ++i) {
+        sig[i] = (K.k[0] * x[3 * i] + K.k[1] * x[3 * i + 1] + K.k[2] * x[3 * i + 2]) / C_LIGHT * P.inv_dt;
+        U[i * st] = u0 - sig[i];
+    }
+    for (int l = 0; l < 6; ++l) {
+        const int r = c_lr[l], s = c_ls[l];
+        double d0 = x[3 * r] - x[3 * s], d1 = x[3 * r + 1] - x[3 * s + 1], d2 = x[3 * r + 2] - x[3 * s + 2];
+        const double inv = 1.0 / sqrt(d0 * d0 + d1 * d1 + d2 * d2);
+        d0 *= inv; d1 *= inv; d2 *= inv;
+        const double un = K.u[0] * d0 + K.u[1] * d1 + K.u[2] * d2, vn = K.v[0] * d0 + K.v[1] * d1 + K.v[2] * d2;
+        const double kn = K.k[0] * d0 + K.k[1] * d1 + K.k[2] * d2;
+        const double xip = un * un - vn * vn, xic = 2.0 * un * vn;
+        const double gl = gyk[l * NY] * (1.0 / (2.0 * (1.0 - kn)));
+        const double cp = gl * (K.c2p * xip + K.s2p * xic), cc = gl * (-K.s2p * xip + K.c2p * xic);
+        U[(3 + l) * st] = u0 - L[l] * P.inv_dt - sig[s];
+        CF[2 * (3 + l) * st] = cp;
+        CF[(2 * (3 + l) + 1) * st] = cc;
+        CF[2 * r * st] -= cp;
+        CF[(2 * r + 1) * st] -= cc;
+    }
+}
+
+__device__ void proj_adj_scalar(const FwdParams &P, Shared &S, int T, double u0, int64_t i0, int nb, int64_t k_lo,
+                                const double *gys, double *ghp, double *ghc, double *w)
+{
+    const int tid = threadIdx.x, h = (T - 2) / 2;
+    double *U = w + 72 * T, *CF = U + 72;   // chunks of 8 link samples: 72 reads
+    double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+    for (int j0 = 0; j0 < NY; j0 += 8) {
+        __syncthreads();
+        if (tid < 8) proj_adj_sample(P, S.skc, u0, k_lo + j0 + tid, S.ti.N, gys + j0 + tid, U + tid, CF + tid, 8);
+        __syncthreads();
+        if (tid < 72) lagrange_to(S, T, U[tid] - floor(U[tid]), w + tid, 72);
+        __syncthreads();
+        for (int r = 0; r < 2; ++r) {
+            const int i = tid + 256 * r;
+            if (i >= nb) continue;
+            for (int id = 0; id < 72; ++id) {
+                const int64_t a = i0 + i - (k_lo + j0 + (id & 7) + (int64_t)floor(U[id])) + h;
+                if (a < 0 || a >= T) continue;
+                acc[r][0] = fma(w[a * 72 + id], CF[2 * (id >> 3) * 8 + (id & 7)], acc[r][0]);
+                acc[r][1] = fma(w[a * 72 + id], CF[(2 * (id >> 3) + 1) * 8 + (id & 7)], acc[r][1]);
+            }
+        }
+    }
+    for (int r = 0; r < 2; ++r)
+        if (tid + 256 * r < nb) {
+            ghp[i0 + tid + 256 * r] = acc[r][0];
+            ghc[i0 + tid + 256 * r] = acc[r][1];
+        }
+    __syncthreads();
+}
+
+// planes of T_q g for orders Q0 .. Q1 - 1 at row p, from x0 = g in fixed point
+template <int Q0, int Q1>
+__device__ __forceinline__ void order_planes(uint16_t *planes, int p, long long x0, int kappa, bool in)
+{
+    long long xa = x0, xb = in ? mul_nu<9>(x0, kappa) : 0;
+#pragma unroll
+    for (int q = 0; q < Q1; ++q) {
+        // xa = T_q g, xb = T_{q+1} g
+        uint16_t *pl = planes + (gplane(false, q) - gplane(false, Q0)) * DL;
+        if (q >= Q0) {
+            if (gdigits(false, q) == 7) put_digits<7>(pl, p, xa);
+            else if (gdigits(false, q) == 6) put_digits<6>(pl, p, xa);
+            else if (gdigits(false, q) == 5) put_digits<5>(pl, p, xa);
+            else if (gdigits(false, q) == 4) put_digits<4>(pl, p, xa);
+            else put_digits<3>(pl, p, xa);
+        }
+        const long long nx = in ? mul_nu<8>(xb, kappa) - xa : 0;
+        xa = xb;
+        xb = nx;
+    }
+}
+
+template <int Q, bool LAST>
+__device__ __forceinline__ void proj_order(float (&acc)[7][4], const unsigned char *a_lane, const unsigned char *w_lane,
+                                           uint32_t sh, int nks)
+{
+    constexpr int base = Q < QA ? 0 : PQA;
+    contract_order<Q, false, LAST>(acc, a_lane + (gplane(false, Q) - base) * DL * 2, w_lane + digit_row(false, Q) * WS, sh, nks);
+}
+
+__global__ void __launch_bounds__(256, 2) k_fx_proj_adj(FwdParams P, FxTab X, BwdParams B, int T)
+{
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    double *gys = reinterpret_cast<double *>(sm_raw);
+    uint16_t *planes = reinterpret_cast<uint16_t *>(sm_raw + K2_PLANES);
+    unsigned char *W = sm_raw + K2_W;
+    double *wn = reinterpret_cast<double *>(sm_raw + K2_PLANES);  // the node weights are done with before the planes
+    __shared__ Shared S;
+    __shared__ int nbs, umin, umax;
+    __shared__ double u0s;
+    const int tid = threadIdx.x, h = (T - 2) / 2;
+    const int lane = tid & 31, warp = tid >> 5, lr4 = lane >> 2, kp = lane & 3;
+    const uint32_t sh = 8 * ((7 - lr4) & 3);
+    lagrange_tables(S, T);
+    if (tid < 32 && !B.h_tile_off) sky_by_warp(P.src.sky1, &S.skc);
+    FwdParams Q = P;   // tiles over strain samples
+    Q.src.tile_off = B.h_tile_off;
+    Q.tile = B.tile_h;
+    const int64_t total = B.h_total_tiles >= 0 ? B.h_total_tiles : B.h_tile_off[P.src.S];
+    for (int64_t g = blockIdx.x; g < total; g += gridDim.x) {
+        int64_t src = 0;
+        if (tid < 32 && Q.src.tile_off) src = find_source(Q, g);
+        if (tid == 0) {
+            S.ti = tile_info_of(Q, g, src, 3);
+            if (Q.src.tile_off) S.skc = P.src.skyc[src];
+            if (!S.ti.ok) atomicOr(P.err, ERR_OFFSETS);
+            const int64_t nbh = S.ti.nh - S.ti.n0;   // clipped against the strain, not the outputs
+            nbs = !S.ti.ok || nbh <= 0 ? 0 : (int)(nbh < B.tile_h ? nbh : B.tile_h);
+            u0s = (P.t0 - S.ti.t0h) / P.dt;
+            umin = 1 << 29;
+            umax = -(1 << 29);
+        }
+        __syncthreads();
+        const int nb = nbs;
+        if (nb <= 0) {
+            __syncthreads();
+            continue;
+        }
+        const double u0 = u0s, fl0 = floor(u0);
+        const int64_t i0 = S.ti.n0, N = S.ti.N;
+        // the link samples whose reads can land on the tile: from the reads' positions near its centre
+        if (tid < 9) {
+            int piece;
+            const double u = read_pos(P, X, S.skc, u0, P.t0 + (double)(i0 + nb / 2 - (int64_t)fl0) * P.dt, tid, &piece) - fl0;
+            atomicMin(&umin, (int)floor(u - 0.25));
+            atomicMax(&umax, (int)floor(u + 0.25));
+        }
+        __syncthreads();
+        const int64_t k_lo = i0 - (int64_t)fl0 - umax - (h + 1);
+        const double t_lo = P.t0 + (double)k_lo * P.dt;
+        projection_segments(P, X, S, t_lo, u0, fl0, NY);
+        const double *gy = B.g_y + 2 * (S.ti.out - P.out);
+        bool any = false;
+        for (int l = 0; l < 6; ++l)
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const int j = tid + 256 * r;
+                const int64_t k = k_lo + j;
+                const double v = k >= 0 && k < N ? __ldg(gy + l * N + k) : 0.0;
+                gys[l * NY + j] = v;
+                any |= v != 0.0;
+                range_update(S, abs_hi(v));
+            }
+        double *ghp = B.g_hp + (S.ti.hp - P.hp), *ghc = B.g_hc + (S.ti.hp - P.hp);
+        if (!__syncthreads_or(any)) {
+            for (int i = tid; i < nb; i += blockDim.x) ghp[i0 + i] = ghc[i0 + i] = 0.0;
+            __syncthreads();
+            continue;
+        }
+        const int nseg = S.nseg, KW = S.mmax - S.mmin + T, nks = (KW + 3 + 15) / 16;
+        const int j0 = umax - S.mmax;   // row of the first link sample that output 0 gathers from
+        int eg = 0;
+        bool bad = S.bad || nks * 16 > 64 || j0 < 0 || j0 + nb + KW - 1 > NY || !range_ok(S, &eg);
+        double out[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int sg = 0; sg < nseg && !bad; ++sg) {
+            if (!projection_stencils<true>(P, X, S, T, t_lo, u0, fl0, sg, KW, W, wn)) {
+                bad = true;
+                break;
+            }
+            const int nq = S.nq, js = S.segj[sg], je = S.segj[sg + 1];
+            const bool last = S.last;
+            long long sum[4] = {0, 0, 0, 0};
+            const unsigned char *a_lane = reinterpret_cast<const unsigned char *>(planes) + 8 * (16 * warp + lr4) + 8 * kp;
+            for (int l = 0; l < 6; ++l) {
+                const unsigned char *w_lane = W + (2 * l + (lr4 >> 2)) * PD * WS + 4 + 4 * kp;
+                float acc[7][4] = {};
+                for (int p = tid; p < DL; p += blockDim.x) {
+                    const int j = p + j0;
+                    const bool in = j >= js && j < je;
+                    order_planes<0, QA>(planes, p, in ? to_fixed(gys[l * NY + j], eg) : 0, 2 * j + 1 - NY, in);
+                }
+                __syncthreads();
+                if (64 * warp < nb) {
+                    proj_order<0, false>(acc, a_lane, w_lane, sh, nks);
+                    if (last) {
+                        if (nq > 1) proj_order<1, true>(acc, a_lane, w_lane, sh, nks);
+                        if (nq > 2) proj_order<2, true>(acc, a_lane, w_lane, sh, nks);
+                    } else {
+                        if (nq > 1) proj_order<1, false>(acc, a_lane, w_lane, sh, nks);
+                        if (nq > 2) proj_order<2, false>(acc, a_lane, w_lane, sh, nks);
+                    }
+                }
+                __syncthreads();
+                if (nq > QA) {
+                    for (int p = tid; p < DL; p += blockDim.x) {
+                        const int j = p + j0;
+                        const bool in = j >= js && j < je;
+                        order_planes<QA, NN>(planes, p, in ? to_fixed(gys[l * NY + j], eg) : 0, 2 * j + 1 - NY, in);
+                    }
+                    __syncthreads();
+                    if (64 * warp < nb) {
+                        if (last) {
+                            proj_order<3, true>(acc, a_lane, w_lane, sh, nks);
+                            if (nq > 4) proj_order<4, true>(acc, a_lane, w_lane, sh, nks);
+                            if (nq > 5) proj_order<5, true>(acc, a_lane, w_lane, sh, nks);
+                            if (nq > 6) proj_order<6, true>(acc, a_lane, w_lane, sh, nks);
+                            if (nq > 7) proj_order<7, true>(acc, a_lane, w_lane, sh, nks);
+                        } else {
+                            proj_order<3, false>(acc, a_lane, w_lane, sh, nks);
+                            if (nq > 4) proj_order<4, false>(acc, a_lane, w_lane, sh, nks);
+                            if (nq > 5) proj_order<5, false>(acc, a_lane, w_lane, sh, nks);
+                            if (nq > 6) proj_order<6, false>(acc, a_lane, w_lane, sh, nks);
+                            if (nq > 7) proj_order<7, false>(acc, a_lane, w_lane, sh, nks);
+                        }
+                    }
+                    __syncthreads();
+                }
+#pragma unroll
+                for (int r = 0; r < 4; ++r) sum[r] += levels<0>(acc, r);
+            }
+            const int unit = eg + S.wexp[0] - 57;
+#pragma unroll
+            for (int r = 0; r < 4; ++r) out[r] += from_fixed(sum[r], unit);
+        }
+        __syncthreads();
+        if (!bad) {
+            double *o = (kp >> 1) ? ghc : ghp;
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const int i = 64 * warp + 4 * (lr4 + (r >> 1) * 8) + 2 * (kp & 1) + (r & 1);
+                if (i < nb) o[i0 + i] = out[r];
+            }
+        } else {
+            proj_adj_scalar(P, S, T, u0, i0, nb, k_lo, gys, ghp, ghc, reinterpret_cast<double *>(sm_raw + K2_PLANES));
+        }
+        __syncthreads();
+    }
+}
+
+// ---------------------------------------------------------------- K3: sky-angle gradient
+// derivatives of the frame (k, u, v) with respect to lambda (0) and beta (1), from the frame itself
+__device__ __forceinline__ void frame_derivatives(const SkyConst &K, double dk[2][3], double du[2][3], double dv[2][3])
+{
+    const double sl = K.u[0], cl = -K.u[1], cb = K.v[2], sb = -K.k[2];
+    dk[0][0] = cb * sl;  dk[0][1] = -cb * cl; dk[0][2] = 0.0;
+    dk[1][0] = sb * cl;  dk[1][1] = sb * sl;  dk[1][2] = -cb;
+    du[0][0] = cl;       du[0][1] = sl;       du[0][2] = 0.0;
+    du[1][0] = 0.0;      du[1][1] = 0.0;      du[1][2] = 0.0;
+    dv[0][0] = sb * sl;  dv[0][1] = -sb * cl; dv[0][2] = 0.0;
+    dv[1][0] = -cb * cl; dv[1][1] = -cb * sl; dv[1][2] = -sb;
+}
+
+// link l's part of the gradient at positions x: e, r the emission and reception reads summed against gy,
+// (value, derivative) of h+ and hx
+__device__ __forceinline__ void sky_terms(const FwdParams &P, const SkyConst &K, const double *x, int l, const double *e,
+                                          const double *r, double *G)
+{
+    double dk[2][3], du[2][3], dv[2][3];
+    frame_derivatives(K, dk, du, dv);
+    const int ir = c_lr[l], is = c_ls[l];
+    double n[3];
+    for (int d = 0; d < 3; ++d) n[d] = x[3 * ir + d] - x[3 * is + d];
+    const double inv = 1.0 / sqrt(n[0] * n[0] + n[1] * n[1] + n[2] * n[2]);
+    for (int d = 0; d < 3; ++d) n[d] *= inv;
+    auto dot = [&](const double *a) { return a[0] * n[0] + a[1] * n[1] + a[2] * n[2]; };
+    const double un = dot(K.u), vn = dot(K.v), kn = dot(K.k);
+    const double xip = un * un - vn * vn, xic = 2.0 * un * vn;
+    const double xp = K.c2p * xip + K.s2p * xic, xc = -K.s2p * xip + K.c2p * xic;
+    const double den = 1.0 / (2.0 * (1.0 - kn));
+    const double dPp = e[0] - r[0], dPc = e[2] - r[2], dH = xp * dPp + xc * dPc;
+    for (int th = 0; th < 2; ++th) {
+        const double da = dot(du[th]), db = dot(dv[th]);
+        const double dxip = 2.0 * (un * da - vn * db), dxic = 2.0 * (da * vn + un * db);
+        const double dxp = K.c2p * dxip + K.s2p * dxic, dxc = -K.s2p * dxip + K.c2p * dxic;
+        const double dden = 2.0 * den * den * dot(dk[th]);
+        const double due = -(dk[th][0] * x[3 * is] + dk[th][1] * x[3 * is + 1] + dk[th][2] * x[3 * is + 2]) / C_LIGHT * P.inv_dt;
+        const double dur = -(dk[th][0] * x[3 * ir] + dk[th][1] * x[3 * ir + 1] + dk[th][2] * x[3 * ir + 2]) / C_LIGHT * P.inv_dt;
+        const double ddH = dxp * dPp + dxc * dPc + xp * (e[1] * due - r[1] * dur) + xc * (e[3] * due - r[3] * dur);
+        G[th] += dden * dH + den * ddH;
+    }
+    G[2] += den * (2.0 * xc * dPp - 2.0 * xp * dPc);
+}
+
+// value and derivative of both polarisations at base + u, straight from memory (Horner form of read_scalar)
+__device__ void read_vd_scalar(const Shared &S, int T, const double *hp, const double *hc, int64_t nh, int64_t base, double u,
+                               double *v)
+{
+    const int h = (T - 2) / 2;
+    const double fl = floor(u), e = u - fl;
+    const int64_t st = base + (int64_t)fl - h;
+    double L = -1.0, dL = 0.0;
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int j = 0; j < T; ++j) {
+        const int64_t i = st + j;
+        const double p = i >= 0 && i < nh ? __ldg(hp + i) : 0.0, c = i >= 0 && i < nh ? __ldg(hc + i) : 0.0;
+        if (j) {
+            const double f = fma(e, S.rc1[j], S.rc0[j]), f1 = S.rc1[j];
+            const double q = -fma(e, S.lc1[j - 1], S.lc0[j - 1]), q1 = -S.lc1[j - 1];
+            dL = fma(dL, q, L * q1);
+            L *= q;
+            a[1] = fma(a[1], f, fma(a[0], f1, dL * p));
+            a[0] = fma(a[0], f, L * p);
+            a[3] = fma(a[3], f, fma(a[2], f1, dL * c));
+            a[2] = fma(a[2], f, L * c);
+        } else {
+            a[0] = L * p;
+            a[2] = L * c;
+        }
+    }
+    for (int i = 0; i < 4; ++i) v[i] = a[i];
+}
+
+// digit bytes of T_q g (K3's right operand) of one row
+template <int N>
+__device__ __forceinline__ void put_bytes(unsigned char *row, long long X)
+{
+    X += DIGIT_BIAS;
+    row[0] = (unsigned char)((int)(X >> 48) + 128);   // |X| < 2^54: the scale leaves a bit for the byte's range
+#pragma unroll
+    for (int i = 1; i < N; ++i) row[i * GB] = (unsigned char)(X >> (8 * (6 - i)));
+}
+
+// correlations of order Q over k-steps [s0, s1): acc by level, the top one carrying the next
+template <int Q>
+__device__ __forceinline__ void correlate(float (&acc)[7][4], const unsigned char *a_lane, const unsigned char *g_lane,
+                                          uint32_t sh, int s0, int s1)
+{
+    constexpr int n = 7 - zq(false, Q), NA = n < 7 ? n + 1 : 7, ND = gdigits(false, Q);
+#pragma unroll 1
+    for (int ks = s0; ks < s1; ++ks) {
+        uint32_t a[NA][4];
+#pragma unroll
+        for (int k = 0; k < NA; ++k) {
+            const uint2 p = *reinterpret_cast<const uint2 *>(a_lane + 32 * ks + k * DL * 2);
+            const uint2 c = *reinterpret_cast<const uint2 *>(a_lane + 32 * ks + (7 + k) * DL * 2);
+            a[k][0] = p.x; a[k][1] = c.x; a[k][2] = p.y; a[k][3] = c.y;
+        }
+#pragma unroll
+        for (int d = 0; d < ND; ++d) {
+            const uint32_t *w = reinterpret_cast<const uint32_t *>(g_lane + 16 * ks + (gplane(false, Q) + d) * GB);
+            const uint32_t u = __funnelshift_r(w[0], w[1], sh);
+            const uint32_t b0 = digits_h2(u, 0x4140u), b1 = digits_h2(u, 0x4342u);
+            if (d < n) {
+#pragma unroll
+                for (int k = 0; k < n - 1 - d; ++k) mma_f16(acc[d + k], a[k], b0, b1);
+                if (n - d < NA) {
+                    uint32_t x[4];
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) x[r] = extend_h2(a[n - 1 - d][r], a[n - d][r]);
+                    mma_f16(acc[n - 1], x, b0, b1);
+                } else {
+                    mma_f16(acc[n - 1], a[n - 1 - d], b0, b1);
+                }
+            } else {  // digit n against the series' first digit: level n
+                uint32_t x[4];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) x[r] = extend_h2(0u, a[0][r]);
+                mma_f16(acc[n - 1], x, b0, b1);
+            }
+        }
+    }
+}
+
+template <int Q>
+__device__ __forceinline__ void correlate_item(double *C, int LG, const unsigned char *a_lane, const unsigned char *g_lane,
+                                               uint32_t sh, int s0, int s1, int lag0, int lane, int link0)
+{
+    constexpr int n = 7 - zq(false, Q);
+    float acc[7][4] = {};
+    correlate<Q>(acc, a_lane, g_lane, sh, s0, s1);
+    const int lr4 = lane >> 2, kp = lane & 3, l = link0 + (kp >> 1);
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        long long v = 0;
+#pragma unroll
+        for (int L = 0; L < n - 1; ++L) v = v * 256 + (long long)__float2int_rn(acc[L][r]);
+        v += (long long)__float2int_rn(acc[n - 1][r] * (1.0f / 256.0f));
+        const int lag = lag0 + 4 * lr4 + 2 * (kp & 1) + (r & 1), pol = r >> 1;
+        // two contributions per place (the halves of the block), so the sum does not depend on their order
+        if (lag < LG) atomicAdd(&C[((l * NN + Q) * 2 + pol) * LG + lag], (double)v * pow2(8 * zq(false, Q) - 54));
+    }
+}
+
+// the (order, half of the block) items 2 q + half of each warp: the orders cost 28, 28, 22, 16, 11, 11, 7, 4
+// products a step
+__constant__ signed char c_items[8][4] = {{0, 14, -1, -1}, {1, 15, -1, -1}, {2, -1, -1, -1}, {3, -1, -1, -1},
+                                          {4, 8, -1, -1},  {5, 9, -1, -1},  {6, 10, 12, -1}, {7, 11, 13, -1}};
+
+__global__ void __launch_bounds__(256, 2) k_fx_sky_adj(FwdParams P, FxTab X, BwdParams B, int T)
+{
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    uint16_t *planes = reinterpret_cast<uint16_t *>(sm_raw);
+    unsigned char *G = sm_raw + K3_G;
+    double *wn = reinterpret_cast<double *>(sm_raw + K3_G), *dwn = wn + T * WNS;   // once the digit rows are done with
+    const int gend = K3_GEND > K3_G + 16 * T * WNS ? K3_GEND : K3_G + 16 * T * WNS;
+    double *C = reinterpret_cast<double *>(sm_raw + ((gend + 15) & ~15));          // [link][order or node][pol][LG]
+    const int LG = X.lags;
+    __shared__ Shared S;
+    __shared__ double dots[NN][6][2][4];   // node, link, (emission, reception): h+ value, derivative, hx value, derivative
+    __shared__ double red[3][8];
+    __shared__ unsigned gmax, gmin;
+    const int tid = threadIdx.x, h = (T - 2) / 2;
+    const int lane = tid & 31, warp = tid >> 5, lr4 = lane >> 2, kp = lane & 3;
+    const uint32_t sh = 8 * ((7 - lr4) & 3);
+    lagrange_tables(S, T);
+    if (tid < 32 && !P.src.tile_off) sky_by_warp(P.src.sky1, &S.skc);
+    const int64_t total = P.total_tiles >= 0 ? P.total_tiles : P.src.tile_off[P.src.S];
+    for (int64_t g = blockIdx.x; g < total; g += gridDim.x) {
+        int64_t src = 0;
+        if (tid < 32 && P.src.tile_off) src = find_source(P, g);
+        if (tid == 0) {
+            S.ti = tile_info_of(P, g, src, 3);
+            if (P.src.tile_off) S.skc = P.src.skyc[src];
+            if (!S.ti.ok) atomicOr(P.err, ERR_OFFSETS);
+            gmax = 0;
+            gmin = 0x7fffffffu;
+        }
+        __syncthreads();
+        double Gs[3] = {0.0, 0.0, 0.0};
+        if (S.ti.ok && S.ti.nb > 0) {
+            const TileInfo &ti = S.ti;
+            const int nb = (int)ti.nb;
+            const int64_t k_lo = ti.n0, N = ti.N;
+            const double u0 = (P.t0 - ti.t0h) / P.dt, fl0 = floor(u0), t_lo = P.t0 + (double)k_lo * P.dt;
+            const double *gy = B.g_y + 2 * (ti.out - P.out);
+            projection_segments(P, X, S, t_lo, u0, fl0, nb);
+            const int nseg = S.nseg, mmin = S.mmin, KW = S.mmax - mmin + T, npass = (KW + 31) / 32;
+            bool bad = S.bad || KW > LG;
+            const int64_t w_lo = k_lo + (int64_t)fl0 + mmin - h;
+            const int WL = nb + KW - 1;
+            bool anyg = false, anyh = false;
+            double vp[3], vc[3];
+            if (!bad) {
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    const int p = tid + i * 256;
+                    const int64_t idx = w_lo + p;
+                    vp[i] = vc[i] = 0.0;
+                    if (p < WL && idx >= 0 && idx < ti.nh) {
+                        vp[i] = __ldg(ti.hp + idx);
+                        vc[i] = __ldg(ti.hc + idx);
+                    }
+                    anyh |= vp[i] != 0.0 || vc[i] != 0.0;
+                    const unsigned a = abs_hi(vp[i]), b = abs_hi(vc[i]);
+                    range_update(S, a > b ? a : b);
+                }
+                for (int l = 0; l < 6; ++l)
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) {
+                        const int j = tid + 256 * r;
+                        const double v = j < nb ? __ldg(gy + l * N + k_lo + j) : 0.0;
+                        anyg |= v != 0.0;
+                        const unsigned m = __reduce_max_sync(0xffffffffu, abs_hi(v));
+                        if (lane == 0 && m) {
+                            atomicMax(&gmax, m);
+                            atomicMin(&gmin, m);
+                        }
+                    }
+            }
+            const bool work = bad || (__syncthreads_or(anyg) && __syncthreads_or(anyh));
+            int ex = 0, eg = 0;
+            if (!bad && work) {
+                bad = !range_ok(S, &ex);
+                const int eb = (int)(gmax >> 20), es = (int)(gmin >> 20);
+                eg = eb - 1021;
+                bad |= !(eb >= 200 && eb <= 1900 && eb - es <= RANGE_BITS);
+            }
+            if (!bad && work) {
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    const int p = tid + i * 256;
+                    if (p < DL) {
+                        digits_to_planes(planes, p, vp[i], ex);
+                        digits_to_planes(planes + 7 * DL, p, vc[i], ex);
+                    }
+                }
+                const int steps = (nb + 3 + 15) / 16, mid = (steps + 1) / 2;
+                for (int sg = 0; sg < nseg; ++sg) {
+                    const int js = S.segj[sg], je = S.segj[sg + 1];
+                    __syncthreads();
+                    for (int i = tid; i < 12 * NN * LG; i += blockDim.x) C[i] = 0.0;
+                    for (int lp = 0; lp < 3; ++lp) {
+                        __syncthreads();
+                        for (int i = tid; i < 2 * GROWS * GB / 4; i += blockDim.x) reinterpret_cast<uint32_t *>(G)[i] = 0x80808080u;
+                        __syncthreads();
+                        for (int i = tid; i < 2 * (je - js); i += blockDim.x) {
+                            const int l2 = i >= je - js, j = js + i - l2 * (je - js);
+                            const long long x0 = to_fixed(__ldg(gy + (2 * lp + l2) * N + k_lo + j), eg);
+                            const int kappa = 2 * j + 1 - NY;
+                            unsigned char *row = G + l2 * GROWS * GB + 7 + j;
+                            long long xa = x0, xb = mul_nu<9>(x0, kappa);
+#pragma unroll
+                            for (int q = 0; q < NN; ++q) {
+                                unsigned char *o = row + gplane(false, q) * GB;
+                                if (gdigits(false, q) == 7) put_bytes<7>(o, xa);
+                                else if (gdigits(false, q) == 6) put_bytes<6>(o, xa);
+                                else if (gdigits(false, q) == 5) put_bytes<5>(o, xa);
+                                else if (gdigits(false, q) == 4) put_bytes<4>(o, xa);
+                                else put_bytes<3>(o, xa);
+                                const long long nx = mul_nu<8>(xb, kappa) - xa;
+                                xa = xb;
+                                xb = nx;
+                            }
+                        }
+                        __syncthreads();
+                        const unsigned char *g_lane = G + (lr4 >> 2) * GROWS * GB + 4 + 4 * kp;
+                        for (int ps = 0; ps < npass; ++ps) {
+                            const unsigned char *a_lane = reinterpret_cast<const unsigned char *>(planes) + 8 * (lr4 + 8 * ps) + 8 * kp;
+                            for (int k = 0; k < 4; ++k) {
+                                const int it = c_items[warp][k];
+                                if (it < 0) break;
+                                const int s0 = (it & 1) ? mid : 0, s1 = (it & 1) ? steps : mid;
+                                switch (it >> 1) {
+                                    case 0: correlate_item<0>(C, LG, a_lane, g_lane, sh, s0, s1, 32 * ps, lane, 2 * lp); break;
+                                    case 1: correlate_item<1>(C, LG, a_lane, g_lane, sh, s0, s1, 32 * ps, lane, 2 * lp); break;
+                                    case 2: correlate_item<2>(C, LG, a_lane, g_lane, sh, s0, s1, 32 * ps, lane, 2 * lp); break;
+                                    case 3: correlate_item<3>(C, LG, a_lane, g_lane, sh, s0, s1, 32 * ps, lane, 2 * lp); break;
+                                    case 4: correlate_item<4>(C, LG, a_lane, g_lane, sh, s0, s1, 32 * ps, lane, 2 * lp); break;
+                                    case 5: correlate_item<5>(C, LG, a_lane, g_lane, sh, s0, s1, 32 * ps, lane, 2 * lp); break;
+                                    case 6: correlate_item<6>(C, LG, a_lane, g_lane, sh, s0, s1, 32 * ps, lane, 2 * lp); break;
+                                    default: correlate_item<7>(C, LG, a_lane, g_lane, sh, s0, s1, 32 * ps, lane, 2 * lp); break;
+                                }
+                            }
+                        }
+                    }
+                    __syncthreads();
+                    // node weights and their derivatives (prefix and suffix products with the product rule, two
+                    // threads per read), the reads on this segment's spline piece
+                    const int *sm = S.segm[sg];
+                    if (sm[9] != S.segm[sg ? sg - 1 : 0][9]) {
+                        if (tid < NN * 3) node_reads(P, X, S, t_lo, u0, tid / 3, tid % 3, sm[9]);
+                        __syncthreads();
+                    }
+                    const int id = tid < WNS ? tid : tid - WNS;
+                    const bool low = tid < WNS, half = tid < 2 * WNS;
+                    double e = 0.0, run = 1.0, drun = 0.0;
+                    double *w = wn + id, *dw = dwn + id;
+                    if (half) {
+                        e = S.nodeu[id] - (fl0 + (double)sm[id % 9]);
+                        if (low) {
+                            for (int a = 0; a < T / 2; ++a) {
+                                w[a * WNS] = run;
+                                dw[a * WNS] = drun;
+                                const double f = fma(e, S.lc1[a], S.lc0[a]);
+                                drun = fma(drun, f, run * S.lc1[a]);
+                                run *= f;
+                            }
+                        } else {
+                            for (int a = T - 1; a >= T / 2; --a) {
+                                const double sg1 = ((T - 1 - a) & 1) ? -1.0 : 1.0;
+                                w[a * WNS] = sg1 * run;
+                                dw[a * WNS] = sg1 * drun;
+                                const double f = fma(e, S.rc1[a], S.rc0[a]);
+                                drun = fma(drun, f, run * S.rc1[a]);
+                                run *= f;
+                            }
+                        }
+                    }
+                    __syncthreads();
+                    if (half) {
+                        if (low) {
+                            for (int a = T / 2; a < T; ++a) {
+                                const double r = w[a * WNS], dr = dw[a * WNS];
+                                w[a * WNS] = run * r;
+                                dw[a * WNS] = fma(drun, r, run * dr);
+                                const double f = fma(e, S.lc1[a], S.lc0[a]);
+                                drun = fma(drun, f, run * S.lc1[a]);
+                                run *= f;
+                            }
+                        } else {
+                            for (int a = T / 2 - 1; a >= 0; --a) {
+                                const double sg1 = ((T - 1 - a) & 1) ? -1.0 : 1.0, r = w[a * WNS], dr = dw[a * WNS];
+                                w[a * WNS] = sg1 * (run * r);
+                                dw[a * WNS] = sg1 * fma(drun, r, run * dr);
+                                const double f = fma(e, S.rc1[a], S.rc0[a]);
+                                drun = fma(drun, f, run * S.rc1[a]);
+                                run *= f;
+                            }
+                        }
+                    }
+                    // correlations at the nodes: sum over the orders (cheb of node NN - 1 - n is that of n with
+                    // odd orders negated)
+                    for (int i = tid; i < 12 * LG; i += blockDim.x) {
+                        const int l = i / (2 * LG), r = i - l * 2 * LG;
+                        double *c = C + l * NN * 2 * LG + r;
+                        double v[NN];
+#pragma unroll
+                        for (int q = 0; q < NN; ++q) v[q] = c[q * 2 * LG];
+#pragma unroll
+                        for (int n = 0; n < NN / 2; ++n) {
+                            double ev = 0.0, od = 0.0;
+#pragma unroll
+                            for (int q = 0; q < NN; q += 2) {
+                                ev = fma(X.cheb[q][n], v[q], ev);
+                                od = fma(X.cheb[q + 1][n], v[q + 1], od);
+                            }
+                            c[n * 2 * LG] = ev + od;
+                            c[(NN - 1 - n) * 2 * LG] = ev - od;
+                        }
+                    }
+                    __syncthreads();
+                    if (tid < NN * 24) {
+                        const int n = tid / 24, l = (tid % 24) >> 2, er = (tid >> 1) & 1, pol = tid & 1;
+                        const int rd = er ? c_lr[l] : 3 + l;
+                        const double *c = C + ((l * NN + n) * 2 + pol) * LG + sm[rd] - mmin;
+                        const double *a = wn + n * 9 + rd, *b = dwn + n * 9 + rd;
+                        double v = 0.0, d = 0.0;
+                        for (int t = 0; t < T; ++t) {
+                            v = fma(a[t * WNS], c[t], v);
+                            d = fma(b[t * WNS], c[t], d);
+                        }
+                        dots[n][l][er][2 * pol] = v;
+                        dots[n][l][er][2 * pol + 1] = d;
+                    }
+                    __syncthreads();
+                    if (tid < NN * 6) {
+                        double t[3] = {0.0, 0.0, 0.0};
+                        sky_terms(P, S.skc, S.npos[tid / 6], tid % 6, dots[tid / 6][tid % 6][0], dots[tid / 6][tid % 6][1], t);
+                        const double unit = pow2(eg) * pow2(ex);
+                        for (int c = 0; c < 3; ++c) Gs[c] += t[c] * unit;
+                    }
+                }
+            }
+            __syncthreads();
+            if (bad)
+                for (int j = tid; j < nb; j += blockDim.x) {
+                    const int64_t k = k_lo + j;
+                    double x[9], L[6], rr[3][4], sig[3];
+                    orbit_all(P.po, P.t0 + (double)k * P.dt, x, L);
+                    for (int i = 0; i < 3; ++i) {
+                        sig[i] = (S.skc.k[0] * x[3 * i] + S.skc.k[1] * x[3 * i + 1] + S.skc.k[2] * x[3 * i + 2]) / C_LIGHT * P.inv_dt;
+                        read_vd_scalar(S, T, ti.hp, ti.hc, ti.nh, k, u0 - sig[i], rr[i]);
+                    }
+                    for (int l = 0; l < 6; ++l) {
+                        const double gl = __ldg(gy + l * N + k);
+                        if (gl == 0.0) continue;
+                        double ee[4], t[3] = {0.0, 0.0, 0.0};
+                        read_vd_scalar(S, T, ti.hp, ti.hc, ti.nh, k, u0 - L[l] * P.inv_dt - sig[c_ls[l]], ee);
+                        sky_terms(P, S.skc, x, l, ee, rr[c_lr[l]], t);
+                        for (int c = 0; c < 3; ++c) Gs[c] = fma(gl, t[c], Gs[c]);
+                    }
+                }
+        }
+        // fixed-order block reduction: warp tree, then warps in order
+        for (int t = 0; t < 3; ++t) {
+            double v = Gs[t];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+            if (lane == 0) red[t][warp] = v;
+        }
+        __syncthreads();
+        if (tid < 3) {
+            double s = 0.0;
+            for (int w = 0; w < 8; ++w) s += red[tid][w];
+            B.partial[3 * g + tid] = s;
+        }
+        __syncthreads();
+    }
+}
+
+}  // namespace
+
+int launch_fx_bwd(int kind, int order, const FwdParams &P, const BwdParams &B, FxPlan *F, int sms, void *stream)
+{
+    int T = order + 1;
+    FxTab X;
+    if (const int e = fx_table_for(F, stream, &X)) return e;
+    void *k = kind == 0 ? (void *)k_fx_tdi_adj : kind == 1 ? (void *)k_fx_proj_adj : (void *)k_fx_sky_adj;
+    size_t smem = kind == 0 ? k1_w(T) + FX_TDI_W : K2_END;
+    if (kind == 2) {
+        const size_t w = K3_G + 16 * (size_t)T * WNS;
+        smem = ((w > K3_GEND ? w : K3_GEND) + 15 & ~(size_t)15) + sizeof(double) * 12 * NN * (size_t)X.lags;
+    }
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return (int)e;
+    int per_sm = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 256, smem);
+    if (e != cudaSuccess) return (int)e;
+    if (per_sm < 1) return (int)cudaErrorLaunchOutOfResources;
+    int64_t grid = (int64_t)per_sm * sms;
+    const int64_t known = kind == 1 ? B.h_total_tiles : P.total_tiles;
+    if (known >= 0 && known < grid) grid = known;
+    if (grid < 1) grid = 1;
+    void *args[] = {(void *)&P, (void *)&X, (void *)&B, (void *)&T};
+    return (int)cudaLaunchKernel(k, dim3((unsigned)grid), dim3(256), args, smem, (cudaStream_t)stream);
+}
+
+}  // namespace lr

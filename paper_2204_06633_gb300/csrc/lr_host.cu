@@ -313,6 +313,38 @@ int constant_delay_table(lr_plan *p, const lr_orbit *o)
     return LR_OK;
 }
 
+// launch constants and stencil table of the tensor-core kernels, once per plan; false when out of memory
+bool fx_create(lr_plan *p)
+{
+    if (p->fx) return true;
+    const lr::FwdParams &P = p->base;
+    p->fx = new (std::nothrow) lr::FxPlan();
+    if (!p->fx) return false;
+    lr::fx_tables(P, p->desc.order, p->desc.proj_orbit->max_delay, p->fx->tab);
+    const size_t bytes = lr::fx_table_bytes(P, p->desc.order);
+    // without the table (no memory for it) the blocks compute their own stencils
+    if (bytes && lr::dev_malloc(&p->fx->mem, bytes) == cudaSuccess && lr::fx_table_build(P, p->desc.order, p->fx)) {
+        cudaFree(p->fx->mem);
+        p->fx->mem = nullptr;
+    }
+    cudaGetLastError();
+    return true;
+}
+
+// whether the adjoint runs on the tensor-core kernels: summed (or constant) delays, stencils that fit and the
+// table of them.  Mixed plans take the same kernels (the table is built at their first adjoint): they are
+// more exact than the float-float ones and several times faster.
+bool fx_backward(lr_plan *p)
+{
+    const lr::FwdParams &P = p->base;
+    if ((P.delay_nested && !P.cd_w) || lr::fx_max_tile(P, p->desc.order) < 128 || !fx_create(p)) return false;
+    return p->fx->tab.tab != nullptr;
+}
+
+// its tiles (of link and of strain samples): the forward's block, so that a time split in units of the plan's
+// tile meets the same blocks
+int fx_backward_tile(const lr_plan *p) { return p->base.fx_tile ? p->base.fx_tile : lr::fx_max_tile(p->base, p->desc.order); }
+
 // FP64 plans whose stencils fit run on the tensor-core kernels (lr_fx64.cu).  Their blocks hold at most
 // fx_max_tile outputs; a larger tile is worked in equal parts, so that a time split in units of the tile
 // keeps every block whole.  Nested delays that vary keep the sample-by-sample kernels.
@@ -325,18 +357,7 @@ void fx_setup(lr_plan *p)
     int block = p->tile < most ? p->tile : most;
     while (block >= 128 && p->tile % block) --block;
     if (block < 128 && p->tile >= 128) return;  // no part of at least 128 outputs
-    if (!p->fx) {
-        p->fx = new (std::nothrow) lr::FxPlan();
-        if (!p->fx) return;
-        lr::fx_tables(P, p->fx->tab);
-        const size_t bytes = lr::fx_table_bytes(P, p->desc.order);
-        // without the table (no memory for it) the blocks compute their own stencils
-        if (bytes && lr::dev_malloc(&p->fx->mem, bytes) == cudaSuccess && lr::fx_table_build(P, p->desc.order, p->fx)) {
-            cudaFree(p->fx->mem);
-            p->fx->mem = nullptr;
-        }
-        cudaGetLastError();
-    }
+    if (!fx_create(p)) return;
     P.fx = p->fx;
     P.fx_tile = block;
     P.tile = block;
@@ -726,7 +747,7 @@ LR_API int lr_plan_check(lr_plan *plan, void *stream)
 namespace {
 
 // Sizes the backward launch parameters and grows the plan's workspace.
-int backward_setup(lr_plan *plan, int64_t gy_elems, int64_t ktiles, lr::FwdParams &P, lr::BwdParams &B)
+int backward_setup(lr_plan *plan, bool fx, int64_t gy_elems, int64_t ktiles, lr::FwdParams &P, lr::BwdParams &B)
 {
     P = plan->base;
     std::memset(&B, 0, sizeof(B));
@@ -757,20 +778,27 @@ int backward_setup(lr_plan *plan, int64_t gy_elems, int64_t ktiles, lr::FwdParam
     }
     B.g_y = plan->d_gy;
     B.partial = plan->d_partial;
+    if (fx) {
+        P.tile = B.tile_h = fx_backward_tile(plan);
+    }
     return LR_OK;
 }
 
 // TDI transpose, sky partials, projection transpose, then the ordered sky reduction.
-int backward_launch(lr_plan *plan, lr::FwdParams &P, lr::BwdParams &B, int64_t S, const int64_t *ktile_off,
+int backward_launch(lr_plan *plan, bool fx, lr::FwdParams &P, lr::BwdParams &B, int64_t S, const int64_t *ktile_off,
                     double *g_sky, void *stream)
 {
     const int sms = plan->ctx->sms;
     const int order = plan->desc.order;
-    // mixed plans: the transposes and the sky gradient in the mixed kernels
+    // otherwise mixed plans take the float-float kernels
     const bool mx = plan->desc.precision == LR_MIXED;
-    int e = mx ? lr::launch_bwd_mx(0, order, P, B, sms, stream) : lr::launch_bwd(0, order, P, B, sms, stream);
-    if (!e && g_sky) e = mx ? lr::launch_bwd_mx(2, order, P, B, sms, stream) : lr::launch_bwd(2, order, P, B, sms, stream);
-    if (!e) e = mx ? lr::launch_bwd_mx(1, order, P, B, sms, stream) : lr::launch_bwd(1, order, P, B, sms, stream);
+    auto run = [&](int kind) {
+        return fx ? lr::launch_fx_bwd(kind, order, P, B, plan->fx, sms, stream)
+                  : mx ? lr::launch_bwd_mx(kind, order, P, B, sms, stream) : lr::launch_bwd(kind, order, P, B, sms, stream);
+    };
+    int e = run(0);
+    if (!e && g_sky) e = run(2);
+    if (!e) e = run(1);
     if (!e && g_sky) e = lr::launch_sky_reduce(B.partial, ktile_off, S, P.total_tiles, g_sky, stream);
     return check_launch(plan->ctx, e);
 }
@@ -1110,8 +1138,10 @@ LR_API int lr_backward(lr_plan *plan, const double *hp, const double *hc, int64_
     lr::FwdParams P;
     lr::BwdParams B;
     const int64_t N = plan->desc.n;
-    const int64_t ktiles = (N + lr::BWD_TILE_K - 1) / lr::BWD_TILE_K;
-    int st = backward_setup(plan, 6 * N, ktiles, P, B);
+    const bool fx = fx_backward(plan);
+    const int tile_k = fx ? fx_backward_tile(plan) : lr::BWD_TILE_K;
+    const int64_t ktiles = (N + tile_k - 1) / tile_k;
+    int st = backward_setup(plan, fx, 6 * N, ktiles, P, B);
     if (st) return st;
     P.src.n1 = N;
     P.src.nh1 = n_h;
@@ -1125,8 +1155,8 @@ LR_API int lr_backward(lr_plan *plan, const double *hp, const double *hc, int64_
     B.g_hp = g_hp;
     B.g_hc = g_hc;
     B.h_tile_off = nullptr;
-    B.h_total_tiles = (n_h + lr::BWD_TILE_H - 1) / lr::BWD_TILE_H;
-    return backward_launch(plan, P, B, 1, nullptr, g_sky, stream);
+    B.h_total_tiles = (n_h + B.tile_h - 1) / B.tile_h;
+    return backward_launch(plan, fx, P, B, 1, nullptr, g_sky, stream);
 }
 
 LR_API int lr_backward_batched(lr_plan *plan, int64_t S, const int64_t *h_off, const int64_t *out_off,
@@ -1144,29 +1174,34 @@ LR_API int lr_backward_batched(lr_plan *plan, int64_t S, const int64_t *h_off, c
     if (e == cudaSuccess) e = cudaStreamSynchronize((cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(plan->ctx, e);
     if (total_n < 0) return LR_ERR_INVALID_ARG;
-    const int64_t ktiles_bound = total_n / lr::BWD_TILE_K + S + 1;
+    const bool fx = fx_backward(plan);
+    const int tile_k = fx ? fx_backward_tile(plan) : lr::BWD_TILE_K;
+    const int64_t ktiles_bound = total_n / tile_k + S + 1;
     lr::FwdParams P;
     lr::BwdParams B;
-    int st = backward_setup(plan, 6 * (total_n > 0 ? total_n : 1), ktiles_bound, P, B);
+    int st = backward_setup(plan, fx, 6 * (total_n > 0 ? total_n : 1), ktiles_bound, P, B);
     if (st) return st;
     if (S + 1 > plan->ktile_cap) {
         if (plan->d_ktile_off) cudaFree(plan->d_ktile_off);
         if (plan->d_htile_off) cudaFree(plan->d_htile_off);
         plan->d_ktile_off = plan->d_htile_off = nullptr;
         plan->ktile_cap = 0;
-        e = lr::dev_malloc((void **)&plan->d_ktile_off, sizeof(int64_t) * (size_t)(S + 1));
+        // the link tiles' table, then the sources' sky frames
+        e = lr::dev_malloc((void **)&plan->d_ktile_off, (sizeof(int64_t) + sizeof(lr::SkyConst)) * (size_t)(S + 1));
         if (e == cudaSuccess) e = lr::dev_malloc((void **)&plan->d_htile_off, sizeof(int64_t) * (size_t)(S + 1));
         if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? LR_ERR_OOM : cuda_fail(plan->ctx, e);
         plan->ktile_cap = S + 1;
     }
-    int le = lr::launch_tile_offsets(out_off, S, lr::BWD_TILE_K, plan->d_ktile_off, P.err, stream);
-    if (!le) le = lr::launch_tile_offsets(h_off, S, lr::BWD_TILE_H, plan->d_htile_off, P.err, stream);
+    lr::SkyConst *skyc = fx ? reinterpret_cast<lr::SkyConst *>(plan->d_ktile_off + plan->ktile_cap) : nullptr;
+    int le = lr::launch_batch_tables(out_off, sky, S, tile_k, plan->d_ktile_off, skyc, P.err, stream);
+    if (!le) le = lr::launch_tile_offsets(h_off, S, B.tile_h, plan->d_htile_off, P.err, stream);
     if (le) return check_launch(plan->ctx, le);
     P.src.h_off = h_off;
     P.src.out_off = out_off;
     P.src.t0h = t0_h;
     P.src.sky = sky;
     P.src.tile_off = plan->d_ktile_off;
+    P.src.skyc = skyc;
     P.src.S = S;
     P.hp = hp;
     P.hc = hc;
@@ -1177,7 +1212,7 @@ LR_API int lr_backward_batched(lr_plan *plan, int64_t S, const int64_t *h_off, c
     B.g_hc = g_hc;
     B.h_tile_off = plan->d_htile_off;
     B.h_total_tiles = -1;
-    return backward_launch(plan, P, B, S, plan->d_ktile_off, g_sky, stream);
+    return backward_launch(plan, fx, P, B, S, plan->d_ktile_off, g_sky, stream);
 }
 
 }  // extern "C"

@@ -110,6 +110,7 @@ struct FxTab {
     const double *tab;
     const int *meta;
     int tab_kw;
+    int lags;   // correlation lags of the sky gradient, a multiple of 16
 };
 // host side of a plan's tensor-core kernels: launch constants, the table's memory and the event of its
 // computation (null once it is known to be done)
