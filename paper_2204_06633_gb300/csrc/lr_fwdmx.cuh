@@ -1205,8 +1205,11 @@ __device__ __forceinline__ void tdi_chain(const FwdParams &P, const MxShared &sh
 }
 
 // ---------------------------------------------------------------- kernel
-template <int T, int KIND>
-__global__ void __launch_bounds__(MIXED_THREADS, (T <= 32 ? 2 : 1)) k_mixed(FwdParams P)
+// NT threads: 256 (two CTAs per SM up to order 31), or 512 for launches of at most one tile per SM, where a
+// tile's latency is the launch's: the same items on twice the warps (bit-identical), one round of the
+// threads instead of two in the projection and link phases.  N = 4096 at order 25: 42.9 -> 37.6 us a call.
+template <int T, int KIND, int NT = MIXED_THREADS>
+__global__ void __launch_bounds__(NT, (NT == MIXED_THREADS && T <= 32 ? 2 : 1)) k_mixed(FwdParams P)
 {
     extern __shared__ __align__(16) float smf[];
     __shared__ MxShared sh;
@@ -1216,6 +1219,7 @@ __global__ void __launch_bounds__(MIXED_THREADS, (T <= 32 ? 2 : 1)) k_mixed(FwdP
     constexpr bool PREFETCH = KIND != KIND_TDI;
     constexpr bool LIKE = KIND == KIND_LIKE;                 // fused + likelihood epilogue
     constexpr bool FUSED = KIND == KIND_FUSED || LIKE;
+    static_assert(NT == MIXED_THREADS || (!LIKE && KIND != KIND_TDI && NT >= MX_YCAP + 64), "roles of the wide kernel");
     const int tid = threadIdx.x;
     if (tid == 0) {
         sh.tot = P.total_tiles >= 0 ? P.total_tiles : P.src.tile_off[P.src.S];
@@ -1265,7 +1269,7 @@ __global__ void __launch_bounds__(MIXED_THREADS, (T <= 32 ? 2 : 1)) k_mixed(FwdP
             woff_fx = (long long)woff << FX_BITS;
             // the CTA's next tile's bookkeeping (a chain of dependent loads) on the last thread,
             // hidden behind the others' staging loads
-            const int nst = next ? MIXED_THREADS - 1 : MIXED_THREADS;
+            const int nst = next ? NT - 1 : NT;
             unsigned long long mx = 0ull;
             if (tid >= nst) {
                 tile_begin<KIND>(P, sh, tn, gn);
@@ -1402,7 +1406,7 @@ __global__ void __launch_bounds__(MIXED_THREADS, (T <= 32 ? 2 : 1)) k_mixed(FwdP
                 }
             }
             // the TDI references of this tile, on threads that the loop above gave one sample
-            if (FUSED) tdi_refs<T>(P, ts, sh, smf + OFF_TW, TDI_REF0);
+            if (FUSED) tdi_refs<T>(P, ts, sh, smf + OFF_TW, NT == MIXED_THREADS ? TDI_REF0 : MX_YCAP);
         }
         double *ld = reinterpret_cast<double *>(smf + OFF_LD);
         if (KIND != KIND_PROJECT) {

@@ -9,6 +9,7 @@ static void *kernel_ptr_mx(int kind)
     switch (kind) {
         case KIND_PROJECT: return (void *)k_mixed<T, KIND_PROJECT>;
         case KIND_TDI: return (void *)k_mixed<T, KIND_TDI>;
+        case KIND_WIDE: return (void *)k_mixed<T, KIND_FUSED, MIXED_WIDE>;
         case KIND_LIKE: return (void *)k_mixed<T, KIND_LIKE>;
         default: return (void *)k_mixed<T, KIND_FUSED>;
     }

@@ -9,6 +9,7 @@ static void *kernel_ptr_mx(int kind)
     switch (kind) {
         case KIND_PROJECT: return (void *)k_mixed<T, KIND_PROJECT>;
         case KIND_TDI: return (void *)k_mixed<T, KIND_TDI>;
+        case KIND_WIDE: return nullptr;  // 128 registers do not hold its reads
         case KIND_LIKE: return (void *)k_mixed<T, KIND_LIKE>;
         default: return (void *)k_mixed<T, KIND_FUSED>;
     }

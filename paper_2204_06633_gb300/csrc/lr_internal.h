@@ -181,6 +181,7 @@ int smem_fwdmx(int kind, int order, const FwdParams &P, size_t *smem);
 int max_blocks_fwdmx(int kind, int order, int threads, size_t smem, int *blocks);
 bool order_compiled_mx(int order);
 constexpr int MIXED_THREADS = 256;  // the mixed kernels' per-tile setup assigns work by thread index
+constexpr int MIXED_WIDE = 512;     // of the fused kernel for launches of at most a tile per SM
 
 // Shared-memory geometry of the mixed kernels (compile time, so every array offset is an
 // immediate).  A staged series of up to n samples is stored in 8 phases: sample j at
@@ -208,6 +209,7 @@ inline int mx_max_tile(int HL, int HR, int lproj_b, int T)
     if (one_pass < t) t = one_pass;
     return t & ~(MX_TDI_BLOCK - 1);
 }
-// launch kinds: projection only, TDI only, fused, fused with the likelihood epilogue
-enum { KIND_PROJECT = 0, KIND_TDI = 1, KIND_FUSED = 2, KIND_LIKE = 3 };
+// launch kinds: projection only, TDI only, fused, fused with the likelihood epilogue; the mixed fused kernel
+// with MIXED_WIDE threads
+enum { KIND_PROJECT = 0, KIND_TDI = 1, KIND_FUSED = 2, KIND_LIKE = 3, KIND_WIDE = 4 };
 }  // namespace lr
