@@ -242,6 +242,7 @@ __device__ __forceinline__ long long piece_at(const PosPiece &p, int r)
 // Tile g of the launch: its source, offsets and sky frame.  In a batch the source is found by
 // galloping forward from s_hint, the source of the CTA's previous tile (a CTA's tiles come in
 // increasing order), then bisecting; the loops are bounded by the 64-bit index width.
+template <bool GEN>
 __device__ inline void mx_tile(const FwdParams &P, int64_t g, int ochan, int64_t &s_hint, TileInfo &ti,
                                SkyConst &sk)
 {
@@ -258,7 +259,7 @@ __device__ inline void mx_tile(const FwdParams &P, int64_t g, int ochan, int64_t
         ti.dat = P.like.data;
         ti.n0 = g * P.tile;
         sk = P.src.skyc1;
-        if (P.gen_strain) ti.gb = make_gb(P.src.gb1);
+        if (GEN) ti.gb = make_gb_lazy(P.src.gb1);
     } else {
         const int64_t *to = P.src.tile_off;
         const int64_t S = P.src.S;
@@ -278,8 +279,8 @@ __device__ inline void mx_tile(const FwdParams &P, int64_t g, int ochan, int64_t
         const int64_t s = lo;
         s_hint = s;
         int64_t ho = 0, ho1 = 0;
-        if (P.gen_strain) {
-            ti.gb = make_gb(P.src.gb[s]);
+        if (GEN) {
+            ti.gb = make_gb_lazy(P.src.gb[s]);
         } else {
             ho = __ldg(P.src.h_off + s);
             ho1 = __ldg(P.src.h_off + s + 1);
@@ -288,7 +289,7 @@ __device__ inline void mx_tile(const FwdParams &P, int64_t g, int ochan, int64_t
         ti.N = oo1 - oo;
         ti.nh = ho1 - ho;
         if (ti.N < 0 || ti.nh < 0) ti.ok = 0;
-        ti.t0h = P.gen_strain ? P.t0 : __ldg(P.src.t0h + s);  // no strain arrays when generated
+        ti.t0h = GEN ? P.t0 : __ldg(P.src.t0h + s);  // no strain arrays when generated
         ti.sky = P.src.sky[s];
         ti.hp = P.hp + ho;
         ti.hc = P.hc + ho;
@@ -298,7 +299,7 @@ __device__ inline void mx_tile(const FwdParams &P, int64_t g, int ochan, int64_t
         ti.n0 = (g - __ldg(to + s)) * P.tile;
         sk = P.src.skyc[s];
     }
-    if (P.gen_strain) {  // the waveform on the output grid, at every index
+    if (GEN) {  // the waveform on the output grid, at every index
         ti.nh = GEN_STRAIN_LEN;
         ti.t0h = P.t0;
     }
@@ -518,29 +519,12 @@ __device__ void build_tables2(float *smf, int base0, int AS, int SS, int npair, 
     }
 }
 
-// Generated strain window of a tile (Galactic binary on the output grid): out of line, so the
-// double-double phase and the sincos stay out of the hot body of kernels that read strain arrays.
-// Samples j0, j0 + stride, ...; returns this thread's largest bit pattern of |h|.
-__device__ __noinline__ unsigned long long stage_generated(const GbConst &g, double t0, double dt, int64_t i0,
-                                                           int wlen, double *pf, int j0, int stride)
-{
-    unsigned long long mx = 0ull;
-    for (int j = j0; j < wlen; j += stride) {
-        double a, b;
-        gb_strain(g, t0, dt, i0 + j, a, b);
-        pf[j] = a;
-        pf[MX_WCAP + j] = b;
-        mx = max(mx, max(abs_bits(a), abs_bits(b)));
-    }
-    return mx;
-}
-
 // ---------------------------------------------------------------- per-tile setup
 // Tile g's bookkeeping (one thread): source, offsets, sky frame, span.
-template <int KIND>
+template <int KIND, bool GEN>
 __device__ void tile_begin(const FwdParams &P, MxShared &sh, TileSetup &ts, int64_t g)
 {
-    mx_tile(P, g, KIND == KIND_PROJECT ? 6 : 3, sh.s_hint, ts.ti, ts.sk);
+    mx_tile<GEN>(P, g, KIND == KIND_PROJECT ? 6 : 3, sh.s_hint, ts.ti, ts.sk);
     if (!ts.ti.ok) atomicOr(P.err, ERR_OFFSETS);
     const int hl = KIND == KIND_PROJECT ? 0 : P.HL, hr = KIND == KIND_PROJECT ? 0 : P.HR;
     ts.k_lo = ts.ti.n0 - hl;
@@ -689,14 +673,56 @@ __device__ void fit_geometry(const FwdParams &P, TileSetup &ts, int f)
     ts.g3[f] = (float)b[3];
 }
 
+// first sample of the strain window relative to the link span (0 when the window exceeds its arrays)
+__device__ __forceinline__ int window_start(const TileSetup &ts, int h)
+{
+    const long long span = (long long)ts.whi - (long long)ts.wlo + (2 * h + 2) + 4;
+    return span > 0 && span <= MX_WCAP ? ts.wlo - h - 2 : 0;
+}
+
+// Rotation tables of a tile's generated strain (lr_gb.cuh), by one warp: the phasors of the anchors (sample
+// 32 a + 16 of the strain window) and of the offsets 0 .. 16 on its 32 lanes through one code path, and the drift
+// constant; turn == 0: the drift is too fast, generate sample by sample.
+constexpr int GB_ANCHORS = (MX_WCAP + GB_STEP - 1) / GB_STEP;
+static_assert(GB_ANCHORS + GB_OFF == 32, "one phasor per lane");
+struct GbTable {
+    double ph[32][2];
+    double kd;
+    int turn;
+};
+__device__ __forceinline__ void gb_table(const FwdParams &P, TileSetup &ts, int woff, int lane, GbTable &t)
+{
+    GbConst g = ts.ti.gb;
+    __syncwarp();
+    if (lane == 31) gb_amplitudes(ts.ti.gb);   // here, off the chain of the tile's bookkeeping
+    const double tc = P.t0 + (double)(ts.k_lo + ts.ny / 2) * P.dt;
+    if (lane == 0) {
+        t.turn = gb_rotation_fits(g, tc, P.dt, (MX_WCAP + MX_YCAP) * P.dt);
+        t.kd = 3.141592653589793 * (2.0 * g.fd2 + 6.0 * g.fdd6 * tc) * P.dt * P.dt;
+    }
+    double t0 = P.t0;
+    int64_t i = ts.k_lo + woff + GB_STEP * lane + GB_STEP / 2;
+    if (lane >= GB_ANCHORS) {  // an offset: the drift's frequency as a phase, from time zero
+        i = lane - GB_ANCHORS;
+        t0 = 0.0;
+        g.phi0 = 6.283185307179586 * ((2.0 * g.fd2 + 3.0 * g.fdd6 * tc) * tc) * ((double)(int)i * P.dt);
+        g.fd2 = g.fdd6 = 0.0;
+    }
+    gb_phasor(g, t0, P.dt, i, t.ph[lane][0], t.ph[lane][1]);
+}
+
 // the setup lanes of a tile (see SETUP_PIECE0); warp 7 fits the geometry cubics once its 12
 // lanes have the nodes
-template <int KIND>
-__device__ __forceinline__ void setup_lanes(const FwdParams &P, TileSetup &ts)
+template <int KIND, bool GEN>
+__device__ __forceinline__ void setup_lanes(const FwdParams &P, TileSetup &ts, int h, GbTable &gb)
 {
     const int tid = threadIdx.x;
-    if (tid >= SETUP_PIECE0 && tid < SETUP_PIECE0 + 30) {
-        setup_piece<KIND>(P, ts, tid - SETUP_PIECE0);
+    if (tid >= SETUP_PIECE0 && tid < SETUP_PIECE0 + (GEN ? 32 : 30)) {
+        if (!GEN || tid < SETUP_PIECE0 + 30) setup_piece<KIND>(P, ts, tid - SETUP_PIECE0);
+        if (GEN) {  // the pieces have given the strain window
+            __syncwarp();
+            gb_table(P, ts, window_start(ts, h), tid - SETUP_PIECE0, gb);
+        }
     } else if (KIND != KIND_TDI && tid >= SETUP_GEO0 && tid < SETUP_GEO0 + 32) {
         const int f = tid - SETUP_GEO0;
         if (f < 12) setup_geometry(P, ts, f);
@@ -1204,15 +1230,42 @@ __device__ __forceinline__ void tdi_chain(const FwdParams &P, const MxShared &sh
     }
 }
 
+// Generated strain window of a tile (Galactic binary on the output grid): samples j0, j0 + stride, ... turned
+// from the rotation tables that the tile's setup left (lr_gb.cuh), or generated one by one where the frequency
+// drifts too fast for them.  Returns this thread's largest bit pattern of |h|.  The sample-by-sample form kept
+// the FP64 pipe busy for ~18 % of the kernel: generated-strain likelihood of 24 sources of 2^16 to 2^20 samples,
+// order 25: 5.62 -> 5.24 ms.
+__device__ __forceinline__ unsigned long long stage_generated(const FwdParams &P, const TileSetup &ts, const GbTable &gb,
+                                                              int woff, int wlen, double *pf, int j0, int stride)
+{
+    const GbConst &g = ts.ti.gb;
+    unsigned long long mx = 0ull;
+    for (int j = j0; j < wlen; j += stride) {
+        double x, y;
+        if (gb.turn) {
+            const int a = j / GB_STEP, b = j % GB_STEP - GB_STEP / 2;
+            gb_turn(g, gb.kd, gb.ph[a], gb.ph[GB_ANCHORS + (b < 0 ? -b : b)], woff + GB_STEP * a + GB_STEP / 2 - ts.ny / 2, b, x, y);
+        } else {
+            gb_strain(g, P.t0, P.dt, ts.k_lo + woff + j, x, y);
+        }
+        pf[j] = x;
+        pf[MX_WCAP + j] = y;
+        mx = max(mx, max(abs_bits(x), abs_bits(y)));
+    }
+    return mx;
+}
+
 // ---------------------------------------------------------------- kernel
 // NT threads: 256 (two CTAs per SM up to order 31), or 512 for launches of at most one tile per SM, where a
 // tile's latency is the launch's: the same items on twice the warps (bit-identical), one round of the
 // threads instead of two in the projection and link phases.  N = 4096 at order 25: 42.9 -> 37.6 us a call.
-template <int T, int KIND, int NT = MIXED_THREADS>
+// GEN: the strain is a Galactic binary generated on the device (a separate instance: none of it in the others).
+template <int T, int KIND, int NT = MIXED_THREADS, bool GEN = false>
 __global__ void __launch_bounds__(NT, (NT == MIXED_THREADS && T <= 32 ? 2 : 1)) k_mixed(FwdParams P)
 {
     extern __shared__ __align__(16) float smf[];
     __shared__ MxShared sh;
+    __shared__ GbTable gbt[GEN ? 2 : 1];  // rotation tables, as sh.ts
     constexpr int h = (T - 2) / 2;
     // fused and projection launches set up the CTA's next tile on the warps a projection phase
     // leaves idle; TDI-only launches set up each tile in place
@@ -1228,9 +1281,9 @@ __global__ void __launch_bounds__(NT, (NT == MIXED_THREADS && T <= 32 ? 2 : 1)) 
     __syncthreads();
     int cur = 0;
     if (PREFETCH && blockIdx.x < sh.tot) {
-        if (tid == 0) tile_begin<KIND>(P, sh, sh.ts[0], blockIdx.x);
+        if (tid == 0) tile_begin<KIND, GEN>(P, sh, sh.ts[0], blockIdx.x);
         __syncthreads();
-        if (sh.ts[0].ti.ok && sh.ts[0].ti.nb > 0) setup_lanes<KIND>(P, sh.ts[0]);
+        if (sh.ts[0].ti.ok && sh.ts[0].ti.nb > 0) setup_lanes<KIND, GEN>(P, sh.ts[0], h, gbt[0]);
         __syncthreads();
     }
     for (int64_t g = blockIdx.x; g < sh.tot; g += gridDim.x, cur ^= PREFETCH ? 1 : 0) {
@@ -1239,17 +1292,17 @@ __global__ void __launch_bounds__(NT, (NT == MIXED_THREADS && T <= 32 ? 2 : 1)) 
         const int64_t gn = g + gridDim.x;
         const bool next = PREFETCH && gn < sh.tot;
         if (!PREFETCH) {
-            if (tid == 0) tile_begin<KIND>(P, sh, ts, g);
+            if (tid == 0) tile_begin<KIND, GEN>(P, sh, ts, g);
             __syncthreads();
-            if (ts.ti.ok && ts.ti.nb > 0) setup_lanes<KIND>(P, ts);
+            if (ts.ti.ok && ts.ti.nb > 0) setup_lanes<KIND, GEN>(P, ts, h, gbt[0]);
             __syncthreads();
         }
         if (!ts.ti.ok || ts.ti.nb <= 0) {
             if (LIKE && tid == 0) like_store(P, g, 0.0, 0.0);
             if (next) {
-                if (tid == 0) tile_begin<KIND>(P, sh, tn, gn);
+                if (tid == 0) tile_begin<KIND, GEN>(P, sh, tn, gn);
                 __syncthreads();
-                if (tn.ti.ok && tn.ti.nb > 0) setup_lanes<KIND>(P, tn);
+                if (tn.ti.ok && tn.ti.nb > 0) setup_lanes<KIND, GEN>(P, tn, h, gbt[GEN ? cur ^ 1 : 0]);
             }
             __syncthreads();
             continue;
@@ -1272,9 +1325,9 @@ __global__ void __launch_bounds__(NT, (NT == MIXED_THREADS && T <= 32 ? 2 : 1)) 
             const int nst = next ? NT - 1 : NT;
             unsigned long long mx = 0ull;
             if (tid >= nst) {
-                tile_begin<KIND>(P, sh, tn, gn);
-            } else if (P.gen_strain) {  // the Galactic binary generated at t0 + i dt
-                mx = stage_generated(ts.ti.gb, P.t0, P.dt, ts.k_lo + woff, wlen, pf, tid, nst);
+                tile_begin<KIND, GEN>(P, sh, tn, gn);
+            } else if (GEN) {  // the Galactic binary generated at t0 + i dt
+                mx = stage_generated(P, ts, gbt[GEN ? cur : 0], woff, wlen, pf, tid, nst);
             } else {
                 for (int j = tid; j < wlen; j += nst) {
                     const int64_t i = ts.k_lo + woff + j;
@@ -1340,7 +1393,7 @@ __global__ void __launch_bounds__(NT, (NT == MIXED_THREADS && T <= 32 ? 2 : 1)) 
             const int nblk = (ny + PB - 1) / PB;
             for (int it = tid; it < 9 * nblk; it += blockDim.x)
                 proj_item<T>(smf, ts, it / nblk, it % nblk, ny, wlen, woff_fx, P.err);
-            if (next && tn.ti.ok && tn.ti.nb > 0) setup_lanes<KIND>(P, tn);
+            if (next && tn.ti.ok && tn.ti.nb > 0) setup_lanes<KIND, GEN>(P, tn, h, gbt[GEN ? cur ^ 1 : 0]);
             __syncthreads();
             // ---- link series, in place over the staged reads: one thread per sample reads all
             //      of the sample's staged reads before writing its six links (same column)

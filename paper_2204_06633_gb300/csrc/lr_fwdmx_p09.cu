@@ -11,6 +11,8 @@ static void *kernel_ptr_mx(int kind)
         case KIND_TDI: return (void *)k_mixed<T, KIND_TDI>;
         case KIND_WIDE: return (void *)k_mixed<T, KIND_FUSED, MIXED_WIDE>;
         case KIND_LIKE: return (void *)k_mixed<T, KIND_LIKE>;
+        case KIND_FUSED_GEN: return (void *)k_mixed<T, KIND_FUSED, MIXED_THREADS, true>;
+        case KIND_LIKE_GEN: return (void *)k_mixed<T, KIND_LIKE, MIXED_THREADS, true>;
         default: return (void *)k_mixed<T, KIND_FUSED>;
     }
 }

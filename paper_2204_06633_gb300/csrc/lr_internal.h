@@ -209,7 +209,7 @@ inline int mx_max_tile(int HL, int HR, int lproj_b, int T)
     if (one_pass < t) t = one_pass;
     return t & ~(MX_TDI_BLOCK - 1);
 }
-// launch kinds: projection only, TDI only, fused, fused with the likelihood epilogue; the mixed fused kernel
-// with MIXED_WIDE threads
-enum { KIND_PROJECT = 0, KIND_TDI = 1, KIND_FUSED = 2, KIND_LIKE = 3, KIND_WIDE = 4 };
+// launch kinds: projection only, TDI only, fused, fused with the likelihood epilogue; of the mixed
+// kernels also the fused one with MIXED_WIDE threads and the two fused ones on generated strain
+enum { KIND_PROJECT = 0, KIND_TDI = 1, KIND_FUSED = 2, KIND_LIKE = 3, KIND_WIDE = 4, KIND_FUSED_GEN = 5, KIND_LIKE_GEN = 6 };
 }  // namespace lr

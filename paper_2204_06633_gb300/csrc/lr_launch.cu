@@ -21,6 +21,7 @@ int launch_forward(int precision, int kind, int order, FwdParams &P, int threads
     const bool mx = precision == LR_MIXED;
     if (!mx && P.fx_tile) return launch_fx64(kind, order, P, sms, stream);
     if (mx) threads = MIXED_THREADS;
+    if (mx && P.gen_strain) kind = kind == KIND_LIKE ? KIND_LIKE_GEN : KIND_FUSED_GEN;
     if (mx && kind == KIND_FUSED && P.total_tiles >= 0 && P.total_tiles <= sms && order < 41) {
         kind = KIND_WIDE;
         threads = MIXED_WIDE;
