@@ -55,6 +55,7 @@ namespace {
 
 // ---------------------------------------------------------------- the block's link series
 // Fills ys[6][NY] with the link series of rows 0 .. ny - 1 (sample k_lo + row).
+template <int NTHR>
 __device__ void project_block(const FwdParams &P, const FxTab &X, Shared &S, int T, int64_t k_lo, int ny, double u0, double *ys,
                               unsigned char *work)
 {
@@ -74,11 +75,12 @@ __device__ void project_block(const FwdParams &P, const FxTab &X, Shared &S, int
     // strain window: row j reads samples w_lo + j .. w_lo + j + KW - 1
     const int64_t w_lo = k_lo + (int64_t)fl0 + mmin - h;
     const int WL = ny + KW - 1;
-    double vp[3], vc[3];
+    constexpr int NV = (DL + NTHR - 1) / NTHR;
+    double vp[NV], vc[NV];
     if (!bad) {
 #pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            const int p = tid + i * 256;
+        for (int i = 0; i < NV; ++i) {
+            const int p = tid + i * NTHR;
             vp[i] = vc[i] = 0.0;
             if (p < WL) {
                 const int64_t idx = w_lo + p;
@@ -100,7 +102,7 @@ __device__ void project_block(const FwdParams &P, const FxTab &X, Shared &S, int
     if (!bad && vmax == 0) {  // a block of zeros (or of subnormal high words): the response is zero
         bool any = false;
 #pragma unroll
-        for (int i = 0; i < 3; ++i) any |= vp[i] != 0.0 || vc[i] != 0.0;
+        for (int i = 0; i < NV; ++i) any |= vp[i] != 0.0 || vc[i] != 0.0;
         if (!__syncthreads_or(any)) {
             for (int i = tid; i < 6 * NY; i += blockDim.x) ys[i] = 0.0;
             __syncthreads();
@@ -110,8 +112,8 @@ __device__ void project_block(const FwdParams &P, const FxTab &X, Shared &S, int
     }
     if (!bad) bad = !range_ok(S, &ex);
     if (!bad) {
-        for (int i = 0; i < 3; ++i) {
-            const int p = tid + i * 256;
+        for (int i = 0; i < NV; ++i) {
+            const int p = tid + i * NTHR;
             if (p < DL) {
                 digits_to_planes(planes, p, vp[i], ex);
                 digits_to_planes(planes + 7 * DL, p, vc[i], ex);
@@ -231,7 +233,7 @@ __device__ void project_block(const FwdParams &P, const FxTab &X, Shared &S, int
 // ---------------------------------------------------------------- the block's X, Y, Z
 // Link rows ys[6][NY] (ny = nb + HL + HR of them, row = output + HL) to outputs; ys is overwritten.
 // Each output is handed to `emit(i, X, Y, Z)` by one thread.
-template <class Emit>
+template <int NTHR, class Emit>
 __device__ void tdi_block(const FwdParams &P, const FxTab &X, Shared &S, int T, int64_t n0, int nb, double *ys, unsigned char *work,
                           Emit emit)
 {
@@ -257,8 +259,8 @@ __device__ void tdi_block(const FwdParams &P, const FxTab &X, Shared &S, int T, 
     // the first and last link rows are spare: no stencil reaches them
     for (int l = 0; l < 6; ++l)
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            const int j = tid + 256 * i;
+        for (int i = 0; i < NY / NTHR; ++i) {
+            const int j = tid + NTHR * i;
             range_update(S, j >= 1 && j < ny - 1 ? abs_hi(ys[l * NY + j]) : 0u);
         }
     const bool fast = S.fast != 0;
@@ -292,7 +294,7 @@ __device__ void tdi_block(const FwdParams &P, const FxTab &X, Shared &S, int T, 
             break;
         }
         int ew;
-        if (!tdi_stencils<false>(P, X, S, T, t_lo, sg, fast, KW, mmin, W, wt, &ew)) {
+        if (!tdi_stencils<false, NTHR>(P, X, S, T, t_lo, sg, fast, KW, mmin, W, wt, &ew)) {
             bad = true;
             break;
         }
@@ -402,8 +404,9 @@ __device__ void tdi_block(const FwdParams &P, const FxTab &X, Shared &S, int T, 
 }
 
 // ---------------------------------------------------------------- kernel
-template <int KIND>
-__global__ void __launch_bounds__(256, 2) k_fx64(FwdParams P, FxTab X, int T)
+// NTHR threads: 256 (two CTAs per SM), or 512 where a launch has at most a block per SM (65536 samples, order 25: 125 -> 113 us)
+template <int KIND, int NTHR>
+__global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx64(FwdParams P, FxTab X, int T)
 {
     extern __shared__ __align__(16) unsigned char sm_raw[];
     double *ys = reinterpret_cast<double *>(sm_raw);
@@ -433,7 +436,7 @@ __global__ void __launch_bounds__(256, 2) k_fx64(FwdParams P, FxTab X, int T)
             const TileInfo &ti = S.ti;
             const int nb = (int)ti.nb;
             if (KIND == KIND_PROJECT) {
-                project_block(P, X, S, T, ti.n0, nb, (P.t0 - ti.t0h) / P.dt, ys, work);
+                project_block<NTHR>(P, X, S, T, ti.n0, nb, (P.t0 - ti.t0h) / P.dt, ys, work);
                 for (int i = tid; i < nb; i += blockDim.x)
 #pragma unroll
                     for (int l = 0; l < 6; ++l) ti.out[l * ti.N + ti.n0 + i] = ys[l * NY + i];
@@ -448,10 +451,10 @@ __global__ void __launch_bounds__(256, 2) k_fx64(FwdParams P, FxTab X, int T)
                         }
                     __syncthreads();
                 } else {
-                    project_block(P, X, S, T, k_lo, ny, (P.t0 - ti.t0h) / P.dt, ys, work);
+                    project_block<NTHR>(P, X, S, T, k_lo, ny, (P.t0 - ti.t0h) / P.dt, ys, work);
                 }
                 double dh = 0.0, hh = 0.0;
-                tdi_block(P, X, S, T, ti.n0, nb, ys, work, [&](int i, double vx, double vy, double vz) {
+                tdi_block<NTHR>(P, X, S, T, ti.n0, nb, ys, work, [&](int i, double vx, double vy, double vz) {
                     const int64_t n = ti.n0 + i;
                     if (ti.out) {
                         ti.out[n] = vx;
@@ -582,13 +585,14 @@ __global__ void __launch_bounds__(256) k_fx_table(FwdParams P, FxTab X, int T, d
     }
 }
 
+template <int NTHR>
 void *kernel_of(int kind)
 {
     switch (kind) {
-        case KIND_PROJECT: return (void *)k_fx64<KIND_PROJECT>;
-        case KIND_TDI: return (void *)k_fx64<KIND_TDI>;
-        case KIND_FUSED: return (void *)k_fx64<KIND_FUSED>;
-        default: return (void *)k_fx64<KIND_LIKE>;
+        case KIND_PROJECT: return (void *)k_fx64<KIND_PROJECT, NTHR>;
+        case KIND_TDI: return (void *)k_fx64<KIND_TDI, NTHR>;
+        case KIND_FUSED: return (void *)k_fx64<KIND_FUSED, NTHR>;
+        default: return (void *)k_fx64<KIND_LIKE, NTHR>;
     }
 }
 
@@ -709,13 +713,14 @@ int fx_table_for(FxPlan *F, void *str, FxTab *X)
 
 int launch_fx64(int kind, int order, const FwdParams &P, int sms, void *stream)
 {
-    void *k = kernel_of(kind);
+    const int nthr = P.total_tiles >= 0 && P.total_tiles <= sms ? 512 : 256;
+    void *k = nthr == 512 ? kernel_of<512>(kind) : kernel_of<256>(kind);
     int T = order + 1;
     const size_t smem = smem_of(T);
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return (int)e;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 256, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, nthr, smem);
     if (e != cudaSuccess) return (int)e;
     if (per_sm < 1) return (int)cudaErrorLaunchOutOfResources;
     int64_t grid = (int64_t)per_sm * sms;
@@ -724,7 +729,7 @@ int launch_fx64(int kind, int order, const FwdParams &P, int sms, void *stream)
     FxTab X;
     if (const int te = fx_table_for(P.fx, stream, &X)) return te;
     void *args[] = {(void *)&P, (void *)&X, (void *)&T};
-    return (int)cudaLaunchKernel(k, dim3((unsigned)grid), dim3(256), args, smem, (cudaStream_t)stream);
+    return (int)cudaLaunchKernel(k, dim3((unsigned)grid), dim3(nthr), args, smem, (cudaStream_t)stream);
 }
 
 }  // namespace lr

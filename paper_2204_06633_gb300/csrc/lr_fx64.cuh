@@ -24,7 +24,8 @@ constexpr int NGT = NY / GT + 1;
 constexpr int NTERM = 42;
 constexpr int WTS = 4 * NTERM + 1;   // row length of the TDI node weights (odd: no bank conflicts)
 constexpr int WNS = NN * 9;
-constexpr int REPS = (12 * 57 + 255) / 256;  // merged TDI taps per thread: at most 12 stencils of 57 taps
+// merged TDI taps per thread: at most 12 stencils of 57 taps
+__host__ __device__ constexpr int tap_reps(int nthr) { return (12 * 57 + nthr - 1) / nthr; }
 constexpr int RANGE_BITS = 12;
 // the last order's coefficient must be below 2^-45 of the stencil's scale: the next one is then below 2^-53
 constexpr double LAST_MAX = 1024.0;
@@ -95,7 +96,7 @@ struct Shared {
     unsigned long long qor[NN];  // OR of the coefficients' magnitudes per order
     int nq, last;                // orders in use; whether those above 0 have their last digit only
     int bad;
-    double red[2 * 8];
+    double red[2 * 16];
 };
 
 __device__ __forceinline__ void mma_f16(float *c, const uint32_t *a, uint32_t b0, uint32_t b1)
@@ -812,7 +813,7 @@ __device__ void find_tdi_segments(const FwdParams &P, Shared &S, double t_lo, in
 // Digit rows W of segment sg's merged TDI stencils (REV: taps in reverse) and their scale *ew_out: from the
 // plan's table (fast), or from the delayed reads' weights at four nodes (wt [T][WTS]).  False when the
 // coefficients do not fit their digits.  Begins and ends with a barrier.
-template <bool REV>
+template <bool REV, int NTHR>
 __device__ __forceinline__ bool tdi_stencils(const FwdParams &P, const FxTab &X, Shared &S, int T, double t_lo, int sg,
                                              bool fast, int KW, int mmin, unsigned char *W, double *wt, int *ew_out)
 {
@@ -848,11 +849,11 @@ __device__ __forceinline__ bool tdi_stencils(const FwdParams &P, const FxTab &X,
     // table around the block's centre
     const double xc = 2.0 * ((t_lo + 0.5 * (NY - 1) * P.dt - P.to.t_first) * P.to.inv_dk - (double)piece) - 1.0;
     const double xs = NY * P.dt * P.to.inv_dk;
-    double b[REPS][NT];
+    double b[tap_reps(NTHR)][NT];
     float bm = 0.0f;
 #pragma unroll
-    for (int rep = 0; rep < REPS; ++rep) {
-        const int i = tid + 256 * rep;
+    for (int rep = 0; rep < tap_reps(NTHR); ++rep) {
+        const int i = tid + NTHR * rep;
         if (i < 12 * KW && fast) {
             table_coefs(P, X, piece, (i / KW) * X.tab_kw + i % KW, xc, xs, b[rep]);
         } else {
@@ -893,8 +894,8 @@ __device__ __forceinline__ bool tdi_stencils(const FwdParams &P, const FxTab &X,
     bool fits = sm_max < 1e30f;
     unsigned long long mag[NT] = {};
 #pragma unroll
-    for (int rep = 0; rep < REPS; ++rep) {
-        const int i = tid + 256 * rep;
+    for (int rep = 0; rep < tap_reps(NTHR); ++rep) {
+        const int i = tid + NTHR * rep;
         if (i < 12 * KW) {
             const int cs = i / KW, tap = i - cs * KW;
             unsigned char *w = W + cs * TD * WS + 7 + (REV ? KW - 1 - tap : tap);

@@ -39,8 +39,13 @@ constexpr int GROWS = gplane(false, NN);                      // 44 rows per lin
 constexpr int K1_PART = 3 * NY * 8, K1_PLANES = K1_PART + 6 * NY * 8;
 // the node weights of blocks off the table share the sums' and planes' place
 __host__ __device__ constexpr int k1_w(int T) { return K1_PART + (T * WTS * 8 > 6 * NY * 8 + TQP * DL * 2 ? T * WTS * 8 : 6 * NY * 8 + TQP * DL * 2); }
-constexpr int K2_PLANES = 6 * NY * 8, K2_W = K2_PLANES + PQB * DL * 2, K2_END = K2_W + FX_PROJ_W;
-constexpr int K3_G = FX_PROJ_PLANES, K3_GEND = K3_G + 2 * GROWS * GB;
+constexpr int K2_STENCILS = 6 * NY * 8, K2_PLANES = K2_STENCILS + FX_PROJ_W, K2_GROUP = PQB * DL * 2;  // one group of planes per 256 threads
+constexpr int K3_G = FX_PROJ_PLANES, K3_PAIR = 2 * GROWS * GB;   // digit rows of a link pair per 256 threads
+__host__ __device__ constexpr int k3_c(int T, int nthr)
+{
+    const int g = nthr / 256 * K3_PAIR, w = 16 * T * WNS;
+    return K3_G + (((g > w ? g : w) + 15) & ~15);
+}
 
 // acc[L] += the level sums of order Q, its digit planes at `a_lane`, its digit rows at `w_lane`
 template <int Q, bool TDI, bool LAST>
@@ -156,7 +161,7 @@ __device__ void tdi_adj_scalar(const FwdParams &P, Shared &S, int T, int64_t k0,
             }
             __syncthreads();
             for (int r = 0; r < 2; ++r) {
-                const int i = tid + 256 * r;
+                const int i = tid + (int)blockDim.x * r;
                 if (i >= nb) continue;
                 for (int j = 0; j < 16; ++j) {
                     const double g = gs[ch * NY + p0 + j];
@@ -182,12 +187,13 @@ __device__ void tdi_adj_scalar(const FwdParams &P, Shared &S, int T, int64_t k0,
             }
         }
     for (int r = 0; r < 2; ++r)
-        if (tid + 256 * r < nb)
-            for (int l = 0; l < 6; ++l) gy[l * N + k0 + tid + 256 * r] = acc[r][l];
+        if (tid + (int)blockDim.x * r < nb)
+            for (int l = 0; l < 6; ++l) gy[l * N + k0 + tid + (int)blockDim.x * r] = acc[r][l];
     __syncthreads();
 }
 
-__global__ void __launch_bounds__(256, 2) k_fx_tdi_adj(FwdParams P, FxTab X, BwdParams B, int T)
+template <int NTHR>
+__global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_tdi_adj(FwdParams P, FxTab X, BwdParams B, int T)
 {
     extern __shared__ __align__(16) unsigned char sm_raw[];
     double *gs = reinterpret_cast<double *>(sm_raw);
@@ -223,8 +229,8 @@ __global__ void __launch_bounds__(256, 2) k_fx_tdi_adj(FwdParams P, FxTab X, Bwd
         bool any = false;
         for (int c = 0; c < 3; ++c)
 #pragma unroll
-            for (int r = 0; r < 2; ++r) {
-                const int p = tid + 256 * r;
+            for (int r = 0; r < NY / NTHR; ++r) {
+                const int p = tid + NTHR * r;
                 const int64_t n = n_lo + p;
                 const double v = p < rows && n >= 0 && n < N ? __ldg(gx + c * N + n) : 0.0;
                 gs[c * NY + p] = v;
@@ -255,7 +261,7 @@ __global__ void __launch_bounds__(256, 2) k_fx_tdi_adj(FwdParams P, FxTab X, Bwd
             const int js = S.segj[sg], je = S.segj[sg + 1];
             int ew;
             if (nks * 16 > 64 || nb + KW - 1 > rows || (!fast && S.mmax >= 0) ||
-                !tdi_stencils<true>(P, X, S, T, t_lo, sg, fast, KW, mmin, W, wt, &ew)) {
+                !tdi_stencils<true, NTHR>(P, X, S, T, t_lo, sg, fast, KW, mmin, W, wt, &ew)) {
                 bad = true;
                 break;
             }
@@ -368,7 +374,7 @@ __device__ void proj_adj_scalar(const FwdParams &P, Shared &S, int T, double u0,
         if (tid < 72) lagrange_to(S, T, U[tid] - floor(U[tid]), w + tid, 72);
         __syncthreads();
         for (int r = 0; r < 2; ++r) {
-            const int i = tid + 256 * r;
+            const int i = tid + (int)blockDim.x * r;
             if (i >= nb) continue;
             for (int id = 0; id < 72; ++id) {
                 const int64_t a = i0 + i - (k_lo + j0 + (id & 7) + (int64_t)floor(U[id])) + h;
@@ -379,9 +385,9 @@ __device__ void proj_adj_scalar(const FwdParams &P, Shared &S, int T, double u0,
         }
     }
     for (int r = 0; r < 2; ++r)
-        if (tid + 256 * r < nb) {
-            ghp[i0 + tid + 256 * r] = acc[r][0];
-            ghc[i0 + tid + 256 * r] = acc[r][1];
+        if (tid + (int)blockDim.x * r < nb) {
+            ghp[i0 + tid + (int)blockDim.x * r] = acc[r][0];
+            ghc[i0 + tid + (int)blockDim.x * r] = acc[r][1];
         }
     __syncthreads();
 }
@@ -416,18 +422,20 @@ __device__ __forceinline__ void proj_order(float (&acc)[7][4], const unsigned ch
     contract_order<Q, false, LAST>(acc, a_lane + (gplane(false, Q) - base) * DL * 2, w_lane + digit_row(false, Q) * WS, sh, nks);
 }
 
-__global__ void __launch_bounds__(256, 2) k_fx_proj_adj(FwdParams P, FxTab X, BwdParams B, int T)
+template <int NTHR>
+__global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_proj_adj(FwdParams P, FxTab X, BwdParams B, int T)
 {
     extern __shared__ __align__(16) unsigned char sm_raw[];
     double *gys = reinterpret_cast<double *>(sm_raw);
-    uint16_t *planes = reinterpret_cast<uint16_t *>(sm_raw + K2_PLANES);
-    unsigned char *W = sm_raw + K2_W;
+    constexpr int NGR = NTHR / 256;   // groups of eight warps: each takes every NGR-th link, in planes of its own
+    unsigned char *W = sm_raw + K2_STENCILS;
     double *wn = reinterpret_cast<double *>(sm_raw + K2_PLANES);  // the node weights are done with before the planes
     __shared__ Shared S;
     __shared__ int nbs, umin, umax;
     __shared__ double u0s;
     const int tid = threadIdx.x, h = (T - 2) / 2;
-    const int lane = tid & 31, warp = tid >> 5, lr4 = lane >> 2, kp = lane & 3;
+    const int lane = tid & 31, warp = (tid >> 5) & 7, grp = tid >> 8, lr4 = lane >> 2, kp = lane & 3;
+    uint16_t *planes = reinterpret_cast<uint16_t *>(sm_raw + K2_PLANES + grp * K2_GROUP);
     const uint32_t sh = 8 * ((7 - lr4) & 3);
     lagrange_tables(S, T);
     if (tid < 32 && !B.h_tile_off) sky_by_warp(P.src.sky1, &S.skc);
@@ -471,8 +479,8 @@ __global__ void __launch_bounds__(256, 2) k_fx_proj_adj(FwdParams P, FxTab X, Bw
         bool any = false;
         for (int l = 0; l < 6; ++l)
 #pragma unroll
-            for (int r = 0; r < 2; ++r) {
-                const int j = tid + 256 * r;
+            for (int r = 0; r < NY / NTHR; ++r) {
+                const int j = tid + NTHR * r;
                 const int64_t k = k_lo + j;
                 const double v = k >= 0 && k < N ? __ldg(gy + l * N + k) : 0.0;
                 gys[l * NY + j] = v;
@@ -499,10 +507,10 @@ __global__ void __launch_bounds__(256, 2) k_fx_proj_adj(FwdParams P, FxTab X, Bw
             const bool last = S.last;
             long long sum[4] = {0, 0, 0, 0};
             const unsigned char *a_lane = reinterpret_cast<const unsigned char *>(planes) + 8 * (16 * warp + lr4) + 8 * kp;
-            for (int l = 0; l < 6; ++l) {
+            for (int l = grp; l < 6; l += NGR) {
                 const unsigned char *w_lane = W + (2 * l + (lr4 >> 2)) * PD * WS + 4 + 4 * kp;
                 float acc[7][4] = {};
-                for (int p = tid; p < DL; p += blockDim.x) {
+                for (int p = tid & 255; p < DL; p += 256) {
                     const int j = p + j0;
                     const bool in = j >= js && j < je;
                     order_planes<0, QA>(planes, p, in ? to_fixed(gys[l * NY + j], eg) : 0, 2 * j + 1 - NY, in);
@@ -520,7 +528,7 @@ __global__ void __launch_bounds__(256, 2) k_fx_proj_adj(FwdParams P, FxTab X, Bw
                 }
                 __syncthreads();
                 if (nq > QA) {
-                    for (int p = tid; p < DL; p += blockDim.x) {
+                    for (int p = tid & 255; p < DL; p += 256) {
                         const int j = p + j0;
                         const bool in = j >= js && j < je;
                         order_planes<QA, NN>(planes, p, in ? to_fixed(gys[l * NY + j], eg) : 0, 2 * j + 1 - NY, in);
@@ -551,16 +559,23 @@ __global__ void __launch_bounds__(256, 2) k_fx_proj_adj(FwdParams P, FxTab X, Bw
             for (int r = 0; r < 4; ++r) out[r] += from_fixed(sum[r], unit);
         }
         __syncthreads();
-        if (!bad) {
+        double *parts = reinterpret_cast<double *>(sm_raw + K2_PLANES);   // the second group's sums
+        if (NGR > 1) {
+            if (grp == 1 && !bad)
+                for (int r = 0; r < 4; ++r) parts[4 * (tid & 255) + r] = out[r];
+            __syncthreads();
+            if (grp == 0 && !bad)
+                for (int r = 0; r < 4; ++r) out[r] += parts[4 * tid + r];
+        }
+        if (!bad && grp == 0) {
             double *o = (kp >> 1) ? ghc : ghp;
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
                 const int i = 64 * warp + 4 * (lr4 + (r >> 1) * 8) + 2 * (kp & 1) + (r & 1);
                 if (i < nb) o[i0 + i] = out[r];
             }
-        } else {
-            proj_adj_scalar(P, S, T, u0, i0, nb, k_lo, gys, ghp, ghc, reinterpret_cast<double *>(sm_raw + K2_PLANES));
         }
+        if (bad) proj_adj_scalar(P, S, T, u0, i0, nb, k_lo, gys, ghp, ghc, reinterpret_cast<double *>(sm_raw + K2_STENCILS));
         __syncthreads();
     }
 }
@@ -714,18 +729,18 @@ __device__ __forceinline__ void correlate_item(double *C, int LG, const unsigned
 __constant__ signed char c_items[8][4] = {{0, 14, -1, -1}, {1, 15, -1, -1}, {2, -1, -1, -1}, {3, -1, -1, -1},
                                           {4, 8, -1, -1},  {5, 9, -1, -1},  {6, 10, 12, -1}, {7, 11, 13, -1}};
 
-__global__ void __launch_bounds__(256, 2) k_fx_sky_adj(FwdParams P, FxTab X, BwdParams B, int T)
+template <int NTHR>
+__global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_sky_adj(FwdParams P, FxTab X, BwdParams B, int T)
 {
     extern __shared__ __align__(16) unsigned char sm_raw[];
     uint16_t *planes = reinterpret_cast<uint16_t *>(sm_raw);
     unsigned char *G = sm_raw + K3_G;
     double *wn = reinterpret_cast<double *>(sm_raw + K3_G), *dwn = wn + T * WNS;   // once the digit rows are done with
-    const int gend = K3_GEND > K3_G + 16 * T * WNS ? K3_GEND : K3_G + 16 * T * WNS;
-    double *C = reinterpret_cast<double *>(sm_raw + ((gend + 15) & ~15));          // [link][order or node][pol][LG]
+    double *C = reinterpret_cast<double *>(sm_raw + k3_c(T, NTHR));          // [link][order or node][pol][LG]
     const int LG = X.lags;
     __shared__ Shared S;
     __shared__ double dots[NN][6][2][4];   // node, link, (emission, reception): h+ value, derivative, hx value, derivative
-    __shared__ double red[3][8];
+    __shared__ double red[3][NTHR / 32];
     __shared__ unsigned gmax, gmin;
     const int tid = threadIdx.x, h = (T - 2) / 2;
     const int lane = tid & 31, warp = tid >> 5, lr4 = lane >> 2, kp = lane & 3;
@@ -757,11 +772,12 @@ __global__ void __launch_bounds__(256, 2) k_fx_sky_adj(FwdParams P, FxTab X, Bwd
             const int64_t w_lo = k_lo + (int64_t)fl0 + mmin - h;
             const int WL = nb + KW - 1;
             bool anyg = false, anyh = false;
-            double vp[3], vc[3];
+            constexpr int NV = (DL + NTHR - 1) / NTHR;
+            double vp[NV], vc[NV];
             if (!bad) {
 #pragma unroll
-                for (int i = 0; i < 3; ++i) {
-                    const int p = tid + i * 256;
+                for (int i = 0; i < NV; ++i) {
+                    const int p = tid + i * NTHR;
                     const int64_t idx = w_lo + p;
                     vp[i] = vc[i] = 0.0;
                     if (p < WL && idx >= 0 && idx < ti.nh) {
@@ -774,8 +790,8 @@ __global__ void __launch_bounds__(256, 2) k_fx_sky_adj(FwdParams P, FxTab X, Bwd
                 }
                 for (int l = 0; l < 6; ++l)
 #pragma unroll
-                    for (int r = 0; r < 2; ++r) {
-                        const int j = tid + 256 * r;
+                    for (int r = 0; r < NY / NTHR; ++r) {
+                        const int j = tid + NTHR * r;
                         const double v = j < nb ? __ldg(gy + l * N + k_lo + j) : 0.0;
                         anyg |= v != 0.0;
                         const unsigned m = __reduce_max_sync(0xffffffffu, abs_hi(v));
@@ -795,8 +811,8 @@ __global__ void __launch_bounds__(256, 2) k_fx_sky_adj(FwdParams P, FxTab X, Bwd
             }
             if (!bad && work) {
 #pragma unroll
-                for (int i = 0; i < 3; ++i) {
-                    const int p = tid + i * 256;
+                for (int i = 0; i < NV; ++i) {
+                    const int p = tid + i * NTHR;
                     if (p < DL) {
                         digits_to_planes(planes, p, vp[i], ex);
                         digits_to_planes(planes + 7 * DL, p, vc[i], ex);
@@ -807,13 +823,17 @@ __global__ void __launch_bounds__(256, 2) k_fx_sky_adj(FwdParams P, FxTab X, Bwd
                     const int js = S.segj[sg], je = S.segj[sg + 1];
                     __syncthreads();
                     for (int i = tid; i < 12 * NN * LG; i += blockDim.x) C[i] = 0.0;
-                    for (int lp = 0; lp < 3; ++lp) {
+                    // link pairs one after the other (256 threads), or the first two side by side and then
+                    // the third with an item per warp
+                    constexpr int NGR = NTHR / 256, ROUNDS = NGR == 1 ? 3 : 2;
+                    for (int round = 0; round < ROUNDS; ++round) {
+                        const int lp0 = NGR * round, np = 3 - lp0 < NGR ? 3 - lp0 : NGR;
                         __syncthreads();
-                        for (int i = tid; i < 2 * GROWS * GB / 4; i += blockDim.x) reinterpret_cast<uint32_t *>(G)[i] = 0x80808080u;
+                        for (int i = tid; i < np * K3_PAIR / 4; i += NTHR) reinterpret_cast<uint32_t *>(G)[i] = 0x80808080u;
                         __syncthreads();
-                        for (int i = tid; i < 2 * (je - js); i += blockDim.x) {
-                            const int l2 = i >= je - js, j = js + i - l2 * (je - js);
-                            const long long x0 = to_fixed(__ldg(gy + (2 * lp + l2) * N + k_lo + j), eg);
+                        for (int i = tid; i < 2 * np * (je - js); i += NTHR) {
+                            const int l2 = i / (je - js), j = js + i - l2 * (je - js);
+                            const long long x0 = to_fixed(__ldg(gy + (2 * lp0 + l2) * N + k_lo + j), eg);
                             const int kappa = 2 * j + 1 - NY;
                             unsigned char *row = G + l2 * GROWS * GB + 7 + j;
                             long long xa = x0, xb = mul_nu<9>(x0, kappa);
@@ -831,11 +851,13 @@ __global__ void __launch_bounds__(256, 2) k_fx_sky_adj(FwdParams P, FxTab X, Bwd
                             }
                         }
                         __syncthreads();
-                        const unsigned char *g_lane = G + (lr4 >> 2) * GROWS * GB + 4 + 4 * kp;
+                        const bool shared_pair = np < NGR;   // all warps on one pair, one item each
+                        const int pr = shared_pair ? 0 : warp >> 3, lp = lp0 + pr;
+                        const unsigned char *g_lane = G + pr * K3_PAIR + (lr4 >> 2) * GROWS * GB + 4 + 4 * kp;
                         for (int ps = 0; ps < npass; ++ps) {
                             const unsigned char *a_lane = reinterpret_cast<const unsigned char *>(planes) + 8 * (lr4 + 8 * ps) + 8 * kp;
-                            for (int k = 0; k < 4; ++k) {
-                                const int it = c_items[warp][k];
+                            for (int k = 0; k < (shared_pair ? 1 : 4); ++k) {
+                                const int it = shared_pair ? warp : c_items[warp & 7][k];
                                 if (it < 0) break;
                                 const int s0 = (it & 1) ? mid : 0, s1 = (it & 1) ? steps : mid;
                                 switch (it >> 1) {
@@ -979,7 +1001,7 @@ __global__ void __launch_bounds__(256, 2) k_fx_sky_adj(FwdParams P, FxTab X, Bwd
         __syncthreads();
         if (tid < 3) {
             double s = 0.0;
-            for (int w = 0; w < 8; ++w) s += red[tid][w];
+            for (int w = 0; w < NTHR / 32; ++w) s += red[tid][w];
             B.partial[3 * g + tid] = s;
         }
         __syncthreads();
@@ -993,24 +1015,25 @@ int launch_fx_bwd(int kind, int order, const FwdParams &P, const BwdParams &B, F
     int T = order + 1;
     FxTab X;
     if (const int e = fx_table_for(F, stream, &X)) return e;
-    void *k = kind == 0 ? (void *)k_fx_tdi_adj : kind == 1 ? (void *)k_fx_proj_adj : (void *)k_fx_sky_adj;
-    size_t smem = kind == 0 ? k1_w(T) + FX_TDI_W : K2_END;
-    if (kind == 2) {
-        const size_t w = K3_G + 16 * (size_t)T * WNS;
-        smem = ((w > K3_GEND ? w : K3_GEND) + 15 & ~(size_t)15) + sizeof(double) * 12 * NN * (size_t)X.lags;
-    }
+    const int64_t known = kind == 1 ? B.h_total_tiles : P.total_tiles;
+    // 512 threads a block where the launch has at most a block per SM
+    const int nthr = known >= 0 && known <= sms ? 512 : 256;
+    void *k = nthr == 512 ? (kind == 0 ? (void *)k_fx_tdi_adj<512> : kind == 1 ? (void *)k_fx_proj_adj<512> : (void *)k_fx_sky_adj<512>)
+                          : (kind == 0 ? (void *)k_fx_tdi_adj<256> : kind == 1 ? (void *)k_fx_proj_adj<256> : (void *)k_fx_sky_adj<256>);
+    const size_t smem = kind == 0 ? k1_w(T) + FX_TDI_W
+                        : kind == 1 ? K2_PLANES + nthr / 256 * K2_GROUP
+                                    : k3_c(T, nthr) + sizeof(double) * 12 * NN * (size_t)X.lags;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return (int)e;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 256, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, nthr, smem);
     if (e != cudaSuccess) return (int)e;
     if (per_sm < 1) return (int)cudaErrorLaunchOutOfResources;
     int64_t grid = (int64_t)per_sm * sms;
-    const int64_t known = kind == 1 ? B.h_total_tiles : P.total_tiles;
     if (known >= 0 && known < grid) grid = known;
     if (grid < 1) grid = 1;
     void *args[] = {(void *)&P, (void *)&X, (void *)&B, (void *)&T};
-    return (int)cudaLaunchKernel(k, dim3((unsigned)grid), dim3(256), args, smem, (cudaStream_t)stream);
+    return (int)cudaLaunchKernel(k, dim3((unsigned)grid), dim3(nthr), args, smem, (cudaStream_t)stream);
 }
 
 }  // namespace lr
