@@ -10,6 +10,8 @@
 //   K3  dLoss/d(lambda, beta, psi) partial sums per tile: the derivative of each link sample
 //                           (patterns, 1/(1 - k.n) and read times through k) against g_y,
 //                           with derivative Lagrange weights; K4 adds the partials in order.
+// They serve the plans that the tensor-core kernels of lr_fxbwd.cu do not take (those of lr_fwd64.cu, and plans
+// without a table of TDI stencils); K4 serves both.  65 536 samples at order 25: K1 1.26 ms here, 0.063 there.
 // All arithmetic is FP64.  Link series are never stored: K1 only needs the orbit, K3 recomputes
 // the strain reads.
 #include <cuda_runtime.h>

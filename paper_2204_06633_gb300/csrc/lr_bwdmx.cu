@@ -3,6 +3,10 @@
 // cotangents on the FP32 pipe, while the orbit splines, the delays and the read positions stay FP64 and every
 // index split is exact integer work on 64-bit fixed point (44 fractional bits).
 //
+// They serve the mixed plans that the tensor-core kernels of lr_fxbwd.cu do not take: varying nested delays, merged
+// stencils of more than 64 taps, no table of TDI stencils.  One year at order 41: 30.3 ms for the three kernels here,
+// 12.4 there.
+//
 // Structure as the FP64 kernels (lr_bwd.cu): deterministic gathers over inverted tap windows.
 //   KM1  g_y = T^T g_xyz   tile of 256 link samples; per window output the six link delays in fixed
 //                          point; per term float-float reference weights at the window centre with

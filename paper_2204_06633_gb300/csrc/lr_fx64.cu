@@ -38,11 +38,13 @@
 // of a row with one 8-byte load and its right registers from four consecutive digit bytes, which become
 // halves by placing them under the exponent of 1024 and subtracting 1152.
 //
-// Measured (fused, order 25, one year of 3 153 600 outputs): 44.45 ms sample by sample, 3.65 ms here, with
-// 1.3e-13 relative error against 64 bits where the sample form has 1.4e-13.  Two blocks share an SM; the
-// tensor pipe is busy a third of the time and the FP64 pipe (weights, transforms) a quarter, the rest is
-// latency of the short FP64 phases.  With 8-sample rows in the projection and the TDI stencils computed in
-// every block it was 4.36 ms.
+// Measured (fused, order 25, one year of 3 153 600 outputs): 44.45 ms sample by sample, 3.4 to 4.0 ms here (the
+// source's position sets how many segments a block has), with 3.0e-12 relative error against 64 bits where
+// the sample form has 3.5e-12; 65 536 outputs: 490 us and 108 us.  Two blocks share an SM; the tensor pipe is
+// busy a third of the time and the FP64 pipe (weights, transforms) a quarter, the rest is latency of the short
+// FP64 phases.  Steps on the way, one year: 4.36 ms with 8-sample rows in the projection and the TDI stencils
+// computed in every block; 65 536 outputs: 113 us with the weights and the links' patterns of the nodes on the
+// same warps, the TDI stencils' scale found in the block, and a barrier more for each of the two scales.
 //
 // Where the expansion does not apply, the block is evaluated sample by sample in FP64 as in lr_fwd64.cu: a
 // NaN or infinity in the series, values that span more than 12 bits between 32-sample stretches (the
@@ -285,8 +287,8 @@ __device__ void tdi_block(const FwdParams &P, const FxTab &X, Shared &S, int T, 
     int done = 0;                                          // outputs kept in ys[0..2][.] by earlier segments
     for (int sg = 0; sg < nseg && !bad; ++sg) {
         const int piece = S.segm[sg][NTERM];
-        const int mmin = fast ? X.meta[2 * piece + 1] : S.mmin;
-        const int KW = fast ? X.meta[2 * piece] : (S.mmax > 0 ? S.mmax : 0) - mmin + T;
+        const int mmin = fast ? X.meta[FX_META * piece + 1] : S.mmin;
+        const int KW = fast ? X.meta[FX_META * piece] : (S.mmax > 0 ? S.mmax : 0) - mmin + T;
         const int nks = (KW + 7 + 15) / 16;
         const int j0 = P.HL + mmin - h;                        // link row of the stencil's first tap for output 0
         if (!fast && (nks * 16 > 64 || j0 < 1 || S.mmax > 0)) {
@@ -294,7 +296,8 @@ __device__ void tdi_block(const FwdParams &P, const FxTab &X, Shared &S, int T, 
             break;
         }
         int ew;
-        if (!tdi_stencils<false, NTHR>(P, X, S, T, t_lo, sg, fast, KW, mmin, W, wt, &ew)) {
+        if (!(fast ? tdi_stencils<false, NTHR>(P, X, S, t_lo, sg, KW, W, &ew)
+                   : tdi_stencils_nodes<false, NTHR>(P, X, S, T, t_lo, sg, KW, mmin, W, wt, &ew))) {
             bad = true;
             break;
         }
@@ -481,7 +484,7 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx64(FwdParams P,
 // One CTA per spline piece of the TDI orbit: where no delayed read's stencil steps within the piece, the
 // merged stencils of the 12 (channel, link) pairs as polynomials of degree 5 in the piece's coordinate on
 // [-1, 1] (weights at six Chebyshev nodes; over a 1e5 s piece the delays move by ~1e-3 samples, so the next
-// order is below 2^-54).  meta: taps (0: no entry) and the first tap's position.  The stencils depend on the
+// order is below 2^-54).  meta: taps (0: no entry), the first tap's position and the scale's exponent.  The stencils depend on the
 // orbit alone; from the table a block's expansion is 20 FP64 operations per tap, against ~130 per read and
 // node computed in the block.
 __global__ void __launch_bounds__(256) k_fx_table(FwdParams P, FxTab X, int T, double *tab, int *meta, int tab_kw)
@@ -490,7 +493,7 @@ __global__ void __launch_bounds__(256) k_fx_table(FwdParams P, FxTab X, int T, d
     constexpr int TQ = FX_TAB_Q, WTT = TQ * NTERM + 1;
     __shared__ double pc[6][4], eps[TQ][NTERM];
     __shared__ double lc1[64], lc0[64], rc1[64], rc0[64];
-    __shared__ int mm[NTERM], mmin, mmax, bad;
+    __shared__ int mm[NTERM], mmin, mmax, bad, wmax;
     const int tid = threadIdx.x, k = blockIdx.x, h = (T - 2) / 2, qn = P.q_terms;
     if (tid < T) {
         lc1[tid] = 1.0 / (double)(tid + 1);
@@ -510,6 +513,7 @@ __global__ void __launch_bounds__(256) k_fx_table(FwdParams P, FxTab X, int T, d
         mmin = 1 << 29;
         mmax = -(1 << 29);
         bad = 0;
+        wmax = 0;
     }
     __syncthreads();
     if (tid < NTERM && tid % 7 < qn) {
@@ -534,7 +538,7 @@ __global__ void __launch_bounds__(256) k_fx_table(FwdParams P, FxTab X, int T, d
     __syncthreads();
     const int KW = (mmax > 0 ? mmax : 0) - mmin + T;
     if (bad || KW > tab_kw || KW + 7 > 64 || P.HL + mmin - h < 1) {
-        if (tid == 0) meta[2 * k] = meta[2 * k + 1] = 0;
+        if (tid < FX_META) meta[FX_META * k + tid] = 0;
         return;
     }
     for (int i = tid; i < TQ * NTERM; i += blockDim.x)
@@ -552,6 +556,7 @@ __global__ void __launch_bounds__(256) k_fx_table(FwdParams P, FxTab X, int T, d
         }
     __syncthreads();
     bool ok = true;
+    float most = 0.0f;   // bound of the stencils over the piece, the orders' magnitudes added
     for (int i = tid; i < 12 * KW; i += blockDim.x) {
         const int cs = i / KW, tap = i - cs * KW, ch = cs >> 2, sl = cs & 3;
         double V[TQ], b[TQ];
@@ -576,12 +581,23 @@ __global__ void __launch_bounds__(256) k_fx_table(FwdParams P, FxTab X, int T, d
         const double m[TQ] = {b[0] - b[2] + b[4], b[1] - 3.0 * b[3] + 5.0 * b[5], 2.0 * b[2] - 8.0 * b[4],
                               4.0 * b[3] - 20.0 * b[5], 8.0 * b[4], 16.0 * b[5]};
         ok &= fabs(m[TQ - 1]) < 9e-13;  // 2^-40: the order left out is then below 2^-54
-        for (int q = 0; q < TQ; ++q) tab[((size_t)k * TQ + q) * 12 * tab_kw + cs * tab_kw + tap] = m[q];
+        double sum = 0.0;
+        for (int q = 0; q < TQ; ++q) {
+            tab[((size_t)k * TQ + q) * 12 * tab_kw + cs * tab_kw + tap] = m[q];
+            sum += fabs(m[q]);
+        }
+        most = fmaxf(most, (float)sum);
     }
+    atomicMax(&wmax, (int)__float_as_uint(most));
     ok = !__syncthreads_or(!ok);
     if (tid == 0) {
-        meta[2 * k] = ok ? KW : 0;
-        meta[2 * k + 1] = mmin;
+        // 2 % for blocks that reach past the piece
+        const float top = __int_as_float(wmax) * 1.02f;
+        const bool in = top > 1e-30f && top < 1e30f;
+        meta[FX_META * k] = ok && in ? KW : 0;
+        meta[FX_META * k + 1] = mmin;
+        meta[FX_META * k + 2] = in ? (int)(__float_as_uint(top) >> 23) - 126 : 0;   // exponent of the scale
+        meta[FX_META * k + 3] = 0;
     }
 }
 
@@ -645,7 +661,7 @@ size_t fx_table_bytes(const FwdParams &P, int order)
 {
     // plans with very many spline pieces work without the table
     const int T = order + 1, kw = T + (P.HL - (T - 2) / 2 - 2) + 1;
-    const size_t per = sizeof(double) * FX_TAB_Q * 12 * (size_t)kw + 2 * sizeof(int);
+    const size_t per = sizeof(double) * FX_TAB_Q * 12 * (size_t)kw + FX_META * sizeof(int);
     return P.to.nint <= FX_TAB_PIECES ? per * (size_t)P.to.nint : 0;
 }
 

@@ -24,11 +24,12 @@ constexpr int NGT = NY / GT + 1;
 constexpr int NTERM = 42;
 constexpr int WTS = 4 * NTERM + 1;   // row length of the TDI node weights (odd: no bank conflicts)
 constexpr int WNS = NN * 9;
+static_assert(2 * WNS <= 160 && NN * 6 == 48, "roles of node_weights");
 // merged TDI taps per thread: at most 12 stencils of 57 taps
 __host__ __device__ constexpr int tap_reps(int nthr) { return (12 * 57 + nthr - 1) / nthr; }
 constexpr int RANGE_BITS = 12;
 // the last order's coefficient must be below 2^-45 of the stencil's scale: the next one is then below 2^-53
-constexpr double LAST_MAX = 1024.0;
+constexpr unsigned long long LAST_MAX = 1024;
 
 // digits of order q that are left out at the top: |b_q| < 2^-8z of the stencil's scale
 __host__ __device__ constexpr int zq(bool tdi, int q)
@@ -87,6 +88,7 @@ struct Shared {
     };
     int segm[MAXSEG][NTERM + 1];  // stencil positions (9 or 42) and the spline piece of each segment
     int segj[MAXSEG + 1];
+    double xc, xs;
     int nseg, nlist, fast;
     unsigned brk[NY / 32];
     int list[NTERM * 8 + 8];
@@ -387,9 +389,9 @@ __device__ __forceinline__ long long to_fixed(double v, int e)
     const long long b = __double_as_longlong(v);
     const int E = (int)((b >> 52) & 0x7ff);
     const unsigned long long m = ((unsigned long long)b & 0xfffffffffffffull) | (E ? 1ull << 52 : 0ull);
-    const int s = E - e - 1020;  // at most 2
+    const int s = E - e - 1020;  // at most 2 for |v| < 2^e
     unsigned long long r;
-    if (s >= 0) r = m << s;
+    if (s >= 0) r = s < 9 ? m << s : 1ull << 61;   // beyond every digit's range
     else r = s > -60 ? ((m >> (-s - 1)) + 1) >> 1 : 0ull;
     return b < 0 ? -(long long)r : (long long)r;
 }
@@ -434,10 +436,11 @@ __device__ __forceinline__ bool coef_digits(unsigned char *w, long long b)
     return top >= -128 && top <= 127;
 }
 
+// coefficient b of a stencil of scale 2^e (integer work: conversions and scalings would be FP64 issue slots)
 template <bool TDI, int Q>
-__device__ __forceinline__ bool coef_store(unsigned char *w, double b, unsigned long long *mag)
+__device__ __forceinline__ bool coef_store(unsigned char *w, double b, int e, unsigned long long *mag)
 {
-    const long long v = __double2ll_rn(b);
+    const long long v = to_fixed(b, e);
     mag[Q] |= (unsigned long long)(v < 0 ? -v : v);
     return coef_digits<zq(TDI, Q)>(w + digit_row(TDI, Q) * WS, v);
 }
@@ -568,26 +571,48 @@ __device__ __forceinline__ void node_weights(const FwdParams &P, const FxTab &X,
     if (tid >= 200 && tid < 200 + NN) S.qor[tid - 200] = 0;
     __syncthreads();
     // Lagrange weights at the nodes, two threads per read: prefix products of the lower half and suffix
-    // products of the upper half, then each carries on through the other's half
-    const int id = tid < WNS ? tid : tid - WNS;
-    const bool low = tid < WNS, half = tid < 2 * WNS;
-    double e = 0.0, run = 1.0;
-    if (half) {
-        e = S.nodeu[id] - (fl0 + (double)sm[id % 9]);
+    // products of the upper half, then each carries on through the other's half.  They fill warps 0 to 4; the
+    // links' patterns take 16 lanes of warps 5, 6 and 7 (an FP64 instruction holds its scheduler's pipe for 64
+    // cycles however few lanes it has, so the four schedulers get 130 to 155 of them each).
+    if (tid < 160) {
+        const int id = tid < WNS ? tid : tid - WNS;
+        const bool low = tid < WNS, half = tid < 2 * WNS;
+        double e = 0.0, run = 1.0;
         double *w = wn + id;
-        if (low) {
-            for (int a = 0; a < T / 2; ++a) {
-                w[a * WNS] = run;
-                run *= fma(e, S.lc1[a], S.lc0[a]);
-            }
-        } else {
-            for (int a = T - 1; a >= T / 2; --a) {
-                w[a * WNS] = ((T - 1 - a) & 1) ? -run : run;
-                run *= fma(e, S.rc1[a], S.rc0[a]);
+        if (half) {
+            e = S.nodeu[id] - (fl0 + (double)sm[id % 9]);
+            if (low) {
+#pragma unroll 4
+                for (int a = 0; a < T / 2; ++a) {
+                    w[a * WNS] = run;
+                    run *= fma(e, S.lc1[a], S.lc0[a]);
+                }
+            } else {
+#pragma unroll 4
+                for (int a = T - 1; a >= T / 2; --a) {
+                    w[a * WNS] = ((T - 1 - a) & 1) ? -run : run;
+                    run *= fma(e, S.rc1[a], S.rc0[a]);
+                }
             }
         }
-    } else if (tid >= 160 && tid < 160 + NN * 6) {
-        const int n = (tid - 160) / 6, l = (tid - 160) % 6, r = c_lr[l], s = c_ls[l];
+        asm volatile("bar.sync 1, 160;" ::: "memory");
+        if (half) {
+            if (low) {
+#pragma unroll 4
+                for (int a = T / 2; a < T; ++a) {
+                    w[a * WNS] *= run;
+                    run *= fma(e, S.lc1[a], S.lc0[a]);
+                }
+            } else {
+#pragma unroll 4
+                for (int a = T / 2 - 1; a >= 0; --a) {
+                    w[a * WNS] *= ((T - 1 - a) & 1) ? -run : run;
+                    run *= fma(e, S.rc1[a], S.rc0[a]);
+                }
+            }
+        }
+    } else if (tid < 256 && (tid & 31) < 16) {
+        const int at = ((tid >> 5) - 5) * 16 + (tid & 31), n = at / 6, l = at % 6, r = c_lr[l], s = c_ls[l];
         const SkyConst &K = S.skc;
         const double *x = S.npos[n];
         double d0 = x[3 * r] - x[3 * s], d1 = x[3 * r + 1] - x[3 * s + 1], d2 = x[3 * r + 2] - x[3 * s + 2];
@@ -606,21 +631,13 @@ __device__ __forceinline__ void node_weights(const FwdParams &P, const FxTab &X,
         if (!isfinite(gf)) S.bad = 1;
     }
     __syncthreads();
-    if (half) {
-        double *w = wn + id;
-        if (low) {
-            for (int a = T / 2; a < T; ++a) {
-                w[a * WNS] *= run;
-                run *= fma(e, S.lc1[a], S.lc0[a]);
-            }
-        } else {
-            for (int a = T / 2 - 1; a >= 0; --a) {
-                w[a * WNS] *= ((T - 1 - a) & 1) ? -run : run;
-                run *= fma(e, S.rc1[a], S.rc0[a]);
-            }
-        }
-    }
-    __syncthreads();
+}
+
+// exponent of a stencil's scale, 2 max|c| with slack for offsets just outside [0, 1)
+__device__ __forceinline__ int stencil_exp(int cmax)
+{
+    const float m = __int_as_float(cmax) * 2.4f;
+    return m > 1e-30f && m < 1e30f ? (int)(__float_as_uint(m) >> 23) - 126 : -126;
 }
 
 // Digit rows W of segment sg's merged stencils (REV: taps in reverse, one scale for all links); false when the
@@ -635,16 +652,14 @@ __device__ bool projection_stencils(const FwdParams &P, const FxTab &X, Shared &
     for (int i = tid; i < FX_PROJ_W / 16; i += blockDim.x)
         reinterpret_cast<uint4 *>(W)[i] = make_uint4(0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u);
     node_weights(P, X, S, T, t_lo, u0, fl0, sg, wn);
-    if (tid < 6) {  // the stencil's scale: 2 max|c| with slack for offsets just outside [0, 1)
-        int c = S.cmax[tid];
-        if (REV)   // one scale for the sum over the links
-            for (int l = 0; l < 6; ++l) c = max(c, S.cmax[l]);
-        const float m = __int_as_float(c) * 2.4f;
-        S.wexp[tid] = m > 1e-30f && m < 1e30f ? (int)(__float_as_uint(m) >> 23) - 126 : -126;
+    int cm[6], call = 0;
+#pragma unroll
+    for (int l = 0; l < 6; ++l) {
+        cm[l] = S.cmax[l];
+        call = max(call, cm[l]);
     }
-    __syncthreads();
-    if (tid < NN * 12) S.ncf[tid / 12][tid % 12] *= pow2(55 - S.wexp[(tid % 12) >> 1]);
-    __syncthreads();
+    if (tid == 0)
+        for (int l = 0; l < 6; ++l) S.wexp[l] = stencil_exp(REV ? call : cm[l]);   // REV: one scale for the sum over the links
     bool fits = !S.bad;
     unsigned long long mag[NN] = {};
     if (fits)
@@ -673,14 +688,17 @@ __device__ bool projection_stencils(const FwdParams &P, const FxTab &X, Shared &
                 for (int n = 0; n < NN / 2; ++n) v = fma((q & 1) ? o[n] : e[n], X.cheb[q][n], v);
                 b[q] = v;
             }
-            fits &= coef_store<false, 0>(w, b[0], mag);
-            fits &= coef_store<false, 1>(w, b[1], mag);
-            fits &= coef_store<false, 2>(w, b[2], mag);
-            fits &= coef_store<false, 3>(w, b[3], mag);
-            fits &= coef_store<false, 4>(w, b[4], mag);
-            fits &= coef_store<false, 5>(w, b[5], mag);
-            fits &= coef_store<false, 6>(w, b[6], mag);
-            fits &= coef_store<false, 7>(w, b[7], mag) && fabs(b[7]) < LAST_MAX;
+            const int ew = stencil_exp(REV ? call : S.cmax[l]);
+            fits &= coef_store<false, 0>(w, b[0], ew, mag);
+            fits &= coef_store<false, 1>(w, b[1], ew, mag);
+            fits &= coef_store<false, 2>(w, b[2], ew, mag);
+            fits &= coef_store<false, 3>(w, b[3], ew, mag);
+            fits &= coef_store<false, 4>(w, b[4], ew, mag);
+            fits &= coef_store<false, 5>(w, b[5], ew, mag);
+            fits &= coef_store<false, 6>(w, b[6], ew, mag);
+            unsigned long long m7[NN] = {};
+            fits &= coef_store<false, 7>(w, b[7], ew, m7) && m7[7] < LAST_MAX;
+            mag[7] |= m7[7];
         }
     orders_in_use<NN>(S, mag);
     if (__syncthreads_or(!fits)) return false;
@@ -689,15 +707,10 @@ __device__ bool projection_stencils(const FwdParams &P, const FxTab &X, Shared &
 }
 
 // ---------------------------------------------------------------- the plan's TDI table
-// Chebyshev coefficients of one tap over the block, from the piece's polynomial (degree 5 in its coordinate
+// Chebyshev coefficients of one tap over the block, from the piece's polynomial p (degree 5 in its coordinate
 // on [-1, 1]) moved to the block's centre xc and scaled by its half width xs
-__device__ __forceinline__ void table_coefs(const FwdParams &P, const FxTab &X, int piece, int at, double xc, double xs, double *b)
+__device__ __forceinline__ void table_coefs(double *p, double xc, double xs, double *b)
 {
-    const double *c = X.tab + (size_t)piece * FX_TAB_Q * 12 * X.tab_kw + at;
-    const int st = 12 * X.tab_kw;
-    double p[FX_TAB_Q];
-#pragma unroll
-    for (int q = 0; q < FX_TAB_Q; ++q) p[q] = __ldg(c + q * st);
 #pragma unroll
     for (int k = 0; k < NT; ++k)
 #pragma unroll
@@ -718,7 +731,7 @@ __device__ int table_segments(const FwdParams &P, const FxTab &X, Shared &S, dou
     row_at(P.to, t_lo, -1, &x, &a);
     const double ua = x + (double)a;
     row_at(P.to, t_lo + (double)(nb - 1) * P.dt, -1, &x, &b);
-    if (b > a + 1 || X.meta[2 * a] == 0 || X.meta[2 * b] == 0) return 0;
+    if (b > a + 1 || X.meta[FX_META * a] == 0 || X.meta[FX_META * b] == 0) return 0;
     S.nseg = 1 + (b > a);
     S.segj[0] = 0;
     S.segm[0][NTERM] = a;
@@ -810,12 +823,61 @@ __device__ void find_tdi_segments(const FwdParams &P, Shared &S, double t_lo, in
     }
 }
 
-// Digit rows W of segment sg's merged TDI stencils (REV: taps in reverse) and their scale *ew_out: from the
-// plan's table (fast), or from the delayed reads' weights at four nodes (wt [T][WTS]).  False when the
-// coefficients do not fit their digits.  Begins and ends with a barrier.
+// Digit rows W of segment sg's merged TDI stencils (REV: taps in reverse) from the plan's table, whose entries
+// are on their way while the rows are filled; *ew_out: their scale.  False when the coefficients do not fit
+// their digits.  Begins and ends with a barrier.
 template <bool REV, int NTHR>
-__device__ __forceinline__ bool tdi_stencils(const FwdParams &P, const FxTab &X, Shared &S, int T, double t_lo, int sg,
-                                             bool fast, int KW, int mmin, unsigned char *W, double *wt, int *ew_out)
+__device__ __forceinline__ bool tdi_stencils(const FwdParams &P, const FxTab &X, Shared &S, double t_lo, int sg, int KW,
+                                             unsigned char *W, int *ew_out)
+{
+    const int tid = threadIdx.x, piece = S.segm[sg][NTERM];
+    double p[tap_reps(NTHR)][FX_TAB_Q];
+    const double *c = X.tab + (size_t)piece * FX_TAB_Q * 12 * X.tab_kw;
+#pragma unroll
+    for (int rep = 0; rep < tap_reps(NTHR); ++rep) {
+        const int i = tid + NTHR * rep;
+        if (i < 12 * KW) {
+            const int at = (i / KW) * X.tab_kw + i % KW;
+#pragma unroll
+            for (int q = 0; q < FX_TAB_Q; ++q) p[rep][q] = __ldg(c + q * 12 * X.tab_kw + at);
+        }
+    }
+    const int ew = X.meta[FX_META * piece + 2];
+    *ew_out = ew;
+    __syncthreads();
+    for (int i = tid; i < FX_TDI_W / 16; i += NTHR)
+        reinterpret_cast<uint4 *>(W)[i] = make_uint4(0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u);
+    if (tid < NT) S.qor[tid] = 0;
+    if (tid == NTHR - 1) {
+        S.xc = 2.0 * ((t_lo + 0.5 * (NY - 1) * P.dt - P.to.t_first) * P.to.inv_dk - (double)piece) - 1.0;
+        S.xs = NY * P.dt * P.to.inv_dk;
+    }
+    __syncthreads();
+    const double xc = S.xc, xs = S.xs;
+    bool fits = true;
+    unsigned long long mag[NT] = {};
+#pragma unroll
+    for (int rep = 0; rep < tap_reps(NTHR); ++rep) {
+        const int i = tid + NTHR * rep;
+        if (i < 12 * KW) {
+            const int cs = i / KW, tap = i - cs * KW;
+            unsigned char *w = W + cs * TD * WS + 7 + (REV ? KW - 1 - tap : tap);
+            double b[NT];
+            table_coefs(p[rep], xc, xs, b);
+            fits &= coef_store<true, 0>(w, b[0], ew, mag);
+            fits &= coef_store<true, 1>(w, b[1], ew, mag);
+            fits &= coef_store<true, 2>(w, b[2], ew, mag);
+            fits &= coef_store<true, 3>(w, b[3], ew, mag);
+        }
+    }
+    orders_in_use<NT>(S, mag);
+    return !__syncthreads_or(!fits);
+}
+
+// The same from the delayed reads' weights at four nodes (wt [T][WTS]), for blocks that the table does not cover.
+template <bool REV, int NTHR>
+__device__ __noinline__ bool tdi_stencils_nodes(const FwdParams &P, const FxTab &X, Shared &S, int T, double t_lo, int sg,
+                                                   int KW, int mmin, unsigned char *W, double *wt, int *ew_out)
 {
     const int tid = threadIdx.x, lane = tid & 31, h = (T - 2) / 2, qn = P.q_terms;
     const int *sm = S.segm[sg];
@@ -823,7 +885,7 @@ __device__ __forceinline__ bool tdi_stencils(const FwdParams &P, const FxTab &X,
     __syncthreads();
     for (int i = tid; i < FX_TDI_W / 16; i += blockDim.x)
         reinterpret_cast<uint4 *>(W)[i] = make_uint4(0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u);
-    if (!fast && tid < NT * 6) {
+    if (tid < NT * 6) {
         const int n = tid / 6, l = tid % 6;
         double x;
         int k;
@@ -836,7 +898,7 @@ __device__ __forceinline__ bool tdi_stencils(const FwdParams &P, const FxTab &X,
     }
     __syncthreads();
     // the node weights take the planes' place; with more than one segment the series is sliced again
-    if (!fast && tid < NT * NTERM) {
+    if (tid < NT * NTERM) {
         const int n = tid / NTERM, tm = tid % NTERM, cc = tm / 7, q = tm % 7 + 1;
         if (q <= qn) {
             double D = 0.0;
@@ -845,18 +907,13 @@ __device__ __forceinline__ bool tdi_stencils(const FwdParams &P, const FxTab &X,
         }
     }
     __syncthreads();
-    // merged stencils: the reads of one (channel, link) added tap by tap at the four nodes, or the plan's
-    // table around the block's centre
-    const double xc = 2.0 * ((t_lo + 0.5 * (NY - 1) * P.dt - P.to.t_first) * P.to.inv_dk - (double)piece) - 1.0;
-    const double xs = NY * P.dt * P.to.inv_dk;
+    // merged stencils: the reads of one (channel, link) added tap by tap
     double b[tap_reps(NTHR)][NT];
     float bm = 0.0f;
 #pragma unroll
     for (int rep = 0; rep < tap_reps(NTHR); ++rep) {
         const int i = tid + NTHR * rep;
-        if (i < 12 * KW && fast) {
-            table_coefs(P, X, piece, (i / KW) * X.tab_kw + i % KW, xc, xs, b[rep]);
-        } else {
+        {
             double V[NT] = {0.0, 0.0, 0.0, 0.0};
             if (i < 12 * KW) {
                 const int cs = i / KW, tap = i - cs * KW, ch = cs >> 2, sl = cs & 3;
@@ -890,7 +947,6 @@ __device__ __forceinline__ bool tdi_stencils(const FwdParams &P, const FxTab &X,
     __syncthreads();
     const float sm_max = __int_as_float(S.cmax[0]) * 1.01f;
     *ew_out = sm_max > 1e-30f && sm_max < 1e30f ? (int)(__float_as_uint(sm_max) >> 23) - 126 : 0;
-    const double ws = pow2(55 - *ew_out);
     bool fits = sm_max < 1e30f;
     unsigned long long mag[NT] = {};
 #pragma unroll
@@ -899,10 +955,10 @@ __device__ __forceinline__ bool tdi_stencils(const FwdParams &P, const FxTab &X,
         if (i < 12 * KW) {
             const int cs = i / KW, tap = i - cs * KW;
             unsigned char *w = W + cs * TD * WS + 7 + (REV ? KW - 1 - tap : tap);
-            fits &= coef_store<true, 0>(w, b[rep][0] * ws, mag);
-            fits &= coef_store<true, 1>(w, b[rep][1] * ws, mag);
-            fits &= coef_store<true, 2>(w, b[rep][2] * ws, mag);
-            fits &= coef_store<true, 3>(w, b[rep][3] * ws, mag);
+            fits &= coef_store<true, 0>(w, b[rep][0], *ew_out, mag);
+            fits &= coef_store<true, 1>(w, b[rep][1], *ew_out, mag);
+            fits &= coef_store<true, 2>(w, b[rep][2], *ew_out, mag);
+            fits &= coef_store<true, 3>(w, b[rep][3], *ew_out, mag);
         }
     }
     orders_in_use<NT>(S, mag);

@@ -17,6 +17,7 @@
 //
 // Measured (one year at order 41, mixed plan): K1 5.97 -> 1.65, K2 12.16 -> 4.45, K3 12.2 -> 6.34 ms;
 // 65536 samples at order 25 (FP64 plan): K1 1.26 -> 0.063, K2 0.42 -> 0.116, K3 0.64 -> 0.175 ms.
+// The tensor pipe's share of K3 is the largest (correlations at all lags, order 41: two passes of 32).
 #include "lr_fx64.cuh"
 
 #include "lr_bwd.h"
@@ -257,11 +258,12 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_tdi_adj(FwdPar
         bool bad = S.bad || !range_ok(S, &eg);
         const int nseg = S.nseg;
         for (int sg = 0; sg < nseg && !bad; ++sg) {
-            const int piece = S.segm[sg][NTERM], mmin = fast ? X.meta[2 * piece + 1] : S.mmin, KW = T - mmin, nks = (KW + 7 + 15) / 16;
+            const int piece = S.segm[sg][NTERM], mmin = fast ? X.meta[FX_META * piece + 1] : S.mmin, KW = T - mmin, nks = (KW + 7 + 15) / 16;
             const int js = S.segj[sg], je = S.segj[sg + 1];
             int ew;
             if (nks * 16 > 64 || nb + KW - 1 > rows || (!fast && S.mmax >= 0) ||
-                !tdi_stencils<true, NTHR>(P, X, S, T, t_lo, sg, fast, KW, mmin, W, wt, &ew)) {
+                !(fast ? tdi_stencils<true, NTHR>(P, X, S, t_lo, sg, KW, W, &ew)
+                       : tdi_stencils_nodes<true, NTHR>(P, X, S, T, t_lo, sg, KW, mmin, W, wt, &ew))) {
                 bad = true;
                 break;
             }
@@ -593,10 +595,10 @@ __device__ __forceinline__ void frame_derivatives(const SkyConst &K, double dk[2
     dv[1][0] = -cb * cl; dv[1][1] = -cb * sl; dv[1][2] = -sb;
 }
 
-// link l's part of the gradient at positions x: e, r the emission and reception reads summed against gy,
-// (value, derivative) of h+ and hx
+// link l's part of the gradient at positions x, angles a0 .. a1 - 1 of (lambda, beta); psi with beta.  e, r: the
+// emission and reception reads summed against gy, (value, derivative) of h+ and hx
 __device__ __forceinline__ void sky_terms(const FwdParams &P, const SkyConst &K, const double *x, int l, const double *e,
-                                          const double *r, double *G)
+                                          const double *r, int a0, int a1, double *G)
 {
     double dk[2][3], du[2][3], dv[2][3];
     frame_derivatives(K, dk, du, dv);
@@ -611,7 +613,7 @@ __device__ __forceinline__ void sky_terms(const FwdParams &P, const SkyConst &K,
     const double xp = K.c2p * xip + K.s2p * xic, xc = -K.s2p * xip + K.c2p * xic;
     const double den = 1.0 / (2.0 * (1.0 - kn));
     const double dPp = e[0] - r[0], dPc = e[2] - r[2], dH = xp * dPp + xc * dPc;
-    for (int th = 0; th < 2; ++th) {
+    for (int th = a0; th < a1; ++th) {
         const double da = dot(du[th]), db = dot(dv[th]);
         const double dxip = 2.0 * (un * da - vn * db), dxic = 2.0 * (da * vn + un * db);
         const double dxp = K.c2p * dxip + K.s2p * dxic, dxc = -K.s2p * dxip + K.c2p * dxic;
@@ -621,7 +623,7 @@ __device__ __forceinline__ void sky_terms(const FwdParams &P, const SkyConst &K,
         const double ddH = dxp * dPp + dxc * dPc + xp * (e[1] * due - r[1] * dur) + xc * (e[3] * due - r[3] * dur);
         G[th] += dden * dH + den * ddH;
     }
-    G[2] += den * (2.0 * xc * dPp - 2.0 * xp * dPc);
+    if (a1 == 2) G[2] += den * (2.0 * xc * dPp - 2.0 * xp * dPc);
 }
 
 // value and derivative of both polarisations at base + u, straight from memory (Horner form of read_scalar)
@@ -658,7 +660,7 @@ template <int N>
 __device__ __forceinline__ void put_bytes(unsigned char *row, long long X)
 {
     X += DIGIT_BIAS;
-    row[0] = (unsigned char)((int)(X >> 48) + 128);   // |X| < 2^54: the scale leaves a bit for the byte's range
+    row[0] = (unsigned char)((int)(X >> 48) + 128);   // |X| < 127.5 * 2^48
 #pragma unroll
     for (int i = 1; i < N; ++i) row[i * GB] = (unsigned char)(X >> (8 * (6 - i)));
 }
@@ -724,10 +726,10 @@ __device__ __forceinline__ void correlate_item(double *C, int LG, const unsigned
     }
 }
 
-// the (order, half of the block) items 2 q + half of each warp: the orders cost 28, 28, 22, 16, 11, 11, 7, 4
-// products a step
-__constant__ signed char c_items[8][4] = {{0, 14, -1, -1}, {1, 15, -1, -1}, {2, -1, -1, -1}, {3, -1, -1, -1},
-                                          {4, 8, -1, -1},  {5, 9, -1, -1},  {6, 10, 12, -1}, {7, 11, 13, -1}};
+// the (order, half of the block) items 2 q + half of each warp, balanced by issue slots per step (119, 119, 113,
+// 94, 76, 76, 59, 43 for orders 0 .. 7: products, digit conversions and loads) over the warps (162 to 189) and
+// over the schedulers, which have warps w and w + 4 (348 and 351)
+__constant__ signed char c_items[8][2] = {{0, 12}, {1, 13}, {2, 14}, {3, 15}, {6, 10}, {7, 11}, {4, 8}, {5, 9}};
 
 template <int NTHR>
 __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_sky_adj(FwdParams P, FxTab X, BwdParams B, int T)
@@ -806,7 +808,7 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_sky_adj(FwdPar
             if (!bad && work) {
                 bad = !range_ok(S, &ex);
                 const int eb = (int)(gmax >> 20), es = (int)(gmin >> 20);
-                eg = eb - 1021;
+                eg = eb - 1022 + ((gmax & 0xfffff) >= 0xfa000);   // the top byte's range is 127.5 / 128 of the scale
                 bad |= !(eb >= 200 && eb <= 1900 && eb - es <= RANGE_BITS);
             }
             if (!bad && work) {
@@ -856,9 +858,8 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_sky_adj(FwdPar
                         const unsigned char *g_lane = G + pr * K3_PAIR + (lr4 >> 2) * GROWS * GB + 4 + 4 * kp;
                         for (int ps = 0; ps < npass; ++ps) {
                             const unsigned char *a_lane = reinterpret_cast<const unsigned char *>(planes) + 8 * (lr4 + 8 * ps) + 8 * kp;
-                            for (int k = 0; k < (shared_pair ? 1 : 4); ++k) {
+                            for (int k = 0; k < (shared_pair ? 1 : 2); ++k) {
                                 const int it = shared_pair ? warp : c_items[warp & 7][k];
-                                if (it < 0) break;
                                 const int s0 = (it & 1) ? mid : 0, s1 = (it & 1) ? steps : mid;
                                 switch (it >> 1) {
                                     case 0: correlate_item<0>(C, LG, a_lane, g_lane, sh, s0, s1, 32 * ps, lane, 2 * lp); break;
@@ -963,9 +964,10 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_sky_adj(FwdPar
                         dots[n][l][er][2 * pol + 1] = d;
                     }
                     __syncthreads();
-                    if (tid < NN * 6) {
+                    if (tid < 128 && (tid & 63) < NN * 6) {   // an angle per thread: lambda, then beta and psi two warps on
                         double t[3] = {0.0, 0.0, 0.0};
-                        sky_terms(P, S.skc, S.npos[tid / 6], tid % 6, dots[tid / 6][tid % 6][0], dots[tid / 6][tid % 6][1], t);
+                        const int th = tid >> 6, n = (tid & 63) / 6, l = (tid & 63) % 6;
+                        sky_terms(P, S.skc, S.npos[n], l, dots[n][l][0], dots[n][l][1], th, th + 1, t);
                         const double unit = pow2(eg) * pow2(ex);
                         for (int c = 0; c < 3; ++c) Gs[c] += t[c] * unit;
                     }
@@ -986,7 +988,7 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_sky_adj(FwdPar
                         if (gl == 0.0) continue;
                         double ee[4], t[3] = {0.0, 0.0, 0.0};
                         read_vd_scalar(S, T, ti.hp, ti.hc, ti.nh, k, u0 - L[l] * P.inv_dt - sig[c_ls[l]], ee);
-                        sky_terms(P, S.skc, x, l, ee, rr[c_lr[l]], t);
+                        sky_terms(P, S.skc, x, l, ee, rr[c_lr[l]], 0, 2, t);
                         for (int c = 0; c < 3; ++c) Gs[c] = fma(gl, t[c], Gs[c]);
                     }
                 }

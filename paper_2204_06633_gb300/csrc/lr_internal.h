@@ -99,14 +99,15 @@ struct LikeArgs {
 // digit planes and stencils
 constexpr int FX_ROWS = 512, FX_NODES = 8, FX_TDI_NODES = 4;
 constexpr int FX_PROJ_PLANES = 14 * (FX_ROWS + 64) * 2, FX_PROJ_W = 12 * 38 * 72;
-constexpr int FX_TAB_Q = 6, FX_TAB_PIECES = 4096;  // polynomial terms and most pieces of the plan's TDI table
+constexpr int FX_TAB_Q = 6, FX_TAB_PIECES = 4096, FX_META = 4;  // polynomial terms and most pieces of the plan's TDI table
 constexpr int FX_TDI_PLANES = 42 * (FX_ROWS + 64) * 2, FX_TDI_W = 12 * 19 * 72;
 struct FxTab {
     double icdt;                                                         // 1 / (c dt)
     double node_j[FX_NODES], cheb[FX_NODES][FX_NODES / 2];               // node rows, transform (half by symmetry)
     double tnode_j[FX_TDI_NODES], tcheb[FX_TDI_NODES][FX_TDI_NODES / 2];
     double tab_node[FX_TAB_Q], tab_cheb[FX_TAB_Q][FX_TAB_Q];             // of the table's own expansion
-    // merged TDI stencils per spline piece [pieces][FX_TAB_Q][12][tab_kw] and (taps, first tap) per piece; null: none
+    // merged TDI stencils per spline piece [pieces][FX_TAB_Q][12][tab_kw] and FX_META ints per piece (taps, first tap,
+    // exponent of the scale); null: none
     const double *tab;
     const int *meta;
     int tab_kw;

@@ -101,3 +101,22 @@ def test_nonfinite_cotangent_stays_local(ctx, flex):
     m = synth.input_margin_samples(DT, p)
     assert bad.any() and np.flatnonzero(bad).min() >= 3000 and np.flatnonzero(bad).max() <= 3000 + 2 * m
     assert np.linalg.norm((got - ref)[~bad]) <= 1e-13 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("N", [479, 3000])
+def test_cotangent_scales(ctx, flex, N):
+    """Cotangents times s, 1 <= s < 2, so that the blocks' largest values pass through all significands (the top
+    byte's range ends at 127.5 / 128 of a power of two): the gradient is linear, s times the oracle's."""
+    p, src = 11, synth.draw_sources(1, seed=12)[0]
+    t0h, hp, hc = synth.gb_input(src, T0, DT, N, p)
+    g = np.random.default_rng(N).normal(size=(3, N))
+    rp, rc, rs, scale = oracle.backward(p, 2, DT, T0, N, flex.orc, flex.orc, hp, hc, t0h, src.lam, src.beta, src.psi, g,
+                                        with_scale=True)
+    bound = np.maximum(1e-11 * np.abs(rs), 4 * (p + 17) * 2.0 ** -53 * scale)
+    plan = lr.Plan(ctx, p, N, DT, flex.gpu, t0=T0)
+    for s in 1.0 + np.arange(128) / 128:
+        got = [host(v) / s for v in plan.backward(dev(hp), dev(hc), t0h, sky(src), dev(g * s))]
+        for a, b in zip(got, (rp, rc)):
+            assert np.linalg.norm(a - b) <= 1e-12 * np.linalg.norm(b)
+        assert np.all(np.abs(got[2] - rs) <= bound), (s, got[2], rs, bound)
+    plan.check()
