@@ -36,7 +36,7 @@ DT, T0, ORDER, S_SOURCES = 10.0, 0.0, 25, 1024
 # (9 unique projection reads x 2 polarisations + 42 TDI reads) = 120 T flops, 51 Lagrange
 # weight vectors x ~3 T flops, ~500 flops of orbit splines and geometry
 FLOPS_PER_SAMPLE = lambda p: 273 * (p + 1) + 500  # noqa: E731
-FP64_NOMINAL_TFLOPS = 1.25   # GB300 FP64 (nominal; our DFMA probe measured 1.20)
+DIGIT_PEAK_TFLOPS = 600.0     # half-precision mma.sync (own probe: 300 T multiply-adds/s)
 # FP32 ALU peak from unit counts and clock: 152 SMs x 128 FP32 lanes x 2 flops x 2.07 GHz
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
 # DRAM bytes (read + write) per output sample of the fused mixed kernel at order 25 and its
@@ -44,6 +44,20 @@ FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
 # / 7 115 014 outputs); the launch traffic is this times the launch's outputs.  Valid only for the
 # kernel build it was taken on (profiles/k_mixed_fused_batched16_p25.md).
 MIXED_P25_DRAM_BYTES_PER_SAMPLE = 235_981_568 / 7_115_014
+
+
+def fp64_roofline(p, samples, seconds):
+    """Of the FP64 kernel, whose taps are products of 8-bit digits on the tensor cores: the digit products of
+    its stencils per output against the measured rate of the instruction it uses.  Merged stencils of T + 3
+    (links, 12, reads within 3 samples of each other, 121 digit products) and T + 7 taps (TDI, 12, delays within
+    70 s, 62 products), with the alignment of their rows, in steps of 16."""
+    up = lambda k: -(-k // 16) * 16  # noqa: E731
+    digits = 2 * 12 * (121 * up(p + 7) + 62 * up(p + 15))
+    tf = digits * samples / seconds / 1e12
+    return {"bound": "tensor", "achieved": tf, "peak": DIGIT_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": tf / DIGIT_PEAK_TFLOPS,
+            "peak_source": "half-precision mma.sync with FP32 accumulators, own probe: 300 T multiply-adds/s",
+            "digit_flops_per_sample": digits,
+            "algorithmic_tflops": FLOPS_PER_SAMPLE(p) * samples / seconds / 1e12}
 
 
 def workload(rank: int, world: int, n_sources: int):
@@ -418,10 +432,7 @@ def run_ours(args):
         fp64 = {"value": link_samples / (ms64 * 1e-3), "unit": "link-samples/s", "ms_per_step": ms64,
                 "tile": plan64.tile,
                 "steps": 2, "warmup": 1, "mixed_speedup": ms64 / ms_step,
-                "roofline": {"bound": "alu", "achieved": FLOPS_PER_SAMPLE(p) * total_samples /
-                             (statistics.mean(l64) * 1e-3) / 1e12, "peak": FP64_NOMINAL_TFLOPS,
-                             "unit": "TFLOP/s", "frac": FLOPS_PER_SAMPLE(p) * total_samples /
-                             (statistics.mean(l64) * 1e-3) / 1e12 / FP64_NOMINAL_TFLOPS}}
+                "roofline": fp64_roofline(p, total_samples, statistics.mean(l64) * 1e-3)}
         if rank == 0 and not args.no_check:
             fp64["parity"] = sampled_error(d_xyz, lens, srcs, out_off, orb, p, 1e-12, exact=True)
             fp64["rel_error_vs_oracle"] = fp64["parity"]["rel_error_vs_oracle"]
@@ -439,20 +450,18 @@ def run_ours(args):
         return
     avg_launch_s = statistics.mean(launch_ms) * 1e-3
     flops = FLOPS_PER_SAMPLE(p) * total_samples
-    if precision == lr.FP64:
-        peak_tflops, src_peak = FP64_NOMINAL_TFLOPS, "GB300 FP64 nominal 1.25 TFLOP/s (own DFMA probe: 1.20)"
-    else:
-        peak_tflops, src_peak = FP32_PEAK_TFLOPS, ("FP32 ALU peak 152 SM x 128 lanes x 2 flop x 2.07 GHz "
-                                                   "(own FFMA probe: 74.9 TFLOP/s)")
+    src_peak = "FP32 ALU peak 152 SM x 128 lanes x 2 flop x 2.07 GHz (own FFMA probe: 74.9 TFLOP/s)"
     traffic = None
     if precision == lr.MIXED and p == 25 and plan.tile == 340:
         traffic = MIXED_P25_DRAM_BYTES_PER_SAMPLE * total_samples
-    roof = {"bound": "alu", "achieved": flops / avg_launch_s / 1e12, "peak": peak_tflops, "unit": "TFLOP/s",
-            "frac": flops / avg_launch_s / 1e12 / peak_tflops, "traffic": traffic, "peak_source": src_peak,
-            "algorithmic_flops_per_sample": FLOPS_PER_SAMPLE(p),
-            "kernel": "k_mixed<T,FUSED>" if precision == lr.MIXED else "k_fused64<T>",
-            "timing": "CUDA events around each batched call on its stream (tile-table kernel + fused kernel; "
-                      "the fused kernel is 99.9 % of it by the ncu launch list)"}
+    roof = {"bound": "alu", "achieved": flops / avg_launch_s / 1e12, "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
+            "frac": flops / avg_launch_s / 1e12 / FP32_PEAK_TFLOPS, "traffic": traffic, "peak_source": src_peak}
+    if precision == lr.FP64:
+        roof = dict(fp64_roofline(p, total_samples, avg_launch_s), traffic=None)
+    roof.update(algorithmic_flops_per_sample=FLOPS_PER_SAMPLE(p),
+                kernel="k_mixed<T,FUSED>" if precision == lr.MIXED else "k_fx64",
+                timing="CUDA events around each batched call on its stream (tile-table kernel + fused kernel; "
+                       "the fused kernel is 99.9 % of it by the ncu launch list)")
     line = {"metric": METRIC, "value": value, "unit": "link-samples/s", "n_gpus": ws, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms_step, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": "f64" if precision == lr.FP64 else "f32 taps + f64 index",
