@@ -40,8 +40,8 @@
 //
 // Measured (fused, order 25, one year of 3 153 600 outputs): 44.45 ms sample by sample, 3.4 to 4.0 ms here (the
 // source's position sets how many segments a block has), with 3.0e-12 relative error against 64 bits where
-// the sample form has 3.5e-12; 65 536 outputs: 490 us and 108 us.  Two blocks share an SM; the tensor pipe is
-// busy a third of the time and the FP64 pipe (weights, transforms) a quarter, the rest is latency of the short
+// the sample form has 3.5e-12; 65 536 outputs: 490 us and 108 us.  Two blocks share an SM; the tensor pipe
+// and the FP64 pipe (weights, transforms) are each busy a quarter of the time, the rest is latency of the short
 // FP64 phases.  Steps on the way, one year: 4.36 ms with 8-sample rows in the projection and the TDI stencils
 // computed in every block; 65 536 outputs: 113 us with the weights and the links' patterns of the nodes on the
 // same warps, the TDI stencils' scale found in the block, and a barrier more for each of the two scales.

@@ -17,7 +17,8 @@
 //
 // Measured (one year at order 41, mixed plan): K1 5.97 -> 1.65, K2 12.16 -> 4.45, K3 12.2 -> 6.34 ms;
 // 65536 samples at order 25 (FP64 plan): K1 1.26 -> 0.063, K2 0.42 -> 0.116, K3 0.64 -> 0.175 ms.
-// The tensor pipe's share of K3 is the largest (correlations at all lags, order 41: two passes of 32).
+// K3 is bound by the FP64 pipe (44 % busy: node weights with derivatives, level sums to FP64) and the barriers
+// around it, with the tensor pipe at 20 %; integer conversion of its level sums was slower (0.914).
 #include "lr_fx64.cuh"
 
 #include "lr_bwd.h"
