@@ -729,6 +729,7 @@ int fx_table_for(FxPlan *F, void *str, FxTab *X)
 
 int launch_fx64(int kind, int order, const FwdParams &P, int sms, void *stream)
 {
+    if (P.src.tile_off && !P.src.skyc && kind != KIND_TDI) return (int)cudaErrorInvalidValue;  // sky frames of a batch
     const int nthr = P.total_tiles >= 0 && P.total_tiles <= sms ? 512 : 256;
     void *k = nthr == 512 ? kernel_of<512>(kind) : kernel_of<256>(kind);
     int T = order + 1;

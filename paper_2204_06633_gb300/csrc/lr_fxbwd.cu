@@ -1015,6 +1015,7 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_sky_adj(FwdPar
 
 int launch_fx_bwd(int kind, int order, const FwdParams &P, const BwdParams &B, FxPlan *F, int sms, void *stream)
 {
+    if (P.src.tile_off && !P.src.skyc && kind != 0) return (int)cudaErrorInvalidValue;  // sky frames of a batch
     int T = order + 1;
     FxTab X;
     if (const int e = fx_table_for(F, stream, &X)) return e;

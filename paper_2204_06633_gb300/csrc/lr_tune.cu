@@ -355,12 +355,13 @@ LR_API int lr_plan_autotune_batch(lr_plan *plan, int64_t S, const int64_t *lengt
     int best = tile0;
     double best_ms = 1e300;
     const std::vector<int> cand = tile_candidates(v);
-    lr::SkyConst *skyc = lr::needs_sky_table(v.precision, v.base) ? reinterpret_cast<lr::SkyConst *>(tables + k + 1) : nullptr;
     for (size_t i = 0; e == cudaSuccess && i < cand.size(); ++i) {
         if (lr::plan_set_tile(plan, cand[i]) != LR_OK) continue;
         lr::PlanView w;
         lr::plan_view(plan, &w);
         lr::FwdParams P = w.base;
+        // the tile decides the kernel family, and with it whether the launch reads the sky frames
+        lr::SkyConst *skyc = lr::needs_sky_table(w.precision, P) ? reinterpret_cast<lr::SkyConst *>(tables + k + 1) : nullptr;
         P.src.skyc = skyc;
         P.src.h_off = d_off;
         P.src.out_off = d_off + k + 1;
