@@ -354,6 +354,7 @@ void fx_setup(lr_plan *p)
     P.fx_tile = 0;
     if (p->desc.precision != LR_FP64 || (P.delay_nested && !P.cd_w)) return;
     const int most = lr::fx_max_tile(P, p->desc.order);
+    if (most < 128) return;  // the merged stencils do not fit, or their halos leave no room
     int block = p->tile < most ? p->tile : most;
     while (block >= 128 && p->tile % block) --block;
     if (block < 128 && p->tile >= 128) return;  // no part of at least 128 outputs

@@ -60,3 +60,21 @@ def test_batch_autotune_of_a_plan_off_the_tensor_cores(ctx, flex, tile, tmp_path
     xyz = plan.response_batched(*args)
     plan.check()
     check_batch(xyz, flex, lens, per, p)
+
+
+@pytest.mark.parametrize("tile", [1, 64, 127, 128])
+@pytest.mark.parametrize("p,dt", [(25, 1.0), (41, 4.0)])
+def test_small_tiles_where_the_stencils_do_not_fit(ctx, p, dt, tile):
+    """Sampling steps so short that a merged stencil passes 64 taps, with a small tile asked for: the plan keeps
+    the sample-by-sample kernels and its tile, one source and batched."""
+    lens = [700, 1, 130]
+    pair = Pair(ctx, synth.orbit_flexing(T0 - 3e5, T0 + 1000 * dt + 3e5))
+    args, per = batch_args(lens, p, dt)
+    s, t0h, hp, hc = per[0]
+    plan = lr.Plan(ctx, p, lens[0], dt, pair.gpu, t0=T0, tile=tile)
+    assert plan.tile == tile
+    one = plan.response(dev(hp), dev(hc), t0h, sky(s))
+    xyz = plan.response_batched(*args)
+    plan.check()
+    check_batch(one, pair, lens[:1], per[:1], p, dt)
+    check_batch(xyz, pair, lens, per, p, dt)
