@@ -243,7 +243,8 @@ LR_API int lr_plan_autotune(lr_plan *plan, int64_t n_samples, int use_cache, voi
     cudaEvent_t a = nullptr, b = nullptr;
     if (e == cudaSuccess) e = cudaEventCreate(&a);
     if (e == cudaSuccess) e = cudaEventCreate(&b);
-    const int tile0 = v.base.tile;
+    int tile0 = 0;  // as the caller sees it, to be put back if no candidate can be timed
+    lr_plan_tile(plan, &tile0);
     int best = tile0;
     double best_ms = 1e300;
     // time a plan-sized single-source call: build the launch as lr_response would
@@ -351,7 +352,8 @@ LR_API int lr_plan_autotune_batch(lr_plan *plan, int64_t S, const int64_t *lengt
     cudaEvent_t a = nullptr, b = nullptr;
     if (e == cudaSuccess) e = cudaEventCreate(&a);
     if (e == cudaSuccess) e = cudaEventCreate(&b);
-    const int tile0 = v.base.tile;
+    int tile0 = 0;  // as the caller sees it, to be put back if no candidate can be timed
+    lr_plan_tile(plan, &tile0);
     int best = tile0;
     double best_ms = 1e300;
     const std::vector<int> cand = tile_candidates(v);

@@ -78,3 +78,17 @@ def test_small_tiles_where_the_stencils_do_not_fit(ctx, p, dt, tile):
     plan.check()
     check_batch(one, pair, lens[:1], per[:1], p, dt)
     check_batch(xyz, pair, lens, per, p, dt)
+
+
+def test_failed_tuning_keeps_the_tile(ctx, flex):
+    """A tile that the tensor-core kernels work in equal parts (512 in parts of 256) is still the plan's tile after
+    a tuning that ran out of memory."""
+    plan = lr.Plan(ctx, 25, 4096, DT, flex.gpu, t0=T0, tile=512)
+    for tune in (lambda: plan.autotune(4096, use_cache=False), lambda: plan.autotune_batch([4096, 300], use_cache=False)):
+        lr.library().lr_debug_fail_allocations(0)
+        try:
+            with pytest.raises(lr.LRError):
+                tune()
+        finally:
+            lr.library().lr_debug_fail_allocations(-1)
+        assert plan.tile == 512
