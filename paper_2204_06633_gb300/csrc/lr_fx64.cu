@@ -698,7 +698,9 @@ void fx_plan_free(FxPlan *F)
 }
 
 // The launch's parameters.  Until the table's kernel is known to be done the stream waits for it; a captured
-// launch cannot (the event was recorded outside the capture), there the host waits.
+// launch cannot (the event was recorded outside the capture), there the host waits.  While a stream is being
+// captured in global mode, by this thread or another, event calls are refused and break that capture: the event
+// belongs to no capture, so they are made in relaxed mode.
 int fx_table_for(FxPlan *F, void *str, FxTab *X)
 {
     const cudaStream_t stream = (cudaStream_t)str;
@@ -708,23 +710,23 @@ int fx_table_for(FxPlan *F, void *str, FxTab *X)
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     cudaError_t e = cudaStreamIsCapturing(stream, &cap);
     if (e != cudaSuccess) return (int)e;
-    if (cap != cudaStreamCaptureStatusNone) {
-        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;  // event calls are refused in the other modes
-        e = cudaThreadExchangeStreamCaptureMode(&mode);
-        if (e != cudaSuccess) return (int)e;
-        e = cudaEventSynchronize(ev);
-        const cudaError_t e2 = cudaThreadExchangeStreamCaptureMode(&mode);
-        if (e == cudaSuccess) e = e2;
-        return (int)e;
-    }
-    e = cudaEventQuery(ev);
-    if (e == cudaErrorNotReady) {
-        cudaGetLastError();
-        return (int)cudaStreamWaitEvent(stream, ev);
-    }
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    e = cudaThreadExchangeStreamCaptureMode(&mode);
     if (e != cudaSuccess) return (int)e;
-    F->ready = nullptr;
-    return (int)cudaEventDestroy(ev);
+    if (cap != cudaStreamCaptureStatusNone) {
+        e = cudaEventSynchronize(ev);
+    } else {
+        e = cudaEventQuery(ev);
+        if (e == cudaErrorNotReady) {
+            cudaGetLastError();
+            e = cudaStreamWaitEvent(stream, ev);
+        } else if (e == cudaSuccess) {
+            F->ready = nullptr;
+            e = cudaEventDestroy(ev);
+        }
+    }
+    const cudaError_t e2 = cudaThreadExchangeStreamCaptureMode(&mode);
+    return (int)(e != cudaSuccess ? e : e2);
 }
 
 int launch_fx64(int kind, int order, const FwdParams &P, int sms, void *stream)

@@ -3,6 +3,7 @@ tensor-core kernels' range give the oracle's results, keep what the caller asked
 that their kernels read."""
 import dataclasses
 import os
+import threading
 
 import numpy as np
 import pytest
@@ -92,3 +93,39 @@ def test_failed_tuning_keeps_the_tile(ctx, flex):
         finally:
             lr.library().lr_debug_fail_allocations(-1)
         assert plan.tile == 512
+
+
+def test_first_call_while_another_thread_captures(ctx, flex):
+    """A plan's first call looks whether its stencil table is done; made while another thread captures a graph in
+    the strictest mode, it runs and leaves the capture whole."""
+    N, p = 3000, 25
+    src = synth.draw_sources(1, seed=2)[0]
+    t0h, hp, hc = synth.gb_input(src, T0, DT, N, p)
+    hp, hc = dev(hp), dev(hc)
+    ref = lr.Plan(ctx, p, N, DT, flex.gpu, t0=T0).response(hp, hc, t0h, sky(src))   # the kernels are loaded
+    plan = lr.Plan(ctx, p, N, DT, flex.gpu, t0=T0)
+    xyz, mine, cap = torch.empty_like(ref), torch.cuda.Stream(), torch.cuda.Stream()
+    a = torch.zeros(8, device="cuda:0")
+    torch.cuda.synchronize()
+    failed = []
+
+    def call():
+        try:
+            plan.response(hp, hc, t0h, sky(src), xyz=xyz, stream=mine)
+        except lr.LRError as e:
+            failed.append(e)
+
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(cap):
+        g.capture_begin(capture_error_mode="global")
+        a.add_(1.0)
+        t = threading.Thread(target=call)
+        t.start()
+        t.join()
+        a.add_(1.0)
+        g.capture_end()
+    assert not failed
+    g.replay()
+    plan.check(mine)
+    torch.cuda.synchronize()
+    assert torch.equal(xyz, ref) and torch.equal(a, torch.full_like(a, 2.0))
