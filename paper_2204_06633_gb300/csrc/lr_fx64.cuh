@@ -723,7 +723,8 @@ __device__ __forceinline__ void table_coefs(double *p, double xc, double xs, dou
 }
 
 // Segments of a block on the plan's expansion table (one per spline piece, at most two): their starts and
-// pieces, or 0 when a piece has no entry.  One thread.
+// pieces, or 0 when a piece has no entry or the block leaves the orbit's knots: the end pieces are continued
+// there, and the table's polynomials and their one stencil position hold within a piece only.  One thread.
 __device__ int table_segments(const FwdParams &P, const FxTab &X, Shared &S, double t_lo, int nb)
 {
     double x;
@@ -731,6 +732,7 @@ __device__ int table_segments(const FwdParams &P, const FxTab &X, Shared &S, dou
     row_at(P.to, t_lo, -1, &x, &a);
     const double ua = x + (double)a;
     row_at(P.to, t_lo + (double)(nb - 1) * P.dt, -1, &x, &b);
+    if (ua < 0.0 || x + (double)b > (double)P.to.nint) return 0;
     if (b > a + 1 || X.meta[FX_META * a] == 0 || X.meta[FX_META * b] == 0) return 0;
     S.nseg = 1 + (b > a);
     S.segj[0] = 0;

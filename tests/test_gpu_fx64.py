@@ -100,3 +100,20 @@ def test_zero_strain_gives_zero(ctx, flex):
     z = torch.zeros(2200, dtype=torch.float64, device="cuda:0")
     assert not plan.response(z, z, -100 * DT, (0.3, 0.2, 0.1)).any()
     plan.check()
+
+
+@pytest.mark.parametrize("past", [0.0, 3e5])
+def test_outputs_past_the_knots(ctx, past):
+    """The orbit's end pieces are continued outside its knots, and the delayed reads with them: blocks before the
+    first knot, across the last one and behind it."""
+    N, p = 3000, 25
+    tk = synth.knot_grid(0.0, 5e5, pad=2)
+    pair = Pair(ctx, synth.Orbit(tk, synth.keplerian_flexing(tk), None))
+    src = dataclasses.replace(synth.draw_sources(1, seed=4)[0], f=3e-3)
+    for t0 in (tk[-1] - 15000.0 + past, tk[0] - 15000.0 - past):
+        t0h, hp, hc = synth.gb_input(src, t0, DT, N, p)
+        plan = lr.Plan(ctx, p, N, DT, pair.gpu, t0=t0)
+        got = host(plan.response(dev(hp), dev(hc), t0h, sky(src)))
+        plan.check()
+        args = (p, 2, DT, t0, N, pair.orc, pair.orc, hp, hc, t0h, src.lam, src.beta, src.psi)
+        assert_close(got, oracle.response(*args), oracle.response(*args, absval=True), p + 1, 1e-12)
