@@ -331,30 +331,43 @@ bool fx_create(lr_plan *p)
     return true;
 }
 
-// whether the adjoint runs on the tensor-core kernels: summed (or constant) delays, stencils that fit and the
-// table of them.  Mixed plans take the same kernels (the table is built at their first adjoint): they are
-// more exact than the float-float ones and several times faster.
-bool fx_backward(lr_plan *p)
+// Whether the tensor-core kernels serve the plan: summed (or constant) delays, merged stencils and halos that
+// leave blocks of 128 outputs, and orbits that a block's expansion can follow.
+//   - The projection transpose finds the link samples of a block from the reads' positions at one time, within a
+//     quarter of a sample: the reads may not drift by more over half a block and the reads' reach.  A LISA orbit
+//     drifts by 0.06 to 0.09.  Before that limit a block's expansion no longer converges and the blocks are
+//     evaluated sample by sample, where the kernels made for that are faster (200 000 samples, order 25, an orbit
+//     eight times as fast: forward 3.6 against 3.3 ms, adjoint 23.8 against 6.9).
+//   - A block holds at most ten segments, one for each spline piece and stencil step: with knots closer than an
+//     eighth of a block every block would be evaluated sample by sample (4.3 against 3.3 ms).
+bool fx_applies(const lr_plan *p)
 {
     const lr::FwdParams &P = p->base;
-    if ((P.delay_nested && !P.cd_w) || lr::fx_max_tile(P, p->desc.order) < 128 || !fx_create(p)) return false;
-    return p->fx->tab.tab != nullptr;
+    if ((P.delay_nested && !P.cd_w) || lr::fx_max_tile(P, p->desc.order) < 128) return false;
+    const double reach = lr::FX_ROWS / 2 + P.sig_b + P.lproj_b + p->T;
+    if (p->desc.proj_orbit->max_rate * reach > 0.25) return false;
+    const double block = lr::FX_ROWS * P.dt;
+    return block <= 8.0 * p->desc.proj_orbit->dk && block <= 8.0 * p->desc.tdi_orbit->dk;
 }
+
+// whether the adjoint runs on the tensor-core kernels (it needs the stencil table).  Mixed plans take the same
+// kernels (the table is built at their first adjoint): they are more exact than the float-float ones and several
+// times faster.
+bool fx_backward(lr_plan *p) { return fx_applies(p) && fx_create(p) && p->fx->tab.tab != nullptr; }
 
 // its tiles (of link and of strain samples): the forward's block, so that a time split in units of the plan's
 // tile meets the same blocks
 int fx_backward_tile(const lr_plan *p) { return p->base.fx_tile ? p->base.fx_tile : lr::fx_max_tile(p->base, p->desc.order); }
 
-// FP64 plans whose stencils fit run on the tensor-core kernels (lr_fx64.cu).  Their blocks hold at most
+// FP64 plans that they serve run on the tensor-core kernels (lr_fx64.cu).  Their blocks hold at most
 // fx_max_tile outputs; a larger tile is worked in equal parts, so that a time split in units of the tile
-// keeps every block whole.  Nested delays that vary keep the sample-by-sample kernels.
+// keeps every block whole.
 void fx_setup(lr_plan *p)
 {
     lr::FwdParams &P = p->base;
     P.fx_tile = 0;
-    if (p->desc.precision != LR_FP64 || (P.delay_nested && !P.cd_w)) return;
+    if (p->desc.precision != LR_FP64 || !fx_applies(p)) return;
     const int most = lr::fx_max_tile(P, p->desc.order);
-    if (most < 128) return;  // the merged stencils do not fit, or their halos leave no room
     int block = p->tile < most ? p->tile : most;
     while (block >= 128 && p->tile % block) --block;
     if (block < 128 && p->tile >= 128) return;  // no part of at least 128 outputs
@@ -668,10 +681,7 @@ LR_API int lr_plan_create(lr_ctx *ctx, const lr_plan_desc *d, lr_plan **out)
             delete p;
             return st;
         }
-        if (d->tile == 0 && (!P.delay_nested || P.cd_w)) {
-            const int most = lr::fx_max_tile(P, d->order);
-            if (most >= 128) P.tile = most;
-        }
+        if (d->tile == 0 && fx_applies(p)) P.tile = lr::fx_max_tile(P, d->order);
     }
     P.ymax = P.tile + P.HL + P.HR;
     P.wmax = P.ymax + 2 * P.sig_b + P.lproj_b + p->T + 4;

@@ -49,3 +49,23 @@ def test_outputs_past_the_knots(ctx, past):
     pair = Pair(ctx, synth.Orbit(tk, synth.keplerian_flexing(tk), None))
     src = dataclasses.replace(synth.draw_sources(1, seed=4)[0], f=3e-3)
     check(ctx, pair, N, p, src, np.random.default_rng(6).normal(size=(3, N)), t0=tk[-1] - 7000.0 + past)
+
+
+@pytest.mark.parametrize("speed,spacing,precision", [(2.0, 5e4, lr.FP64), (4.0, 25e3, lr.FP64), (20.0, 1e3, lr.FP64),
+                                                     (60.0, 1e3, lr.FP64), (2.0, 5e4, lr.MIXED)])
+def test_fast_orbits(ctx, speed, spacing, precision):
+    """The orbit run through faster: its reads drift by up to 1.5 samples over half a block of 512."""
+    N, p = 2500, 25
+    tk = synth.knot_grid(-1e5, N * DT + 1e5, spacing=spacing)
+    pair = Pair(ctx, synth.Orbit(tk, synth.keplerian_flexing(tk * speed), None))
+    src = dataclasses.replace(synth.draw_sources(1, seed=4)[0], f=3e-3, beta=0.02)
+    check(ctx, pair, N, p, src, np.random.default_rng(8).normal(size=(3, N)), precision=precision)
+
+
+def test_close_knots(ctx):
+    """More spline pieces in a block than it has segments."""
+    N, p = 1500, 25
+    tk = synth.knot_grid(-2e4, N * DT + 2e4, spacing=500.0)
+    pair = Pair(ctx, synth.Orbit(tk, synth.keplerian_flexing(tk), None))
+    src = dataclasses.replace(synth.draw_sources(1, seed=4)[0], f=3e-3)
+    check(ctx, pair, N, p, src, np.random.default_rng(8).normal(size=(3, N)))
