@@ -13,7 +13,8 @@
 //       expansion nodes, the gradient is the inner product of dV_n/dtheta with the correlations
 //       C_q[c] = sum_k T_q(nu_k) gy[k] h[k + c], which are contractions over the block's samples; the node
 //       values (weights, their derivatives, geometry) are then needed 8 times per block, not per sample.
-// Segments (stencil steps, spline knots), ranges and the blocks evaluated sample by sample are as in lr_fx64.cu.
+// Segments (stencil steps, spline knots), ranges and the blocks evaluated sample by sample are as in lr_fx64.cu; K3
+// bounds the orders of its products from the geometry at the nodes (sky_series_fits).
 //
 // Measured (one year at order 41, mixed plan): K1 5.97 -> 1.65, K2 12.16 -> 4.45, K3 12.2 -> 6.34 ms;
 // 65536 samples at order 25 (FP64 plan): K1 1.26 -> 0.063, K2 0.42 -> 0.116, K3 0.64 -> 0.175 ms.
@@ -597,9 +598,11 @@ __device__ __forceinline__ void frame_derivatives(const SkyConst &K, double dk[2
 }
 
 // link l's part of the gradient at positions x, angles a0 .. a1 - 1 of (lambda, beta); psi with beta.  e, r: the
-// emission and reception reads summed against gy, (value, derivative) of h+ and hx
+// emission and reception reads summed against gy, (value, derivative) of h+ and hx.  geo, where not null, gets the
+// link's coefficients of h+ and hx and their derivatives with respect to those angles: [6], two for the values
+// (with the first angle), then two per angle.
 __device__ __forceinline__ void sky_terms(const FwdParams &P, const SkyConst &K, const double *x, int l, const double *e,
-                                          const double *r, int a0, int a1, double *G)
+                                          const double *r, int a0, int a1, double *G, double *geo)
 {
     double dk[2][3], du[2][3], dv[2][3];
     frame_derivatives(K, dk, du, dv);
@@ -614,6 +617,10 @@ __device__ __forceinline__ void sky_terms(const FwdParams &P, const SkyConst &K,
     const double xp = K.c2p * xip + K.s2p * xic, xc = -K.s2p * xip + K.c2p * xic;
     const double den = 1.0 / (2.0 * (1.0 - kn));
     const double dPp = e[0] - r[0], dPc = e[2] - r[2], dH = xp * dPp + xc * dPc;
+    if (geo && a0 == 0) {
+        geo[0] = den * xp;
+        geo[1] = den * xc;
+    }
     for (int th = a0; th < a1; ++th) {
         const double da = dot(du[th]), db = dot(dv[th]);
         const double dxip = 2.0 * (un * da - vn * db), dxic = 2.0 * (da * vn + un * db);
@@ -623,8 +630,63 @@ __device__ __forceinline__ void sky_terms(const FwdParams &P, const SkyConst &K,
         const double dur = -(dk[th][0] * x[3 * ir] + dk[th][1] * x[3 * ir + 1] + dk[th][2] * x[3 * ir + 2]) / C_LIGHT * P.inv_dt;
         const double ddH = dxp * dPp + dxc * dPc + xp * (e[1] * due - r[1] * dur) + xc * (e[3] * due - r[3] * dur);
         G[th] += dden * dH + den * ddH;
+        if (geo) {
+            geo[2 + 2 * th] = fma(dden, xp, den * dxp);
+            geo[3 + 2 * th] = fma(dden, xc, den * dxc);
+        }
     }
     if (a1 == 2) G[2] += den * (2.0 * xc * dPp - 2.0 * xp * dPc);
+}
+
+// Whether the expansion of one coefficient series of a link over the block (g: its node values, a stride apart)
+// holds, together with that of the reads' weights.  The gradient's products are taken at eight nodes, and the
+// correlations of order q carry 8 zq(q) bits less than those of order 0, so the orders of (coefficient) x (weights)
+// have to fall as the digits assume and the first one left out has to be small.  Orders of the coefficient relative
+// to `scale`; those of the weights by those of sinc: with a drift of +-delta samples over the block the j-th is
+// at most 2 (pi delta / 2)^j / (j! (j + 1)).  Checked against the exact terms of single blocks (a 3 mHz source, order
+// 25): the bound of order 8 is 7e-15 for sources far from the arms, 1e-11 at 0.01 rad from one, where the terms are
+// 9e-12 off, 1.6e-9 at 5e-3 (1e-9), 5e-4 at 1e-3 (2e-4).
+__device__ __forceinline__ bool sky_series_fits(const FxTab &X, const double *g, int stride, float scale, float delta)
+{
+    double e[NN / 2], o[NN / 2];
+#pragma unroll
+    for (int n = 0; n < NN / 2; ++n) {
+        const double a = g[n * stride], b = g[(NN - 1 - n) * stride];
+        e[n] = a + b;
+        o[n] = a - b;
+    }
+    float c[NN], w[NN + 1];
+    const float inv = 1.0f / scale;
+#pragma unroll
+    for (int q = 0; q < NN; ++q) {
+        double v = 0.0;
+#pragma unroll
+        for (int n = 0; n < NN / 2; ++n) v = fma((q & 1) ? o[n] : e[n], X.cheb[q][n], v);
+        c[q] = fabsf((float)v) * inv;
+    }
+    float run = 2.0f;
+    w[0] = 1.0f;
+#pragma unroll
+    for (int j = 1; j <= NN; ++j) {
+        run *= 1.5707964f * delta / (float)j;
+        w[j] = run / (float)(j + 1);
+    }
+    bool ok = true;
+#pragma unroll
+    for (int q = 1; q <= NN; ++q) {
+        float p = 0.0f;
+#pragma unroll
+        for (int i = 0; i < NN && i <= q; ++i) p = fmaf(c[i], w[q - i], p);
+        if (q < NN) {
+            ok &= p <= 16.0f / (float)(1ull << (8 * zq(false, q)));
+        } else {
+            // the coefficient's own next order, from the decay over its last two pairs
+            const float last = fmaxf(c[NN - 1], c[NN - 2]), before = fmaxf(c[NN - 3], c[NN - 4]);
+            p += last <= before ? last * (last / fmaxf(before, 1e-30f)) : last;
+            ok &= p <= 2.8e-14f;   // 2^-45
+        }
+    }
+    return ok;   // false for NaN
 }
 
 // value and derivative of both polarisations at base + u, straight from memory (Horner form of read_scalar)
@@ -745,6 +807,7 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_sky_adj(FwdPar
     __shared__ double dots[NN][6][2][4];   // node, link, (emission, reception): h+ value, derivative, hx value, derivative
     __shared__ double red[3][NTHR / 32];
     __shared__ unsigned gmax, gmin;
+    __shared__ int gscale[2];   // largest coefficient at the nodes, largest derivative (floats)
     const int tid = threadIdx.x, h = (T - 2) / 2;
     const int lane = tid & 31, warp = tid >> 5, lr4 = lane >> 2, kp = lane & 3;
     const uint32_t sh = 8 * ((7 - lr4) & 3);
@@ -879,6 +942,7 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_sky_adj(FwdPar
                     // node weights and their derivatives (prefix and suffix products with the product rule, two
                     // threads per read), the reads on this segment's spline piece
                     const int *sm = S.segm[sg];
+                    if (tid < 2) gscale[tid] = 0;
                     if (sm[9] != S.segm[sg ? sg - 1 : 0][9]) {
                         if (tid < NN * 3) node_reads(P, X, S, t_lo, u0, tid / 3, tid % 3, sm[9]);
                         __syncthreads();
@@ -965,14 +1029,32 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_sky_adj(FwdPar
                         dots[n][l][er][2 * pol + 1] = d;
                     }
                     __syncthreads();
+                    double *geo = wn;   // [node][link][6]: the weights are done with
                     if (tid < 128 && (tid & 63) < NN * 6) {   // an angle per thread: lambda, then beta and psi two warps on
                         double t[3] = {0.0, 0.0, 0.0};
                         const int th = tid >> 6, n = (tid & 63) / 6, l = (tid & 63) % 6;
-                        sky_terms(P, S.skc, S.npos[n], l, dots[n][l][0], dots[n][l][1], th, th + 1, t);
+                        double *q = geo + 6 * (tid & 63);
+                        sky_terms(P, S.skc, S.npos[n], l, dots[n][l][0], dots[n][l][1], th, th + 1, t, q);
                         const double unit = pow2(eg) * pow2(ex);
                         for (int c = 0; c < 3; ++c) Gs[c] += t[c] * unit;
+                        if (th == 0) atomicMax(&gscale[0], __float_as_int((float)fmax(fabs(q[0]), fabs(q[1]))) & 0x7fffffff);
+                        atomicMax(&gscale[1], __float_as_int((float)fmax(fabs(q[2 + 2 * th]), fabs(q[3 + 2 * th]))) & 0x7fffffff);
+                    }
+                    __syncthreads();
+                    bool fits = true;
+                    if (tid < 36) {
+                        const int l = tid / 6, i = tid % 6;
+                        const double de = S.nodeu[3 + l] - S.nodeu[(NN - 1) * 9 + 3 + l];
+                        const double dr = S.nodeu[c_lr[l]] - S.nodeu[(NN - 1) * 9 + c_lr[l]];
+                        const float delta = 0.51f * (float)fmax(fabs(de), fabs(dr));   // half the drift; the nodes end at 0.98
+                        fits = sky_series_fits(X, geo + 6 * l + i, 36, __int_as_float(gscale[i > 1]), delta);
+                    }
+                    if (__syncthreads_or(!fits)) {
+                        bad = true;
+                        break;
                     }
                 }
+                if (bad) Gs[0] = Gs[1] = Gs[2] = 0.0;
             }
             __syncthreads();
             if (bad)
@@ -989,7 +1071,7 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_sky_adj(FwdPar
                         if (gl == 0.0) continue;
                         double ee[4], t[3] = {0.0, 0.0, 0.0};
                         read_vd_scalar(S, T, ti.hp, ti.hc, ti.nh, k, u0 - L[l] * P.inv_dt - sig[c_ls[l]], ee);
-                        sky_terms(P, S.skc, x, l, ee, rr[c_lr[l]], 0, 2, t);
+                        sky_terms(P, S.skc, x, l, ee, rr[c_lr[l]], 0, 2, t, nullptr);
                         for (int c = 0; c < 3; ++c) Gs[c] = fma(gl, t[c], Gs[c]);
                     }
                 }

@@ -69,3 +69,30 @@ def test_close_knots(ctx):
     pair = Pair(ctx, synth.Orbit(tk, synth.keplerian_flexing(tk), None))
     src = dataclasses.replace(synth.draw_sources(1, seed=4)[0], f=3e-3)
     check(ctx, pair, N, p, src, np.random.default_rng(8).normal(size=(3, N)))
+
+
+@pytest.mark.skipif(not oracle.quad_available(), reason="no binary128 libm in this toolchain")
+@pytest.mark.parametrize("off", [3e-2, 1e-2, 5e-3, 1e-3, 2e-4, 5e-5])
+def test_sky_gradient_beside_an_arm(ctx, flex, off):
+    """One block, the closest approach to an arm in its middle: the patterns turn within it, the faster the nearer
+    the source is.  Against binary128; 1 - k.n has few significant bits there, so the FP64 oracle is off by up to
+    3e-8 itself, and the bound is 16 times its error (as many bits lost, in other operations) where that is more
+    than 1e-11 (1e-12 for the strain gradients)."""
+    N, p, mid = 492, 11, 246
+    pos = synth.keplerian_flexing(np.array([mid * DT]))[:, :, 0]
+    d = (pos[0] - pos[1]) / np.linalg.norm(pos[0] - pos[1])
+    src = dataclasses.replace(synth.draw_sources(1, seed=4)[0], f=1e-2, lam=float(np.arctan2(-d[1], -d[0]) + off),
+                              beta=float(np.arcsin(-d[2])))
+    t0h, hp, hc = synth.gb_input(src, T0, DT, N, p)
+    g = np.random.default_rng(8).normal(size=(3, N))
+    g[:, :mid - 180] = g[:, mid + 180:] = 0.0
+    orb, oracle_args = flex.orb, (hp, hc, t0h, *sky(src), g)
+    exact = oracle.backward_quad(p, 2, DT, T0, N, orb.t_knots, orb.pos, orb.delays, *oracle_args)
+    r64 = oracle.backward(p, 2, DT, T0, N, flex.orc, flex.orc, *oracle_args)
+    for precision in (lr.FP64, lr.MIXED):
+        plan = lr.Plan(ctx, p, N, DT, flex.gpu, t0=T0, precision=precision)
+        got = [host(v) for v in plan.backward(dev(hp), dev(hc), t0h, sky(src), dev(g))]
+        plan.check()
+        for a, b, c, rel in zip(got, exact, r64, (1e-12, 1e-12, 1e-11)):
+            err, own = np.linalg.norm(a - b), np.linalg.norm(c - b)
+            assert err <= max(rel * np.linalg.norm(b), 16 * own), (err / np.linalg.norm(b), own / np.linalg.norm(b))
