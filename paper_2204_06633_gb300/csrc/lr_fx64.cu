@@ -58,24 +58,25 @@ namespace {
 // ---------------------------------------------------------------- the block's link series
 // Fills ys[6][NY] with the link series of rows 0 .. ny - 1 (sample k_lo + row).
 template <int NTHR>
-__device__ void project_block(const FwdParams &P, const FxTab &X, Shared &S, int T, int64_t k_lo, int ny, double u0, double *ys,
+__device__ void project_block(const FwdParams &P, const FxTab &X, Shared &S, int T, int64_t k_lo, int ny, double u, double *ys,
                               unsigned char *work)
 {
     const int tid = threadIdx.x, h = (T - 2) / 2;
-    const double fl0 = floor(u0);
+    const int64_t f0 = (int64_t)floor(u);
+    const double u0 = u - floor(u);
     const double t_lo = P.t0 + (double)k_lo * P.dt;
     const TileInfo &ti = S.ti;
     uint16_t *planes = reinterpret_cast<uint16_t *>(work);
     unsigned char *W = work + FX_PROJ_PLANES;
     double *wn = reinterpret_cast<double *>(work + FX_PROJ_PLANES + FX_PROJ_W);
 
-    projection_segments(P, X, S, t_lo, u0, fl0, ny);
+    projection_segments(P, X, S, t_lo, u0, ny);
     const int nseg = S.nseg;
     const int mmin = S.mmin, KW = S.mmax - mmin + T;   // taps of a merged stencil
     const int nks = (KW + 3 + 15) / 16;
     bool bad = S.bad || nks * 16 > 64;
     // strain window: row j reads samples w_lo + j .. w_lo + j + KW - 1
-    const int64_t w_lo = k_lo + (int64_t)fl0 + mmin - h;
+    const int64_t w_lo = k_lo + f0 + mmin - h;
     const int WL = ny + KW - 1;
     constexpr int NV = (DL + NTHR - 1) / NTHR;
     double vp[NV], vc[NV];
@@ -125,7 +126,7 @@ __device__ void project_block(const FwdParams &P, const FxTab &X, Shared &S, int
     const uint32_t lane = tid & 31, warp = tid >> 5, lr4 = lane >> 2, kp = lane & 3;
     const uint32_t sh = 8 * ((7 - lr4) & 3);
     for (int sg = 0; sg < nseg && !bad; ++sg) {
-        if (!projection_stencils<false>(P, X, S, T, t_lo, u0, fl0, sg, KW, W, wn)) {
+        if (!projection_stencils<false>(P, X, S, T, t_lo, u0, sg, KW, W, wn)) {
             bad = true;
             break;
         }
@@ -180,7 +181,7 @@ __device__ void project_block(const FwdParams &P, const FxTab &X, Shared &S, int
     if (!bad) return;
     // sample by sample, on the strain window of all reads that the plan's bounds allow
     double *hwp = reinterpret_cast<double *>(work), *hwc = hwp + FX_PROJ_PLANES / 16;
-    const int64_t s_lo = k_lo + (int64_t)fl0 - P.sig_b - P.lproj_b - h - 2;
+    const int64_t s_lo = k_lo + f0 - P.sig_b - P.lproj_b - h - 2;
     const int slen = ny + 2 * P.sig_b + P.lproj_b + T + 4;
     bool nonfinite = false;
     for (int j = tid; j < slen; j += blockDim.x) {
@@ -207,8 +208,8 @@ __device__ void project_block(const FwdParams &P, const FxTab &X, Shared &S, int
             orbit_all(P.po, P.t0 + (double)k * P.dt, x, L);
             for (int i = 0; i < 3; ++i) {
                 sig[i] = (K.k[0] * x[3 * i] + K.k[1] * x[3 * i + 1] + K.k[2] * x[3 * i + 2]) / C_LIGHT * P.inv_dt;
-                rp[i] = read_scalar(S, T, hwp, k, u0 - sig[i], s_lo, slen, P.err);
-                rc[i] = read_scalar(S, T, hwc, k, u0 - sig[i], s_lo, slen, P.err);
+                rp[i] = read_scalar(S, T, hwp, k + f0, u0 - sig[i], s_lo, slen, P.err);
+                rc[i] = read_scalar(S, T, hwc, k + f0, u0 - sig[i], s_lo, slen, P.err);
             }
             for (int a = 0; a < 3; ++a) {
                 const int r = a, s = (a + 1) % 3, lf = a, lb = 5 - a;
@@ -220,10 +221,10 @@ __device__ void project_block(const FwdParams &P, const FxTab &X, Shared &S, int
                 const double xip = un * un - vn * vn, xic = 2.0 * un * vn;
                 const double xp = K.c2p * xip + K.s2p * xic, xc = -K.s2p * xip + K.c2p * xic;
                 const double uf = u0 - L[lf] * P.inv_dt - sig[s], ub = u0 - L[lb] * P.inv_dt - sig[r];
-                double ep = read_scalar(S, T, hwp, k, uf, s_lo, slen, P.err), ec = read_scalar(S, T, hwc, k, uf, s_lo, slen, P.err);
+                double ep = read_scalar(S, T, hwp, k + f0, uf, s_lo, slen, P.err), ec = read_scalar(S, T, hwc, k + f0, uf, s_lo, slen, P.err);
                 y[lf] = (xp * (ep - rp[r]) + xc * (ec - rc[r])) / (2.0 * (1.0 - kn));
-                ep = read_scalar(S, T, hwp, k, ub, s_lo, slen, P.err);
-                ec = read_scalar(S, T, hwc, k, ub, s_lo, slen, P.err);
+                ep = read_scalar(S, T, hwp, k + f0, ub, s_lo, slen, P.err);
+                ec = read_scalar(S, T, hwc, k + f0, ub, s_lo, slen, P.err);
                 y[lb] = (xp * (ep - rp[s]) + xc * (ec - rc[s])) / (2.0 * (1.0 + kn));
             }
         }

@@ -474,10 +474,12 @@ __device__ __forceinline__ void count_orders(Shared &S)
 }
 
 // ---------------------------------------------------------------- projection stencils
+// Positions of the reads are relative to row + floor((t0 - t0h) / dt); u0 is the fraction that is left of that
+// offset.  The whole part goes into indices alone: a strain that begins 10^6 samples before the outputs would take
+// 20 bits from the reads' fractions (6e-12 of the response, and no block's expansion would fit).
 // Segments of rows 0 .. rows - 1 (row 0 at time t_lo) in which no read's stencil steps and the orbit's spline
 // piece stays: fills segj, segm, nseg, mmin, mmax and the reads at the expansion nodes.
-__device__ void projection_segments(const FwdParams &P, const FxTab &X, Shared &S, double t_lo, double u0, double fl0,
-                                    int rows)
+__device__ void projection_segments(const FwdParams &P, const FxTab &X, Shared &S, double t_lo, double u0, int rows)
 {
     const int tid = threadIdx.x;
     // stencil positions on the grid samples, and the reads at the expansion nodes (on row 0's spline piece)
@@ -494,7 +496,7 @@ __device__ void projection_segments(const FwdParams &P, const FxTab &X, Shared &
             for (int i = 0; i < 3; ++i) {
                 const int rd = i == 0 ? s : 3 + c_by_emitter[s][i - 1];
                 const double fl = floor(u[i]);
-                S.mg[g][rd] = (int)(fl - fl0);
+                S.mg[g][rd] = (int)fl;
                 S.fg[g][rd] = (float)(u[i] - fl);
             }
         } else {
@@ -534,7 +536,7 @@ __device__ void projection_segments(const FwdParams &P, const FxTab &X, Shared &
         const int j = g * GP + lane + 1;   // rows g GP + 1 .. (g + 1) GP against the row before
         int piece;
         const double u = read_pos(P, X, S.skc, u0, t_lo + (double)j * P.dt, rd < 9 ? rd : 0, &piece);
-        const int m = rd < 9 ? (int)(floor(u) - fl0) : piece;
+        const int m = rd < 9 ? (int)floor(u) : piece;
         const int prev = __shfl_up_sync(0xffffffffu, m, 1);
         if (m != (lane ? prev : S.mg[g][rd]) && j < NY) atomicOr(&S.brk[j >> 5], 1u << (j & 31));
     }
@@ -548,7 +550,7 @@ __device__ void projection_segments(const FwdParams &P, const FxTab &X, Shared &
         if (sg) {
             int piece;
             const double u = read_pos(P, X, S.skc, u0, t_lo + (double)S.segj[sg] * P.dt, rd < 9 ? rd : 0, &piece);
-            m = rd < 9 ? (int)(floor(u) - fl0) : piece;
+            m = rd < 9 ? (int)floor(u) : piece;
         }
         S.segm[sg][rd] = m;
         if (rd < 9) {
@@ -562,7 +564,7 @@ __device__ void projection_segments(const FwdParams &P, const FxTab &X, Shared &
 // Lagrange weights wn[T][node, read] and pattern coefficients of segment sg at the expansion nodes.  Starts
 // with a barrier in the caller; ends after the last write (a barrier is needed before reading).
 __device__ __forceinline__ void node_weights(const FwdParams &P, const FxTab &X, Shared &S, int T, double t_lo, double u0,
-                                             double fl0, int sg, double *wn)
+                                             int sg, double *wn)
 {
     const int tid = threadIdx.x;
     const int *sm = S.segm[sg];
@@ -580,7 +582,7 @@ __device__ __forceinline__ void node_weights(const FwdParams &P, const FxTab &X,
         double e = 0.0, run = 1.0;
         double *w = wn + id;
         if (half) {
-            e = S.nodeu[id] - (fl0 + (double)sm[id % 9]);
+            e = S.nodeu[id] - (double)sm[id % 9];
             if (low) {
 #pragma unroll 4
                 for (int a = 0; a < T / 2; ++a) {
@@ -644,14 +646,14 @@ __device__ __forceinline__ int stencil_exp(int cmax)
 // expansion does not fit.  Begins and ends with a barrier.
 template <bool REV>
 __device__ bool projection_stencils(const FwdParams &P, const FxTab &X, Shared &S, int T, double t_lo, double u0,
-                                    double fl0, int sg, int KW, unsigned char *W, double *wn)
+                                    int sg, int KW, unsigned char *W, double *wn)
 {
     const int tid = threadIdx.x, mmin = S.mmin;
     const int *sm = S.segm[sg];
     __syncthreads();  // the previous segment's stencils and nodes are free
     for (int i = tid; i < FX_PROJ_W / 16; i += blockDim.x)
         reinterpret_cast<uint4 *>(W)[i] = make_uint4(0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u);
-    node_weights(P, X, S, T, t_lo, u0, fl0, sg, wn);
+    node_weights(P, X, S, T, t_lo, u0, sg, wn);
     int cm[6], call = 0;
 #pragma unroll
     for (int l = 0; l < 6; ++l) {

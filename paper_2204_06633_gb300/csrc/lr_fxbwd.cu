@@ -365,7 +365,7 @@ __device__ void proj_adj_sample(const FwdParams &P, const SkyConst &K, double u0
     }
 }
 
-__device__ void proj_adj_scalar(const FwdParams &P, Shared &S, int T, double u0, int64_t i0, int nb, int64_t k_lo,
+__device__ void proj_adj_scalar(const FwdParams &P, Shared &S, int T, double u0, int64_t f0, int64_t i0, int nb, int64_t k_lo,
                                 const double *gys, double *ghp, double *ghc, double *w)
 {
     const int tid = threadIdx.x, h = (T - 2) / 2;
@@ -381,7 +381,7 @@ __device__ void proj_adj_scalar(const FwdParams &P, Shared &S, int T, double u0,
             const int i = tid + (int)blockDim.x * r;
             if (i >= nb) continue;
             for (int id = 0; id < 72; ++id) {
-                const int64_t a = i0 + i - (k_lo + j0 + (id & 7) + (int64_t)floor(U[id])) + h;
+                const int64_t a = i0 + i - (k_lo + f0 + j0 + (id & 7) + (int64_t)floor(U[id])) + h;
                 if (a < 0 || a >= T) continue;
                 acc[r][0] = fma(w[a * 72 + id], CF[2 * (id >> 3) * 8 + (id & 7)], acc[r][0]);
                 acc[r][1] = fma(w[a * 72 + id], CF[(2 * (id >> 3) + 1) * 8 + (id & 7)], acc[r][1]);
@@ -466,19 +466,19 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_proj_adj(FwdPa
             __syncthreads();
             continue;
         }
-        const double u0 = u0s, fl0 = floor(u0);
-        const int64_t i0 = S.ti.n0, N = S.ti.N;
+        const int64_t i0 = S.ti.n0, N = S.ti.N, f0 = (int64_t)floor(u0s);
+        const double u0 = u0s - floor(u0s);
         // the link samples whose reads can land on the tile: from the reads' positions near its centre
         if (tid < 9) {
             int piece;
-            const double u = read_pos(P, X, S.skc, u0, P.t0 + (double)(i0 + nb / 2 - (int64_t)fl0) * P.dt, tid, &piece) - fl0;
+            const double u = read_pos(P, X, S.skc, u0, P.t0 + (double)(i0 + nb / 2 - f0) * P.dt, tid, &piece);
             atomicMin(&umin, (int)floor(u - 0.25));
             atomicMax(&umax, (int)floor(u + 0.25));
         }
         __syncthreads();
-        const int64_t k_lo = i0 - (int64_t)fl0 - umax - (h + 1);
+        const int64_t k_lo = i0 - f0 - umax - (h + 1);
         const double t_lo = P.t0 + (double)k_lo * P.dt;
-        projection_segments(P, X, S, t_lo, u0, fl0, NY);
+        projection_segments(P, X, S, t_lo, u0, NY);
         const double *gy = B.g_y + 2 * (S.ti.out - P.out);
         bool any = false;
         for (int l = 0; l < 6; ++l)
@@ -503,7 +503,7 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_proj_adj(FwdPa
         bool bad = S.bad || nks * 16 > 64 || j0 < 0 || j0 + nb + KW - 1 > NY || !range_ok(S, &eg);
         double out[4] = {0.0, 0.0, 0.0, 0.0};
         for (int sg = 0; sg < nseg && !bad; ++sg) {
-            if (!projection_stencils<true>(P, X, S, T, t_lo, u0, fl0, sg, KW, W, wn)) {
+            if (!projection_stencils<true>(P, X, S, T, t_lo, u0, sg, KW, W, wn)) {
                 bad = true;
                 break;
             }
@@ -579,7 +579,7 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_proj_adj(FwdPa
                 if (i < nb) o[i0 + i] = out[r];
             }
         }
-        if (bad) proj_adj_scalar(P, S, T, u0, i0, nb, k_lo, gys, ghp, ghc, reinterpret_cast<double *>(sm_raw + K2_STENCILS));
+        if (bad) proj_adj_scalar(P, S, T, u0, f0, i0, nb, k_lo, gys, ghp, ghc, reinterpret_cast<double *>(sm_raw + K2_STENCILS));
         __syncthreads();
     }
 }
@@ -830,12 +830,13 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_sky_adj(FwdPar
             const TileInfo &ti = S.ti;
             const int nb = (int)ti.nb;
             const int64_t k_lo = ti.n0, N = ti.N;
-            const double u0 = (P.t0 - ti.t0h) / P.dt, fl0 = floor(u0), t_lo = P.t0 + (double)k_lo * P.dt;
+            const double u = (P.t0 - ti.t0h) / P.dt, u0 = u - floor(u), t_lo = P.t0 + (double)k_lo * P.dt;
+            const int64_t f0 = (int64_t)floor(u);
             const double *gy = B.g_y + 2 * (ti.out - P.out);
-            projection_segments(P, X, S, t_lo, u0, fl0, nb);
+            projection_segments(P, X, S, t_lo, u0, nb);
             const int nseg = S.nseg, mmin = S.mmin, KW = S.mmax - mmin + T, npass = (KW + 31) / 32;
             bool bad = S.bad || KW > LG;
-            const int64_t w_lo = k_lo + (int64_t)fl0 + mmin - h;
+            const int64_t w_lo = k_lo + f0 + mmin - h;
             const int WL = nb + KW - 1;
             bool anyg = false, anyh = false;
             constexpr int NV = (DL + NTHR - 1) / NTHR;
@@ -952,7 +953,7 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_sky_adj(FwdPar
                     double e = 0.0, run = 1.0, drun = 0.0;
                     double *w = wn + id, *dw = dwn + id;
                     if (half) {
-                        e = S.nodeu[id] - (fl0 + (double)sm[id % 9]);
+                        e = S.nodeu[id] - (double)sm[id % 9];
                         if (low) {
                             for (int a = 0; a < T / 2; ++a) {
                                 w[a * WNS] = run;
@@ -1064,13 +1065,13 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_sky_adj(FwdPar
                     orbit_all(P.po, P.t0 + (double)k * P.dt, x, L);
                     for (int i = 0; i < 3; ++i) {
                         sig[i] = (S.skc.k[0] * x[3 * i] + S.skc.k[1] * x[3 * i + 1] + S.skc.k[2] * x[3 * i + 2]) / C_LIGHT * P.inv_dt;
-                        read_vd_scalar(S, T, ti.hp, ti.hc, ti.nh, k, u0 - sig[i], rr[i]);
+                        read_vd_scalar(S, T, ti.hp, ti.hc, ti.nh, k + f0, u0 - sig[i], rr[i]);
                     }
                     for (int l = 0; l < 6; ++l) {
                         const double gl = __ldg(gy + l * N + k);
                         if (gl == 0.0) continue;
                         double ee[4], t[3] = {0.0, 0.0, 0.0};
-                        read_vd_scalar(S, T, ti.hp, ti.hc, ti.nh, k, u0 - L[l] * P.inv_dt - sig[c_ls[l]], ee);
+                        read_vd_scalar(S, T, ti.hp, ti.hc, ti.nh, k + f0, u0 - L[l] * P.inv_dt - sig[c_ls[l]], ee);
                         sky_terms(P, S.skc, x, l, ee, rr[c_lr[l]], 0, 2, t, nullptr);
                         for (int c = 0; c < 3; ++c) Gs[c] = fma(gl, t[c], Gs[c]);
                     }

@@ -117,3 +117,23 @@ def test_outputs_past_the_knots(ctx, past):
         plan.check()
         args = (p, 2, DT, t0, N, pair.orc, pair.orc, hp, hc, t0h, src.lam, src.beta, src.psi)
         assert_close(got, oracle.response(*args), oracle.response(*args, absval=True), p + 1, 1e-12)
+
+
+@pytest.mark.parametrize("early", [1, 20011, 1000037])
+def test_strain_that_begins_long_before_the_outputs(ctx, flex, early):
+    """The reads' fractions do not depend on how far before the outputs the strain begins: the same response, bit
+    for bit, and the same gradients."""
+    N, p = 3000, 25
+    src = dataclasses.replace(synth.draw_sources(1, seed=4)[0], f=3e-3)
+    t0h, hp, hc = synth.gb_input(src, T0, DT, N, p)
+    plan = lr.Plan(ctx, p, N, DT, flex.gpu, t0=T0)
+    g = dev(np.random.default_rng(3).normal(size=(3, N)))
+    z = np.zeros(early)
+    out = []
+    for a, b, t in ((hp, hc, t0h), (np.r_[z, hp], np.r_[z, hc], t0h - early * DT)):
+        out.append((plan.response(dev(a), dev(b), t, sky(src)), plan.backward(dev(a), dev(b), t, sky(src), g)))
+    plan.check()
+    (x0, g0), (x1, g1) = out
+    assert torch.equal(x0, x1) and torch.equal(g0[2], g1[2])
+    for a, b in zip(g0[:2], g1[:2]):
+        assert float(torch.linalg.norm(b[early:] - a)) <= 1e-13 * float(torch.linalg.norm(a))
