@@ -36,7 +36,8 @@ __host__ __device__ constexpr int gplane(bool tdi, int q)  // planes before orde
 }
 constexpr int TQP = gplane(true, NT);                         // 22 planes of a channel
 constexpr int QA = 3, PQA = gplane(false, QA), PQB = gplane(false, NN) - PQA;  // a link in two rounds: 21 and 23 planes
-constexpr int GB = 516;                                       // bytes of a digit row of T_q g (K3): distinct banks per link
+constexpr int GB = 520;                                       // bytes of a digit row of T_q g (K3): distinct banks per link
+static_assert(GB % 4 == 0 && GB >= 4 + 12 + 16 * (NY / 16 - 1) + 8, "the last step's loads of a full block stay in the row");
 constexpr int GROWS = gplane(false, NN);                      // 44 rows per link
 
 constexpr int K1_PART = 3 * NY * 8, K1_PLANES = K1_PART + 6 * NY * 8;
