@@ -356,8 +356,13 @@ bool fx_applies(const lr_plan *p)
 bool fx_backward(lr_plan *p) { return fx_applies(p) && fx_create(p) && p->fx->tab.tab != nullptr; }
 
 // its tiles (of link and of strain samples): the forward's block, so that a time split in units of the plan's
-// tile meets the same blocks
-int fx_backward_tile(const lr_plan *p) { return p->base.fx_tile ? p->base.fx_tile : lr::fx_max_tile(p->base, p->desc.order); }
+// tile meets the same blocks, or several of a small one (the work of a block hardly depends on its outputs:
+// 200 000 samples with a tile of 16, 7.6 ms in blocks of 16, 0.8 in blocks of 464)
+int fx_backward_tile(const lr_plan *p)
+{
+    const int most = lr::fx_max_tile(p->base, p->desc.order), block = p->base.fx_tile;
+    return block >= 128 ? block : block ? most / block * block : most;
+}
 
 // FP64 plans that they serve run on the tensor-core kernels (lr_fx64.cu).  Their blocks hold at most
 // fx_max_tile outputs; a larger tile is worked in equal parts, so that a time split in units of the tile

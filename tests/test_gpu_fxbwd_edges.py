@@ -96,3 +96,28 @@ def test_sky_gradient_beside_an_arm(ctx, flex, off):
         for a, b, c, rel in zip(got, exact, r64, (1e-12, 1e-12, 1e-11)):
             err, own = np.linalg.norm(a - b), np.linalg.norm(c - b)
             assert err <= max(rel * np.linalg.norm(b), 16 * own), (err / np.linalg.norm(b), own / np.linalg.norm(b))
+
+
+
+@pytest.mark.parametrize("tile", [1, 16, 127])
+def test_small_tiles(ctx, flex, tile):
+    """The adjoint's blocks hold as many of a small tile's as fit.  Three times the default tile's time allows for
+    smaller blocks, another number of waves and the spread of timings (in blocks of 16 they took ten times as long)."""
+    N, p = 60000, 25
+    src = dataclasses.replace(synth.draw_sources(1, seed=4)[0], f=3e-3)
+    g = np.random.default_rng(8).normal(size=(3, 3000))
+    check(ctx, flex, 3000, p, src, g, tile=tile)
+    t0h, hp, hc = (torch.as_tensor(v, device="cuda:0") if isinstance(v, np.ndarray) else v
+                   for v in synth.gb_input(src, T0, DT, N, p))
+    g, ms = torch.randn(3, N, dtype=torch.float64, device="cuda:0"), {}
+    for t in (0, tile):
+        plan = lr.Plan(ctx, p, N, DT, flex.gpu, t0=T0, tile=t)
+        plan.backward(hp, hc, t0h, sky(src), g)
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        for _ in range(10):
+            plan.backward(hp, hc, t0h, sky(src), g)
+        b.record()
+        b.synchronize()
+        ms[t] = a.elapsed_time(b)
+    assert ms[tile] <= 3.0 * ms[0], ms
