@@ -47,8 +47,8 @@
 // same warps, the TDI stencils' scale found in the block, and a barrier more for each of the two scales.
 //
 // Where the expansion does not apply, the block is evaluated sample by sample in FP64 as in lr_fwd64.cu: a
-// NaN or infinity in the series, values that span more than 12 bits between 32-sample stretches (the
-// fixed point is relative to the block's largest value), coefficients above the digits reserved for their
+// NaN or infinity in the series, outputs that read values far below the block's largest (the fixed point is
+// relative to it: RANGE_PROJ, RANGE_TDI), coefficients above the digits reserved for their
 // order (a source within ~1 degree of an arm direction, an orbit that moves faster), too many segments.
 #include "lr_fx64.cuh"
 
@@ -96,12 +96,14 @@ __device__ void project_block(const FwdParams &P, const FxTab &X, Shared &S, int
             }
             const unsigned a = abs_hi(vp[i]), b = abs_hi(vc[i]);
             if (!P.gen_strain && (a > b ? a : b) >= 0x7ff00000u) atomicOr(P.err, ERR_NONFINITE);
-            range_update(S, a > b ? a : b);
+            const unsigned w = warp_max(a > b ? a : b);
+            if ((tid & 31) == 0 && p < DL) S.st[0][p >> 5] = w;
         }
     }
     __syncthreads();
     int ex = 0;
-    const unsigned vmax = S.vmax;
+    unsigned vmax = 1;
+    const bool in_range = !bad && range_ok(S.st, 1, NSTR, KW, RANGE_PROJ, &vmax, &ex);
     if (!bad && vmax == 0) {  // a block of zeros (or of subnormal high words): the response is zero
         bool any = false;
 #pragma unroll
@@ -113,7 +115,7 @@ __device__ void project_block(const FwdParams &P, const FxTab &X, Shared &S, int
         }
         bad = true;
     }
-    if (!bad) bad = !range_ok(S, &ex);
+    bad |= !in_range;
     if (!bad) {
         for (int i = 0; i < NV; ++i) {
             const int p = tid + i * NTHR;
@@ -252,28 +254,33 @@ __device__ void tdi_block(const FwdParams &P, const FxTab &X, Shared &S, int T, 
     if (tid == 32) {
         S.nlist = 0;
         S.bad = 0;
-        S.vmax = 0;
-        S.vmin = 0x7fffffffu;
         S.mmin = 1 << 29;
         S.mmax = -(1 << 29);
     }
     if (tid == 64) S.fast = X.tab ? table_segments(P, X, S, t_lo, nb) : 0;
     __syncthreads();
     // the first and last link rows are spare: no stencil reaches them
-    for (int l = 0; l < 6; ++l)
 #pragma unroll
-        for (int i = 0; i < NY / NTHR; ++i) {
-            const int j = tid + NTHR * i;
-            range_update(S, j >= 1 && j < ny - 1 ? abs_hi(ys[l * NY + j]) : 0u);
-        }
+    for (int i = 0; i < NY / NTHR; ++i) {
+        const int j = tid + NTHR * i;
+        unsigned w[6];
+#pragma unroll
+        for (int l = 0; l < 6; ++l) w[l] = warp_max(j >= 1 && j < ny - 1 ? abs_hi(ys[l * NY + j]) : 0u);
+        constexpr SlotTab slots = make_slots();
+#pragma unroll
+        for (int ch = 0; ch < 3; ++ch)
+            if (lane == 0)
+                S.st[ch][j >> 5] = max(max(w[slots.link[ch][0]], w[slots.link[ch][1]]), max(w[slots.link[ch][2]], w[slots.link[ch][3]]));
+    }
     const bool fast = S.fast != 0;
     if (!fast) find_tdi_segments(P, S, t_lo, nb);
     __syncthreads();
     const int nseg = S.nseg;
     bool bad = S.bad;
     int ey = 0;
-    const bool zero = S.vmax == 0;
-    if (zero) {
+    unsigned vmax;
+    const bool in_range = range_ok(S.st, 3, NY / 32, T + P.HL - h - 2, RANGE_TDI, &vmax, &ey);
+    if (vmax == 0) {
         bool any = false;
         for (int i = tid; i < 6 * NY; i += blockDim.x) any |= i % NY < ny && ys[i] != 0.0;
         if (!__syncthreads_or(any)) {
@@ -283,7 +290,7 @@ __device__ void tdi_block(const FwdParams &P, const FxTab &X, Shared &S, int T, 
         }
         bad = true;
     }
-    if (!bad) bad = !range_ok(S, &ey);
+    bad |= !in_range;
     long long *part = reinterpret_cast<long long *>(ys);  // [2][3][NY], one segment: the planes hold the series
     int done = 0;                                          // outputs kept in ys[0..2][.] by earlier segments
     for (int sg = 0; sg < nseg && !bad; ++sg) {

@@ -27,7 +27,16 @@ constexpr int WNS = NN * 9;
 static_assert(2 * WNS <= 160 && NN * 6 == 48, "roles of node_weights");
 // merged TDI taps per thread: at most 12 stencils of 57 taps
 __host__ __device__ constexpr int tap_reps(int nthr) { return (12 * 57 + nthr - 1) / nthr; }
-constexpr int RANGE_BITS = 12;
+constexpr int NSTR = DL / 32;     // stretches of 32 samples of a staged series
+// Most binary orders between a block's largest value and the largest of any window that an output reads.  The
+// fixed point is relative to the block, so a quiet output beside a loud stretch loses those bits; beyond the
+// limit the block is evaluated sample by sample.  Error of such outputs against binary128, digits over sample
+// kernels (orders 11 to 41, a stretch 2^k of the rest): projection and TDI at 0.1 mHz 0.07 to 0.13 for k = 0, 0.5 to
+// 0.8 for 3, 1.1 to 1.7 for 4, 17 to 26 for 8; TDI alone at 1 mHz 0.9 to 1.1, 1.0 to 1.3, 1.4 to 1.8, 16 to 23; strain
+// gradients 0.66 for k = 0, 0.89 for 6, 2.1 for 8.  One order less for TDI would send a quarter of the blocks of a
+// 0.1 mHz source to the sample form, where the link series cross zero.  The sky gradient is a sum over the block,
+// in which the loud part has its own term.
+constexpr int RANGE_PROJ = 3, RANGE_TDI = 4, RANGE_ADJ = 5, RANGE_SKY = 12;
 // the last order's coefficient must be below 2^-45 of the stencil's scale: the next one is then below 2^-53
 constexpr unsigned long long LAST_MAX = 1024;
 
@@ -94,7 +103,7 @@ struct Shared {
     int list[NTERM * 8 + 8];
     int mmin, mmax;
     int cmax[6], wexp[6];
-    unsigned vmax, vmin;
+    unsigned st[3][NSTR];   // largest high word per stretch, of each set of series that one output reads
     unsigned long long qor[NN];  // OR of the coefficients' magnitudes per order
     int nq, last;                // orders in use; whether those above 0 have their last digit only
     int bad;
@@ -364,22 +373,26 @@ __device__ __forceinline__ void collect_segments(Shared &S, int rows)
 
 __device__ __forceinline__ unsigned abs_hi(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
 
-// largest and smallest non-zero of the 32-sample stretches' maxima (high words)
-__device__ __forceinline__ void range_update(Shared &S, unsigned m)
-{
-    const unsigned w = __reduce_max_sync(0xffffffffu, m);
-    if ((threadIdx.x & 31) == 0 && w) {
-        atomicMax(&S.vmax, w);
-        atomicMin(&S.vmin, w);
-    }
-}
+__device__ __forceinline__ unsigned warp_max(unsigned v) { return __reduce_max_sync(0xffffffffu, v); }
 
-// the exponent e with max < 2^e when the values fit the fixed point; false otherwise
-__device__ __forceinline__ bool range_ok(const Shared &S, int *e)
+// From the stretches' maxima (sets of n): the block's largest high word, the exponent e with max < 2^e, and whether
+// every window of taps samples that holds anything but zeros comes within `bits` orders of it.  Every warp for itself.
+__device__ __forceinline__ bool range_ok(const unsigned (*st)[NSTR], int sets, int n, int taps, int bits, unsigned *vmax, int *e)
 {
-    const int eb = (int)(S.vmax >> 20), es = (int)(S.vmin >> 20);
+    const int lane = threadIdx.x & 31;
+    unsigned hi = 0, lo = 0x7fffffffu;
+    for (int c = 0; c < sets; ++c) {
+        const unsigned m = lane < n ? st[c][lane] : 0u, next = __shfl_down_sync(0xffffffffu, m, 1);
+        hi = max(hi, m);
+        const unsigned w = taps > 32 ? max(m, next) : m;   // a window of more than 32 samples is in two stretches at least
+        if (w && lane < (taps > 32 ? n - 1 : n)) lo = min(lo, w);
+    }
+    hi = warp_max(hi);
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    *vmax = hi;
+    const int eb = (int)(hi >> 20), es = (int)(lo >> 20);
     *e = eb - 1022;
-    return eb >= 200 && eb <= 1900 && eb - es <= RANGE_BITS;
+    return eb >= 200 && eb <= 1900 && eb - es <= bits;
 }
 
 // v * 2^(55 - e), |v| < 2^e, rounded to an integer: shifts of the significand (FP64 conversions issue at a
@@ -510,8 +523,6 @@ __device__ void projection_segments(const FwdParams &P, const FxTab &X, Shared &
     if (tid == 192) {
         S.nlist = 0;
         S.bad = 0;
-        S.vmax = 0;
-        S.vmin = 0x7fffffffu;
         S.mmin = 1 << 29;
         S.mmax = -(1 << 29);
     }

@@ -100,13 +100,6 @@ __device__ __forceinline__ void put_digits(uint16_t *pl, int p, long long X)
     }
 }
 
-__device__ __forceinline__ void reset_range(Shared &S)
-{
-    S.bad = 0;
-    S.vmax = 0;
-    S.vmin = 0x7fffffffu;
-}
-
 __device__ __forceinline__ void lagrange_tables(Shared &S, int T)
 {
     const int tid = threadIdx.x, h = (T - 2) / 2;
@@ -217,7 +210,7 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_tdi_adj(FwdPar
         if (tid == 0) {
             S.ti = tile_info_of(P, g, src, 3);
             if (!S.ti.ok) atomicOr(P.err, ERR_OFFSETS);
-            reset_range(S);
+            S.bad = 0;
         }
         __syncthreads();
         if (!S.ti.ok || S.ti.nb <= 0) {
@@ -231,16 +224,22 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_tdi_adj(FwdPar
         const double *gx = B.g_xyz + (S.ti.out - P.out);
         double *gy = B.g_y + 2 * (S.ti.out - P.out);
         bool any = false;
-        for (int c = 0; c < 3; ++c)
 #pragma unroll
-            for (int r = 0; r < NY / NTHR; ++r) {
-                const int p = tid + NTHR * r;
-                const int64_t n = n_lo + p;
+        for (int r = 0; r < NY / NTHR; ++r) {
+            const int p = tid + NTHR * r;
+            const int64_t n = n_lo + p;
+            unsigned w[3];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
                 const double v = p < rows && n >= 0 && n < N ? __ldg(gx + c * N + n) : 0.0;
                 gs[c * NY + p] = v;
                 any |= v != 0.0;
-                range_update(S, abs_hi(v));
+                w[c] = warp_max(abs_hi(v));
             }
+            if (lane == 0)   // a link sample gathers from two of the channels
+#pragma unroll
+                for (int c = 0; c < 3; ++c) S.st[c][p >> 5] = max(w[c], w[(c + 1) % 3]);
+        }
         if (tid < NY / 32) S.brk[tid] = 0;
         if (tid == 0) {
             S.fast = table_segments(P, X, S, t_lo, rows);
@@ -258,7 +257,8 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_tdi_adj(FwdPar
         const bool fast = S.fast != 0;
         if (!fast) find_tdi_segments(P, S, t_lo, rows);
         __syncthreads();
-        bool bad = S.bad || !range_ok(S, &eg);
+        unsigned vmax;
+        bool bad = !range_ok(S.st, 3, NY / 32, X.tab_kw, RANGE_ADJ, &vmax, &eg) || S.bad;
         const int nseg = S.nseg;
         for (int sg = 0; sg < nseg && !bad; ++sg) {
             const int piece = S.segm[sg][NTERM], mmin = fast ? X.meta[FX_META * piece + 1] : S.mmin, KW = T - mmin, nks = (KW + 7 + 15) / 16;
@@ -482,16 +482,20 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_proj_adj(FwdPa
         projection_segments(P, X, S, t_lo, u0, NY);
         const double *gy = B.g_y + 2 * (S.ti.out - P.out);
         bool any = false;
-        for (int l = 0; l < 6; ++l)
 #pragma unroll
-            for (int r = 0; r < NY / NTHR; ++r) {
-                const int j = tid + NTHR * r;
-                const int64_t k = k_lo + j;
+        for (int r = 0; r < NY / NTHR; ++r) {
+            const int j = tid + NTHR * r;
+            const int64_t k = k_lo + j;
+            unsigned w = 0;
+            for (int l = 0; l < 6; ++l) {
                 const double v = k >= 0 && k < N ? __ldg(gy + l * N + k) : 0.0;
                 gys[l * NY + j] = v;
                 any |= v != 0.0;
-                range_update(S, abs_hi(v));
+                w = max(w, abs_hi(v));
             }
+            w = warp_max(w);
+            if (lane == 0) S.st[0][j >> 5] = w;
+        }
         double *ghp = B.g_hp + (S.ti.hp - P.hp), *ghc = B.g_hc + (S.ti.hp - P.hp);
         if (!__syncthreads_or(any)) {
             for (int i = tid; i < nb; i += blockDim.x) ghp[i0 + i] = ghc[i0 + i] = 0.0;
@@ -501,7 +505,9 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_proj_adj(FwdPa
         const int nseg = S.nseg, KW = S.mmax - S.mmin + T, nks = (KW + 3 + 15) / 16;
         const int j0 = umax - S.mmax;   // row of the first link sample that output 0 gathers from
         int eg = 0;
-        bool bad = S.bad || nks * 16 > 64 || j0 < 0 || j0 + nb + KW - 1 > NY || !range_ok(S, &eg);
+        unsigned vmax;
+        bool bad = !range_ok(S.st, 1, NY / 32, KW, RANGE_ADJ, &vmax, &eg);
+        bad |= S.bad || nks * 16 > 64 || j0 < 0 || j0 + nb + KW - 1 > NY;
         double out[4] = {0.0, 0.0, 0.0, 0.0};
         for (int sg = 0; sg < nseg && !bad; ++sg) {
             if (!projection_stencils<true>(P, X, S, T, t_lo, u0, sg, KW, W, wn)) {
@@ -807,7 +813,6 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_sky_adj(FwdPar
     __shared__ Shared S;
     __shared__ double dots[NN][6][2][4];   // node, link, (emission, reception): h+ value, derivative, hx value, derivative
     __shared__ double red[3][NTHR / 32];
-    __shared__ unsigned gmax, gmin;
     __shared__ int gscale[2];   // largest coefficient at the nodes, largest derivative (floats)
     const int tid = threadIdx.x, h = (T - 2) / 2;
     const int lane = tid & 31, warp = tid >> 5, lr4 = lane >> 2, kp = lane & 3;
@@ -822,8 +827,6 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_sky_adj(FwdPar
             S.ti = tile_info_of(P, g, src, 3);
             if (P.src.tile_off) S.skc = P.src.skyc[src];
             if (!S.ti.ok) atomicOr(P.err, ERR_OFFSETS);
-            gmax = 0;
-            gmin = 0x7fffffffu;
         }
         __syncthreads();
         double Gs[3] = {0.0, 0.0, 0.0};
@@ -854,28 +857,29 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_sky_adj(FwdPar
                     }
                     anyh |= vp[i] != 0.0 || vc[i] != 0.0;
                     const unsigned a = abs_hi(vp[i]), b = abs_hi(vc[i]);
-                    range_update(S, a > b ? a : b);
+                    const unsigned w = warp_max(a > b ? a : b);
+                    if (lane == 0 && p < DL) S.st[0][p >> 5] = w;
                 }
-                for (int l = 0; l < 6; ++l)
 #pragma unroll
-                    for (int r = 0; r < NY / NTHR; ++r) {
-                        const int j = tid + NTHR * r;
+                for (int r = 0; r < NY / NTHR; ++r) {
+                    const int j = tid + NTHR * r;
+                    unsigned w = 0;
+                    for (int l = 0; l < 6; ++l) {
                         const double v = j < nb ? __ldg(gy + l * N + k_lo + j) : 0.0;
                         anyg |= v != 0.0;
-                        const unsigned m = __reduce_max_sync(0xffffffffu, abs_hi(v));
-                        if (lane == 0 && m) {
-                            atomicMax(&gmax, m);
-                            atomicMin(&gmin, m);
-                        }
+                        w = max(w, abs_hi(v));
                     }
+                    w = warp_max(w);
+                    if (lane == 0) S.st[1][j >> 5] = w;
+                }
             }
             const bool work = bad || (__syncthreads_or(anyg) && __syncthreads_or(anyh));
             int ex = 0, eg = 0;
             if (!bad && work) {
-                bad = !range_ok(S, &ex);
-                const int eb = (int)(gmax >> 20), es = (int)(gmin >> 20);
-                eg = eb - 1022 + ((gmax & 0xfffff) >= 0xfa000);   // the top byte's range is 127.5 / 128 of the scale
-                bad |= !(eb >= 200 && eb <= 1900 && eb - es <= RANGE_BITS);
+                unsigned hmax, gmax;
+                bad = !range_ok(S.st, 1, NSTR, KW, RANGE_SKY, &hmax, &ex);
+                bad |= !range_ok(S.st + 1, 1, NY / 32, KW, RANGE_SKY, &gmax, &eg);
+                eg += (gmax & 0xfffff) >= 0xfa000;   // the top byte's range is 127.5 / 128 of the scale
             }
             if (!bad && work) {
 #pragma unroll

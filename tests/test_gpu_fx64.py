@@ -137,3 +137,48 @@ def test_strain_that_begins_long_before_the_outputs(ctx, flex, early):
     assert torch.equal(x0, x1) and torch.equal(g0[2], g1[2])
     for a, b in zip(g0[:2], g1[:2]):
         assert float(torch.linalg.norm(b[early:] - a)) <= 1e-13 * float(torch.linalg.norm(a))
+
+
+@pytest.mark.skipif(not oracle.quad_available(), reason="no binary128 libm in this toolchain")
+@pytest.mark.parametrize("k", [0, 2, 3, 4, 8, 11])
+@pytest.mark.parametrize("f", [1e-4, 1e-3, 1e-2])
+def test_quiet_outputs_beside_a_loud_stretch(ctx, f, k):
+    """A stretch 2^k above the rest of its block: the outputs that do not read it are as close to binary128 as the
+    sample kernels' (a quarter more allows for chance), whether the block's fixed point takes them or not."""
+    N, p = 700, 11
+    orb = synth.orbit_flexing(T0 - 3e5, T0 + N * DT + 3e5)
+    pair = Pair(ctx, orb)
+    src = dataclasses.replace(synth.draw_sources(1, seed=4)[0], f=f)
+    t0h, hp, hc = synth.gb_input(src, T0, DT, N, p)
+    m = (len(hp) - N) // 2
+    loud = np.zeros(len(hp))
+    loud[m + 300:m + 380] = 1.0
+    hp, hc = (1.0 + (2.0 ** k - 1.0) * loud) * hp, (1.0 + (2.0 ** k - 1.0) * loud) * hc
+    quiet = oracle.response(p, 2, DT, T0, N, pair.orc, pair.orc, loud, loud, t0h, *sky(src), absval=True).max(0) == 0.0
+    quiet[492:] = False   # the block of the loud stretch
+    assert 150 < quiet.sum() < 400
+    exact = oracle.response_quad(p, 2, DT, T0, N, orb.t_knots, orb.pos, orb.delays, hp, hc, t0h, *sky(src))
+    err = []
+    for tile in (0, BY_SAMPLE):
+        plan = lr.Plan(ctx, p, N, DT, pair.gpu, t0=T0, tile=tile)
+        err.append(np.linalg.norm((host(plan.response(dev(hp), dev(hc), t0h, sky(src))) - exact)[:, quiet]))
+        plan.check()
+    assert err[0] <= max(1.25 * err[1], 1e-14 * np.linalg.norm(exact[:, quiet])), err
+
+
+@pytest.mark.parametrize("k", [0, 4, 8, 11])
+def test_quiet_channel_beside_loud_links(ctx, flex, k):
+    """X does not read the links between spacecraft 2 and 3: however loud they are, its distance from the oracle is
+    that of the sample kernels' to a factor of 4 (two bits of the block's fixed point, and the oracle's own error)."""
+    N, p = 1434, 11
+    src = dataclasses.replace(synth.draw_sources(1, seed=4)[0], f=1e-3)
+    t0h, hp, hc = synth.gb_input(src, T0, DT, N, p)
+    y = oracle.project(p, DT, T0, N, flex.orc, hp, hc, t0h, *sky(src))
+    ref = oracle.tdi(p, 2, DT, T0, N, flex.orc, y, 0)[0]
+    y[[1, 4]] *= 2.0 ** k
+    err = []
+    for tile in (0, BY_SAMPLE):
+        plan = lr.Plan(ctx, p, N, DT, flex.gpu, t0=T0, tile=tile)
+        err.append(np.linalg.norm(host(plan.tdi(dev(y)))[0] - ref))
+        plan.check()
+    assert err[0] <= 4.0 * err[1], err

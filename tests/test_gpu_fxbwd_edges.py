@@ -121,3 +121,29 @@ def test_small_tiles(ctx, flex, tile):
         b.synchronize()
         ms[t] = a.elapsed_time(b)
     assert ms[tile] <= 3.0 * ms[0], ms
+
+
+@pytest.mark.skipif(not oracle.quad_available(), reason="no binary128 libm in this toolchain")
+@pytest.mark.parametrize("k", [0, 5, 8, 11])
+def test_quiet_gradients_beside_a_loud_stretch(ctx, flex, k):
+    """A stretch of the cotangent 2^k above the rest: the strain gradients that it does not reach are within twice
+    the FP64 oracle's own distance from binary128."""
+    N, p = 700, 11
+    src = dataclasses.replace(synth.draw_sources(1, seed=4)[0], f=1e-3)
+    t0h, hp, hc = synth.gb_input(src, T0, DT, N, p)
+    g = np.random.default_rng(2).normal(size=(3, N))
+    loud = np.zeros((3, N))
+    loud[:, 300:380] = 1.0
+    args = (hp, hc, t0h, *sky(src))
+    quiet = oracle.backward(p, 2, DT, T0, N, flex.orc, flex.orc, *args, loud)[0] == 0.0
+    m = (len(hp) - N) // 2
+    quiet[:m] = quiet[m + 492:] = False   # the block of the loud stretch
+    assert 150 < quiet.sum() < 450
+    g *= 1.0 + (2.0 ** k - 1.0) * loud
+    exact = oracle.backward_quad(p, 2, DT, T0, N, flex.orb.t_knots, flex.orb.pos, flex.orb.delays, *args, g)
+    r64 = oracle.backward(p, 2, DT, T0, N, flex.orc, flex.orc, *args, g)
+    plan = lr.Plan(ctx, p, N, DT, flex.gpu, t0=T0)
+    got = [host(v) for v in plan.backward(dev(hp), dev(hc), t0h, sky(src), dev(g))]
+    plan.check()
+    for a, b, c in zip(got[:2], exact, r64):
+        assert np.linalg.norm((a - b)[quiet]) <= 2.0 * np.linalg.norm((c - b)[quiet])
