@@ -333,69 +333,116 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_tdi_adj(FwdPar
 }
 
 // ---------------------------------------------------------------- K2: projection transpose
-// the nine reads' coefficients of one link sample: U positions, CF[18] (read, polarisation)
-__device__ void proj_adj_sample(const FwdParams &P, const SkyConst &K, double u0, int64_t k, int64_t N, const double *gyk,
-                                double *U, double *CF, int st)
-{
-    for (int rd = 0; rd < 9; ++rd) {
-        U[rd * st] = u0;
-        CF[2 * rd * st] = CF[(2 * rd + 1) * st] = 0.0;
-    }
-    if (k < 0 || k >= N) return;
-    double x[9], L[6], sig[3];
-    orbit_all(P.po, P.t0 + (double)k * P.dt, x, L);
-    for (int i = 0; i < 3; ++i) {
-        sig[i] = (K.k[0] * x[3 * i] + K.k[1] * x[3 * i + 1] + K.k[2] * x[3 * i + 2]) / C_LIGHT * P.inv_dt;
-        U[i * st] = u0 - sig[i];
-    }
-    for (int l = 0; l < 6; ++l) {
-        const int r = c_lr[l], s = c_ls[l];
-        double d0 = x[3 * r] - x[3 * s], d1 = x[3 * r + 1] - x[3 * s + 1], d2 = x[3 * r + 2] - x[3 * s + 2];
-        const double inv = 1.0 / sqrt(d0 * d0 + d1 * d1 + d2 * d2);
-        d0 *= inv; d1 *= inv; d2 *= inv;
-        const double un = K.u[0] * d0 + K.u[1] * d1 + K.u[2] * d2, vn = K.v[0] * d0 + K.v[1] * d1 + K.v[2] * d2;
-        const double kn = K.k[0] * d0 + K.k[1] * d1 + K.k[2] * d2;
-        const double xip = un * un - vn * vn, xic = 2.0 * un * vn;
-        const double gl = gyk[l * NY] * (1.0 / (2.0 * (1.0 - kn)));
-        const double cp = gl * (K.c2p * xip + K.s2p * xic), cc = gl * (-K.s2p * xip + K.c2p * xic);
-        U[(3 + l) * st] = u0 - L[l] * P.inv_dt - sig[s];
-        CF[2 * (3 + l) * st] = cp;
-        CF[(2 * (3 + l) + 1) * st] = cc;
-        CF[2 * r * st] -= cp;
-        CF[(2 * r + 1) * st] -= cc;
-    }
-}
-
-__device__ void proj_adj_scalar(const FwdParams &P, Shared &S, int T, double u0, int64_t f0, int64_t i0, int nb, int64_t k_lo,
-                                const double *gys, double *ghp, double *ghc, double *w)
+// Sample by sample, for blocks that the expansion or the fixed point does not cover: chunks of 64 link samples,
+// over all that the plan's bounds let the block's strain samples meet.  The reads' positions and coefficients of a
+// chunk are shared between the threads by spacecraft and by link, the weights of two reads at a time are formed by
+// 128 threads, and every strain sample gathers from the rows of the chunk whose stencils hold it.  Eight threads
+// forming the reads of eight link samples, and every strain sample looking at all rows, took ten times as long
+// (200 000 samples, order 25, all blocks: 16 ms for this kernel; XXX now).
+constexpr int CR = 64;
+__device__ void proj_adj_scalar(const FwdParams &P, const FxTab &X, Shared &S, int T, double u0, int64_t f0, int64_t i0, int nb,
+                                const double *gy, double *ghp, double *ghc, double *w)
 {
     const int tid = threadIdx.x, h = (T - 2) / 2;
-    double *U = w + 72 * T, *CF = U + 72;   // chunks of 8 link samples: 72 reads
+    const int64_t N = S.ti.N;
+    // weights [T][2 CR], before them the spacecraft's positions [9][CR]; the nine reads' positions and coefficients, whole parts
+    double *pos = w, *U = w + (size_t)(2 * T > 9 ? 2 * T : 9) * CR, *CF = U + 9 * CR;
+    int *M = reinterpret_cast<int *>(CF + 18 * CR);
+    __shared__ int lo[9], hi[9];   // stencil positions of a chunk's reads
     double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
-    for (int j0 = 0; j0 < NY; j0 += 8) {
+    const int64_t ka = i0 - f0 - P.sig_b - h - 3, kb = i0 + nb - f0 + P.sig_b + P.lproj_b + h + 3;
+    const int64_t k_end = kb < N ? kb : N;
+    for (int64_t k0 = ka > 0 ? ka : 0; k0 < k_end; k0 += CR) {
         __syncthreads();
-        if (tid < 8) proj_adj_sample(P, S.skc, u0, k_lo + j0 + tid, S.ti.N, gys + j0 + tid, U + tid, CF + tid, 8);
+        if (tid < 9) {
+            lo[tid] = 1 << 29;
+            hi[tid] = -(1 << 29);
+        }
+        for (int i = tid; i < 3 * CR; i += blockDim.x) {
+            const int s = i / CR, j = i % CR;
+            double x, u[3], ps[9];
+            int piece;
+            const Coef4 *row = row_at(P.po, P.t0 + (double)(k0 + j) * P.dt, -1, &x, &piece);
+            reads_of(P, X, S.skc, row, x, s, u0, u, ps);
+#pragma unroll
+            for (int d = 0; d < 3; ++d) pos[(3 * s + d) * CR + j] = ps[3 * s + d];
+            U[s * CR + j] = u[0];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) U[(3 + c_by_emitter[s][e]) * CR + j] = u[1 + e];
+        }
         __syncthreads();
-        if (tid < 72) lagrange_to(S, T, U[tid] - floor(U[tid]), w + tid, 72);
+        for (int i = tid; i < 6 * CR; i += blockDim.x) {
+            const int l = i / CR, j = i % CR, r = c_lr[l], s = c_ls[l];
+            const SkyConst &K = S.skc;
+            double d0 = pos[3 * r * CR + j] - pos[3 * s * CR + j], d1 = pos[(3 * r + 1) * CR + j] - pos[(3 * s + 1) * CR + j],
+                   d2 = pos[(3 * r + 2) * CR + j] - pos[(3 * s + 2) * CR + j];
+            const double inv = 1.0 / sqrt(d0 * d0 + d1 * d1 + d2 * d2);
+            d0 *= inv; d1 *= inv; d2 *= inv;
+            const double un = K.u[0] * d0 + K.u[1] * d1 + K.u[2] * d2, vn = K.v[0] * d0 + K.v[1] * d1 + K.v[2] * d2;
+            const double kn = K.k[0] * d0 + K.k[1] * d1 + K.k[2] * d2;
+            const double xip = un * un - vn * vn, xic = 2.0 * un * vn;
+            const double gl = k0 + j < k_end ? __ldg(gy + l * N + k0 + j) * (1.0 / (2.0 * (1.0 - kn))) : 0.0;
+            CF[2 * (3 + l) * CR + j] = gl * (K.c2p * xip + K.s2p * xic);
+            CF[(2 * (3 + l) + 1) * CR + j] = gl * (-K.s2p * xip + K.c2p * xic);
+        }
+        for (int i = tid; i < 9 * CR; i += blockDim.x) {   // a warp's lanes are of one read
+            const int rd = i / CR;
+            const double u = U[i];
+            const int m = (int)floor(u);
+            M[i] = m;
+            const int a = __reduce_min_sync(0xffffffffu, m), b = __reduce_max_sync(0xffffffffu, m);
+            if ((tid & 31) == 0) {
+                atomicMin(&lo[rd], a);
+                atomicMax(&hi[rd], b);
+            }
+            if (k0 + i % CR < k_end && (m > P.sig_b + 1 || m < -P.sig_b - P.lproj_b - 2)) atomicOr(P.err, ERR_WINDOW);
+        }
         __syncthreads();
-        for (int r = 0; r < 2; ++r) {
-            const int i = tid + (int)blockDim.x * r;
-            if (i >= nb) continue;
-            for (int id = 0; id < 72; ++id) {
-                const int64_t a = i0 + i - (k_lo + f0 + j0 + (id & 7) + (int64_t)floor(U[id])) + h;
-                if (a < 0 || a >= T) continue;
-                acc[r][0] = fma(w[a * 72 + id], CF[2 * (id >> 3) * 8 + (id & 7)], acc[r][0]);
-                acc[r][1] = fma(w[a * 72 + id], CF[(2 * (id >> 3) + 1) * 8 + (id & 7)], acc[r][1]);
+        for (int i = tid; i < 6 * CR; i += blockDim.x) {   // receptions: the two links of a receiver
+            const int r = (i / CR) >> 1, pol = (i / CR) & 1, j = i % CR, l2 = r ? 6 - r : 3;
+            CF[(2 * r + pol) * CR + j] = -(CF[(2 * (3 + r) + pol) * CR + j] + CF[(2 * (3 + l2) + pol) * CR + j]);
+        }
+        const int64_t at = k0 + f0 - i0;   // strain sample (within the block) that the chunk's first row reads at position 0
+        for (int rd = 0; rd < 9; rd += 2) {
+            bool any = false;
+            for (int x = rd; x < rd + 2 && x < 9; ++x) any |= at + hi[x] + CR + h + 1 >= 0 && at + lo[x] - h < nb;
+            if (!any) continue;   // uniform over the block
+            __syncthreads();
+            if (tid < 2 * CR && rd + tid / CR < 9) {
+                const double u = U[rd * CR + tid];
+                lagrange_to(S, T, u - (double)M[rd * CR + tid], w + tid, 2 * CR);
+            }
+            __syncthreads();
+            for (int x = 0; x < 2 && rd + x < 9; ++x) {
+                const double *cp = CF + 2 * (rd + x) * CR, *cc = cp + CR;
+                const int *m = M + (rd + x) * CR;
+#pragma unroll
+                for (int o = 0; o < 2; ++o) {
+                    const int i = tid + (int)blockDim.x * o;
+                    const int64_t c = i - at;   // rows j with c - h - 1 <= j + m[j] <= c + h
+                    const int64_t ja = c - h - 1 - hi[rd + x], jb = c + h - lo[rd + x];
+                    if (i >= nb || jb < 0 || ja >= CR) continue;
+                    for (int j = ja > 0 ? (int)ja : 0; j < CR && j <= jb; ++j) {
+                        const int a = (int)(c - j) - m[j] + h;
+                        if (a < 0 || a >= T) continue;
+                        const double wt = w[a * 2 * CR + x * CR + j];
+                        acc[o][0] = fma(wt, cp[j], acc[o][0]);
+                        acc[o][1] = fma(wt, cc[j], acc[o][1]);
+                    }
+                }
             }
         }
     }
-    for (int r = 0; r < 2; ++r)
-        if (tid + (int)blockDim.x * r < nb) {
-            ghp[i0 + tid + (int)blockDim.x * r] = acc[r][0];
-            ghc[i0 + tid + (int)blockDim.x * r] = acc[r][1];
+#pragma unroll
+    for (int o = 0; o < 2; ++o)
+        if (tid + (int)blockDim.x * o < nb) {
+            ghp[i0 + tid + (int)blockDim.x * o] = acc[o][0];
+            ghc[i0 + tid + (int)blockDim.x * o] = acc[o][1];
         }
     __syncthreads();
 }
+// its arrays fit in the stencils' and planes' place at every order compiled
+static_assert((2 * 42 + 27) * CR * 8 + 9 * CR * 4 <= FX_PROJ_W + K2_GROUP, "proj_adj_scalar's shared memory");
 
 // planes of T_q g for orders Q0 .. Q1 - 1 at row p, from x0 = g in fixed point
 template <int Q0, int Q1>
@@ -436,7 +483,7 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_proj_adj(FwdPa
     unsigned char *W = sm_raw + K2_STENCILS;
     double *wn = reinterpret_cast<double *>(sm_raw + K2_PLANES);  // the node weights are done with before the planes
     __shared__ Shared S;
-    __shared__ int nbs, umin, umax;
+    __shared__ int nbs, umax;
     __shared__ double u0s;
     const int tid = threadIdx.x, h = (T - 2) / 2;
     const int lane = tid & 31, warp = (tid >> 5) & 7, grp = tid >> 8, lr4 = lane >> 2, kp = lane & 3;
@@ -458,7 +505,6 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_proj_adj(FwdPa
             const int64_t nbh = S.ti.nh - S.ti.n0;   // clipped against the strain, not the outputs
             nbs = !S.ti.ok || nbh <= 0 ? 0 : (int)(nbh < B.tile_h ? nbh : B.tile_h);
             u0s = (P.t0 - S.ti.t0h) / P.dt;
-            umin = 1 << 29;
             umax = -(1 << 29);
         }
         __syncthreads();
@@ -473,7 +519,6 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_proj_adj(FwdPa
         if (tid < 9) {
             int piece;
             const double u = read_pos(P, X, S.skc, u0, P.t0 + (double)(i0 + nb / 2 - f0) * P.dt, tid, &piece);
-            atomicMin(&umin, (int)floor(u - 0.25));
             atomicMax(&umax, (int)floor(u + 0.25));
         }
         __syncthreads();
@@ -586,7 +631,7 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_proj_adj(FwdPa
                 if (i < nb) o[i0 + i] = out[r];
             }
         }
-        if (bad) proj_adj_scalar(P, S, T, u0, f0, i0, nb, k_lo, gys, ghp, ghc, reinterpret_cast<double *>(sm_raw + K2_STENCILS));
+        if (bad) proj_adj_scalar(P, X, S, T, u0, f0, i0, nb, gy, ghp, ghc, reinterpret_cast<double *>(sm_raw + K2_STENCILS));
         __syncthreads();
     }
 }

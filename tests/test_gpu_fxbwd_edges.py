@@ -147,3 +147,20 @@ def test_quiet_gradients_beside_a_loud_stretch(ctx, flex, k):
     plan.check()
     for a, b, c in zip(got[:2], exact, r64):
         assert np.linalg.norm((a - b)[quiet]) <= 2.0 * np.linalg.norm((c - b)[quiet])
+
+
+@pytest.mark.parametrize("p,N,gen", [(1, 700, 2), (3, 31, 2), (11, 492, 1), (25, 478, 2), (25, 1434, 1), (41, 2000, 2)])
+def test_blocks_evaluated_sample_by_sample(ctx, flex, p, N, gen):
+    """One loud cotangent sample in each block, in the first, a middle and the last output of the span."""
+    src = dataclasses.replace(synth.draw_sources(1, seed=7)[0], f=3e-3)
+    g = np.random.default_rng(N).normal(size=(3, N))
+    g[0, 0] = g[1, N // 2] = g[2, -1] = 1e5
+    t0h, hp, hc = synth.gb_input(src, T0, DT, N, p)
+    plan = lr.Plan(ctx, p, N, DT, flex.gpu, t0=T0, generation=gen)
+    got = [host(v) for v in plan.backward(dev(hp), dev(hc), t0h, sky(src), dev(g))]
+    plan.check()
+    rp, rc, rs, scale = oracle.backward(p, gen, DT, T0, N, flex.orc, flex.orc, hp, hc, t0h, src.lam, src.beta, src.psi, g,
+                                        with_scale=True)
+    for a, b in zip(got, (rp, rc)):
+        assert np.linalg.norm(a - b) <= 1e-12 * np.linalg.norm(b)
+    assert np.all(np.abs(got[2] - rs) <= np.maximum(1e-11 * np.abs(rs), 4 * (p + 17) * 2.0 ** -53 * scale))
