@@ -132,62 +132,77 @@ __device__ __forceinline__ void sky_by_warp(const lr_sky &sky, SkyConst *out)
 }
 
 // ---------------------------------------------------------------- K1: TDI transpose
-// Chunks of 16 outputs: the weights of a chain's seven reads at each, then every link sample gathers the taps
-// that land on it (blocks that the table or the fixed point does not cover).
-__device__ void tdi_adj_scalar(const FwdParams &P, Shared &S, int T, int64_t k0, int nb, const double *gs, double *gy,
-                               int64_t N, double *w)
+// Sample by sample, for blocks that the table or the fixed point does not cover: chunks of 64 outputs, the weights of
+// two delayed reads at a time by 128 threads, then every link sample gathers from the chunk's rows whose stencils
+// hold it, into a sum of its own.  Every link sample looking at all rows of a chunk, and adding to one of six
+// registers by comparing the link, took five times as long (200 000 samples, order 25, all blocks: 18 ms for this
+// kernel; XXX now).
+constexpr int CR = 64;
+__device__ void tdi_adj_scalar(const FwdParams &P, Shared &S, int T, int64_t k0, int nb, int rows, const double *gs, double *gy,
+                               int64_t N, double *acc)
 {
     const int tid = threadIdx.x, h = (T - 2) / 2, qn = P.q_terms;
-    const int64_t n_lo = k0 - h - 1;
-    int *mo = reinterpret_cast<int *>(w + 112 * T);
-    double acc[2][6];
-    for (int r = 0; r < 2; ++r)
-        for (int l = 0; l < 6; ++l) acc[r][l] = 0.0;
-    for (int p0 = 0; p0 < NY; p0 += 16)
-        for (int cc = 0; cc < 6; ++cc) {
-            const int ch = cc >> 1, c = cc & 1;
+    // sums [6][NY], the chunk's delays [6][CR], weights [T][2 CR], stencil positions [2 CR]
+    double *L = acc + 6 * NY, *w = L + 6 * CR;
+    int *M = reinterpret_cast<int *>(w + (size_t)2 * T * CR);
+    __shared__ int lo[4], hi[4];
+    __syncthreads();
+    for (int i = tid; i < nb; i += blockDim.x) {
+        for (int l = 0; l < 6; ++l) acc[l * NY + i] = 0.0;
+        for (int cc = 0; cc < 6; ++cc) {   // the undelayed terms
+            const double g = gs[(cc >> 1) * NY + i + h + 1];
+            acc[c_tdifx.link[cc >> 1][cc & 1][0] * NY + i] += (cc & 1) ? -g : g;
+        }
+    }
+    for (int p0 = 0; p0 < rows; p0 += CR) {
+        __syncthreads();
+        for (int i = tid; i < 6 * CR; i += blockDim.x) {
+            const int l = i / CR, j = i % CR;
+            double x;
+            int piece;
+            const Coef4 *row = row_at(P.to, P.t0 + (double)(k0 - h - 1 + p0 + j) * P.dt, -1, &x, &piece);
+            L[i] = cubic(ldg4(row + 9 + l), x) * P.inv_dt;
+        }
+        for (int t = 0; t < 6 * qn; t += 2) {   // 18 or 42 delayed terms
             __syncthreads();
-            if (tid < 112) {
-                const int j = tid & 15, q = (tid >> 4) + 1;
-                if (q <= qn) {
-                    int piece;
-                    const double u = -chain_delay(P, P.t0 + (double)(n_lo + p0 + j) * P.dt, cc * 7 + q - 1, &piece), fl = floor(u);
-                    mo[tid] = (int)fl;
-                    lagrange_to(S, T, u - fl, w + tid, 112);
+            if (tid < 2 * CR) {
+                const int cc = (t + tid / CR) / qn, q = (t + tid / CR) % qn + 1, j = tid % CR;
+                double D = 0.0;
+                for (int k = 1; k <= q; ++k) D += L[c_tdifx.pair[cc >> 1][cc & 1][k] * CR + j];
+                const int m = (int)floor(-D), a = __reduce_min_sync(0xffffffffu, m), b = __reduce_max_sync(0xffffffffu, m);
+                M[tid] = m;
+                if ((tid & 31) == 0) {
+                    lo[tid >> 5] = a;
+                    hi[tid >> 5] = b;
                 }
+                lagrange_to(S, T, -D - (double)m, w + tid, 2 * CR);
             }
             __syncthreads();
-            for (int r = 0; r < 2; ++r) {
-                const int i = tid + (int)blockDim.x * r;
-                if (i >= nb) continue;
-                for (int j = 0; j < 16; ++j) {
-                    const double g = gs[ch * NY + p0 + j];
-                    if (g == 0.0) continue;
-                    for (int q = 0; q <= qn; ++q) {
-                        const int64_t n = n_lo + p0 + j;
-                        double t;
-                        if (q == 0) {
-                            if (n != k0 + i) continue;
-                            t = g;
-                        } else {
-                            const int id = (q - 1) * 16 + j;
-                            const int a = (int)(k0 + i - (n + mo[id])) + h;
-                            if (a < 0 || a >= T) continue;
-                            t = w[a * 112 + id] * g;
-                        }
-                        const int l = c_tdifx.link[ch][c][q];
-#pragma unroll
-                        for (int m = 0; m < 6; ++m)
-                            if (m == l) acc[r][m] += c ? -t : t;
+            for (int x = 0; x < 2; ++x) {
+                const int cc = (t + x) / qn, q = (t + x) % qn + 1, l = c_tdifx.link[cc >> 1][cc & 1][q];
+                const int mlo = min(lo[2 * x], lo[2 * x + 1]), mhi = max(hi[2 * x], hi[2 * x + 1]);
+                const double *g = gs + (cc >> 1) * NY + p0;
+                for (int i = tid; i < nb; i += blockDim.x) {
+                    const int c = i + h + 1 - p0;   // rows j with c - h - 1 <= j + M[j] <= c + h
+                    const int ja = max(c - h - 1 - mhi, 0), jb = min(c + h - mlo, CR - 1);
+                    if (ja > jb) continue;
+                    double sum = 0.0;
+                    for (int j = ja; j <= jb; ++j) {
+                        const int a = c - j - M[x * CR + j] + h;
+                        if (a >= 0 && a < T) sum = fma(w[a * 2 * CR + x * CR + j], g[j], sum);
                     }
+                    acc[l * NY + i] += (cc & 1) ? -sum : sum;
                 }
             }
         }
-    for (int r = 0; r < 2; ++r)
-        if (tid + (int)blockDim.x * r < nb)
-            for (int l = 0; l < 6; ++l) gy[l * N + k0 + tid + (int)blockDim.x * r] = acc[r][l];
+    }
+    for (int i = tid; i < nb; i += blockDim.x)
+        for (int l = 0; l < 6; ++l) gy[l * N + k0 + i] = acc[l * NY + i];
     __syncthreads();
 }
+// its arrays fit in the place of the sums, the planes or node weights, and the stencils
+constexpr int k1_scalar(int T) { return 6 * NY * 8 + 6 * CR * 8 + 2 * T * CR * 8 + 2 * CR * 4; }
+static_assert(k1_scalar(32) <= k1_w(32) - K1_PART + FX_TDI_W && k1_scalar(42) <= k1_w(42) - K1_PART + FX_TDI_W, "tdi_adj_scalar's shared memory");
 
 template <int NTHR>
 __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_tdi_adj(FwdParams P, FxTab X, BwdParams B, int T)
@@ -327,7 +342,7 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_tdi_adj(FwdPar
                 }
         }
         __syncthreads();
-        if (bad) tdi_adj_scalar(P, S, T, k0, nb, gs, gy, N, reinterpret_cast<double *>(sm_raw + K1_PART));
+        if (bad) tdi_adj_scalar(P, S, T, k0, nb, rows, gs, gy, N, reinterpret_cast<double *>(sm_raw + K1_PART));
         __syncthreads();
     }
 }
@@ -339,7 +354,6 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_tdi_adj(FwdPar
 // 128 threads, and every strain sample gathers from the rows of the chunk whose stencils hold it.  Eight threads
 // forming the reads of eight link samples, and every strain sample looking at all rows, took ten times as long
 // (200 000 samples, order 25, all blocks: 16 ms for this kernel; XXX now).
-constexpr int CR = 64;
 __device__ void proj_adj_scalar(const FwdParams &P, const FxTab &X, Shared &S, int T, double u0, int64_t f0, int64_t i0, int nb,
                                 const double *gy, double *ghp, double *ghc, double *w)
 {
