@@ -643,8 +643,9 @@ int fx_max_tile(const FwdParams &P, int order)
     return fwd < adj ? fwd : adj;
 }
 
-void fx_tables(const FwdParams &P, int order, double max_delay, FxTab &X)
+void fx_tables(const FwdParams &P, int order, int precision, double max_delay, FxTab &X)
 {
+    X.range_adj = precision == LR_MIXED ? RANGE_ADJ_MIXED : RANGE_ADJ;
     const double pi = 3.14159265358979323846;
     X.icdt = P.inv_dt / C_LIGHT;
     // lags between a link sample and the strain it reads: the reads lie within two arms, one more while one steps

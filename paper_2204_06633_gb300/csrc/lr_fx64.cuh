@@ -35,8 +35,10 @@ constexpr int NSTR = DL / 32;     // stretches of 32 samples of a staged series
 // 0.8 for 3, 1.1 to 1.7 for 4, 17 to 26 for 8; TDI alone at 1 mHz 0.9 to 1.1, 1.0 to 1.3, 1.4 to 1.8, 16 to 23; strain
 // gradients 0.66 for k = 0, 0.89 for 6, 2.1 for 8.  One order less for TDI would send a quarter of the blocks of a
 // 0.1 mHz source to the sample form, where the link series cross zero.  The sky gradient is a sum over the block,
-// in which the loud part has its own term.
-constexpr int RANGE_PROJ = 3, RANGE_TDI = 4, RANGE_ADJ = 5, RANGE_SKY = 12;
+// in which the loud part has its own term.  Mixed plans' adjoints keep 43 bits of the quietest part, more than the
+// float-float kernels that they would run on otherwise (5e-13 from FP64, the digits 7e-14 at k = 11), in a tenth of the
+// time of the sample form.
+constexpr int RANGE_PROJ = 3, RANGE_TDI = 4, RANGE_ADJ = 5, RANGE_ADJ_MIXED = 12, RANGE_SKY = 12;
 // the last order's coefficient must be below 2^-45 of the stencil's scale: the next one is then below 2^-53
 constexpr unsigned long long LAST_MAX = 1024;
 

@@ -6,8 +6,8 @@ namespace lr {
 // largest tile (outputs per block) that the tensor-core kernels take for this plan's halos, bounds and
 // order; 0 when they do not apply
 int fx_max_tile(const FwdParams &P, int order);
-// expansion nodes and transforms; max_delay bounds the projection's light times (s)
-void fx_tables(const FwdParams &P, int order, double max_delay, FxTab &X);
+// expansion nodes and transforms; max_delay bounds the projection's light times (s); precision: the plan's
+void fx_tables(const FwdParams &P, int order, int precision, double max_delay, FxTab &X);
 // the plan's table of merged TDI stencils over the orbit's spline pieces: its size (0: none) and its
 // computation into F->mem, asynchronous (F->ready); a cudaError_t value
 size_t fx_table_bytes(const FwdParams &P, int order);

@@ -273,7 +273,7 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_tdi_adj(FwdPar
         if (!fast) find_tdi_segments(P, S, t_lo, rows);
         __syncthreads();
         unsigned vmax;
-        bool bad = !range_ok(S.st, 3, NY / 32, X.tab_kw, RANGE_ADJ, &vmax, &eg) || S.bad;
+        bool bad = !range_ok(S.st, 3, NY / 32, X.tab_kw, X.range_adj, &vmax, &eg) || S.bad;
         const int nseg = S.nseg;
         for (int sg = 0; sg < nseg && !bad; ++sg) {
             const int piece = S.segm[sg][NTERM], mmin = fast ? X.meta[FX_META * piece + 1] : S.mmin, KW = T - mmin, nks = (KW + 7 + 15) / 16;
@@ -565,7 +565,7 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_proj_adj(FwdPa
         const int j0 = umax - S.mmax;   // row of the first link sample that output 0 gathers from
         int eg = 0;
         unsigned vmax;
-        bool bad = !range_ok(S.st, 1, NY / 32, KW, RANGE_ADJ, &vmax, &eg);
+        bool bad = !range_ok(S.st, 1, NY / 32, KW, X.range_adj, &vmax, &eg);
         bad |= S.bad || nks * 16 > 64 || j0 < 0 || j0 + nb + KW - 1 > NY;
         double out[4] = {0.0, 0.0, 0.0, 0.0};
         for (int sg = 0; sg < nseg && !bad; ++sg) {

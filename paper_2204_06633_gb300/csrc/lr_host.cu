@@ -320,7 +320,7 @@ bool fx_create(lr_plan *p)
     const lr::FwdParams &P = p->base;
     p->fx = new (std::nothrow) lr::FxPlan();
     if (!p->fx) return false;
-    lr::fx_tables(P, p->desc.order, p->desc.proj_orbit->max_delay, p->fx->tab);
+    lr::fx_tables(P, p->desc.order, p->desc.precision, p->desc.proj_orbit->max_delay, p->fx->tab);
     const size_t bytes = lr::fx_table_bytes(P, p->desc.order);
     // without the table (no memory for it) the blocks compute their own stencils
     if (bytes && lr::dev_malloc(&p->fx->mem, bytes) == cudaSuccess && lr::fx_table_build(P, p->desc.order, p->fx)) {

@@ -112,6 +112,7 @@ struct FxTab {
     const int *meta;
     int tab_kw;
     int lags;   // correlation lags of the sky gradient, a multiple of 16
+    int range_adj;   // binary orders that a block's cotangents may span (lr_fx64.cuh)
 };
 // host side of a plan's tensor-core kernels: launch constants, the table's memory and the event of its
 // computation (null once it is known to be done)

@@ -127,7 +127,7 @@ def test_small_tiles(ctx, flex, tile):
 @pytest.mark.parametrize("k", [0, 5, 8, 11])
 def test_quiet_gradients_beside_a_loud_stretch(ctx, flex, k):
     """A stretch of the cotangent 2^k above the rest: the strain gradients that it does not reach are within twice
-    the FP64 oracle's own distance from binary128."""
+    the FP64 oracle's own distance from binary128, those of a mixed plan within 1e-12."""
     N, p = 700, 11
     src = dataclasses.replace(synth.draw_sources(1, seed=4)[0], f=1e-3)
     t0h, hp, hc = synth.gb_input(src, T0, DT, N, p)
@@ -145,8 +145,12 @@ def test_quiet_gradients_beside_a_loud_stretch(ctx, flex, k):
     plan = lr.Plan(ctx, p, N, DT, flex.gpu, t0=T0)
     got = [host(v) for v in plan.backward(dev(hp), dev(hc), t0h, sky(src), dev(g))]
     plan.check()
-    for a, b, c in zip(got[:2], exact, r64):
+    mixed = lr.Plan(ctx, p, N, DT, flex.gpu, t0=T0, precision=lr.MIXED)
+    got_mixed = [host(v) for v in mixed.backward(dev(hp), dev(hc), t0h, sky(src), dev(g))]
+    mixed.check()
+    for a, b, c, d in zip(got[:2], exact, r64, got_mixed):
         assert np.linalg.norm((a - b)[quiet]) <= 2.0 * np.linalg.norm((c - b)[quiet])
+        assert np.linalg.norm((d - b)[quiet]) <= 1e-12 * np.linalg.norm(b[quiet])
 
 
 @pytest.mark.parametrize("p,N,gen", [(1, 700, 2), (3, 31, 2), (11, 492, 1), (25, 478, 2), (25, 1434, 1), (41, 2000, 2)])
