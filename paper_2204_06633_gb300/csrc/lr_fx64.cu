@@ -103,7 +103,7 @@ __device__ void project_block(const FwdParams &P, const FxTab &X, Shared &S, int
     __syncthreads();
     int ex = 0;
     unsigned vmax = 1;
-    const bool in_range = !bad && range_ok(S.st, 1, NSTR, KW, RANGE_PROJ, &vmax, &ex);
+    const bool in_range = !bad && range_ok<0>(S.st, 1, WL, KW, RANGE_PROJ, &vmax, &ex);
     if (!bad && vmax == 0) {  // a block of zeros (or of subnormal high words): the response is zero
         bool any = false;
 #pragma unroll
@@ -279,7 +279,7 @@ __device__ void tdi_block(const FwdParams &P, const FxTab &X, Shared &S, int T, 
     bool bad = S.bad;
     int ey = 0;
     unsigned vmax;
-    const bool in_range = range_ok(S.st, 3, NY / 32, T + P.HL - h - 2, RANGE_TDI, &vmax, &ey);
+    const bool in_range = range_ok<1>(S.st, 3, ny, T + P.HL - h - 2, RANGE_TDI, &vmax, &ey);
     if (vmax == 0) {
         bool any = false;
         for (int i = tid; i < 6 * NY; i += blockDim.x) any |= i % NY < ny && ys[i] != 0.0;

@@ -32,9 +32,10 @@ constexpr int NSTR = DL / 32;     // stretches of 32 samples of a staged series
 // fixed point is relative to the block, so a quiet output beside a loud stretch loses those bits; beyond the
 // limit the block is evaluated sample by sample.  Error of such outputs against binary128, digits over sample
 // kernels (orders 11 to 41, a stretch 2^k of the rest): projection and TDI at 0.1 mHz 0.07 to 0.13 for k = 0, 0.5 to
-// 0.8 for 3, 1.1 to 1.7 for 4, 17 to 26 for 8; TDI alone at 1 mHz 0.9 to 1.1, 1.0 to 1.3, 1.4 to 1.8, 16 to 23; strain
-// gradients 0.66 for k = 0, 0.89 for 6, 2.1 for 8.  One order less for TDI would send a quarter of the blocks of a
-// 0.1 mHz source to the sample form, where the link series cross zero.  The sky gradient is a sum over the block,
+// 0.8 for 3, 1.1 to 1.7 for 4, 17 to 26 for 8; TDI alone at 1 mHz 0.9 to 1.1, 1.0 to 1.3, 1.4 to 1.8, 2.4 to
+// 3.4 for 5, 16 to 23; strain gradients 0.66 for k = 0, 0.89 for 6, 2.1 for 8.  Link series cross zero: a 0.1 mHz
+// source's stretches of 32 samples reach 2^5, any two of them 2^4, and 1 % of its blocks (a fifth at an order less)
+// would be evaluated sample by sample without TDI's extra order for single stretches.  The sky gradient is a sum over the block,
 // in which the loud part has its own term.  Mixed plans' adjoints keep 43 bits of the quietest part, more than the
 // float-float kernels that they would run on otherwise (5e-13 from FP64, the digits 7e-14 at k = 11), in a tenth of the
 // time of the sample form.
@@ -377,24 +378,30 @@ __device__ __forceinline__ unsigned abs_hi(double v) { return (unsigned)__double
 
 __device__ __forceinline__ unsigned warp_max(unsigned v) { return __reduce_max_sync(0xffffffffu, v); }
 
-// From the stretches' maxima (sets of n): the block's largest high word, the exponent e with max < 2^e, and whether
-// every window of taps samples that holds anything but zeros comes within `bits` orders of it.  Every warp for itself.
+// From the stretches' maxima (of `sets` sets, over n samples): the block's largest high word, the exponent e with max
+// < 2^e, and whether every window of taps samples that holds anything but zeros comes within `bits` orders of it
+// (SLACK more where the window may lie in one stretch and the two around it come within `bits`).  Every warp for
+// itself.
+template <int SLACK>
 __device__ __forceinline__ bool range_ok(const unsigned (*st)[NSTR], int sets, int n, int taps, int bits, unsigned *vmax, int *e)
 {
-    const int lane = threadIdx.x & 31;
-    unsigned hi = 0, lo = 0x7fffffffu;
+    const int lane = threadIdx.x & 31, stretches = (n + 31) >> 5;
+    const bool whole = n - 32 * lane >= (taps < 32 ? taps : 32);   // a window fits in the lane's stretch
+    unsigned hi = 0, one = 0x7fffffffu, two = 0x7fffffffu;
     for (int c = 0; c < sets; ++c) {
-        const unsigned m = lane < n ? st[c][lane] : 0u, next = __shfl_down_sync(0xffffffffu, m, 1);
+        const unsigned m = lane < stretches ? st[c][lane] : 0u, next = __shfl_down_sync(0xffffffffu, m, 1), w = max(m, next);
         hi = max(hi, m);
-        const unsigned w = taps > 32 ? max(m, next) : m;   // a window of more than 32 samples is in two stretches at least
-        if (w && lane < (taps > 32 ? n - 1 : n)) lo = min(lo, w);
+        if (m && whole) one = min(one, m);
+        if (w && lane < stretches - 1) two = min(two, w);
     }
     hi = warp_max(hi);
-    lo = __reduce_min_sync(0xffffffffu, lo);
+    one = __reduce_min_sync(0xffffffffu, one);
+    two = __reduce_min_sync(0xffffffffu, two);
     *vmax = hi;
-    const int eb = (int)(hi >> 20), es = (int)(lo >> 20);
+    const int eb = (int)(hi >> 20);
     *e = eb - 1022;
-    return eb >= 200 && eb <= 1900 && eb - es <= bits;
+    // a window of more than 32 samples is in two stretches at least
+    return eb >= 200 && eb <= 1900 && (taps > 32 || eb - (int)(one >> 20) <= bits + SLACK) && eb - (int)(two >> 20) <= bits;
 }
 
 // v * 2^(55 - e), |v| < 2^e, rounded to an integer: shifts of the significand (FP64 conversions issue at a

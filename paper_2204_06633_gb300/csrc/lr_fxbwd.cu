@@ -135,8 +135,7 @@ __device__ __forceinline__ void sky_by_warp(const lr_sky &sky, SkyConst *out)
 // Sample by sample, for blocks that the table or the fixed point does not cover: chunks of 64 outputs, the weights of
 // two delayed reads at a time by 128 threads, then every link sample gathers from the chunk's rows whose stencils
 // hold it, into a sum of its own.  Every link sample looking at all rows of a chunk, and adding to one of six
-// registers by comparing the link, took five times as long (200 000 samples, order 25, all blocks: 18 ms for this
-// kernel; XXX now).
+// registers by comparing the link, took 17.8 ms for 200 000 samples at order 25 (every block); 4.5 now.
 constexpr int CR = 64;
 __device__ void tdi_adj_scalar(const FwdParams &P, Shared &S, int T, int64_t k0, int nb, int rows, const double *gs, double *gy,
                                int64_t N, double *acc)
@@ -273,7 +272,7 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_tdi_adj(FwdPar
         if (!fast) find_tdi_segments(P, S, t_lo, rows);
         __syncthreads();
         unsigned vmax;
-        bool bad = !range_ok(S.st, 3, NY / 32, X.tab_kw, X.range_adj, &vmax, &eg) || S.bad;
+        bool bad = !range_ok<0>(S.st, 3, rows, X.tab_kw, X.range_adj, &vmax, &eg) || S.bad;
         const int nseg = S.nseg;
         for (int sg = 0; sg < nseg && !bad; ++sg) {
             const int piece = S.segm[sg][NTERM], mmin = fast ? X.meta[FX_META * piece + 1] : S.mmin, KW = T - mmin, nks = (KW + 7 + 15) / 16;
@@ -352,8 +351,8 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_tdi_adj(FwdPar
 // over all that the plan's bounds let the block's strain samples meet.  The reads' positions and coefficients of a
 // chunk are shared between the threads by spacecraft and by link, the weights of two reads at a time are formed by
 // 128 threads, and every strain sample gathers from the rows of the chunk whose stencils hold it.  Eight threads
-// forming the reads of eight link samples, and every strain sample looking at all rows, took ten times as long
-// (200 000 samples, order 25, all blocks: 16 ms for this kernel; XXX now).
+// forming the reads of eight link samples, and every strain sample looking at all rows, took 5.07 ms for 200 000
+// samples at order 25 (every block); 1.48 now.
 __device__ void proj_adj_scalar(const FwdParams &P, const FxTab &X, Shared &S, int T, double u0, int64_t f0, int64_t i0, int nb,
                                 const double *gy, double *ghp, double *ghc, double *w)
 {
@@ -565,7 +564,7 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_proj_adj(FwdPa
         const int j0 = umax - S.mmax;   // row of the first link sample that output 0 gathers from
         int eg = 0;
         unsigned vmax;
-        bool bad = !range_ok(S.st, 1, NY / 32, KW, X.range_adj, &vmax, &eg);
+        bool bad = !range_ok<0>(S.st, 1, NY, KW, X.range_adj, &vmax, &eg);
         bad |= S.bad || nks * 16 > 64 || j0 < 0 || j0 + nb + KW - 1 > NY;
         double out[4] = {0.0, 0.0, 0.0, 0.0};
         for (int sg = 0; sg < nseg && !bad; ++sg) {
@@ -936,8 +935,8 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_sky_adj(FwdPar
             int ex = 0, eg = 0;
             if (!bad && work) {
                 unsigned hmax, gmax;
-                bad = !range_ok(S.st, 1, NSTR, KW, RANGE_SKY, &hmax, &ex);
-                bad |= !range_ok(S.st + 1, 1, NY / 32, KW, RANGE_SKY, &gmax, &eg);
+                bad = !range_ok<0>(S.st, 1, WL, KW, RANGE_SKY, &hmax, &ex);
+                bad |= !range_ok<0>(S.st + 1, 1, nb, KW, RANGE_SKY, &gmax, &eg);
                 eg += (gmax & 0xfffff) >= 0xfa000;   // the top byte's range is 127.5 / 128 of the scale
             }
             if (!bad && work) {
