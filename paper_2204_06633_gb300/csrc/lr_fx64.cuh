@@ -280,6 +280,15 @@ __device__ __forceinline__ double read_scalar(const Shared &S, int T, const doub
 }
 
 // ---------------------------------------------------------------- positions of the reads
+// whole part of a read's position, kept where differences of two fit an int: positions run away where an orbit's
+// end pieces are continued far outside its knots, and the blocks there are sent to the sample form
+constexpr int STENCIL_FAR = 1 << 28;
+__device__ __forceinline__ int stencil_at(double u)
+{
+    const int m = (int)floor(u);
+    return m < -STENCIL_FAR ? -STENCIL_FAR : m > STENCIL_FAR ? STENCIL_FAR : m;
+}
+
 __device__ __forceinline__ const Coef4 *piece_row(const OrbitDev &o, int k) { return reinterpret_cast<const Coef4 *>(o.coef) + (size_t)k * NSERIES; }
 
 // spline piece of time t and the coordinate within it; forced >= 0: that piece, continued
@@ -518,7 +527,7 @@ __device__ void projection_segments(const FwdParams &P, const FxTab &X, Shared &
             for (int i = 0; i < 3; ++i) {
                 const int rd = i == 0 ? s : 3 + c_by_emitter[s][i - 1];
                 const double fl = floor(u[i]);
-                S.mg[g][rd] = (int)fl;
+                S.mg[g][rd] = stencil_at(fl);
                 S.fg[g][rd] = (float)(u[i] - fl);
             }
         } else {
@@ -556,7 +565,7 @@ __device__ void projection_segments(const FwdParams &P, const FxTab &X, Shared &
         const int j = g * GP + lane + 1;   // rows g GP + 1 .. (g + 1) GP against the row before
         int piece;
         const double u = read_pos(P, X, S.skc, u0, t_lo + (double)j * P.dt, rd < 9 ? rd : 0, &piece);
-        const int m = rd < 9 ? (int)floor(u) : piece;
+        const int m = rd < 9 ? stencil_at(u) : piece;
         const int prev = __shfl_up_sync(0xffffffffu, m, 1);
         if (m != (lane ? prev : S.mg[g][rd]) && j < NY) atomicOr(&S.brk[j >> 5], 1u << (j & 31));
     }
@@ -570,12 +579,13 @@ __device__ void projection_segments(const FwdParams &P, const FxTab &X, Shared &
         if (sg) {
             int piece;
             const double u = read_pos(P, X, S.skc, u0, t_lo + (double)S.segj[sg] * P.dt, rd < 9 ? rd : 0, &piece);
-            m = rd < 9 ? (int)floor(u) : piece;
+            m = rd < 9 ? stencil_at(u) : piece;
         }
         S.segm[sg][rd] = m;
         if (rd < 9) {
             atomicMin(&S.mmin, m);
             atomicMax(&S.mmax, m);
+            if (m <= -STENCIL_FAR || m >= STENCIL_FAR) S.bad = 1;
         }
     }
     __syncthreads();
@@ -794,7 +804,7 @@ __device__ void find_tdi_segments(const FwdParams &P, Shared &S, double t_lo, in
         for (int q = 1; q <= qn; ++q) {
             D += S.lg[g][c_tdifx.pair[cc >> 1][cc & 1][q]];
             const double fl = floor(-D);
-            S.mgt[g][cc * 7 + q - 1] = (int)fl;
+            S.mgt[g][cc * 7 + q - 1] = stencil_at(fl);
             S.fgt[g][cc * 7 + q - 1] = (float)(-D - fl);
         }
     }
@@ -823,7 +833,7 @@ __device__ void find_tdi_segments(const FwdParams &P, Shared &S, double t_lo, in
             const int j = g * GT + c + (int)lane;
             int piece;
             const double D = chain_delay(P, t_lo + (double)j * P.dt, tm < NTERM ? tm : 0, &piece);
-            const int m = tm < NTERM ? (int)floor(-D) : piece;
+            const int m = tm < NTERM ? stencil_at(-D) : piece;
             int prev = __shfl_up_sync(0xffffffffu, m, 1);
             if (lane == 0) prev = c ? last : m;
             last = __shfl_sync(0xffffffffu, m, 31);
@@ -838,7 +848,7 @@ __device__ void find_tdi_segments(const FwdParams &P, Shared &S, double t_lo, in
         const int sg = i / (NTERM + 1), tm = i % (NTERM + 1);
         int piece;
         const double D = chain_delay(P, t_lo + (double)S.segj[sg] * P.dt, tm < NTERM ? tm : 0, &piece);
-        const int m = tm < NTERM ? (int)floor(-D) : piece;
+        const int m = tm < NTERM ? stencil_at(-D) : piece;
         S.segm[sg][tm] = m;
         if (tm < NTERM && tm % 7 < qn) {
             atomicMin(&S.mmin, m);

@@ -532,7 +532,8 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_proj_adj(FwdPa
         if (tid < 9) {
             int piece;
             const double u = read_pos(P, X, S.skc, u0, P.t0 + (double)(i0 + nb / 2 - f0) * P.dt, tid, &piece);
-            atomicMax(&umax, (int)floor(u + 0.25));
+            const int m = stencil_at(u + 0.25);   // beyond the plan's bounds: a window that holds no tile
+            atomicMax(&umax, m > P.sig_b + 2 || m < -P.sig_b - P.lproj_b - 2 ? STENCIL_FAR : m);
         }
         __syncthreads();
         const int64_t k_lo = i0 - f0 - umax - (h + 1);
@@ -555,17 +556,18 @@ __global__ void __launch_bounds__(NTHR, NTHR == 256 ? 2 : 1) k_fx_proj_adj(FwdPa
             if (lane == 0) S.st[0][j >> 5] = w;
         }
         double *ghp = B.g_hp + (S.ti.hp - P.hp), *ghc = B.g_hc + (S.ti.hp - P.hp);
-        if (!__syncthreads_or(any)) {
+        const int nseg = S.nseg, KW = S.mmax - S.mmin + T, nks = (KW + 3 + 15) / 16;
+        const int j0 = umax - S.mmax;   // row of the first link sample that output 0 gathers from
+        const bool lost = j0 < 0 || j0 + nb + KW - 1 > NY;   // link samples outside the rows may land on the tile
+        if (!__syncthreads_or(any) && !lost) {
             for (int i = tid; i < nb; i += blockDim.x) ghp[i0 + i] = ghc[i0 + i] = 0.0;
             __syncthreads();
             continue;
         }
-        const int nseg = S.nseg, KW = S.mmax - S.mmin + T, nks = (KW + 3 + 15) / 16;
-        const int j0 = umax - S.mmax;   // row of the first link sample that output 0 gathers from
         int eg = 0;
         unsigned vmax;
         bool bad = !range_ok<0>(S.st, 1, NY, KW, X.range_adj, &vmax, &eg);
-        bad |= S.bad || nks * 16 > 64 || j0 < 0 || j0 + nb + KW - 1 > NY;
+        bad |= S.bad || nks * 16 > 64 || lost;
         double out[4] = {0.0, 0.0, 0.0, 0.0};
         for (int sg = 0; sg < nseg && !bad; ++sg) {
             if (!projection_stencils<true>(P, X, S, T, t_lo, u0, sg, KW, W, wn)) {

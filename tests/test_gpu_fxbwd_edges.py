@@ -168,3 +168,23 @@ def test_blocks_evaluated_sample_by_sample(ctx, flex, p, N, gen):
     for a, b in zip(got, (rp, rc)):
         assert np.linalg.norm(a - b) <= 1e-12 * np.linalg.norm(b)
     assert np.all(np.abs(got[2] - rs) <= np.maximum(1e-11 * np.abs(rs), 4 * (p + 17) * 2.0 ** -53 * scale))
+
+
+@pytest.mark.parametrize("precision", [lr.FP64, lr.MIXED])
+def test_positions_beyond_every_window(ctx, flex, precision):
+    """Outputs 10^11 s past the knots, where the continued end pieces put the reads 10^13 samples away: recorded as
+    reads outside the plan's bounds, and the next call is as ever."""
+    N, p = 700, 11
+    src = synth.draw_sources(1, seed=4)[0]
+    t0h, hp, hc = synth.gb_input(src, T0, DT, N, p)
+    g = np.random.default_rng(1).normal(size=(3, N))
+    plan = lr.Plan(ctx, p, N, DT, flex.gpu, t0=T0 + 1e11, precision=precision)
+    calls = [lambda: plan.backward(dev(hp), dev(hc), t0h + 1e11, sky(src), dev(g))]
+    if precision == lr.FP64:   # of a mixed plan only the adjoint is on these kernels
+        calls.append(lambda: plan.response(dev(hp), dev(hc), t0h + 1e11, sky(src)))
+    for call in calls:
+        call()
+        with pytest.raises(lr.LRError) as e:
+            plan.check()
+        assert e.value.status == 8   # LR_ERR_DEVICE
+    check(ctx, flex, N, p, src, g, precision=precision)
