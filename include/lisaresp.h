@@ -32,13 +32,30 @@
  *   - Array arguments of compute calls are DEVICE pointers owned by the caller (float64,
  *     contiguous), unless documented as host.  The library never frees or keeps them.
  *   - The library allocates only its own tables (orbit spline coefficients, plan tables,
- *     batch tile tables, the device error word) and frees them in the *_destroy calls.
+ *     batch tile tables, the device error word) and frees them in the *_destroy calls.  An FP64
+ *     plan on the tensor-core kernels holds a table of TDI stencils, 576 (order + 2 + the longest
+ *     chained delay in samples) bytes per spline piece of the TDI orbit (11 to 28 KB at orders 11 to
+ *     41 and dt = 10 s, 6 MB for a year of 1e5 s pieces at order 25); a mixed plan the same from its
+ *     first adjoint on.  Orbits of more than 4096 pieces get none, and a plan that cannot allocate it works
+ *     without.
  *   - Compute calls are asynchronous on `stream` (a cudaStream_t passed as void*, NULL =
  *     legacy default stream) and return after enqueueing.  Argument and range checks happen
  *     on the host before any launch.  Device-side faults the kernels detect (a stencil index
  *     outside its staged window, a bounded wait that ran out) are recorded in the plan's
  *     error word and reported by lr_plan_check().
  *   - Handles are not thread-safe: use one plan per host thread / stream.
+ *
+ * Accuracy
+ *   - FP64 plans with summed or constant delays, and the adjoint of mixed ones, evaluate blocks of
+ *     up to 512 samples in fixed point, 2^-55 of the largest value that the block reads.  A block is
+ *     taken this way only while every output's own reads come within a few binary orders of that
+ *     value (3 for the strain, 4 to 5 for the links of a TDI channel, 5 for cotangents; 12 in mixed
+ *     plans and in the sum of the sky gradient); other blocks are evaluated sample by sample in FP64,
+ *     in 5 to 40 times the time.  A quiet output beside a stretch 2^k louder is as far from
+ *     the exact result as the sample-by-sample evaluation up to k = 3, at most 1.8 times as far at
+ *     k = 4, and 3.4 times for lr_tdi alone at k = 5.
+ *   - The same holds for blocks in which the weights or the geometry turn too fast: a source within
+ *     about 0.02 rad of an arm's direction, orbits several times faster than LISA's.
  *
  * Errors: every call returns an lr_status; no exception crosses the ABI.
  */
@@ -97,8 +114,10 @@ typedef struct {
     const lr_orbit *tdi_orbit;   /* delays used by TDI; may differ (hybrid templates) */
     int tile;             /* output samples per CTA tile; 0 = default.  Mixed plans stage a tile in
                              fixed shared-memory arrays: at most 340 outputs at order 25 and dt =
-                             10 s (less for longer TDI halos); a larger tile is LR_ERR_RANGE */
-    int threads;          /* threads per CTA; 0 = default */
+                             10 s (less for longer TDI halos); a larger tile is LR_ERR_RANGE.  FP64 plans
+                             on the tensor-core kernels work a tile in equal blocks of 128 to 500 outputs */
+    int threads;          /* threads per CTA of the sample-by-sample FP64 kernels; 0 = default.  The other
+                             kernels choose their own */
 } lr_plan_desc;
 
 /* ------------------------------------------------------------------ misc */
@@ -197,8 +216,8 @@ LR_API int lr_response_batched(lr_plan *plan, int64_t S, const int64_t *h_off, c
                                double *xyz, void *stream);
 /* Batched forward on HOST buffers: the same arguments and results as lr_response_batched, but
  * h_off, out_off, t0_h, sky, hp, hc and xyz are host arrays (h_off[0] = out_off[0] = 0, both
- * non-decreasing).  The batch is cut into chunks of whole sources (about 2^25 outputs each) and
- * (LR_PIPELINE_CHUNK_OUTPUTS in the environment overrides the chunk size)
+ * non-decreasing).  The batch is cut into chunks of whole sources (about an eighth of the outputs
+ * each, at least 2^18 and at most 2^25; LR_PIPELINE_CHUNK_OUTPUTS in the environment overrides that) and
  * the copy-in of one chunk, the fused kernel on the previous one and the copy-out of the one
  * before run concurrently on three library streams, in two plan-owned device slots (allocated on
  * first use and grown when a larger chunk arrives; freed with the plan).  Work queued earlier on
@@ -278,9 +297,12 @@ LR_API int lr_response_batched_noalloc(lr_plan *plan, int64_t S, const int64_t *
  * read from arrays: the fused kernels compute the strain window each tile reads directly from the
  * parameters (lr_gb), on the output grid t0 + i dt at every index i (no zero extension: the
  * waveform exists at all times), so no strain crosses HBM.  The phase is formed in double-double
- * and reduced modulo one cycle before the FP64 sincos (a few 1e-16 rad at any t and f0).
+ * and reduced modulo one cycle before the FP64 sincos (a few 1e-16 rad at any t and f0).  Mixed plans
+ * form it so for every 32nd sample and rotate from there, with the frequency's drift to first order
+ * (about 2e-16 of h more), unless the drift's second order would matter (fdot above about 6e-16 Hz/s
+ * at dt = 10 s); FP64 plans form it for every sample.
  *
- * h+, hx [n] at t0 + j dt into DEVICE arrays, the same generator as the fused kernels.  Errors:
+ * h+, hx [n] at t0 + j dt into DEVICE arrays, sample by sample as FP64 plans generate it.  Errors:
  * LR_ERR_INVALID_ARG for null pointers or n < 0, LR_ERR_NONFINITE for a non-finite parameter. */
 LR_API int lr_gb_polarisations(const lr_gb *gb /* HOST */, double t0, double dt, int64_t n, double *hp, double *hc,
                                void *stream);

@@ -4,7 +4,7 @@
 // index split is exact integer work on 64-bit fixed point (44 fractional bits).
 //
 // They serve the mixed plans that the tensor-core kernels of lr_fxbwd.cu do not take: varying nested delays, merged
-// stencils of more than 64 taps, no table of TDI stencils.  One year at order 41: 30.3 ms for the three kernels here,
+// stencils of more than 64 taps, fast orbits, close knots, no table of TDI stencils.  One year at order 41: 30.3 ms for the three kernels here,
 // 12.4 there.
 //
 // Structure as the FP64 kernels (lr_bwd.cu): deterministic gathers over inverted tap windows.

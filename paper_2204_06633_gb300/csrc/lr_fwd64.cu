@@ -8,7 +8,8 @@
 //
 // Most FP64 plans run the tensor-core kernel of lr_fx64.cu instead (one year at order 25: 44.45 against 3.4 to
 // 4.0 ms).  These kernels remain for the plans that it does not take: nested delays that vary, sampling steps so
-// short that the merged stencils pass 64 taps, and tiles asked for that no block of 128 outputs or more divides.
+// short that the merged stencils pass 64 taps, orbits several times faster than LISA's or with knots closer than an
+// eighth of a block, and tiles asked for that no block of 128 outputs or more divides.
 #include <cuda_runtime.h>
 
 #include "lr_device.cuh"

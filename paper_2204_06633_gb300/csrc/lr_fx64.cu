@@ -16,9 +16,12 @@
 //      truncation is below 2^-54 of W for drifts of 1e-4 samples per sample (v/c of the orbit);
 //   3. the b_q and the staged series are 56-bit fixed point in seven balanced base-256 digits, each digit
 //      exact in half precision, and A_{q,L}[j] = sum_c sum_{i+k=L} digit_i(b_q)[c] digit_k(h)[j + c], L = 0..6,
-//      is accumulated in FP32: products are at most 2^14 and fewer than 2^10 of them meet in the levels
-//      below 5, so those sums are exact integers; level 6 carries level 7 (each series digit extended by
-//      the next one to 11 bits), which keeps the products left out below 2^-56;
+//      is accumulated in FP32 (slices of an exact product on low-precision units, as in Ozaki's scheme):
+//      products are at most 2^14, 5 taps x links of them meet at level 4, which is 290 in the projection,
+//      1140 in TDI, 1254 and 1360 in the adjoint's K2 and K3.  Sums below 2^24 are exact integers; to pass it
+//      three quarters of 1360 digit pairs would have to be at the end of their range with agreeing signs (digits
+//      of either sign sum to less than 2^20).  Level 6 carries level 7 (each series digit extended by the
+//      next one to 11 bits), which keeps the products left out below 2^-56;
 //   4. sum_q A_q T_q(nu) is Clenshaw's recurrence in 64-bit integers: nu is a multiple of 2^-9, so each
 //      step is a small integer product and a shift.
 // The digits that a higher q cannot have (|b_q| falls by ~2^-7 per order) are left out: 121 of 224 digit

@@ -711,8 +711,11 @@ __device__ __forceinline__ void sky_terms(const FwdParams &P, const SkyConst &K,
 // have to fall as the digits assume and the first one left out has to be small.  Orders of the coefficient relative
 // to `scale`; those of the weights by those of sinc: with a drift of +-delta samples over the block the j-th is
 // at most 2 (pi delta / 2)^j / (j! (j + 1)).  Checked against the exact terms of single blocks (a 3 mHz source, order
-// 25): the bound of order 8 is 7e-15 for sources far from the arms, 1e-11 at 0.01 rad from one, where the terms are
-// 9e-12 off, 1.6e-9 at 5e-3 (1e-9), 5e-4 at 1e-3 (2e-4).
+// 25): the bound of order 8 is 1e-11 at 0.01 rad from an arm, where the terms are 9e-12 off, 1.6e-9 at 5e-3 (1e-9),
+// 5e-4 at 1e-3 (2e-4).  Far from the arms it is rounding: an arm's direction is the difference of positions sixty
+// times its length, and the bound of 4000 random blocks is 6e-15 in the middle and 7e-14 at most.  A limit of 3e-14
+// sent one block in a hundred to the sample form, and most launches waited for one (a year at order 41: 12.1 to
+// 13.2 ms in one source's case).
 __device__ __forceinline__ bool sky_series_fits(const FxTab &X, const double *g, int stride, float scale, float delta)
 {
     double e[NN / 2], o[NN / 2];
@@ -750,7 +753,7 @@ __device__ __forceinline__ bool sky_series_fits(const FxTab &X, const double *g,
             // the coefficient's own next order, from the decay over its last two pairs
             const float last = fmaxf(c[NN - 1], c[NN - 2]), before = fmaxf(c[NN - 3], c[NN - 4]);
             p += last <= before ? last * (last / fmaxf(before, 1e-30f)) : last;
-            ok &= p <= 2.8e-14f;   // 2^-45
+            ok &= p <= 4.5e-13f;   // 2^-41: a source within about 0.016 rad of an arm
         }
     }
     return ok;   // false for NaN
