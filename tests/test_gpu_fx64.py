@@ -182,3 +182,15 @@ def test_quiet_channel_beside_loud_links(ctx, flex, k):
         err.append(np.linalg.norm(host(plan.tdi(dev(y)))[0] - ref))
         plan.check()
     assert err[0] <= 4.0 * err[1], err
+
+
+@pytest.mark.parametrize("spacing,pieces", [(1500.0, 60), (6000.0, 4100)])
+def test_close_and_very_many_knots(ctx, spacing, pieces):
+    """Blocks over three and four spline pieces, which the stencil table does not serve, and an orbit of more pieces
+    than a table is made for."""
+    N, p = 3000, 25
+    tk = -2e4 + spacing * np.arange(pieces + 1)
+    pair = Pair(ctx, synth.Orbit(tk, synth.keplerian_flexing(tk), None))
+    src = dataclasses.replace(synth.draw_sources(1, seed=4)[0], f=3e-3)
+    for kind in ("response", "tdi"):
+        run_case(ctx, src, N, p, pair, kind=kind)

@@ -188,3 +188,14 @@ def test_positions_beyond_every_window(ctx, flex, precision):
             plan.check()
         assert e.value.status == 8   # LR_ERR_DEVICE
     check(ctx, flex, N, p, src, g, precision=precision)
+
+
+@pytest.mark.parametrize("spacing,pieces", [(1500.0, 60), (6000.0, 4100)])
+def test_knots_off_the_stencil_table(ctx, spacing, pieces):
+    """Blocks over three and four spline pieces; an orbit of more pieces than a stencil table is made for, whose
+    adjoint stays on the sample kernels."""
+    N, p = 1500, 25
+    tk = -2e4 + spacing * np.arange(pieces + 1)
+    pair = Pair(ctx, synth.Orbit(tk, synth.keplerian_flexing(tk), None))
+    src = dataclasses.replace(synth.draw_sources(1, seed=4)[0], f=3e-3)
+    check(ctx, pair, N, p, src, np.random.default_rng(8).normal(size=(3, N)))
