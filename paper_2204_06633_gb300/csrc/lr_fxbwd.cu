@@ -168,7 +168,7 @@ __device__ void tdi_adj_scalar(const FwdParams &P, Shared &S, int T, int64_t k0,
                 const int cc = (t + tid / CR) / qn, q = (t + tid / CR) % qn + 1, j = tid % CR;
                 double D = 0.0;
                 for (int k = 1; k <= q; ++k) D += L[c_tdifx.pair[cc >> 1][cc & 1][k] * CR + j];
-                const int m = (int)floor(-D), a = __reduce_min_sync(0xffffffffu, m), b = __reduce_max_sync(0xffffffffu, m);
+                const int m = stencil_at(-D), a = __reduce_min_sync(0xffffffffu, m), b = __reduce_max_sync(0xffffffffu, m);
                 M[tid] = m;
                 if ((tid & 31) == 0) {
                     lo[tid >> 5] = a;
@@ -401,7 +401,7 @@ __device__ void proj_adj_scalar(const FwdParams &P, const FxTab &X, Shared &S, i
         for (int i = tid; i < 9 * CR; i += blockDim.x) {   // a warp's lanes are of one read
             const int rd = i / CR;
             const double u = U[i];
-            const int m = (int)floor(u);
+            const int m = stencil_at(u);
             M[i] = m;
             const int a = __reduce_min_sync(0xffffffffu, m), b = __reduce_max_sync(0xffffffffu, m);
             if ((tid & 31) == 0) {
